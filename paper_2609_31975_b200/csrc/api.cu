@@ -20,7 +20,23 @@ namespace {
 constexpr int kMaxUpDownGrid = 304;  // upper bound of the up/down grid (2 CTAs per SM on 148 SMs)
 constexpr int kMaxChunk = 4;         // tokens per pass of the general kernels
 constexpr int kMaxSplits = 16;       // union-row splits of the batched down projection
-constexpr int kMaxMmaTokens = 64;    // tokens per pass of the batched tensor-core kernels
+constexpr int kMaxMmaTokens = 64;    // tokens per pass of the mma.sync kernels, and of the tcgen05 ones on int8 limbs
+constexpr int kMaxUmmaTokens = sffn::kUmmaMaxCols;  // tokens per pass of the tcgen05 kernels
+constexpr int kOddWidthMinTokens = 5;  // quantised rows of an odd multiple of 128: batches from here on the tcgen05 kernels
+
+inline int round8(int v) { return (v + 7) & ~7; }
+
+// Row widths that are odd multiples of 128: batches over quantised rows of such widths used to run token by token with h
+// in fp32.  On the tensor cores h enters the down projection there as two bf16 values (16 bits; the tokens' limbs on the
+// single-token route hold fewer: 4e-5 against 2e-6 from the formulas in 64 bits); at the other widths it is one.
+inline int h_terms_for(int D, bool quantised) { return quantised && D % 256 != 0 ? 2 : 1; }
+
+// Most splits of the batched down projection's contraction over `cols` token columns (device-independent bound; what a
+// device uses is umma_down_splits).
+inline int most_splits(int D, int cols) {
+  const int s = (cols <= kMaxMmaTokens ? 2 : 1) * (kMaxUpDownGrid / 2) / (D >= 128 ? D / 128 : 1);
+  return s < 1 ? 1 : s > kMaxSplits ? kMaxSplits : s;
+}
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -45,14 +61,18 @@ Layout make_layout(int D, int H, int r_max, int B_max, int dtype) {
   L.v = take((size_t)B_max * (r_max > 0 ? r_max : 1) * 4);
   L.n = take((size_t)B_max * (r_max > 0 ? r_max : 1) * 4);
   const size_t part_general = (size_t)kMaxUpDownGrid * kMaxChunk * D * 4;
-  const size_t part_batched = (size_t)kMaxSplits * (B_max < kMaxMmaTokens ? B_max : kMaxMmaTokens) * D * 4;
+  const size_t bu = B_max < kMaxUmmaTokens ? B_max : kMaxUmmaTokens;  // tokens of a pass
+  const size_t bu8 = round8((int)bu);
+  const size_t narrow = (size_t)kMaxSplits * (B_max < kMaxMmaTokens ? B_max : kMaxMmaTokens);
+  const size_t wide = (size_t)most_splits(D, kMaxMmaTokens + 1) * bu;
+  const size_t part_batched = (narrow > wide ? narrow : wide) * D * 4;
   L.partial = take(part_general > part_batched ? part_general : part_batched);
   L.xstage = take((size_t)B_max * D * esz);
   L.ystage = take((size_t)B_max * D * 4);
   L.fused = take(sffn::fused_workspace_bytes(D, H, r_max));
   L.hm_stride = (H + 63) / 64 * 64 + 64;
-  L.hmT = take((size_t)(B_max < kMaxMmaTokens ? B_max : kMaxMmaTokens) * L.hm_stride * 2);
-  L.x2 = take((size_t)2 * (B_max < kMaxMmaTokens ? B_max : kMaxMmaTokens) * (r_max > 0 ? r_max : 1) * 2);
+  L.hmT = take(h_terms_for(D, true) * bu8 * L.hm_stride * 2);
+  L.x2 = take(2 * bu8 * (r_max > 0 ? r_max : 1) * 2);
   L.union_flag = take((size_t)H + 256);  // fired flags accumulated over the chunks of a batch of more than 64 tokens
   // int8 rows on the tensor cores: the tokens (and the LoPA vector) as four int8 limbs each, and their scales
   const size_t bt = B_max < kMaxMmaTokens ? B_max : kMaxMmaTokens;
@@ -258,9 +278,9 @@ thread_local int g_last_cuda_line = 0;
     }                                 \
   } while (0)
 
-// Batched tensor-core path (bf16, B >= 2): gate GEMM -> compaction of the union -> up GEMM over the
+// Batched tensor-core path (bf16 tokens, B >= 2): gate GEMM -> compaction of the union -> up GEMM over the
 // union rows -> down GEMM (split over D-slices and union chunks) -> fixed-order sum of the splits.
-// Tokens are taken kMaxMmaTokens at a time; the union (and the list) is that of the whole batch.
+// One pass: at most umma_pass_tokens tokens (64 on the mma.sync kernels); the union (and the list) is that of the pass.
 int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const float* b_g,
                 const void* W_up, const void* W_down, int act, float* y, bool dense, bool umma,
                 const sffn_q8_scales* q8, int qbits, cudaStream_t s) {
@@ -271,7 +291,10 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
   // int8 rows whose K blocks are whole (128 codes): multiplied as int8 against the tokens' int8 limbs, nothing to expand
   // (the down projection keeps the expansion: its B operand, Hm, has no scale known before the whole of it exists)
   // (int4 rows: the nibbles expanded to int8 on the way, for the same MMAs)
-  const bool native = q8 && B <= kMaxMmaTokens && umma_rows_native_i8_supported(D, B) &&
+  // More than 64 tokens (four limbs each: 256 columns) take the expansion to bf16 in all three GEMMs.
+  // Odd multiples of 128 expand as well: bf16 tokens enter exactly, where limbs with one scale per token would cost a token
+  // with an outlier some of what the single-token route, which has a scale per chunk, keeps.
+  const bool native = q8 && D % 256 == 0 && B <= kMaxMmaTokens && umma_rows_native_i8_supported(D, B) &&
                       umma_rows_native_i8_supported(g->kind == SFFN_GATE_LOPA ? g->r : D, B);
   const int wq_rows = native ? (qbits == 8 ? 1 : 2) : wq;
   void* xlimb = h->ws + h->L.xlimb;
@@ -293,19 +316,17 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
   const bool lopa = g->kind == SFFN_GATE_LOPA;
   const int grid_rows = 2 * h->sm_count;
 
+  const int h_terms = h_terms_for(D, q8 != nullptr);
   if (lopa && umma) {  // v = V x on the tensor cores: the rows kernel with the identity as its epilogue
-    for (int b0 = 0; b0 < B; b0 += kMaxMmaTokens) {
-      const int nb = B - b0 < kMaxMmaTokens ? B - b0 : kMaxMmaTokens;
-      UmmaRowsParams p{};
-      p.W = g->V; p.R = g->r; p.K = D;
-      p.qbits = wq_rows; p.w_scale = q8 ? q8->s_V : nullptr;
-      p.X = xb + (size_t)b0 * D * 2; p.x_stride = D; p.ncols_valid = nb; p.B = nb;
-      if (native) { p.X = xlimb; p.ncols_valid = 4 * nb; p.tok_scale = xscale; }
-      p.act = kUmmaActIdentity; p.a_out = vbuf + (size_t)b0 * rs; p.a_stride = rs;
-      p.status = h->at<int32_t>(h->L.status);
-      SFFN_CUDA(launch_umma_rows(false, p, native ? 4 * nb : nb, h->sm_count, s));
-      ++h->launches;
-    }
+    UmmaRowsParams p{};
+    p.W = g->V; p.R = g->r; p.K = D;
+    p.qbits = wq_rows; p.w_scale = q8 ? q8->s_V : nullptr;
+    p.X = xb; p.x_stride = D; p.ncols_valid = B; p.B = B;
+    if (native) { p.X = xlimb; p.ncols_valid = 4 * B; p.tok_scale = xscale; }
+    p.act = kUmmaActIdentity; p.a_out = vbuf; p.a_stride = rs;
+    p.status = h->at<int32_t>(h->L.status);
+    SFFN_CUDA(launch_umma_rows(false, p, native ? 4 * B : B, h->sm_count, s));
+    ++h->launches;
   } else if (lopa) {  // v = V x on the CUDA-core row kernel (r rows only), then RMSNorm
     for (int b0 = 0; b0 < B;) {
       const int nb = B - b0 >= 4 ? 4 : B - b0 >= 2 ? 2 : 1;
@@ -328,67 +349,60 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
   uint32_t* words = reinterpret_cast<uint32_t*>(flag);  // the flag buffer holds either form
   int gate_tile_rows = 0, gate_tiles = 0;
   umma_gate_tiling(H, h->sm_count, &gate_tile_rows, &gate_tiles);
-  for (int b0 = 0; b0 < B; b0 += kMaxMmaTokens) {
-    const int nb = B - b0 < kMaxMmaTokens ? B - b0 : kMaxMmaTokens;
-    void* x2 = h->ws + h->L.x2;
-    const float* nsrc = (g->use_rmsnorm ? nbuf : vbuf) + (size_t)b0 * rs;
-    const void* xtok = xb + (size_t)b0 * D * 2;
-    if (b0 > 0 && !dense) return SFFN_ERR_UNSUPPORTED;  // flags of later chunks would need OR-ing
-    if (umma) {
-      UmmaRowsParams p{};
-      p.R = H; p.B = nb; p.b_g = b_g; p.act = act; p.status = h->at<int32_t>(h->L.status);
-      p.qbits = wq_rows; p.w_scale = q8 ? q8->s_gate : nullptr;
-      p.xtok = xtok; p.xtok_stride = D;
-      p.a_out = actbuf + (size_t)b0 * H; p.a_stride = H;
-      p.flag = (dense || own_list) ? nullptr : flag;
-      p.words_out = own_list ? words : nullptr;
-      int cols = nb;
-      if (lopa && native) {
-        // RMSNorm (or none) and the split into int8 limbs in one launch
-        SFFN_CUDA(launch_rmsnorm_limbs(vbuf + (size_t)b0 * rs, nb, g->r, rs, g->rms_gain, g->rms_eps,
-                                       g->use_rmsnorm != 0, nlimb, nscale, s));
-        ++h->launches;
-        p.W = g->U; p.K = g->r; p.X = nlimb; p.x_stride = g->r; p.tok_scale = nscale;
-        p.g_idx = g->g_idx; p.g_sign = g->g_sign;
-        cols = 4 * nb;
-      } else if (lopa) {
-        // RMSNorm (or none) and the split into bf16 pairs in one launch
-        SFFN_CUDA(launch_rmsnorm_split(vbuf + (size_t)b0 * rs, nb, g->r, rs, g->rms_gain, g->rms_eps,
-                                       g->use_rmsnorm != 0, x2, s));
-        ++h->launches;
-        p.W = g->U; p.K = g->r; p.X = x2; p.x_stride = g->r; p.split_cols = 1;
-        p.g_idx = g->g_idx; p.g_sign = g->g_sign;
-        cols = 2 * nb;
-      } else if (native) {
-        p.W = g->W_g; p.K = D; p.X = xlimb; p.x_stride = D; p.tok_scale = xscale;
-        cols = 4 * nb;
-      } else {
-        p.W = g->W_g; p.K = D; p.X = xtok; p.x_stride = D;
-      }
-      p.ncols_valid = cols;
-      SFFN_CUDA(launch_umma_rows(false, p, cols, h->sm_count, s));
+  void* x2 = h->ws + h->L.x2;
+  if (umma) {
+    UmmaRowsParams p{};
+    p.R = H; p.B = B; p.b_g = b_g; p.act = act; p.status = h->at<int32_t>(h->L.status);
+    p.qbits = wq_rows; p.w_scale = q8 ? q8->s_gate : nullptr;
+    p.xtok = x; p.xtok_stride = D;
+    p.a_out = actbuf; p.a_stride = H;
+    p.flag = (dense || own_list) ? nullptr : flag;
+    p.words_out = own_list ? words : nullptr;
+    int cols = B;
+    if (lopa && native) {
+      // RMSNorm (or none) and the split into int8 limbs in one launch
+      SFFN_CUDA(launch_rmsnorm_limbs(vbuf, B, g->r, rs, g->rms_gain, g->rms_eps, g->use_rmsnorm != 0, nlimb, nscale, s));
+      ++h->launches;
+      p.W = g->U; p.K = g->r; p.X = nlimb; p.x_stride = g->r; p.tok_scale = nscale;
+      p.g_idx = g->g_idx; p.g_sign = g->g_sign;
+      cols = 4 * B;
+    } else if (lopa) {
+      // RMSNorm (or none) and the split into bf16 pairs in one launch
+      p.x_cols = round8(B);
+      SFFN_CUDA(launch_rmsnorm_split(vbuf, B, g->r, rs, g->rms_gain, g->rms_eps, g->use_rmsnorm != 0, p.x_cols, x2, s));
+      ++h->launches;
+      p.W = g->U; p.K = g->r; p.X = x2; p.x_stride = g->r;
+      p.g_idx = g->g_idx; p.g_sign = g->g_sign;
+      cols = 2 * p.x_cols;
+    } else if (native) {
+      p.W = g->W_g; p.K = D; p.X = xlimb; p.x_stride = D; p.tok_scale = xscale;
+      cols = 4 * B;
     } else {
-      RowsMmaParams p{};
-      p.status = h->at<int32_t>(h->L.status);
-      p.R = H; p.B = nb; p.b_g = b_g; p.act = act;
-      p.xtok = xtok; p.xtok_stride = D;
-      p.a_out = actbuf + (size_t)b0 * H; p.a_stride = H;
-      p.flag = dense ? nullptr : flag;
-      int cols = nb;
-      if (lopa) {
-        SFFN_CUDA(launch_split_bf16(nsrc, nb, g->r, rs, x2, s));
-        ++h->launches;
-        p.W = g->U; p.K = g->r; p.X = x2; p.x_stride = g->r; p.split_cols = 1;
-        p.g_idx = g->g_idx; p.g_sign = g->g_sign;
-        cols = 2 * nb;
-      } else {
-        p.W = g->W_g; p.K = D; p.X = xtok; p.x_stride = D;
-      }
-      p.ncols_valid = cols;
-      SFFN_CUDA(launch_rows_mma(false, p, cols, grid_rows, s));
+      p.W = g->W_g; p.K = D; p.X = x; p.x_stride = D;
     }
-    ++h->launches;
+    p.ncols_valid = cols;
+    SFFN_CUDA(launch_umma_rows(false, p, cols, h->sm_count, s));
+  } else {
+    RowsMmaParams p{};
+    p.status = h->at<int32_t>(h->L.status);
+    p.R = H; p.B = B; p.b_g = b_g; p.act = act;
+    p.xtok = x; p.xtok_stride = D;
+    p.a_out = actbuf; p.a_stride = H;
+    p.flag = dense ? nullptr : flag;
+    int cols = B;
+    if (lopa) {
+      SFFN_CUDA(launch_split_bf16(g->use_rmsnorm ? nbuf : vbuf, B, g->r, rs, x2, s));
+      ++h->launches;
+      p.W = g->U; p.K = g->r; p.X = x2; p.x_stride = g->r; p.split_cols = 1;
+      p.g_idx = g->g_idx; p.g_sign = g->g_sign;
+      cols = 2 * B;
+    } else {
+      p.W = g->W_g; p.K = D; p.X = x; p.x_stride = D;
+    }
+    p.ncols_valid = cols;
+    SFFN_CUDA(launch_rows_mma(false, p, cols, grid_rows, s));
   }
+  ++h->launches;
   if (!dense) {
     if (!own_list) {
       SFFN_CUDA(launch_compact(flag, H, idx, count, s));
@@ -396,53 +410,60 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
     }
     h->list_state = 1;
   }
-  int splits = h->sm_count / (D / 256);
-  splits = splits < 1 ? 1 : splits > kMaxSplits ? kMaxSplits : splits;
   float* partial = h->at<float>(h->L.partial);
   void* hmT = h->ws + h->L.hmT;
-  for (int b0 = 0; b0 < B; b0 += kMaxMmaTokens) {
-    const int nb = B - b0 < kMaxMmaTokens ? B - b0 : kMaxMmaTokens;
-    const int32_t* lidx = dense ? nullptr : idx;
-    const int32_t* lcount = dense ? nullptr : count;
-    if (umma) {
-      UmmaRowsParams p{};
-      p.W = W_up; p.R = H; p.K = D;
-      p.qbits = wq_rows; p.w_scale = q8 ? q8->s_up : nullptr; p.out_scale = q8 ? q8->s_down : nullptr;
-      if (own_list) {
-        p.words_in = words; p.n_words = 4 * gate_tiles; p.gate_tile_rows = gate_tile_rows;
-        p.gate_rows_per_word = gate_tile_rows <= 64 ? 16 : 32;
-        p.idx_out = idx; p.count_out = count; p.walk_all = umma_may_walk(nb) ? count + 1 : nullptr;
-      } else {
-        p.idx = lidx; p.count = lcount;
-      }
-      p.X = xb + (size_t)b0 * D * 2; p.x_stride = D; p.ncols_valid = nb; p.B = nb;
-      if (native) { p.X = xlimb; p.ncols_valid = 4 * nb; p.tok_scale = xscale; }
-      p.a = actbuf + (size_t)b0 * H; p.a_stride = H;
-      p.hmT = hmT; p.hm_stride = h->L.hm_stride; p.status = h->at<int32_t>(h->L.status);
-      p.act_up = h->act_up;
-      SFFN_CUDA(launch_umma_rows(true, p, native ? 4 * nb : nb, h->sm_count, s));
+  const int32_t* lidx = dense ? nullptr : idx;
+  const int32_t* lcount = dense ? nullptr : count;
+  const int h_cols = round8(B);
+  if (umma) {
+    UmmaRowsParams p{};
+    p.W = W_up; p.R = H; p.K = D;
+    p.qbits = wq_rows; p.w_scale = q8 ? q8->s_up : nullptr; p.out_scale = q8 ? q8->s_down : nullptr;
+    if (own_list) {
+      p.words_in = words; p.n_words = 4 * gate_tiles; p.gate_tile_rows = gate_tile_rows;
+      p.gate_rows_per_word = gate_tile_rows <= 64 ? 16 : 32;
+      p.idx_out = idx; p.count_out = count; p.walk_all = umma_may_walk(B) ? count + 1 : nullptr;
     } else {
-      RowsMmaParams p{};
-      p.status = h->at<int32_t>(h->L.status);
-      p.W = W_up; p.R = H; p.K = D; p.idx = lidx; p.count = lcount;
-      p.X = xb + (size_t)b0 * D * 2; p.x_stride = D; p.ncols_valid = nb; p.B = nb;
-      p.a = actbuf + (size_t)b0 * H; p.a_stride = H;
-      p.hmT = hmT; p.hm_stride = h->L.hm_stride;
-      p.act_up = h->act_up;
-      SFFN_CUDA(launch_rows_mma(true, p, nb, grid_rows, s));
+      p.idx = lidx; p.count = lcount;
     }
-    int nsplit = splits;
-    if (q8 && !umma_down_supported(D, nb)) return SFFN_ERR_UNSUPPORTED;
-    if (umma && umma_down_supported(D, nb)) {
+    p.X = x; p.x_stride = D; p.ncols_valid = B; p.B = B;
+    if (native) { p.X = xlimb; p.ncols_valid = 4 * B; p.tok_scale = xscale; }
+    p.a = actbuf; p.a_stride = H;
+    p.hmT = hmT; p.hm_stride = h->L.hm_stride; p.h_terms = h_terms; p.h_cols = h_cols;
+    p.status = h->at<int32_t>(h->L.status);
+    p.act_up = h->act_up;
+    SFFN_CUDA(launch_umma_rows(true, p, native ? 4 * B : B, h->sm_count, s));
+  } else {
+    RowsMmaParams p{};
+    p.status = h->at<int32_t>(h->L.status);
+    p.W = W_up; p.R = H; p.K = D; p.idx = lidx; p.count = lcount;
+    p.X = x; p.x_stride = D; p.ncols_valid = B; p.B = B;
+    p.a = actbuf; p.a_stride = H;
+    p.hmT = hmT; p.hm_stride = h->L.hm_stride;
+    p.act_up = h->act_up;
+    SFFN_CUDA(launch_rows_mma(true, p, B, grid_rows, s));
+  }
+  ++h->launches;
+  // the down projection: all tokens at once, or (h in several terms) as many as its 256 columns hold
+  const int down_max = umma ? kUmmaMaxCols / h_terms / 8 * 8 : B;
+  for (int b0 = 0; b0 < B; b0 += down_max) {
+    const int nb = B - b0 < down_max ? B - b0 : down_max;
+    int splits;
+    if (umma) {
       UmmaDownParams d{};
       d.W_down = W_down; d.R = H; d.D = D; d.qbits = wq;
       d.idx = lidx; d.count = lcount;
-      d.hmT = hmT; d.hm_stride = h->L.hm_stride; d.B = nb;
-      d.splits = nsplit = umma_down_splits(D, h->sm_count, kMaxSplits);
-      d.walk_all = (own_list && umma_may_walk(nb)) ? count + 1 : nullptr;
+      d.hmT = hmT; d.hm_stride = h->L.hm_stride; d.terms = h_terms; d.h_cols = h_cols;
+      d.tok0 = b0; d.B = nb; d.cols = round8(nb);
+      // (the workspace holds most_splits() partials of nb tokens; the first argument bounds what the SMs can use)
+      const int cap = nb <= kMaxMmaTokens ? kMaxSplits : most_splits(D, nb);
+      d.splits = splits = umma_down_splits(D, h_terms * d.cols, h->sm_count, cap);
+      d.walk_all = (own_list && umma_may_walk(B)) ? count + 1 : nullptr;
       d.partial = partial; d.status = h->at<int32_t>(h->L.status);
       SFFN_CUDA(launch_umma_down(d, s));
     } else {
+      splits = h->sm_count / (D / 256);
+      splits = splits < 1 ? 1 : splits > kMaxSplits ? kMaxSplits : splits;
       DownMmaParams d{};
       d.status = h->at<int32_t>(h->L.status);
       d.W_down = W_down; d.R = H; d.D = D;
@@ -451,11 +472,15 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
       d.partial = partial;
       SFFN_CUDA(launch_down_mma(d, splits, s));
     }
-    SFFN_CUDA(launch_reduce(partial, nsplit, nb, D, y + (size_t)b0 * D, D, s));
-    h->launches += 3;
+    SFFN_CUDA(launch_reduce(partial, splits, nb, D, y + (size_t)b0 * D, D, s));
+    h->launches += 2;
   }
   return SFFN_OK;
 }
+
+// Tokens that one pass of the tcgen05 kernels takes: 256 columns of the gate GEMM's token operand, which the LoPA
+// vector's high and low parts share.
+int umma_pass_tokens(bool lopa) { return lopa ? kMaxUmmaTokens / 2 : kMaxUmmaTokens; }
 
 // General path: gate (all tokens, chunks of <= 4) -> compaction -> up/down + reduce per chunk.
 int run_general(sffn_handle* h, const void* x, int B, const sffn_gate* g, const float* b_g,
@@ -564,15 +589,20 @@ int run(sffn_handle* h, const void* x, int B, const sffn_gate* g, const float* b
   const int wkind = q8 ? (qbits == 4 ? sffn::kWQ4 : sffn::kWQ8) : h->dtype == SFFN_BF16 ? sffn::kWBF16 : sffn::kWF32;
   const bool lopa_gate = g->kind == SFFN_GATE_LOPA;
   const int gate_k = lopa_gate ? g->r : h->D;
-  const int chunk = B < kMaxMmaTokens ? B : kMaxMmaTokens;
-  // a batch the tensor-core kernels can take (bf16 tokens; bf16, int8 or int4 rows; more than 64 tokens: in chunks of 64)
-  const int gate_cols_chunk = lopa_gate ? 2 * chunk : chunk;
-  // rows of weight codes: the tcgen05 kernels only (they expand the codes to bf16 on the way to the tensor cores)
-  const bool q_tensor_ok = !q8 || (h->path != SFFN_PATH_MMA_SYNC && sffn::umma_rows_supported(gate_k, gate_cols_chunk) &&
-                                   sffn::umma_rows_supported(h->D, chunk) && sffn::umma_down_supported(h->D, chunk) &&
-                                   (!lopa_gate || sffn::umma_rows_supported(h->D, chunk)));
-  const bool tensor_batch = h->dtype == SFFN_BF16 && B >= 2 && h->path != SFFN_PATH_GENERAL && q_tensor_ok &&
-                            h->path != SFFN_PATH_FUSED && sffn::batched_mma_supported(h->D, gate_k, gate_cols_chunk);
+  // A batch the tensor-core kernels can take: bf16 tokens; bf16, int8 or int4 rows of a multiple of 256 elements, and a
+  // LoPA rank of a multiple of 64 (a standard gate on quantised rows: of 128 elements, see h_terms_for; the other batches
+  // of such widths run in fp32 throughout, which the tensor cores' sums do not match: 2e-6 against 2e-7).  At the odd
+  // widths the tensor cores pay from a few tokens on (int8, 1152 x 3500, B = 3 / 4 / 8: 27 / 28 / 28 us against 28 / 37 /
+  // 73 us token by token; 6528 x 20000: 151 / 157 / 184 against 131 / 175 / 348 us).  Larger batches are cut into passes of as many tokens as one launch chain holds: a
+  // pass reads every gate row and the rows of its own union, so fewer passes read fewer bytes (bf16, 4096 x 14336, 200
+  // tokens: 4 passes of 64 took 333 us).  The mma.sync kernels (selected, or a bf16 LoPA rank that is no multiple of 64)
+  // take passes of 64 and rows of a multiple of 256 elements.
+  const bool umma_ok = h->path != SFFN_PATH_MMA_SYNC && sffn::umma_rows_supported(gate_k, 1) &&
+                       sffn::umma_rows_supported(h->D, 1) && sffn::umma_down_supported(h->D, 1) &&
+                       (h->D % 256 == 0 || (q8 && !lopa_gate && B >= kOddWidthMinTokens));
+  const int pass_max = umma_ok ? umma_pass_tokens(lopa_gate) : kMaxMmaTokens;
+  const bool tensor_batch = h->dtype == SFFN_BF16 && B >= 2 && h->path != SFFN_PATH_GENERAL && h->path != SFFN_PATH_FUSED &&
+                            (umma_ok || (!q8 && sffn::batched_mma_supported(h->D, gate_k, 1)));
   // Any other batch (fp32 operands, a row width the tensor-core kernels do not tile, SFFN_PATH_FUSED): the single-token
   // kernel once per token, where it serves the shape.  The CUDA-core batch kernels are slower than B single-token calls
   // (int8, 4096 x 14336, B = 16: 1.66 ms against 0.33 ms; bf16 rows of 4000 elements: 1.03 ms against 0.46 ms; fp32:
@@ -625,16 +655,14 @@ int run(sffn_handle* h, const void* x, int B, const sffn_gate* g, const float* b
     return SFFN_OK;
   }
   if (tensor_batch) {
-    // chunks of at most 64 tokens; with more than one chunk the fired sets are accumulated into the batch's union
+    // with more than one pass the fired sets are accumulated into the batch's union
     uint8_t* uni = h->at<uint8_t>(h->L.union_flag);
-    const bool parts = B > kMaxMmaTokens;
+    const bool parts = B > pass_max;
     if (parts && !dense) SFFN_CUDA(cudaMemsetAsync(uni, 0, h->H, s));
-    for (int b0 = 0; b0 < B; b0 += kMaxMmaTokens) {
-      const int nb = B - b0 < kMaxMmaTokens ? B - b0 : kMaxMmaTokens;
-      const int cols = lopa_gate ? 2 * nb : nb;
-      const bool umma_ok = sffn::umma_rows_supported(gate_k, cols) && sffn::umma_rows_supported(h->D, nb);
+    for (int b0 = 0; b0 < B; b0 += pass_max) {
+      const int nb = B - b0 < pass_max ? B - b0 : pass_max;
       const int rc2 = run_batched(h, static_cast<const char*>(x) + (size_t)b0 * h->D * 2, nb, g, b_g, W_up, W_down, act,
-                                  y + (size_t)b0 * h->D, dense, umma_ok && h->path != SFFN_PATH_MMA_SYNC, q8, qbits, s);
+                                  y + (size_t)b0 * h->D, dense, umma_ok, q8, qbits, s);
       if (rc2 != SFFN_OK) return rc2;
       if (parts && !dense) {
         SFFN_CUDA(sffn::launch_mark_union(h->at<int32_t>(h->L.idx), h->at<int32_t>(h->L.status) + 1, h->H, uni, s));

@@ -32,6 +32,10 @@
 // down projection's are folded into Hm).  With the weights as the A operand the tensor core takes 32 bytes of
 // bf16 per cycle and SM whatever the token count, i.e. 16 codes per cycle: quantised batches are bound by that
 // rate, not by their bytes.
+// Up to 256 token columns go through in one pass.  Wide batches (npad > 128) leave room for two accumulators and a ring
+// of four stages of ~40 KB; they are bound by the token rows every CTA reads again (200 tokens x 4096: 1.6 MB a CTA
+// through L2 beside 0.8 MB of weights), still far cheaper than further passes over the weights (200 tokens, 4096 x
+// 14336, bf16: 135 us in one pass against 333 us in four of at most 64).
 // Every wait is bounded by a cycle budget; on expiry the status word is set, all roles wind down and the TMEM
 // columns are released before the CTA exits.
 #include "umma_kernels.cuh"
@@ -606,6 +610,12 @@ __global__ void __launch_bounds__(kThreadsRows + ((QB == 8 || QB == 4 || QB == 2
     }
     if (!okw) return false;
     tc_fence_after();
+    // h of one (neuron, token): one bf16 value, or (quantised rows of some widths) two that add up to 16 bits of it
+    auto store_h = [&](__nv_bfloat16* dst, float h) {
+      const __nv_bfloat16 t = __float2bfloat16(h);
+      *dst = t;
+      if (kQ && p.h_terms == 2) dst[(size_t)p.h_cols * p.hm_stride] = __float2bfloat16(h - __bfloat162float(t));
+    };
     if constexpr (kNat) {
       // int32 accumulators, four columns per token (its limbs, most significant first, 7 bits apart):
       // value = token scale * row scale * (i0 + i1 / 128 + i2 / 128^2 + i3 / 128^3)
@@ -651,41 +661,32 @@ __global__ void __launch_bounds__(kThreadsRows + ((QB == 8 || QB == 4 || QB == 2
 #pragma unroll
         for (int q = 0; q < 8; ++q)
           if (row_ok && c0 + q < B)
-            hm[(size_t)(c0 + q) * p.hm_stride] =
-                __float2bfloat16(kQ ? av[q] * activation(act_up, v[q] * sc) * osc : av[q] * activation(act_up, v[q]));
+            store_h(hm + (size_t)(c0 + q) * p.hm_stride,
+                    kQ ? av[q] * activation(act_up, v[q] * sc) * osc : av[q] * activation(act_up, v[q]));
       }
     } else {
       const int act = p.act;
       float* arow = p.a_out + j;
       const __nv_bfloat16* xg = static_cast<const __nv_bfloat16*>(p.xtok) + (gi >= 0 ? gi : 0);
-      if (p.split_cols) {
-        for (int c0 = 8 * part; c0 < npad; c0 += 8 * nparts) {
-          float v[8];
-          tmem_ld8(taddr + c0, nacc, npad, v);
+      // LoPA: a token's vector is the sum of two bf16 vectors (columns b and x_cols + b), whose products are added here
+      const int cols = p.x_cols ? p.x_cols : npad;
+      for (int c0 = 8 * part; c0 < cols; c0 += 8 * nparts) {
+        float v[8];
+        tmem_ld8(taddr + c0, nacc, npad, v);
+        if (p.x_cols) {
+          float w[8];
+          tmem_ld8(taddr + p.x_cols + c0, nacc, npad, w);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int b = c0 / 2 + q;
-            if (row_ok && b < B) {
-              float z = kQ ? (v[2 * q] + v[2 * q + 1]) * sc + bias : v[2 * q] + v[2 * q + 1] + bias;
-              if (gi >= 0) z += sg * __bfloat162float(xg[(size_t)b * p.xtok_stride]);
-              fired |= z > 0.f;
-              arow[(size_t)b * p.a_stride] = activation(act, z);
-            }
-          }
+          for (int q = 0; q < 8; ++q) v[q] += w[q];
         }
-      } else {
-        for (int c0 = 8 * part; c0 < npad; c0 += 8 * nparts) {
-          float v[8];
-          tmem_ld8(taddr + c0, nacc, npad, v);
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const int b = c0 + q;
-            if (row_ok && b < B) {
-              float z = kQ ? v[q] * sc + bias : v[q] + bias;
-              if (gi >= 0) z += sg * __bfloat162float(xg[(size_t)b * p.xtok_stride]);
-              fired |= z > 0.f;
-              arow[(size_t)b * p.a_stride] = activation(act, z);
-            }
+        for (int q = 0; q < 8; ++q) {
+          const int b = c0 + q;
+          if (row_ok && b < B) {
+            float z = kQ ? v[q] * sc + bias : v[q] + bias;
+            if (gi >= 0) z += sg * __bfloat162float(xg[(size_t)b * p.xtok_stride]);
+            fired |= z > 0.f;
+            arow[(size_t)b * p.a_stride] = activation(act, z);
           }
         }
       }
@@ -845,7 +846,10 @@ __global__ void __launch_bounds__(kThreadsRows + ((QB == 8 || QB == 4 || QB == 2
       __nv_bfloat16* hm = static_cast<__nv_bfloat16*>(p.hmT);
       const int end = (n_rows + 63) & ~63;
       for (int li = n_rows + (warp - 4) * 32 + lane; li < end; li += 128)
-        for (int b = 0; b < p.B; ++b) hm[(size_t)b * p.hm_stride + li] = __float2bfloat16(0.f);
+        for (int b = 0; b < p.B; ++b) {
+          hm[(size_t)b * p.hm_stride + li] = __float2bfloat16(0.f);
+          if (kQ && p.h_terms == 2) hm[(size_t)(p.h_cols + b) * p.hm_stride + li] = __float2bfloat16(0.f);
+        }
     }
     int tcount = 0;
     for (int tile = blockIdx.x; tile + (share_last ? (int)gridDim.x : 0) < n_tiles; tile += gridDim.x, ++tcount) {
@@ -980,7 +984,8 @@ __global__ void __launch_bounds__(kThreads + (QB ? 32 * kExpandWarps : 0), 2) um
 
   if (warp < kProducerWarps) {
     // ======================= producers (slot s belongs to warp s mod 4) =========================
-    const uint32_t tx_bytes = (uint32_t)((QB ? kRawBytes : kAAtomBytes) + npad * 128);
+    const int terms = QB ? p.terms : 1;
+    const uint32_t tx_bytes = (uint32_t)((QB ? kRawBytes : kAAtomBytes) + terms * p.cols * 128);
     const int half = lane >> 4, quad = lane & 15;
     constexpr int kHalfBytes = QB ? kRawBytes / 2 : kAAtomBytes / 2;  // landed bytes of 64 rows x 64 columns
     constexpr int kColDiv = QB == 4 ? 2 : 1;                          // codes per byte
@@ -1019,7 +1024,8 @@ __global__ void __launch_bounds__(kThreads + (QB ? 32 * kExpandWarps : 0), 2) um
         // every row: 64 consecutive rows per column half; rows past the matrix read as zero
         tma_tile_2d(wdst + lane * kHalfBytes, &map_wt, (d0 + lane * kAtomK) / kColDiv, u0, full + 8 * s);
       }
-      if (lane == 0) tma_tile_2d(abase + kAAtomBytes, &map_hm, u0, 0, full + 8 * s);
+      if (lane < terms)
+        tma_tile_2d(abase + kAAtomBytes + lane * p.cols * 128, &map_hm, u0, lane * p.h_cols + p.tok0, full + 8 * s);
     }
   } else if (QB && warp >= kThreads / 32) {
     // ======================= expanders (quantised rows): the stage's codes -> its two bf16 blocks =
@@ -1077,9 +1083,15 @@ __global__ void __launch_bounds__(kThreads + (QB ? 32 * kExpandWarps : 0), 2) um
       okw = __shfl_sync(0xffffffffu, okw, 0);
       if (okw) {
         tc_fence_after();
-        for (int c0 = 0; c0 < npad; c0 += 8) {
+        for (int c0 = 0; c0 < p.cols; c0 += 8) {
           float v[8];
           tmem_ld8(taddr + c0, nacc, npad, v);
+          if (QB && p.terms == 2) {
+            float w[8];
+            tmem_ld8(taddr + p.cols + c0, nacc, npad, w);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] += w[q];
+          }
 #pragma unroll
           for (int q = 0; q < 8; ++q)
             if (c0 + q < B) out[(size_t)(c0 + q) * p.D] = v[q];
@@ -1098,11 +1110,12 @@ __global__ void __launch_bounds__(kThreads + (QB ? 32 * kExpandWarps : 0), 2) um
   }
 }
 
-// LoPA gate, batched: n = RMSNorm(v) (or v itself), written as bf16 pairs for the tensor cores: row 2b of
-// x2 holds the high parts of token b's vector, row 2b+1 the low parts (v - bf16(v)), so that the gate's
-// U n keeps close to fp32 accuracy.  One CTA per token.
+// LoPA gate, batched: n = RMSNorm(v) (or v itself) as a sum of two bf16 vectors for the tensor cores: row b of
+// x2 holds the high part of token b's vector, row cols + b the low part (v - bf16(v)), so that the gate's U n keeps
+// close to fp32 accuracy.  One CTA per token.
 __global__ void __launch_bounds__(256) rmsnorm_split_kernel(const float* v, int r, int v_stride, const float* gain,
-                                                            float eps, int use_rms, __nv_bfloat16* x2) {
+                                                            float eps, int use_rms, int cols,
+                                                            __nv_bfloat16* x2) {
   __shared__ float red[8];
   pdl_launch_dependents();
   pdl_wait();
@@ -1123,8 +1136,8 @@ __global__ void __launch_bounds__(256) rmsnorm_split_kernel(const float* v, int 
   for (int k = threadIdx.x; k < r; k += blockDim.x) {
     const float n = use_rms ? (gain ? gain[k] : 1.f) * vb[k] * inv : vb[k];
     const __nv_bfloat16 hi = __float2bfloat16(n);
-    x2[(size_t)(2 * b) * r + k] = hi;
-    x2[(size_t)(2 * b + 1) * r + k] = __float2bfloat16(n - __bfloat162float(hi));
+    x2[(size_t)b * r + k] = hi;
+    x2[(size_t)(cols + b) * r + k] = __float2bfloat16(n - __bfloat162float(hi));
   }
 }
 
@@ -1210,7 +1223,7 @@ bool umma_own_list_supported(int R, int sm_count) {
 
 bool umma_may_walk(int B) { return B >= kWalkMinTokens; }
 
-bool umma_rows_supported(int K, int cols) { return K % kAtomK == 0 && K >= kAtomK && cols >= 1 && cols <= 128; }
+bool umma_rows_supported(int K, int cols) { return K % kAtomK == 0 && K >= kAtomK && cols >= 1 && cols <= kUmmaMaxCols; }
 // int8 rows multiplied as int8 (tokens as four int8 limbs each): K blocks of 128 codes, up to 64 tokens.
 bool umma_rows_native_i8_supported(int K, int tokens) { return K % 128 == 0 && K >= 128 && tokens >= 1 && tokens <= 64; }
 
@@ -1316,6 +1329,8 @@ cudaError_t launch_rows_mode(const UmmaRowsParams& p, int grid, size_t smem, cud
 
 cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, cudaStream_t s) {
   p.npad = (cols + 15) / 16 * 16;
+  if (p.h_terms > 1 && !(up && p.h_terms == 2 && (p.qbits == 8 || p.qbits == 4))) return cudaErrorInvalidValue;
+  if (p.x_cols && (p.x_cols % 8 || cols != 2 * p.x_cols)) return cudaErrorInvalidValue;
   p.wait_cycles = fused_test_knobs().wait_cycles;
   p.drop_stage = fused_test_knobs().drop_stage;
   const int grid = p.R < 8 * sm_count ? (p.R + 7) / 8 : sm_count;
@@ -1325,7 +1340,8 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
   alignas(64) CUtensorMap map_w, map_x;
   if (p.qbits != 0 && p.qbits != 8 && p.qbits != 4 && p.qbits != 1 && p.qbits != 2) return cudaErrorInvalidValue;
   const bool i8 = p.qbits == 1 || p.qbits == 2;  // kind::i8 MMAs: X holds the tokens' int8 limbs
-  if (i8 && (p.K % 128 || p.npad > 256 || !p.tok_scale)) return cudaErrorInvalidValue;
+  if (p.npad > kUmmaMaxCols) return cudaErrorInvalidValue;
+  if (i8 && (p.K % 128 || !p.tok_scale)) return cudaErrorInvalidValue;
   // weights: all R rows; boxes of one tile's rows for the gate, single-row boxes for the gather
   if (!make_weight_map(&map_w, p.W, p.K, p.R, up ? 1 : tile_rows_for(p.R, grid), p.qbits)) return cudaErrorNotSupported;
   // tokens: only the rows that exist; the box covers npad rows and the rest reads as zero
@@ -1343,20 +1359,24 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
   return launch_rows_mode<kUp>(p, grid, smem, s, map_w, map_x, WalkMap<false>{});
 }
 
-int umma_down_splits(int D, int sm_count, int max_splits) {
+// Token columns up to which two CTAs of the down kernel share an SM (each with two accumulators in half of the TMEM, and
+// at least four ring stages); wider batches give one CTA the whole SM.
+constexpr int kDownPairCols = 64;
+
+int umma_down_splits(int D, int cols, int sm_count, int max_splits) {
   const int d_tiles = D / kTileRows;
-  int splits = 2 * sm_count / (d_tiles > 0 ? d_tiles : 1);  // two CTAs per SM
+  int splits = (cols <= kDownPairCols ? 2 : 1) * sm_count / (d_tiles > 0 ? d_tiles : 1);
   return splits < 1 ? 1 : splits > max_splits ? max_splits : splits;
 }
 
-bool umma_down_supported(int D, int cols) { return D % kTileRows == 0 && cols >= 1 && cols <= 64; }
+bool umma_down_supported(int D, int cols) { return D % kTileRows == 0 && cols >= 1 && cols <= kUmmaMaxCols; }
 
 namespace {
 template <int QB>
 cudaError_t launch_down_q(const UmmaDownParams& p, int grid, size_t smem, cudaStream_t s, const CUtensorMap& map_wg,
                           const CUtensorMap& map_wt, const CUtensorMap& map_hm) {
   static unsigned long long configured = 0;
-  const cudaError_t e = allow_dynamic_smem(umma_down_kernel<QB>, 113 * 1024, configured);
+  const cudaError_t e = allow_dynamic_smem(umma_down_kernel<QB>, 227 * 1024, configured);
   if (e != cudaSuccess) return e;
   return launch_pdl(umma_down_kernel<QB>, dim3(grid), dim3(kThreads + (QB ? 32 * kExpandWarps : 0)), smem, s, p, map_wg,
                     map_wt, map_hm);
@@ -1365,10 +1385,14 @@ cudaError_t launch_down_q(const UmmaDownParams& p, int grid, size_t smem, cudaSt
 
 cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s) {
   if (p.qbits != 0 && p.qbits != 8 && p.qbits != 4) return cudaErrorInvalidValue;
-  p.npad = (p.B + 15) / 16 * 16;
+  if (p.terms < 1) p.terms = 1;
+  if (p.terms > 2 || (p.terms == 2 && !p.qbits)) return cudaErrorInvalidValue;
+  const int own = p.terms * p.cols;  // token columns that carry something
+  p.npad = (own + 15) / 16 * 16;
+  if (p.cols % 8 || p.cols < p.B || p.npad > kUmmaMaxCols) return cudaErrorInvalidValue;
   p.wait_cycles = fused_test_knobs().wait_cycles;
   const int stage_bytes = kAAtomBytes + p.npad * 128 + p.qbits * kTileRows * kAtomK / 8;
-  int stages = (111 * 1024 - 1024 - 1024) / stage_bytes;
+  int stages = ((own <= kDownPairCols ? 111 : 225) * 1024 - 1024 - 1024) / stage_bytes;
   if (stages > 12) stages = 12;
   stages &= ~1;
   if (stages < 2) return cudaErrorInvalidValue;
@@ -1379,8 +1403,8 @@ cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s) {
   // W_down [H, D]: inner dimension d; single-row boxes for the gather, 64-row boxes for the dense walk
   if (!make_weight_map(&map_wg, p.W_down, p.D, p.R, 1, p.qbits)) return cudaErrorNotSupported;
   if (!make_weight_map(&map_wt, p.W_down, p.D, p.R, kAtomK, p.qbits)) return cudaErrorNotSupported;
-  // HmT [B][hm_stride]: inner dimension u; token rows past B read as zero
-  if (!make_map(&map_hm, p.hmT, p.hm_stride, p.B, (size_t)p.hm_stride, p.npad)) return cudaErrorNotSupported;
+  // HmT [terms * h_cols][hm_stride]: inner dimension u; one box of `cols` token rows per term
+  if (!make_map(&map_hm, p.hmT, p.hm_stride, p.terms * p.h_cols, (size_t)p.hm_stride, p.cols)) return cudaErrorNotSupported;
   const int g = grid;
   return p.qbits == 8   ? launch_down_q<8>(p, g, smem, s, map_wg, map_wt, map_hm)
          : p.qbits == 4 ? launch_down_q<4>(p, g, smem, s, map_wg, map_wt, map_hm)
@@ -1399,8 +1423,8 @@ cudaError_t launch_rmsnorm_limbs(const float* v, int B, int r, int v_stride, con
 }
 
 cudaError_t launch_rmsnorm_split(const float* v, int B, int r, int v_stride, const float* gain, float eps,
-                                 bool use_rms, void* x2, cudaStream_t s) {
-  return launch_pdl(rmsnorm_split_kernel, dim3(B), dim3(256), 0, s, v, r, v_stride, gain, eps, use_rms ? 1 : 0,
+                                 bool use_rms, int cols, void* x2, cudaStream_t s) {
+  return launch_pdl(rmsnorm_split_kernel, dim3(B), dim3(256), 0, s, v, r, v_stride, gain, eps, use_rms ? 1 : 0, cols,
                     static_cast<__nv_bfloat16*>(x2));
 }
 

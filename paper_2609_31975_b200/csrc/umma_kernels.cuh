@@ -9,6 +9,9 @@ namespace sffn {
 // Value of UmmaRowsParams::act that stores the raw products (no bias is usually given, no activation).
 constexpr int kUmmaActIdentity = 3;
 
+// Token columns one pass of these kernels takes (the N of their MMAs).
+constexpr int kUmmaMaxCols = 256;
+
 struct UmmaRowsParams {
   const void* W;         // [*, K] bf16 (or int8 / packed int4 codes, see qbits), rows selected by idx (or 0..R-1)
   int R, K;
@@ -32,7 +35,7 @@ struct UmmaRowsParams {
   int x_stride;
   int ncols_valid;
   int B;                 // tokens
-  int split_cols;        // GATE: 1 = columns 2b, 2b+1 are the high / low bf16 parts of token b's vector
+  int x_cols;            // GATE: nonzero (a multiple of 8) = token b's vector is the sum of columns b and x_cols + b
   const float* b_g;
   const int32_t* g_idx;
   const int8_t* g_sign;
@@ -44,8 +47,9 @@ struct UmmaRowsParams {
   uint32_t* words_out;   // GATE: the same as bit masks, word 4 * tile + epilogue warp, or null
   const float* a;        // UP: gate values
   int a_stride;
-  void* hmT;             // UP: bf16 [B][hm_stride]
+  void* hmT;             // UP: bf16 [h_terms * h_cols][hm_stride]: h of token b is the sum of rows b and (2 terms) h_cols + b
   int hm_stride;
+  int h_terms, h_cols;   //   2 terms: quantised rows only (0: 1)
   int act_up;            // UP: activation on the up projection (double activation), kUmmaActIdentity = none
   int32_t* status;       // device status word
   int npad, ring_bytes;  // filled by the launcher
@@ -59,9 +63,12 @@ struct UmmaDownParams {
   int qbits;             // 0: bf16 rows; 8 / 4: rows of weight codes
   const int32_t* idx;    // list of rows (readable up to the next multiple of 64 past its length), or null = all R rows
   const int32_t* count;  // device length of the list, or null (= R)
-  const void* hmT;       // bf16 [B][hm_stride]; entries from the list's end to the next multiple of 64 are zero
+  const void* hmT;       // bf16 [terms * h_cols][hm_stride] (see UmmaRowsParams); entries from the list's end to the next
+                         // multiple of 64 are zero
   int hm_stride;         // multiple of 64
-  int B;
+  int terms, h_cols;     // terms of h (0: 1) and the rows between them
+  int tok0, B;           // tokens [tok0, tok0 + B) of those rows
+  int cols;              // B rounded up to a multiple of 8 (token columns of one term)
   int splits;            // the list is cut into this many runs of 64-row blocks
   const int32_t* walk_all;  // device word: nonzero = walk every row of W_down instead of the list (set by the up kernel), or null
   float* partial;        // [splits][B][D]
@@ -70,7 +77,7 @@ struct UmmaDownParams {
   long long wait_cycles; // budget of every device-side wait (filled by the launcher)
 };
 
-int umma_down_splits(int D, int sm_count, int max_splits);
+int umma_down_splits(int D, int cols, int sm_count, int max_splits);  // cols: token columns of all terms
 bool umma_down_supported(int D, int cols);
 cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s);
 bool umma_rows_supported(int K, int cols);
@@ -86,6 +93,6 @@ cudaError_t launch_token_limbs(const void* x, int B, int K, int x_stride, void* 
 cudaError_t launch_rmsnorm_limbs(const float* v, int B, int r, int v_stride, const float* gain, float eps, bool use_rms,
                                  void* limbs, float* scale, cudaStream_t s);
 cudaError_t launch_rmsnorm_split(const float* v, int B, int r, int v_stride, const float* gain, float eps,
-                                 bool use_rms, void* x2, cudaStream_t s);
+                                 bool use_rms, int cols, void* x2, cudaStream_t s);
 
 }  // namespace sffn

@@ -154,6 +154,33 @@ def test_int8_batches_tcgen05_edge_shapes(mod, D, H, B, s):
     assert torch.equal(y, y2)
 
 
+@pytest.mark.parametrize("D,H,B,kind", [
+    (128, 300, 5, "standard"),      # one column tile of the down projection, one K block
+    (384, 1001, 130, "standard"),   # an odd multiple of 128: h in two bf16 values, the down projection in two passes
+    (640, 2000, 64, "standard"),    # the most tokens that run on int8 limbs
+    (512, 2000, 65, "standard"),    # one more: codes expanded to bf16 in all three GEMMs
+    (512, 1201, 256, "standard"),   # a full pass
+    (512, 1201, 257, "standard"),   # and one token more
+    (512, 1201, 129, "lopa"),       # the same for the LoPA gate, whose vector takes two columns a token
+])
+def test_int8_wide_batches_and_odd_row_widths(mod, D, H, B, kind):
+    r = 128
+    ffn = mod.SparseFFN(D, H, torch.bfloat16, r_max=r, B_max=B)
+    gate, w = make_std(D, H, 16, 0.9) if kind == "standard" else make_lopa(mod, D, H, r, 16, 0.9)
+    w["b_g"] = syn.bias_from_firing_profile(syn.zipf_firing_profile(H, 1.1, 0.02, 0.9, seed=5)).to(DEV)
+    x = syn.tokens(B, D, torch.bfloat16, 16, DEV)
+    ref = run_oracle_q8(x, gate, w, "relu")
+    y = ffn.sparse_ffn_forward_q8(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0, ffn.status_words()
+    # h as one bf16 value: 2^-9 a term (the default tolerance); as two: 2^-17 = 8e-6, plus 384 / 16 accumulations that
+    # truncate at 2^-23 each
+    tol = dict(rel_l2=1e-5, max_abs=5e-5) if D % 256 else {}
+    assert_y_close(y, ref["y"], what=f"q8 wide {kind} {D}x{H} B={B}", **tol)
+    assert_active_set(ffn.last_active(), ref, what=f"q8 wide {kind} {D}x{H} B={B}")
+    assert torch.equal(y, ffn.sparse_ffn_forward_q8(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu"))
+
+
 @pytest.mark.parametrize("path", ["general", "fused"])
 def test_int8_full_and_zero_sparsity_and_double_activation(mod, path):
     D, H = 768, 1500

@@ -202,6 +202,27 @@ def test_batches_of_more_than_64_tokens_run_in_chunks_with_the_union_of_all(mod,
     assert torch.equal(y1, y2)
 
 
+@pytest.mark.parametrize("kind,B", [("standard", 72), ("standard", 200), ("standard", 256), ("standard", 257), ("lopa", 128), ("lopa", 129)])
+def test_one_pass_takes_up_to_256_tokens(mod, kind, B):
+    # 72: token columns that are no multiple of 16; 128 / 256: a full pass; one more: two passes and the union of both
+    D, H, r = 256, 2500, 64
+    ffn = mod.SparseFFN(D, H, torch.bfloat16, r_max=r, B_max=B)
+    if kind == "standard":
+        gate, w = make_std(D, H, torch.bfloat16, 47, 0.9)
+    else:
+        gate, w = make_lopa(mod, D, H, r, torch.bfloat16, 47, 0.9, "diag", True, True, True)
+    w["b_g"] = syn.bias_from_firing_profile(syn.zipf_firing_profile(H, 1.1, 0.02, 0.9, seed=5)).to(DEV)
+    x = syn.tokens(B, D, torch.bfloat16, 47, DEV)
+    launches0 = ffn.launch_count()
+    y = ffn.sparse_ffn_forward(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+    most = 256 if kind == "standard" else 128
+    assert (ffn.launch_count() - launches0 > 6) == (B > most)
+    run_both_paths(mod, ffn, x, gate, w, "relu", ("auto",), what=f"{kind} B={B}")
+    yd = ffn.dense_ffn_forward(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+    assert_y_close(yd, run_oracle(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu", route="dense")["y"], what=f"dense {kind} B={B}")
+    assert torch.equal(y, ffn.sparse_ffn_forward(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu"))
+
+
 @pytest.mark.parametrize("dtype,D", [(torch.float32, 512), (torch.bfloat16, 520), (torch.float32, 776)])
 @pytest.mark.parametrize("kind", ["standard", "lopa"])
 @pytest.mark.parametrize("B", [2, 5, 70])
