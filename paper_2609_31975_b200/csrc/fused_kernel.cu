@@ -98,6 +98,9 @@ struct FusedParams {
   long long* trace;       // SFFN_TRACE builds: [grid][16] time stamps, or null
 };
 
+// Floats of one exchange buffer of an act group: the four warps' sums of two rows, the stop flag, padding to 16 bytes.
+constexpr int kRedStride = 12;
+
 // Shared-memory carve-up, identical on host and device.
 struct SmemLayout {
   int gate_ring, act_ring, sx, sn, aval, slot_a, red, ctl, bars, row_params, row_scales, slot_scales, gated_bars, gated_vals, xlimb, total;
@@ -116,7 +119,7 @@ struct SmemLayout {
     sn = take(lopa ? K * 4 : 0);
     aval = take(slab_max * 4);
     slot_a = take((n_act_slots + act_extra) * 4);
-    red = take(6 * (2 * 4 + 1) * 4);  // two buffers per act group (four warps each), up to three groups
+    red = take(6 * kRedStride * 4);  // two buffers per act group (four warps each), up to three groups
     ctl = take(8 * 4);
     bars = take(2 * (n_gate_slots + n_act_slots + act_extra) * 8 + 8);  // + one for the CTA's rows of V (LoPA)
     row_params = take((lopa || scaled) ? (1 + (lopa ? 2 : 0) + (scaled ? 1 : 0)) * slab_max * 4 : 0);  // per-neuron gate parameters
@@ -153,6 +156,18 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// Whether a phase has completed, without waiting for it.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(ok)
       : "r"(bar), "r"(parity)
@@ -453,7 +468,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
       }
       mbar_init(v_bar, 1);
       for (int i = 0; i < 8; ++i) ctl[i] = 0;
-      for (int i = 0; i < 6 * (2 * 4 + 1); ++i) red[i] = 0.f;
+      for (int i = 0; i < 6 * kRedStride; ++i) red[i] = 0.f;
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -981,21 +996,32 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
       t_idle = 0;
       const bool take = row < slab_rows && lane < prefix && (p.dense || st != 0x80000000u);
       unsigned fired = __ballot_sync(0xffffffffu, take);
-      // Every lane issues the copy of its own row: up to NA rows go out per step, each into the ring slot of its
-      // place among the fired rows (one lane issuing them one after the other manages a row every ~500 cycles, which
-      // is what bounds a call with a short gate).
+      // Every lane issues the copy of its own row into the ring slot of its place among the fired rows (one lane issuing
+      // them one after the other manages a row every ~500 cycles, which is what bounds a call with a short gate).  Where
+      // the ring is short (wide rows) a step takes the leading rows whose slots are free right now, and waits only when
+      // the first one's is not: a step that waits for the slots of a whole lap lets such a ring run empty once per lap
+      // (3840 x 14230, r = 480, fp32: 25.0 -> 24.1 us a call).  With more than eight slots the look at them costs more than
+      // it brings (1 % at 1408 x 3072, int8).
       while (fired && ok) {
         const int place = __popc(fired & ((1u << lane) - 1u));
-        const int nb = min(__popc(fired), NR);
-        const bool mine = ((fired >> lane) & 1u) != 0 && place < nb;
+        const int most = min(__popc(fired), NR);
+        const bool cand = ((fired >> lane) & 1u) != 0 && place < most;
+        int ms = slot + place;
+        uint32_t mp = par;
+        if (ms >= NR) { ms -= NR; mp ^= 1; }
+        // first use of a slot inside the gate ring: not before the gate warps have read every gate row
+        const bool in_gate = !GATED && ms >= NAown && n_seq + place < NA;
+        int nb = most;
+        if (NR <= 8 && most > 1) {
+          const bool free_now = cand && mbar_test(pempty + 8 * ms, mp) && !(in_gate && ctl[kGateDone] < n_gslots);
+          const unsigned busy = __ballot_sync(0xffffffffu, cand && !free_now);
+          if (busy) nb = max(1, __popc(fired & ((1u << (__ffs(busy) - 1)) - 1u)));
+        }
+        const bool mine = cand && place < nb;
         bool good = true;
         if (mine) {
-          int ms = slot + place;
-          uint32_t mp = par;
-          if (ms >= NR) { ms -= NR; mp ^= 1; }
           bool free_slot = mbar_wait<true>(pempty + 8 * ms, mp, ctl, p.status, p.wait_cycles, 42);
-          if (!GATED && free_slot && ms >= NAown && n_seq + place < NA) {
-            // first use of a slot inside the gate ring: not before the gate warps have read every gate row
+          if (free_slot && in_gate) {
             const long long t0 = clock64();
             while (ctl[kGateDone] < n_gslots) {
               if (ctl[kAbort]) { free_slot = false; break; }
@@ -1148,7 +1174,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
         }
       };
       for (int round = 0;; ++round) {
-        float* rp = red + (round & 1) * (2 * kGAW + 1);
+        float* rp = red + (round & 1) * kRedStride;
         const int us1 = us + 1 == NU ? 0 : us + 1;
         const uint32_t upar1 = us + 1 == NU ? upar ^ 1 : upar;
         const bool got0 = mbar_wait(full_up + 8 * us, upar, ctl, p.status, p.wait_cycles, 45);
@@ -1239,115 +1265,160 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
     int slot = (pair ? 2 : 1) * grp;
     uint32_t par = 0;
     while (slot >= NA) { slot -= NA; par ^= 1; }
+    // Quantised rows, standard gate: the limbs and scales of this thread's chunks of the token, in registers where the
+    // accumulators leave room.
+    constexpr bool kLimbReg = (kLimbs || kLimbs4) && CPT * EPV <= 32;
+    uint4 lr[kLimbReg ? CPT : 1][kLimbs4 ? 2 * kUpLimbs : kUpLimbs];
+    float lsc[kLimbReg ? CPT : 1];
+    if constexpr (kLimbReg) {
+#pragma unroll
+      for (int i = 0; i < CPT; ++i) {
+        const int c = gat + i * kGT < nvecD ? gat + i * kGT : 0;
+        lsc[i] = xsc[c];
+#pragma unroll
+        for (int l = 0; l < kUpLimbs; ++l) {
+          if constexpr (kLimbs4) {
+            lr[i][2 * l] = xl[(l * nvecD + c) * 2];
+            lr[i][2 * l + 1] = xl[(l * nvecD + c) * 2 + 1];
+          } else {
+            lr[i][l] = xl[l * nvecD + c];
+          }
+        }
+      }
+    }
+    // One row's chunk i against the token: added onto the packed sums pk, pkb (fp32 routes) or the sum part (integers).
+    auto up_chunk = [&](int i, const uint4& w, float& part, float2& pk, float2& pkb) {
+      const int c = gat + i * kGT;
+      if constexpr (kLimbs || kLimbs4) {
+        int ia[kUpLimbs];
+        const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int l = 0; l < kUpLimbs; ++l) {
+          ia[l] = 0;
+          if constexpr (kLimbs4) {
+            uint4 h0, h1;
+            if constexpr (kLimbReg) { h0 = lr[i][2 * l]; h1 = lr[i][2 * l + 1]; }
+            else { const int cc = c < nvecD ? c : 0; h0 = xl[(l * nvecD + cc) * 2]; h1 = xl[(l * nvecD + cc) * 2 + 1]; }
+            const uint32_t xe[4] = {h0.x, h0.z, h1.x, h1.z}, xo[4] = {h0.y, h0.w, h1.y, h1.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              ia[l] = __dp4a((int)((ww[k] << 4) & 0xf0f0f0f0u), (int)xe[k], ia[l]);
+              ia[l] = __dp4a((int)(ww[k] & 0xf0f0f0f0u), (int)xo[k], ia[l]);
+            }
+          } else {
+            uint4 xv;
+            if constexpr (kLimbReg) xv = lr[i][l]; else xv = xl[l * nvecD + (c < nvecD ? c : 0)];
+            ia[l] = __dp4a((int)ww[0], (int)xv.x, ia[l]); ia[l] = __dp4a((int)ww[1], (int)xv.y, ia[l]);
+            ia[l] = __dp4a((int)ww[2], (int)xv.z, ia[l]); ia[l] = __dp4a((int)ww[3], (int)xv.w, ia[l]);
+          }
+        }
+        // the chunk's integer sums, scaled by its limb scale, join the fp32 sum (a row of zeros past the row's end adds 0)
+        float sc;
+        if constexpr (kLimbReg) sc = lsc[i]; else sc = xsc[c < nvecD ? c : 0];
+        part = fmaf(fmaf(small_int_as_float(ia[1]), 0.0078125f, small_int_as_float(ia[0])), sc, part);
+      } else if constexpr (EPV == 16) {
+        if (c < nvecD) pk = chunk_dot_q8(w, sx, c, nvecD, pk);
+      } else if constexpr (kXReg) {
+        // packed FMAs on two pairs of running sums per row: half the instructions, chains a quarter as long
+        float f[EPV];
+        Elem<T>::unpack(w, f);
+#pragma unroll
+        for (int e = 0; e < EPV; e += 4) {
+          pk = fma2(make_float2(f[e], f[e + 1]), make_float2(xr[i][e], xr[i][e + 1]), pk);
+          pkb = fma2(make_float2(f[e + 2], f[e + 3]), make_float2(xr[i][e + 2], xr[i][e + 3]), pkb);
+        }
+      } else {
+        if (c < nvecD) part = chunk_dot<T>(w, sx, c, nvecD, part);
+      }
+    };
+    auto up_sum = [&](float part, float2 pk, float2 pkb) -> float {
+      if constexpr (kLimbs4) return part * 0.0625f;  // the bytes were 16 x code
+      else if constexpr (kLimbs) return part;
+      else if constexpr (EPV == 16) return pk.x + pk.y;
+      else if constexpr (kXReg) return (pk.x + pk.y) + (pkb.x + pkb.y);
+      else return part;
+    };
+    // chunk i of a row; zeros past the row's end
+    auto row_chunk = [&](const uint4* row, int i) -> uint4 {
+      uint4 v = make_uint4(0u, 0u, 0u, 0u);
+      if (gat + i * kGT < nvecD) v = row[gat + i * kGT];
+      return v;
+    };
+    auto down_chunk = [&](int i, const uint4& w, float h) {
+      float f[EPV];
+      Elem<T>::unpack(w, f);
+#pragma unroll
+      for (int e = 0; e < EPV; e += 2) {
+        const float2 t = fma2(make_float2(h, h), make_float2(f[e], f[e + 1]), make_float2(acc[i][e], acc[i][e + 1]));
+        acc[i][e] = t.x;
+        acc[i][e + 1] = t.y;
+      }
+    };
+    // The W_down chunks of a round are read while its W_up sums are still on their way through the warps, where the
+    // registers hold them: a round is a chain of latencies (load, multiply, shuffles, barrier, load, multiply), not of
+    // work.  At 4096 columns a round of two rows took 1.1 us with the loads in line and a branch around every chunk.
+    constexpr bool kEarlyDown = CPT * EPV <= 32 && CPT <= 4;
+    constexpr int kBatch = CPT <= 4 ? CPT : CPT * EPV <= 32 ? 4 : 2;  // chunks of each row in registers at a time
     for (int round = 0;; ++round) {
-      float* rp = red + (2 * grp + (round & 1)) * (2 * kGAW + 1);
+      float* rp = red + (2 * grp + (round & 1)) * kRedStride;
       const int slot1 = slot + 1 == NA ? 0 : slot + 1;
       const uint32_t par1 = slot + 1 == NA ? par ^ 1 : par;
       const bool got0 = mbar_wait(full_act + 8 * slot, par, ctl, p.status, p.wait_cycles, 45);
+      const bool there1 = pair && mbar_test(full_act + 8 * slot1, par1);
       const float a0 = got0 ? slot_a[slot] : -1.f;
       bool got1 = true;
-      float a1 = -1.f;
-      if (pair && a0 >= 0.f) {
+      float a1 = there1 ? slot_a[slot1] : -1.f;
+      if (a0 < 0.f) a1 = -1.f;
+      if (pair && a0 >= 0.f && !there1) {
         got1 = mbar_wait(full_act + 8 * slot1, par1, ctl, p.status, p.wait_cycles, 46);
         a1 = got1 ? slot_a[slot1] : -1.f;
       }
       const unsigned char* s0 = act_slot(slot);
       const unsigned char* s1 = act_slot(slot1);
-      float part0 = 0.f, part1 = 0.f;
-      float2 pk0 = make_float2(0.f, 0.f), pk1 = pk0, pk0b = pk0, pk1b = pk0;  // packed partial sums
-      int ia0[kTokenLimbs] = {0, 0}, ia1[kTokenLimbs] = {0, 0};                             // quantised rows, standard gate: a chunk's integer sums per limb
+      const uint4* wd0 = reinterpret_cast<const uint4*>(s0 + row_bytes);
+      const uint4* wd1 = reinterpret_cast<const uint4*>(s1 + row_bytes);
+      uint4 d0[kEarlyDown ? CPT : 1], d1[kEarlyDown ? CPT : 1];
       if (a0 >= 0.f) {
         const uint4* wu0 = reinterpret_cast<const uint4*>(s0);
         const uint4* wu1 = reinterpret_cast<const uint4*>(s1);
+        float part0 = 0.f, part1 = 0.f;
+        float2 pk0 = make_float2(0.f, 0.f), pk1 = pk0, pk0b = pk0, pk1b = pk0;  // packed partial sums
+        if (a1 >= 0.f) {
 #pragma unroll
-        for (int i = 0; i < CPT; ++i) {
-          const int c = gat + i * kGT;
-          if (c < nvecD) {
-            if constexpr (kLimbs4) {
-              const uint4 u0 = wu0[c], u1 = wu1[c];
-              const uint32_t w0[4] = {u0.x, u0.y, u0.z, u0.w}, w1[4] = {u1.x, u1.y, u1.z, u1.w};
+          for (int i0 = 0; i0 < CPT; i0 += kBatch) {
+            uint4 w0[kBatch], w1[kBatch];
 #pragma unroll
-              for (int l = 0; l < kUpLimbs; ++l) {
-                const uint4 h0 = xl[(l * nvecD + c) * 2], h1 = xl[(l * nvecD + c) * 2 + 1];
-                const uint32_t xe[4] = {h0.x, h0.z, h1.x, h1.z}, xo[4] = {h0.y, h0.w, h1.y, h1.w};
+            for (int i = 0; i < kBatch; ++i) { w0[i] = row_chunk(wu0, i0 + i); w1[i] = row_chunk(wu1, i0 + i); }
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                  ia0[l] = __dp4a((int)((w0[k] << 4) & 0xf0f0f0f0u), (int)xe[k], ia0[l]);
-                  ia0[l] = __dp4a((int)(w0[k] & 0xf0f0f0f0u), (int)xo[k], ia0[l]);
-                  if (a1 >= 0.f) {
-                    ia1[l] = __dp4a((int)((w1[k] << 4) & 0xf0f0f0f0u), (int)xe[k], ia1[l]);
-                    ia1[l] = __dp4a((int)(w1[k] & 0xf0f0f0f0u), (int)xo[k], ia1[l]);
-                  }
-                }
-              }
-              {  // the chunk's integer sums, scaled by its limb scale, join the fp32 sums
-                const float sc = xsc[c];
-                const float v0 = fmaf(small_int_as_float(ia0[1]), 0.0078125f, small_int_as_float(ia0[0]));
-                const float v1 = fmaf(small_int_as_float(ia1[1]), 0.0078125f, small_int_as_float(ia1[0]));
-                part0 = fmaf(v0, sc, part0);
-                part1 = fmaf(v1, sc, part1);
-                ia0[0] = ia0[1] = ia1[0] = ia1[1] = 0;
-              }
-            } else if constexpr (kLimbs) {
-              const uint4 u0 = wu0[c], u1 = wu1[c];
-#pragma unroll
-              for (int l = 0; l < kUpLimbs; ++l) {
-                const uint4 xv = xl[l * nvecD + c];
-                ia0[l] = __dp4a((int)u0.x, (int)xv.x, ia0[l]); ia0[l] = __dp4a((int)u0.y, (int)xv.y, ia0[l]);
-                ia0[l] = __dp4a((int)u0.z, (int)xv.z, ia0[l]); ia0[l] = __dp4a((int)u0.w, (int)xv.w, ia0[l]);
-                if (a1 >= 0.f) {
-                  ia1[l] = __dp4a((int)u1.x, (int)xv.x, ia1[l]); ia1[l] = __dp4a((int)u1.y, (int)xv.y, ia1[l]);
-                  ia1[l] = __dp4a((int)u1.z, (int)xv.z, ia1[l]); ia1[l] = __dp4a((int)u1.w, (int)xv.w, ia1[l]);
-                }
-              }
-              {  // the chunk's integer sums, scaled by its limb scale, join the fp32 sums
-                const float sc = xsc[c];
-                const float v0 = fmaf(small_int_as_float(ia0[1]), 0.0078125f, small_int_as_float(ia0[0]));
-                const float v1 = fmaf(small_int_as_float(ia1[1]), 0.0078125f, small_int_as_float(ia1[0]));
-                part0 = fmaf(v0, sc, part0);
-                part1 = fmaf(v1, sc, part1);
-                ia0[0] = ia0[1] = ia1[0] = ia1[1] = 0;
-              }
-            } else if constexpr (EPV == 16) {
-              pk0 = chunk_dot_q8(wu0[c], sx, c, nvecD, pk0);
-              if (a1 >= 0.f) pk1 = chunk_dot_q8(wu1[c], sx, c, nvecD, pk1);
-            } else if constexpr (kXReg) {
-              // packed FMAs on two pairs of running sums per row: half the instructions, chains a quarter as long
-              float f[EPV];
-              Elem<T>::unpack(wu0[c], f);
-#pragma unroll
-              for (int e = 0; e < EPV; e += 4) {
-                pk0 = fma2(make_float2(f[e], f[e + 1]), make_float2(xr[i][e], xr[i][e + 1]), pk0);
-                pk0b = fma2(make_float2(f[e + 2], f[e + 3]), make_float2(xr[i][e + 2], xr[i][e + 3]), pk0b);
-              }
-              if (a1 >= 0.f) {
-                Elem<T>::unpack(wu1[c], f);
-#pragma unroll
-                for (int e = 0; e < EPV; e += 4) {
-                  pk1 = fma2(make_float2(f[e], f[e + 1]), make_float2(xr[i][e], xr[i][e + 1]), pk1);
-                  pk1b = fma2(make_float2(f[e + 2], f[e + 3]), make_float2(xr[i][e + 2], xr[i][e + 3]), pk1b);
-                }
-              }
-            } else {
-              part0 = chunk_dot<T>(wu0[c], sx, c, nvecD, part0);
-              if (a1 >= 0.f) part1 = chunk_dot<T>(wu1[c], sx, c, nvecD, part1);
+            for (int i = 0; i < kBatch; ++i) {
+              up_chunk(i0 + i, w0[i], part0, pk0, pk0b);
+              up_chunk(i0 + i, w1[i], part1, pk1, pk1b);
             }
           }
-        }
-        if constexpr (kLimbs || kLimbs4) {
-          if (kLimbs4) {  // the bytes were 16 x code
-            part0 *= 0.0625f;
-            part1 *= 0.0625f;
+          part0 = up_sum(part0, pk0, pk0b);
+          part1 = up_sum(part1, pk1, pk1b);
+          if constexpr (kEarlyDown) {
+#pragma unroll
+            for (int i = 0; i < CPT; ++i) { d0[i] = row_chunk(wd0, i); d1[i] = row_chunk(wd1, i); }
           }
-        } else if constexpr (EPV == 16) {
-          part0 = pk0.x + pk0.y;
-          part1 = pk1.x + pk1.y;
-        } else if constexpr (kXReg) {
-          part0 = (pk0.x + pk0.y) + (pk0b.x + pk0b.y);
-          part1 = (pk1.x + pk1.y) + (pk1b.x + pk1b.y);
+          part0 = warp_sum(part0);
+          part1 = warp_sum(part1);
+        } else {
+#pragma unroll
+          for (int i0 = 0; i0 < CPT; i0 += kBatch) {
+            uint4 w0[kBatch];
+#pragma unroll
+            for (int i = 0; i < kBatch; ++i) w0[i] = row_chunk(wu0, i0 + i);
+#pragma unroll
+            for (int i = 0; i < kBatch; ++i) up_chunk(i0 + i, w0[i], part0, pk0, pk0b);
+          }
+          part0 = up_sum(part0, pk0, pk0b);
+          if constexpr (kEarlyDown) {
+#pragma unroll
+            for (int i = 0; i < CPT; ++i) d0[i] = row_chunk(wd0, i);
+          }
+          part0 = warp_sum(part0);
         }
-        part0 = warp_sum(part0);
-        part1 = warp_sum(part1);
         if (lane == 0) {
           rp[gaw] = part0;
           rp[kGAW + gaw] = part1;
@@ -1355,9 +1426,10 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
       }
       if (a0 < 0.f || !got1) rp[2 * kGAW] = 1.f;  // stop marker first in the round, or a failed wait
       named_bar_sync(2 + 6 * grp, kGT);
+      const float4 r0 = reinterpret_cast<const float4*>(rp)[0], r1 = reinterpret_cast<const float4*>(rp)[1];
       if (rp[2 * kGAW] != 0.f) break;
-      float u0 = (rp[0] + rp[1]) + (rp[2] + rp[3]);
-      float u1 = (rp[kGAW] + rp[kGAW + 1]) + (rp[kGAW + 2] + rp[kGAW + 3]);
+      float u0 = (r0.x + r0.y) + (r0.z + r0.w);
+      float u1 = (r1.x + r1.y) + (r1.z + r1.w);
       if (kScaled) {  // int8 rows: u = s_up (codes . x); the W_down row's scale rides on h
         u0 *= slot_su[slot];
         u1 *= slot_su[slot1];
@@ -1367,30 +1439,15 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
         h0 *= slot_sd[slot];
         h1 *= slot_sd[slot1];
       }
-      const uint4* wd0 = reinterpret_cast<const uint4*>(s0 + row_bytes);
-      const uint4* wd1 = reinterpret_cast<const uint4*>(s1 + row_bytes);
+      if (a1 >= 0.f) {
 #pragma unroll
-      for (int i = 0; i < CPT; ++i) {
-        const int c = gat + i * kGT;
-        if (c < nvecD) {
-          float f[EPV];
-          Elem<T>::unpack(wd0[c], f);
-#pragma unroll
-          for (int e = 0; e < EPV; e += 2) {
-            const float2 t = fma2(make_float2(h0, h0), make_float2(f[e], f[e + 1]), make_float2(acc[i][e], acc[i][e + 1]));
-            acc[i][e] = t.x;
-            acc[i][e + 1] = t.y;
-          }
-          if (a1 >= 0.f) {
-            Elem<T>::unpack(wd1[c], f);
-#pragma unroll
-            for (int e = 0; e < EPV; e += 2) {
-              const float2 t = fma2(make_float2(h1, h1), make_float2(f[e], f[e + 1]), make_float2(acc[i][e], acc[i][e + 1]));
-              acc[i][e] = t.x;
-              acc[i][e + 1] = t.y;
-            }
-          }
+        for (int i = 0; i < CPT; ++i) {
+          down_chunk(i, kEarlyDown ? d0[kEarlyDown ? i : 0] : row_chunk(wd0, i), h0);
+          down_chunk(i, kEarlyDown ? d1[kEarlyDown ? i : 0] : row_chunk(wd1, i), h1);
         }
+      } else {
+#pragma unroll
+        for (int i = 0; i < CPT; ++i) down_chunk(i, kEarlyDown ? d0[kEarlyDown ? i : 0] : row_chunk(wd0, i), h0);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(empty_act + 8 * slot);
@@ -1567,6 +1624,19 @@ Geometry plan(int wkind, int D, int H, int K, bool lopa, int grid) {
   if (scaled && g.cpt * epv > 64) return g;
   int nr = 8192 / gate_row_bytes;
   nr = nr < 1 ? 1 : nr > 32 ? 32 : nr;
+  // Short rows: 8 KB of them would leave CTAs without a slot, or warps of a CTA.  A share of up to eight rows gives every
+  // gate warp its own (int4, 384 x 1024: 32 rows a slot took 12.4 us, one 7.1).  Beyond that, as measured per storage
+  // type: int8 rows are dotted two at a time (1408 x 3072: 5 rows a slot 10.5 us, 2 rows 9.3), int4 rows by three (2944 x
+  // 6272: 5 rows 13.0 us, 3 rows 11.6; four, which share more reads of the limbs, where they still make two slots a gate
+  // warp: 3840 x 10240 12.9 us, 3 rows 13.2), fp32 / bf16 rows up to
+  // eight at a time but in three slots or more (704 x 2048: 2 rows 7.2 us, 5 rows 6.8).  LoPA: at most eight
+  // (int4: four) rows, four slots or more (int4, 2048 x 6000, r = 256: 32 rows a slot 20.5 us, 4 rows 15.6).
+  const int rows_of_cta = (H + grid - 1) / grid;
+  const int cap = lopa ? (wkind == kWQ4 ? 4 : gate_row_bytes <= 1024 ? 8 : nr) : wkind == kWQ8 ? 2 : wkind == kWQ4 ? (rows_of_cta >= 64 ? 4 : 3) : nr;
+  const int least = lopa ? 4 : 3;  // slots
+  if (nr > cap) nr = cap;
+  if (rows_of_cta <= 8 && !lopa) nr = 1;
+  else if (nr > (rows_of_cta + least - 1) / least) nr = (rows_of_cta + least - 1) / least;
   if (lopa) {
     // Short gate (LoPA): when the CTA's whole share of U fits in three slots per gate warp with a few more rows per
     // slot, take them: every row is then on its way before the token arrives and none waits for a slot to come free

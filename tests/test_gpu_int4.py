@@ -159,3 +159,14 @@ def test_int4_argument_checks(mod):
         mod.SparseFFN(D2, H, torch.bfloat16, B_max=1).sparse_ffn_forward_q4(
             syn.tokens(1, D2, torch.bfloat16, 36, DEV)[0], gate2, w2["b_g"], w2["W_up"], w2["W_down"])
     assert e.value.code == 2
+
+
+@pytest.mark.parametrize("D,H", [(384, 1184), (384, 1185), (128, 148), (2944, 7104), (2944, 9472), (1024, 3000)])
+def test_int4_ring_slots_of_short_and_long_shares(mod, D, H):
+    # 8 rows a CTA (a slot each), 9 (slots of three), 1, 48 (slots of three), 64 (slots of four), ragged last slots
+    ffn = mod.SparseFFN(D, H, torch.bfloat16, r_max=64, B_max=1)
+    x = syn.tokens(1, D, torch.bfloat16, 61, DEV)[0]
+    gate, w = make_std(D, H, 61, 0.8)
+    check(ffn, x, gate, w, "relu", ("fused", "general"), f"q4 slots {D}x{H}")
+    gate, w = make_lopa(mod, D, H, 64, 61, 0.8)
+    check(ffn, x, gate, w, "sqrelu", ("auto", "general"), f"q4 lopa slots {D}x{H}")

@@ -92,6 +92,22 @@ def test_standard_gate_small_shapes(mod, gate_engine, D, H, dtype):
             run_both_paths(mod, ffn, x[t], gate, w, act, ("general", "fused"), what=f"{D}x{H} s={s} {act}")
 
 
+@pytest.mark.parametrize("D,H,r", [(384, 1184, 0), (384, 1185, 0), (704, 2048, 0), (256, 1000, 64), (3840, 6000, 256)])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_ring_slots_of_short_shares_and_rounds_of_short_rings(mod, D, H, r, dtype):
+    # 8 and 9 rows a CTA; slots of several short rows; rings of few wide slots whose rows are queued as slots come free
+    ffn = mod.SparseFFN(D, H, dtype, r_max=r, B_max=1)
+    gate, w = make_lopa(mod, D, H, r, dtype, 23, 0.6) if r else make_std(D, H, dtype, 23, 0.6)
+    for act_up in (None, "silu"):
+        ffn.set_up_activation(act_up)
+        x = syn.tokens(1, D, dtype, 23, DEV)[0]
+        ref = run_oracle(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu", act_up=act_up)
+        ffn.set_path("fused")
+        y = ffn.sparse_ffn_forward(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+        assert_y_close(y, ref["y"], rel_l2=1e-5, max_abs=1e-5, what=f"{D}x{H} r={r}")  # fp32 sums of at most 6000 terms
+        assert_active_set(ffn.last_active(), ref, what=f"{D}x{H} r={r}")
+
+
 @pytest.mark.parametrize("D,H", [(3840, 300), (5120, 200), (8192, 160), (16384, 96)])
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 def test_wide_rows(mod, gate_engine, D, H, dtype):
