@@ -22,14 +22,16 @@ constexpr int kMaxChunk = 4;         // tokens per pass of the general kernels
 constexpr int kMaxSplits = 16;       // union-row splits of the batched down projection
 constexpr int kMaxMmaTokens = 64;    // tokens per pass of the mma.sync kernels, and of the tcgen05 ones on int8 limbs
 constexpr int kMaxUmmaTokens = sffn::kUmmaMaxCols;  // tokens per pass of the tcgen05 kernels
-constexpr int kOddWidthMinTokens = 5;  // quantised rows of an odd multiple of 128: batches from here on the tcgen05 kernels
+constexpr int kOddWidthMinTokens = 5;  // rows of an odd multiple of 128: batches from here on the tcgen05 kernels ...
+constexpr int kExactMinTokens = 6;     // ... and where those have to form exact sums
 
 inline int round8(int v) { return (v + 7) & ~7; }
 
-// Row widths that are odd multiples of 128: batches over quantised rows of such widths used to run token by token with h
-// in fp32.  On the tensor cores h enters the down projection there as two bf16 values (16 bits; the tokens' limbs on the
-// single-token route hold fewer: 4e-5 against 2e-6 from the formulas in 64 bits); at the other widths it is one.
-inline int h_terms_for(int D, bool quantised) { return quantised && D % 256 != 0 ? 2 : 1; }
+// Row widths that are odd multiples of 128: batches of such widths used to run token by token, with every sum and h in
+// fp32.  On the tensor cores h enters the down projection there as three bf16 values (24 bits) and all sums are exact ones
+// (see umma_kernels.cu); under a standard gate on quantised rows, where the single-token route knows the token to 3e-5
+// only, as two (error from the formulas in 64 bits 4e-5 before, 2e-6 now).  At the other widths it is one.
+inline int h_terms_for(int D, bool exact, bool quantised) { return exact ? 3 : quantised && D % 256 != 0 ? 2 : 1; }
 
 // Most splits of the batched down projection's contraction over `cols` token columns (device-independent bound; what a
 // device uses is umma_down_splits).
@@ -71,8 +73,10 @@ Layout make_layout(int D, int H, int r_max, int B_max, int dtype) {
   L.ystage = take((size_t)B_max * D * 4);
   L.fused = take(sffn::fused_workspace_bytes(D, H, r_max));
   L.hm_stride = (H + 63) / 64 * 64 + 64;
-  L.hmT = take(h_terms_for(D, true) * bu8 * L.hm_stride * 2);
-  L.x2 = take(2 * bu8 * (r_max > 0 ? r_max : 1) * 2);
+  const size_t be8 = bu8 < sffn::kUmmaExactTokens ? bu8 : sffn::kUmmaExactTokens;  // tokens of a pass with exact sums
+  const size_t h_rows = D % 256 == 0 ? bu8 : 2 * bu8 > 3 * be8 ? 2 * bu8 : 3 * be8;
+  L.hmT = take(h_rows * L.hm_stride * 2);
+  L.x2 = take((2 * bu8 > 3 * be8 ? 2 * bu8 : 3 * be8) * (r_max > 0 ? r_max : 1) * 2);
   L.union_flag = take((size_t)H + 256);  // fired flags accumulated over the chunks of a batch of more than 64 tokens
   // int8 rows on the tensor cores: the tokens (and the LoPA vector) as four int8 limbs each, and their scales
   const size_t bt = B_max < kMaxMmaTokens ? B_max : kMaxMmaTokens;
@@ -278,6 +282,16 @@ thread_local int g_last_cuda_line = 0;
     }                                 \
   } while (0)
 
+// Whether a batch takes the tcgen05 kernels with exact sums (see h_terms_for).
+bool exact_batch(int D, bool quantised, bool lopa) { return D % 256 != 0 && (!quantised || lopa); }
+
+// Tokens that one pass of the tcgen05 kernels takes: 256 columns of the gate GEMM's token operand, which the LoPA
+// vector's high and low parts share; with exact sums 64, or what fits 128 columns at three terms each.
+int umma_pass_tokens(int D, bool quantised, bool lopa) {
+  if (exact_batch(D, quantised, lopa)) return lopa ? sffn::kUmmaExactCols / 3 / 8 * 8 : sffn::kUmmaExactTokens;
+  return lopa ? kMaxUmmaTokens / 2 : kMaxUmmaTokens;
+}
+
 // Batched tensor-core path (bf16 tokens, B >= 2): gate GEMM -> compaction of the union -> up GEMM over the
 // union rows -> down GEMM (split over D-slices and union chunks) -> fixed-order sum of the splits.
 // One pass: at most umma_pass_tokens tokens (64 on the mma.sync kernels); the union (and the list) is that of the pass.
@@ -316,7 +330,8 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
   const bool lopa = g->kind == SFFN_GATE_LOPA;
   const int grid_rows = 2 * h->sm_count;
 
-  const int h_terms = h_terms_for(D, q8 != nullptr);
+  const bool exact = umma && exact_batch(D, q8 != nullptr, g->kind == SFFN_GATE_LOPA);
+  const int h_terms = h_terms_for(D, exact, q8 != nullptr);
   if (lopa && umma) {  // v = V x on the tensor cores: the rows kernel with the identity as its epilogue
     UmmaRowsParams p{};
     p.W = g->V; p.R = g->r; p.K = D;
@@ -324,6 +339,7 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
     p.X = xb; p.x_stride = D; p.ncols_valid = B; p.B = B;
     if (native) { p.X = xlimb; p.ncols_valid = 4 * B; p.tok_scale = xscale; }
     p.act = kUmmaActIdentity; p.a_out = vbuf; p.a_stride = rs;
+    p.exact = exact;
     p.status = h->at<int32_t>(h->L.status);
     SFFN_CUDA(launch_umma_rows(false, p, native ? 4 * B : B, h->sm_count, s));
     ++h->launches;
@@ -353,6 +369,7 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
   if (umma) {
     UmmaRowsParams p{};
     p.R = H; p.B = B; p.b_g = b_g; p.act = act; p.status = h->at<int32_t>(h->L.status);
+    p.exact = exact;
     p.qbits = wq_rows; p.w_scale = q8 ? q8->s_gate : nullptr;
     p.xtok = x; p.xtok_stride = D;
     p.a_out = actbuf; p.a_stride = H;
@@ -367,13 +384,13 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
       p.g_idx = g->g_idx; p.g_sign = g->g_sign;
       cols = 4 * B;
     } else if (lopa) {
-      // RMSNorm (or none) and the split into bf16 pairs in one launch
+      // RMSNorm (or none) and the split into bf16 pairs (exact sums: triples) in one launch
       p.x_cols = round8(B);
-      SFFN_CUDA(launch_rmsnorm_split(vbuf, B, g->r, rs, g->rms_gain, g->rms_eps, g->use_rmsnorm != 0, p.x_cols, x2, s));
+      SFFN_CUDA(launch_rmsnorm_split(vbuf, B, g->r, rs, g->rms_gain, g->rms_eps, g->use_rmsnorm != 0, p.x_cols, exact, x2, s));
       ++h->launches;
       p.W = g->U; p.K = g->r; p.X = x2; p.x_stride = g->r;
       p.g_idx = g->g_idx; p.g_sign = g->g_sign;
-      cols = 2 * p.x_cols;
+      cols = (exact ? 3 : 2) * p.x_cols;
     } else if (native) {
       p.W = g->W_g; p.K = D; p.X = xlimb; p.x_stride = D; p.tok_scale = xscale;
       cols = 4 * B;
@@ -415,6 +432,7 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
   const int32_t* lidx = dense ? nullptr : idx;
   const int32_t* lcount = dense ? nullptr : count;
   const int h_cols = round8(B);
+  const bool may_walk = umma_may_walk(B) && !exact;
   if (umma) {
     UmmaRowsParams p{};
     p.W = W_up; p.R = H; p.K = D;
@@ -422,7 +440,7 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
     if (own_list) {
       p.words_in = words; p.n_words = 4 * gate_tiles; p.gate_tile_rows = gate_tile_rows;
       p.gate_rows_per_word = gate_tile_rows <= 64 ? 16 : 32;
-      p.idx_out = idx; p.count_out = count; p.walk_all = umma_may_walk(B) ? count + 1 : nullptr;
+      p.idx_out = idx; p.count_out = count; p.walk_all = may_walk ? count + 1 : nullptr;
     } else {
       p.idx = lidx; p.count = lcount;
     }
@@ -430,6 +448,7 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
     if (native) { p.X = xlimb; p.ncols_valid = 4 * B; p.tok_scale = xscale; }
     p.a = actbuf; p.a_stride = H;
     p.hmT = hmT; p.hm_stride = h->L.hm_stride; p.h_terms = h_terms; p.h_cols = h_cols;
+    p.exact = exact;
     p.status = h->at<int32_t>(h->L.status);
     p.act_up = h->act_up;
     SFFN_CUDA(launch_umma_rows(true, p, native ? 4 * B : B, h->sm_count, s));
@@ -444,8 +463,8 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
     SFFN_CUDA(launch_rows_mma(true, p, B, grid_rows, s));
   }
   ++h->launches;
-  // the down projection: all tokens at once, or (h in several terms) as many as its 256 columns hold
-  const int down_max = umma ? kUmmaMaxCols / h_terms / 8 * 8 : B;
+  // the down projection: all tokens at once, or (h in several terms) as many as its columns hold
+  const int down_max = umma ? (exact ? kUmmaExactCols : kUmmaMaxCols) / h_terms / 8 * 8 : B;
   for (int b0 = 0; b0 < B; b0 += down_max) {
     const int nb = B - b0 < down_max ? B - b0 : down_max;
     int splits;
@@ -453,12 +472,12 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
       UmmaDownParams d{};
       d.W_down = W_down; d.R = H; d.D = D; d.qbits = wq;
       d.idx = lidx; d.count = lcount;
-      d.hmT = hmT; d.hm_stride = h->L.hm_stride; d.terms = h_terms; d.h_cols = h_cols;
+      d.hmT = hmT; d.hm_stride = h->L.hm_stride; d.terms = h_terms; d.h_cols = h_cols; d.exact = exact;
       d.tok0 = b0; d.B = nb; d.cols = round8(nb);
       // (the workspace holds most_splits() partials of nb tokens; the first argument bounds what the SMs can use)
       const int cap = nb <= kMaxMmaTokens ? kMaxSplits : most_splits(D, nb);
       d.splits = splits = umma_down_splits(D, h_terms * d.cols, h->sm_count, cap);
-      d.walk_all = (own_list && umma_may_walk(B)) ? count + 1 : nullptr;
+      d.walk_all = (own_list && may_walk) ? count + 1 : nullptr;
       d.partial = partial; d.status = h->at<int32_t>(h->L.status);
       SFFN_CUDA(launch_umma_down(d, s));
     } else {
@@ -477,10 +496,6 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
   }
   return SFFN_OK;
 }
-
-// Tokens that one pass of the tcgen05 kernels takes: 256 columns of the gate GEMM's token operand, which the LoPA
-// vector's high and low parts share.
-int umma_pass_tokens(bool lopa) { return lopa ? kMaxUmmaTokens / 2 : kMaxUmmaTokens; }
 
 // General path: gate (all tokens, chunks of <= 4) -> compaction -> up/down + reduce per chunk.
 int run_general(sffn_handle* h, const void* x, int B, const sffn_gate* g, const float* b_g,
@@ -589,18 +604,19 @@ int run(sffn_handle* h, const void* x, int B, const sffn_gate* g, const float* b
   const int wkind = q8 ? (qbits == 4 ? sffn::kWQ4 : sffn::kWQ8) : h->dtype == SFFN_BF16 ? sffn::kWBF16 : sffn::kWF32;
   const bool lopa_gate = g->kind == SFFN_GATE_LOPA;
   const int gate_k = lopa_gate ? g->r : h->D;
-  // A batch the tensor-core kernels can take: bf16 tokens; bf16, int8 or int4 rows of a multiple of 256 elements, and a
-  // LoPA rank of a multiple of 64 (a standard gate on quantised rows: of 128 elements, see h_terms_for; the other batches
-  // of such widths run in fp32 throughout, which the tensor cores' sums do not match: 2e-6 against 2e-7).  At the odd
-  // widths the tensor cores pay from a few tokens on (int8, 1152 x 3500, B = 3 / 4 / 8: 27 / 28 / 28 us against 28 / 37 /
-  // 73 us token by token; 6528 x 20000: 151 / 157 / 184 against 131 / 175 / 348 us).  Larger batches are cut into passes of as many tokens as one launch chain holds: a
-  // pass reads every gate row and the rows of its own union, so fewer passes read fewer bytes (bf16, 4096 x 14336, 200
-  // tokens: 4 passes of 64 took 333 us).  The mma.sync kernels (selected, or a bf16 LoPA rank that is no multiple of 64)
-  // take passes of 64 and rows of a multiple of 256 elements.
+  // A batch the tensor-core kernels can take: bf16 tokens; bf16, int8 or int4 rows of a multiple of 256 elements, or of
+  // 128 from a few tokens on (see h_terms_for); a LoPA rank of a multiple of 64.  At the odd multiples of 128 the other
+  // route is the single-token kernel once per token: int8, standard gate, 1152 x 3500, B = 3 / 4 / 8: 27 / 28 / 28 us
+  // against 28 / 37 / 73 token by token, 6528 x 20000: 151 / 157 / 184 against 131 / 175 / 348; with exact sums (bf16 rows,
+  // LoPA gates), bf16, 1152 x 3500, B = 6 / 16: 37 / 41 us against 52 / 137, 6528 x 20000: 260 / 318 against 370 / 985.
+  // Larger batches are cut into passes of as many tokens as one launch chain holds: a pass reads every gate row and the
+  // rows of its own union, so fewer passes read fewer bytes (bf16, 4096 x 14336, 200 tokens: 4 passes of 64 took 333 us, one
+  // takes 137).  The mma.sync kernels (selected, or a bf16 LoPA rank that is no multiple of 64) take passes of 64 and rows
+  // of a multiple of 256 elements.
   const bool umma_ok = h->path != SFFN_PATH_MMA_SYNC && sffn::umma_rows_supported(gate_k, 1) &&
                        sffn::umma_rows_supported(h->D, 1) && sffn::umma_down_supported(h->D, 1) &&
-                       (h->D % 256 == 0 || (q8 && !lopa_gate && B >= kOddWidthMinTokens));
-  const int pass_max = umma_ok ? umma_pass_tokens(lopa_gate) : kMaxMmaTokens;
+                       (h->D % 256 == 0 || B >= (exact_batch(h->D, q8 != nullptr, lopa_gate) ? kExactMinTokens : kOddWidthMinTokens));
+  const int pass_max = umma_ok ? umma_pass_tokens(h->D, q8 != nullptr, lopa_gate) : kMaxMmaTokens;
   const bool tensor_batch = h->dtype == SFFN_BF16 && B >= 2 && h->path != SFFN_PATH_GENERAL && h->path != SFFN_PATH_FUSED &&
                             (umma_ok || (!q8 && sffn::batched_mma_supported(h->D, gate_k, 1)));
   // Any other batch (fp32 operands, a row width the tensor-core kernels do not tile, SFFN_PATH_FUSED): the single-token

@@ -345,10 +345,74 @@ struct WalkMap<false> {
   __device__ const CUtensorMap* get() const { return nullptr; }
 };
 
+// Exact sums (EX): the tensor cores truncate when they add onto an accumulator, so a sum over K = 2688 comes out low by
+// 1e-6 of its typical size, ten times what fp32 rounding leaves.  Here every two MMAs (K = 32) start an accumulator of
+// their own; the epilogue warps add a stage's accumulators in fp32 registers, which round to nearest.  An issuer has one
+// place in TMEM (the accumulators of one of its stages) and commits once per stage, to the epilogue warps, which give the
+// ring slot and then the place back: a commit per K block took twice as long.  Two sets of four epilogue warps share the
+// token columns (at most kExactTokens, in up to three terms: kUmmaExactCols columns).  h, and the LoPA vector, enter as
+// three bf16 terms (24 bits).  Error from 64 bits 1.1e-7 to 1.6e-7 over 384 to 7808 columns, the single-token kernels'
+// 1.2e-7 to 1.7e-7.  Bound by the round trip of a stage through issuer and epilogue: 0.5 us to 1 us per K block, 12 us to 35
+// us per kernel more than without (2688 x 7168, 6 / 60 tokens), against token-by-token calls of 97 / 918 us.
+constexpr int kExactTokens = kUmmaExactTokens;
+constexpr int kExactHalf = kExactTokens / 2;
+constexpr int kExactHalfTerms = 24;   // the same for passes whose tokens come in three terms: 40 tokens, in sets of 24 and 16
+constexpr int kExactMmas = 2;         // MMAs that share an accumulator
+constexpr int kExactPer = kAtomK / 16 / kExactMmas;  // accumulators of a K block
+__host__ __device__ constexpr int exact_issuers(int npad) { return npad <= 64 ? 4 : 2; }
+// K blocks of a stage, so that a place takes 128 (two issuers: 256) columns
+__host__ __device__ constexpr int exact_atoms(int npad) { return npad <= 16 ? 4 : npad <= 32 ? 2 : 1; }
+
+// Adds the accumulators of one stage (npad columns apart: `accs` of them, each of up to three terms `stride` columns apart)
+// up and then onto this thread's sums of the token columns [c0, c1), with what those additions round off carried along
+// (Kahan 1965).
+template <int HALF>
+__device__ __forceinline__ void add_stage(uint32_t taddr, int accs, int npad, int c0, int c1, int terms, int stride, float* sum, float* low) {
+#pragma unroll
+  for (int g = 0; g < HALF; g += 16) {
+    if (c0 + g < c1) {
+      const bool two = g + 8 < HALF && c0 + g + 8 < c1;  // 16 columns or eight
+      const uint32_t at = taddr + c0 + g;
+      uint32_t r[16];
+      float part[16];
+      int acc = 1, off = 0;
+      tmem_ld8_raw(at, r);
+      if (two) tmem_ld8_raw(at + 8, r + 8);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+      for (int q = 0; q < 16; ++q) part[q] = __uint_as_float(r[q]);
+#pragma unroll 1
+      for (int i = accs * terms - 1; i > 0; --i) {
+        if (acc == accs) { acc = 0; off += stride; }
+        tmem_ld8_raw(at + acc * npad + off, r);
+        if (two) tmem_ld8_raw(at + acc * npad + off + 8, r + 8);
+        ++acc;
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int q = 0; q < 16; ++q) part[q] += __uint_as_float(r[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < 16; ++q)
+        if (g + q < HALF) {  // (the upper eight are not used where there are none)
+          const float y = part[q] - low[g + q], t = sum[g + q] + y;
+          low[g + q] = (t - sum[g + q]) - y;
+          sum[g + q] = t;
+        }
+    }
+  }
+}
+// Meets `threads` threads at named barrier `id`; true for all of them if any of them came with true.
+__device__ __forceinline__ bool named_bar_any(int id, int threads, bool v) {
+  uint32_t any;
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, %2, %3, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+               : "=r"(any) : "r"(v ? 1u : 0u), "r"(id), "r"(threads) : "memory");
+  return any != 0;
+}
+
 enum RowsMode { kGate = 0, kUp = 1, kUpMayWalk = 2 };  // kUpMayWalk: wide batches, see walk_all below
 
-template <int MODE, int QB>
-__global__ void __launch_bounds__(kThreadsRows + ((QB == 8 || QB == 4 || QB == 2) ? 32 * kExpandWarps : 0), 1) umma_rows_kernel(const UmmaRowsParams p,
+template <int MODE, int QB, bool EX = false>
+__global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || QB == 4 || QB == 2) ? 32 * kExpandWarps : 0), 1) umma_rows_kernel(const UmmaRowsParams p,
                                                                   const __grid_constant__ CUtensorMap map_w,
                                                                   const __grid_constant__ CUtensorMap map_x,
                                                                   const __grid_constant__ WalkMap<MODE == kUpMayWalk> map_t) {
@@ -383,7 +447,11 @@ __global__ void __launch_bounds__(kThreadsRows + ((QB == 8 || QB == 4 || QB == 2
   // Set-up that needs nothing from earlier kernels runs while the predecessor in the stream finishes.
   pdl_launch_dependents();
   const int max_acc = npad > 128 ? 2 : kMaxIssuers;  // 512 TMEM columns: wide token blocks leave room for two accumulators
-  const uint32_t tmem_cols = tmem_cols_for(max_acc * npad);
+  static_assert(!EX || !kNat, "exact sums: bf16 operands");
+  const int place_cols = exact_atoms(npad) * kExactPer * npad;  // EX: columns of an issuer's place
+  const uint32_t place_full = afree + 8 * kExpandSlots, place_empty = place_full + 8 * kMaxIssuers;
+  constexpr int kExpand0 = kThreadsRows + (EX ? 128 : 0);  // first expander thread
+  const uint32_t tmem_cols = tmem_cols_for(EX ? exact_issuers(npad) * place_cols : max_acc * npad);
   if (tid == 0) {
     for (int s = 0; s < kMaxStages; ++s) {
       mbar_init(full + 8 * s, 1);  // the producer's expect_tx arrive; the copies complete the bytes
@@ -393,6 +461,11 @@ __global__ void __launch_bounds__(kThreadsRows + ((QB == 8 || QB == 4 || QB == 2
       for (int t = 0; t < kExpandSlots; ++t) {
         mbar_init(ready + 8 * t, kExpandWarps / 2);
         mbar_init(afree + 8 * t, 1);
+      }
+    if (EX)
+      for (int q = 0; q < kMaxIssuers; ++q) {
+        mbar_init(place_full + 8 * q, 1);
+        mbar_init(place_empty + 8 * q, 8);  // one arrival per epilogue warp
       }
     mbar_init(acc_empty, 128);
     *abort_flag = 0;
@@ -546,6 +619,10 @@ __global__ void __launch_bounds__(kThreadsRows + ((QB == 8 || QB == 4 || QB == 2
   int issuers = (S >= 8 && S % 4 == 0) ? 4 : kExp && S >= 4 ? 4 : 2;
   S &= (kExp && S >= 4) ? ~3 : ~1;
   issuers = issuers > max_acc ? max_acc : issuers;
+  if (EX) {
+    issuers = exact_issuers(npad);
+    S &= ~3;
+  }
   const int kstages = (kblocks + atoms - 1) / atoms;
   // accumulator row that this thread's TMEM lane holds (-1: none); the same for every warp of a lane quarter
   const int row_thr = m64 ? (lane < 16 ? (warp & 3) * 16 + lane : -1) : (warp & 3) * 32 + lane;
@@ -566,7 +643,7 @@ __global__ void __launch_bounds__(kThreadsRows + ((QB == 8 || QB == 4 || QB == 2
   // tile's accumulators, then (gate) adds the fixed-matrix term and the bias, applies the activation and
   // stores the gate values, reporting whether any token fired; (union rows) scales by the gate values
   // and stores HmT.  Returns false if the wait was abandoned.
-  const bool share_last = npad >= 32;  // four or more column groups: worth spreading over all warps
+  const bool share_last = !EX && npad >= 32;  // four or more column groups: worth spreading over all warps
   // `shared`: all twelve warps take part.  Only the epilogue warps have followed the accumulator barrier through
   // every earlier tile (a warp that joins for the last tile could find it still in an earlier phase, which a parity
   // wait cannot tell from "complete"), so they wait for it and the others meet them at a named barrier.
@@ -694,6 +771,79 @@ __global__ void __launch_bounds__(kThreadsRows + ((QB == 8 || QB == 4 || QB == 2
     return true;
   };
 
+  // EX: the same for the token columns of this warp's set, from sums added in registers; stage `it` of the CTA's sequence
+  // comes from ring slot it mod S and issuer it mod issuers (S is a multiple of their number).
+  constexpr int kHalf = QB ? kExactHalfTerms : kExactHalf;  // quantised rows: LoPA gates only
+  auto exact_epilogue = [&](int tile, int tcount, int set, int& it, int& s, bool& fired) -> bool {
+    float sum[kHalf], low[kHalf];
+#pragma unroll
+    for (int c = 0; c < kHalf; ++c) sum[c] = low[c] = 0.f;
+    const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+    const int li = tile * tile_rows + row_thr;
+    const bool row_ok = row_thr >= 0 && row_thr < tile_rows && li < n_rows;
+    int j = !row_ok ? 0 : own_list ? rows_sm[tcount * kTileRows + row_thr] : p.idx ? p.idx[li] : li;
+    if (!SFFN_IN_BOUNDS(j >= 0 && j < p.R, p.status, 40)) j = 0;
+    const int terms = p.x_cols ? 3 : 1, cols = p.x_cols ? p.x_cols : npad;
+    const int half = ((cols + 1) / 2 + 7) & ~7, c0 = set * half, c1 = set ? cols : half;
+    for (int kb = 0; kb < kstages; ++kb, ++it, ++s) {
+      if (s == S) s = 0;
+      const int m = it & (issuers - 1);
+      int ok = 1;
+      if (lane == 0) ok = mbar_wait(place_full + 8 * m, (it / issuers) & 1, abort_flag, p.status, p.wait_cycles) ? 1 : 0;
+      if (!__shfl_sync(0xffffffffu, ok, 0)) return false;
+      if (warp == 4 && lane == 0) {  // the stage's MMAs are done with their operands
+        mbar_arrive(empty + 8 * s);
+        if (kExp) mbar_arrive(afree + 8 * (it % kExpandSlots));
+      }
+      tc_fence_after();
+      add_stage<kHalf>(taddr + m * place_cols, min(atoms, kblocks - kb * atoms) * kExactPer, npad, c0, c1, terms, p.x_cols, sum, low);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(place_empty + 8 * m);
+    }
+    if (MODE == kGate) pdl_wait();
+    const float sc = (kQ && row_ok && p.w_scale) ? p.w_scale[j] : 1.f;
+    if (!row_ok) return true;
+    const int B = p.B < c1 ? p.B : c1;
+    if (UP) {
+      const float osc = (kQ && p.out_scale) ? p.out_scale[j] : 1.f;
+      __nv_bfloat16* hm = static_cast<__nv_bfloat16*>(p.hmT) + li;
+      const size_t term = (size_t)p.h_cols * p.hm_stride;
+#pragma unroll
+      for (int i = 0; i < kHalf; ++i) {
+        const int b = c0 + i;
+        if (b < B) {
+          float h = p.a[(size_t)b * p.a_stride + j] * activation(p.act_up, kQ ? sum[i] * sc : sum[i]);
+          if (kQ) h *= osc;
+          // 24 bits of h as three bf16 values
+          const __nv_bfloat16 h0 = __float2bfloat16(h);
+          h -= __bfloat162float(h0);
+          const __nv_bfloat16 h1 = __float2bfloat16(h);
+          __nv_bfloat16* dst = hm + (size_t)b * p.hm_stride;
+          dst[0] = h0;
+          dst[term] = h1;
+          dst[2 * term] = __float2bfloat16(h - __bfloat162float(h1));
+        }
+      }
+    } else {
+      const float bias = p.b_g ? p.b_g[j] : 0.f;
+      const int gi = p.g_idx ? p.g_idx[j] : -1;
+      const float sg = (p.g_sign && p.g_sign[j] < 0) ? -1.f : 1.f;
+      const __nv_bfloat16* xg = static_cast<const __nv_bfloat16*>(p.xtok) + (gi >= 0 ? gi : 0);
+#pragma unroll
+      for (int i = 0; i < kHalf; ++i) {
+        const int b = c0 + i;
+        if (b < B) {
+          float z = kQ ? sum[i] * sc + bias : sum[i] + bias;
+          if (gi >= 0) z += sg * __bfloat162float(xg[(size_t)b * p.xtok_stride]);
+          fired |= z > 0.f;
+          p.a_out[(size_t)b * p.a_stride + j] = activation(p.act, z);
+        }
+      }
+    }
+    return true;
+  };
+
   if (warp < kProducerWarps) {
     // ======================= producers =========================================================
     // Stages are numbered it = 0, 1, ... over this CTA's (tile, K block) sequence and use ring slot
@@ -769,14 +919,14 @@ __global__ void __launch_bounds__(kThreadsRows + ((QB == 8 || QB == 4 || QB == 2
     } else {
       produce(0, total, true, true);
     }
-  } else if (kExp && warp >= kThreadsRows / 32) {
+  } else if (kExp && warp >= kExpand0 / 32) {
     // ======================= expanders (quantised rows): codes -> bf16 block of the slot ==========
     // Two pairs of warps; a pair takes the slots of its parity (S is even), in the producers' order, so it meets
     // every phase of its slots and cannot fall two phases behind; while one pair waits the other one converts.
     const int my_tiles = (int)blockIdx.x < n_tiles ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     const int total = my_tiles * kstages;
-    const int pair = (tid - kThreadsRows) / (16 * kExpandWarps);
-    const int et = (tid - kThreadsRows) % (16 * kExpandWarps);
+    const int pair = (tid - kExpand0) / (16 * kExpandWarps);
+    const int et = (tid - kExpand0) % (16 * kExpandWarps);
     int s = 0, ph = 0, kb = 0;
     for (int it = 0; it < total; ++it, ++s, ++kb) {
       if (s == S) { s = 0; ph ^= 1; }
@@ -796,10 +946,38 @@ __global__ void __launch_bounds__(kThreadsRows + ((QB == 8 || QB == 4 || QB == 2
       __syncwarp();
       if (lane == 0) mbar_arrive(ready + 8 * t);
     }
-  } else if (warp >= 8) {
+  } else if (warp >= 8 && warp < kThreadsRows / 32) {
     // ======================= MMA issuers =======================================================
     const int m = warp - 8;
-    if (lane == 0 && m < nacc) {
+    if constexpr (EX) {
+      if (lane == 0 && m < issuers) {
+        const uint32_t idesc = make_idesc(npad, mrows);
+        const uint32_t place = tmem_base + m * place_cols;
+        const int my_tiles = (int)blockIdx.x < n_tiles ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+        int s = 0, ph = 0, kb = 0;
+        for (int it = 0; it < my_tiles * kstages; ++it, ++s, ++kb) {
+          if (s == S) { s = 0; ph ^= 1; }
+          if (kb == kstages) kb = 0;
+          if ((it & (issuers - 1)) != m) continue;  // another issuer's slot
+          const int t = it % kExpandSlots;
+          if (kExp ? !mbar_wait(ready + 8 * t, (it / kExpandSlots) & 1, abort_flag, p.status, p.wait_cycles)
+                   : !mbar_wait(full + 8 * s, ph, abort_flag, p.status, p.wait_cycles)) break;
+          if (!mbar_wait(place_empty + 8 * m, ((it / issuers) & 1) ^ 1, abort_flag, p.status, p.wait_cycles)) break;
+          tc_fence_after();
+          const uint32_t sbase = ring0 + s * stage_bytes;
+          const uint32_t wbase = kExp ? stage0 + t * a_bytes : sbase;
+          const int na = min(atoms, kblocks - kb * atoms);
+          for (int a = 0; a < na; ++a) {
+            const uint64_t adesc = make_desc(wbase + a * a_block_bytes);
+            const uint64_t bdesc = make_desc(sbase + b_off + a * b_block_bytes);
+#pragma unroll
+            for (int k = 0; k < kAtomK / 16; ++k)
+              umma(place + (a * kExactPer + k / kExactMmas) * npad, adesc + 2 * k, bdesc + 2 * k, idesc, k % kExactMmas ? 1u : 0u);
+          }
+          umma_commit(place_full + 8 * m);
+        }
+      }
+    } else if (lane == 0 && m < nacc) {
       const uint32_t idesc = kNat ? make_idesc_i8(npad, mrows) : make_idesc(npad, mrows);
       const uint32_t acc = tmem_base + m * npad;
       int tcount = 0;
@@ -841,20 +1019,37 @@ __global__ void __launch_bounds__(kThreadsRows + ((QB == 8 || QB == 4 || QB == 2
     __syncwarp();
   } else {
     // ======================= epilogue warps (wide batches: every tile but the CTA's last) =========
-    if (UP && blockIdx.x == 0) {
+    const int set = EX && warp >= kThreadsRows / 32 ? 1 : 0;
+    if (UP && blockIdx.x == 0 && set == 0) {
       // the down projection walks the list in blocks of 64 rows: entries past its end must read as zero
       __nv_bfloat16* hm = static_cast<__nv_bfloat16*>(p.hmT);
       const int end = (n_rows + 63) & ~63;
       for (int li = n_rows + (warp - 4) * 32 + lane; li < end; li += 128)
         for (int b = 0; b < p.B; ++b) {
           hm[(size_t)b * p.hm_stride + li] = __float2bfloat16(0.f);
-          if (kQ && p.h_terms == 2) hm[(size_t)(p.h_cols + b) * p.hm_stride + li] = __float2bfloat16(0.f);
+          if (EX || (kQ && p.h_terms == 2)) hm[(size_t)(p.h_cols + b) * p.hm_stride + li] = __float2bfloat16(0.f);
+          if (EX) hm[(size_t)(2 * p.h_cols + b) * p.hm_stride + li] = __float2bfloat16(0.f);
         }
     }
-    int tcount = 0;
+    int tcount = 0, it = 0, s = 0;
     for (int tile = blockIdx.x; tile + (share_last ? (int)gridDim.x : 0) < n_tiles; tile += gridDim.x, ++tcount) {
       bool fired = false;
-      if (!epilogue(tile, tcount, 0, 1, false, fired)) break;
+      if constexpr (EX) {
+        const bool done = exact_epilogue(tile, tcount, set, it, s, fired);
+        if (UP) {
+          if (!done) break;
+          continue;
+        }
+        // the two sets of warps hold the flags of half of the tokens each; both leave together
+        uint8_t* fired_sm = reinterpret_cast<uint8_t*>(scan_wt) + (tcount & 1) * 2 * kTileRows;  // the scan scratch is free here
+        const int me = (warp & 3) * 32 + lane;
+        fired_sm[set * kTileRows + me] = fired ? 1 : 0;
+        if (named_bar_any(2, 256, !done)) break;
+        if (set) continue;
+        fired = (fired_sm[me] | fired_sm[kTileRows + me]) != 0;
+      } else {
+        if (!epilogue(tile, tcount, 0, 1, false, fired)) break;
+      }
       const int row_in_tile = row_thr;
       const int li = tile * tile_rows + row_in_tile;
       const bool valid = row_in_tile >= 0 && row_in_tile < tile_rows && li < n_rows;
@@ -863,6 +1058,7 @@ __global__ void __launch_bounds__(kThreadsRows + ((QB == 8 || QB == 4 || QB == 2
         const unsigned m = __ballot_sync(0xffffffffu, fired && valid);
         if (lane == 0) p.words_out[4 * tile + (warp & 3)] = m;
       }
+      if (EX) continue;
       tc_fence_before();
       mbar_arrive(acc_empty);
     }
@@ -916,8 +1112,8 @@ __global__ void __launch_bounds__(kThreadsRows + ((QB == 8 || QB == 4 || QB == 2
 // gathered row delivers 64 contiguous d per swizzle row) and HmT[b][u] is the K-major B operand.
 // Same pipeline as above: 4 producer warps (gather4 per lane: 2 column halves x 16 row quads = one 64-row
 // stage), 2 MMA issuers with their own accumulators, 4 epilogue warps; two CTAs share an SM.
-template <int QB>
-__global__ void __launch_bounds__(kThreads + (QB ? 32 * kExpandWarps : 0), 2) umma_down_kernel(const UmmaDownParams p,
+template <int QB, bool EX = false>
+__global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarps : 0), EX ? 1 : 2) umma_down_kernel(const UmmaDownParams p,
                                                                   const __grid_constant__ CUtensorMap map_wg,
                                                                   const __grid_constant__ CUtensorMap map_wt,
                                                                   const __grid_constant__ CUtensorMap map_hm) {
@@ -942,13 +1138,22 @@ __global__ void __launch_bounds__(kThreads + (QB ? 32 * kExpandWarps : 0), 2) um
   const int d0 = dt * kTileRows;
 
   pdl_launch_dependents();
-  const uint32_t tmem_cols = tmem_cols_for(2 * npad);
+  // EX: see exact sums above; S is a multiple of the issuers, warps 12-15 are the second epilogue set
+  const int place_cols = kExactPer * npad, issuers = exact_issuers(npad);
+  const uint32_t place_full = ready + 8 * S, place_empty = place_full + 8 * kMaxIssuers;
+  constexpr int kExpand0 = EX ? 512 : kThreads;  // first expander thread
+  const uint32_t tmem_cols = tmem_cols_for(EX ? issuers * place_cols : 2 * npad);
   if (tid == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(full + 8 * s, 1);
       mbar_init(empty + 8 * s, 1);
       if (QB) mbar_init(ready + 8 * s, kExpandWarps / 2);
     }
+    if (EX)
+      for (int q = 0; q < kMaxIssuers; ++q) {
+        mbar_init(place_full + 8 * q, 1);
+        mbar_init(place_empty + 8 * q, 8);
+      }
     *abort_flag = 0;
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_wg) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_wt) : "memory");
@@ -984,7 +1189,7 @@ __global__ void __launch_bounds__(kThreads + (QB ? 32 * kExpandWarps : 0), 2) um
 
   if (warp < kProducerWarps) {
     // ======================= producers (slot s belongs to warp s mod 4) =========================
-    const int terms = QB ? p.terms : 1;
+    const int terms = QB || EX ? p.terms : 1;
     const uint32_t tx_bytes = (uint32_t)((QB ? kRawBytes : kAAtomBytes) + terms * p.cols * 128);
     const int half = lane >> 4, quad = lane & 15;
     constexpr int kHalfBytes = QB ? kRawBytes / 2 : kAAtomBytes / 2;  // landed bytes of 64 rows x 64 columns
@@ -1027,11 +1232,11 @@ __global__ void __launch_bounds__(kThreads + (QB ? 32 * kExpandWarps : 0), 2) um
       if (lane < terms)
         tma_tile_2d(abase + kAAtomBytes + lane * p.cols * 128, &map_hm, u0, lane * p.h_cols + p.tok0, full + 8 * s);
     }
-  } else if (QB && warp >= kThreads / 32) {
+  } else if (QB && warp >= kExpand0 / 32) {
     // ======================= expanders (quantised rows): the stage's codes -> its two bf16 blocks =
     // two pairs of warps, each with the slots of its parity (S is even)
-    const int pair = (tid - kThreads) / (16 * kExpandWarps);
-    const int et = (tid - kThreads) % (16 * kExpandWarps);
+    const int pair = (tid - kExpand0) / (16 * kExpandWarps);
+    const int et = (tid - kExpand0) % (16 * kExpandWarps);
     int s = 0, ph = 0;
     for (int kb = 0; kb < kblocks; ++kb, ++s) {
       if (s == S) { s = 0; ph ^= 1; }
@@ -1045,10 +1250,29 @@ __global__ void __launch_bounds__(kThreads + (QB ? 32 * kExpandWarps : 0), 2) um
       __syncwarp();
       if (lane == 0) mbar_arrive(ready + 8 * s);
     }
-  } else if (warp >= 8) {
+  } else if (warp >= 8 && warp < 12) {
     // ======================= MMA issuers (slot s belongs to issuer s mod 2) =====================
     const int m = warp - 8;
-    if (lane == 0 && m < nacc) {
+    if constexpr (EX) {
+      if (lane == 0 && m < issuers) {
+        const uint32_t idesc = make_idesc(npad) | (1u << 15);  // A is MN-major
+        const uint32_t place = tmem_base + m * place_cols;
+        int s = 0, ph = 0;
+        for (int kb = 0; kb < kblocks; ++kb, ++s) {
+          if (s == S) { s = 0; ph ^= 1; }
+          if ((kb & (issuers - 1)) != m) continue;
+          if (!mbar_wait((QB ? ready : full) + 8 * s, ph, abort_flag, p.status, p.wait_cycles)) break;
+          if (!mbar_wait(place_empty + 8 * m, ((kb / issuers) & 1) ^ 1, abort_flag, p.status, p.wait_cycles)) break;
+          tc_fence_after();
+          const uint32_t sbase = stage0 + s * stage_bytes;
+          const uint64_t bdesc = make_desc(sbase + kAAtomBytes);
+#pragma unroll
+          for (int k = 0; k < kAtomK / 16; ++k)
+            umma(place + k / kExactMmas * npad, make_desc_mn(sbase + k * 2048, 8192, 1024), bdesc + 2 * k, idesc, k % kExactMmas ? 1u : 0u);
+          umma_commit(place_full + 8 * m);
+        }
+      }
+    } else if (lane == 0 && m < nacc) {
       const uint32_t idesc = make_idesc(npad) | (1u << 15);  // A is MN-major
       const uint32_t acc = tmem_base + m * npad;
       int s = 0, ph = 0;
@@ -1070,13 +1294,37 @@ __global__ void __launch_bounds__(kThreads + (QB ? 32 * kExpandWarps : 0), 2) um
     __syncwarp();
   } else {
     // ======================= epilogue: lane = output column d, TMEM columns = tokens ============
-    const int ew = warp - 4;
+    const int ew = warp & 3;
     const int d = d0 + ew * 32 + lane;
     const int B = p.B;
     float* out = p.partial + (size_t)sp * B * p.D + d;
     const uint32_t taddr = tmem_base + ((uint32_t)(ew * 32) << 16);
+    const int set = EX && warp >= 12 ? 1 : 0;
     if (kblocks <= 0) {
-      for (int b = 0; b < B; ++b) out[(size_t)b * p.D] = 0.f;
+      for (int b = 0; set == 0 && b < B; ++b) out[(size_t)b * p.D] = 0.f;
+    } else if constexpr (EX) {
+      constexpr int kHalf = QB ? kExactHalfTerms : kExactHalf;
+      float sum[kHalf], low[kHalf];
+#pragma unroll
+      for (int c = 0; c < kHalf; ++c) sum[c] = low[c] = 0.f;
+      const int half = ((p.cols + 1) / 2 + 7) & ~7, c0 = set * half, c1 = set ? p.cols : half;
+      int ok = 1, s = 0;
+      for (int kb = 0; kb < kblocks; ++kb, ++s) {
+        if (s == S) s = 0;
+        const int m = kb & (issuers - 1);
+        if (lane == 0) ok = mbar_wait(place_full + 8 * m, (kb / issuers) & 1, abort_flag, p.status, p.wait_cycles) ? 1 : 0;
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (!ok) break;
+        if (warp == 4 && lane == 0) mbar_arrive(empty + 8 * s);  // the stage's MMAs are done with their operands
+        tc_fence_after();
+        add_stage<kHalf>(taddr + m * place_cols, kExactPer, npad, c0, c1, p.terms, p.cols, sum, low);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(place_empty + 8 * m);
+      }
+#pragma unroll
+      for (int i = 0; i < kHalf; ++i)
+        if (ok && c0 + i < c1 && c0 + i < B) out[(size_t)(c0 + i) * p.D] = sum[i];
     } else {
       int okw = 1;
       if (lane == 0) okw = mbar_wait(acc_full, 0, abort_flag, p.status, p.wait_cycles) ? 1 : 0;
@@ -1112,9 +1360,9 @@ __global__ void __launch_bounds__(kThreads + (QB ? 32 * kExpandWarps : 0), 2) um
 
 // LoPA gate, batched: n = RMSNorm(v) (or v itself) as a sum of two bf16 vectors for the tensor cores: row b of
 // x2 holds the high part of token b's vector, row cols + b the low part (v - bf16(v)), so that the gate's U n keeps
-// close to fp32 accuracy.  One CTA per token.
+// close to fp32 accuracy.  `exact`: row 2 cols + b holds what those two leave (24 bits in all).  One CTA per token.
 __global__ void __launch_bounds__(256) rmsnorm_split_kernel(const float* v, int r, int v_stride, const float* gain,
-                                                            float eps, int use_rms, int cols,
+                                                            float eps, int use_rms, int cols, int exact,
                                                             __nv_bfloat16* x2) {
   __shared__ float red[8];
   pdl_launch_dependents();
@@ -1137,7 +1385,10 @@ __global__ void __launch_bounds__(256) rmsnorm_split_kernel(const float* v, int 
     const float n = use_rms ? (gain ? gain[k] : 1.f) * vb[k] * inv : vb[k];
     const __nv_bfloat16 hi = __float2bfloat16(n);
     x2[(size_t)b * r + k] = hi;
-    x2[(size_t)(cols + b) * r + k] = __float2bfloat16(n - __bfloat162float(hi));
+    const float low = n - __bfloat162float(hi);
+    const __nv_bfloat16 mid = __float2bfloat16(low);
+    x2[(size_t)(cols + b) * r + k] = mid;
+    if (exact) x2[(size_t)(2 * cols + b) * r + k] = __float2bfloat16(low - __bfloat162float(mid));
   }
 }
 
@@ -1299,6 +1550,14 @@ cudaError_t launch_rows_mode(const UmmaRowsParams& p, int grid, size_t smem, cud
                              const CUtensorMap& map_x, const Map& map_t) {
   static unsigned long long configured[4] = {0, 0, 0, 0};
   cudaError_t e;
+  if constexpr (MODE != kUpMayWalk) {
+    if (p.exact) {
+      static unsigned long long configured_ex[3] = {0, 0, 0};
+      auto k = p.qbits == 8 ? umma_rows_kernel<MODE, 8, true> : p.qbits == 4 ? umma_rows_kernel<MODE, 4, true> : umma_rows_kernel<MODE, 0, true>;
+      if ((e = allow_dynamic_smem(k, 227 * 1024, configured_ex[p.qbits == 8 ? 1 : p.qbits == 4 ? 2 : 0])) != cudaSuccess) return e;
+      return launch_pdl(k, dim3(grid), dim3(kThreadsRows + 128 + (p.qbits ? 32 * kExpandWarps : 0)), smem, s, p, map_w, map_x, map_t);
+    }
+  }
   if (p.qbits == 1) {
     auto k = umma_rows_kernel<MODE, 1>;
     if ((e = allow_dynamic_smem(k, 227 * 1024, configured[3])) != cudaSuccess) return e;
@@ -1329,8 +1588,9 @@ cudaError_t launch_rows_mode(const UmmaRowsParams& p, int grid, size_t smem, cud
 
 cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, cudaStream_t s) {
   p.npad = (cols + 15) / 16 * 16;
-  if (p.h_terms > 1 && !(up && p.h_terms == 2 && (p.qbits == 8 || p.qbits == 4))) return cudaErrorInvalidValue;
-  if (p.x_cols && (p.x_cols % 8 || cols != 2 * p.x_cols)) return cudaErrorInvalidValue;
+  if (p.exact ? (p.B > (p.qbits ? kExactHalfTerms + 16 : kExactTokens) || p.npad > kUmmaExactCols || p.qbits == 1 || p.qbits == 2 || (up && p.h_terms != 3))
+              : p.h_terms > 1 && !(up && p.h_terms == 2 && (p.qbits == 8 || p.qbits == 4))) return cudaErrorInvalidValue;
+  if (p.x_cols && (p.x_cols % 8 || cols != (p.exact ? 3 : 2) * p.x_cols)) return cudaErrorInvalidValue;
   p.wait_cycles = fused_test_knobs().wait_cycles;
   p.drop_stage = fused_test_knobs().drop_stage;
   const int grid = p.R < 8 * sm_count ? (p.R + 7) / 8 : sm_count;
@@ -1349,7 +1609,7 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
                    : !make_map(&map_x, p.X, p.K, p.ncols_valid, (size_t)p.x_stride, p.npad))
     return cudaErrorNotSupported;
   if (!up) return launch_rows_mode<kGate>(p, grid, smem, s, map_w, map_x, WalkMap<false>{});
-  if (p.walk_all && umma_may_walk(p.B)) {
+  if (p.walk_all && umma_may_walk(p.B) && !p.exact) {
     // wide batches: the union may cover most rows; the kernel then walks every row with tiled boxes of the tile
     // height of R rows (decided on the device from the union's size, so it depends on this call's inputs only)
     WalkMap<true> map_t;
@@ -1372,13 +1632,13 @@ int umma_down_splits(int D, int cols, int sm_count, int max_splits) {
 bool umma_down_supported(int D, int cols) { return D % kTileRows == 0 && cols >= 1 && cols <= kUmmaMaxCols; }
 
 namespace {
-template <int QB>
+template <int QB, bool EX = false>
 cudaError_t launch_down_q(const UmmaDownParams& p, int grid, size_t smem, cudaStream_t s, const CUtensorMap& map_wg,
                           const CUtensorMap& map_wt, const CUtensorMap& map_hm) {
   static unsigned long long configured = 0;
-  const cudaError_t e = allow_dynamic_smem(umma_down_kernel<QB>, 227 * 1024, configured);
+  const cudaError_t e = allow_dynamic_smem(umma_down_kernel<QB, EX>, 227 * 1024, configured);
   if (e != cudaSuccess) return e;
-  return launch_pdl(umma_down_kernel<QB>, dim3(grid), dim3(kThreads + (QB ? 32 * kExpandWarps : 0)), smem, s, p, map_wg,
+  return launch_pdl(umma_down_kernel<QB, EX>, dim3(grid), dim3((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarps : 0)), smem, s, p, map_wg,
                     map_wt, map_hm);
 }
 }  // namespace
@@ -1386,18 +1646,18 @@ cudaError_t launch_down_q(const UmmaDownParams& p, int grid, size_t smem, cudaSt
 cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s) {
   if (p.qbits != 0 && p.qbits != 8 && p.qbits != 4) return cudaErrorInvalidValue;
   if (p.terms < 1) p.terms = 1;
-  if (p.terms > 2 || (p.terms == 2 && !p.qbits)) return cudaErrorInvalidValue;
+  if (p.exact ? p.terms != 3 || p.cols > kExactTokens || p.npad > kUmmaExactCols : p.terms > 2 || (p.terms == 2 && !p.qbits)) return cudaErrorInvalidValue;
   const int own = p.terms * p.cols;  // token columns that carry something
   p.npad = (own + 15) / 16 * 16;
   if (p.cols % 8 || p.cols < p.B || p.npad > kUmmaMaxCols) return cudaErrorInvalidValue;
   p.wait_cycles = fused_test_knobs().wait_cycles;
   const int stage_bytes = kAAtomBytes + p.npad * 128 + p.qbits * kTileRows * kAtomK / 8;
-  int stages = ((own <= kDownPairCols ? 111 : 225) * 1024 - 1024 - 1024) / stage_bytes;
+  int stages = ((own <= kDownPairCols && !p.exact ? 111 : 225) * 1024 - 1024 - 1024) / stage_bytes;
   if (stages > 12) stages = 12;
-  stages &= ~1;
+  stages &= p.exact ? ~3 : ~1;
   if (stages < 2) return cudaErrorInvalidValue;
   p.stages = stages;
-  const size_t smem = 1024 + (size_t)stages * stage_bytes + (3 * stages + 4) * 8 + 64;
+  const size_t smem = 1024 + (size_t)stages * stage_bytes + (3 * stages + 4 + 2 * kMaxIssuers) * 8 + 64;
   const int grid = (p.D / kTileRows) * p.splits;
   alignas(64) CUtensorMap map_wg, map_wt, map_hm;
   // W_down [H, D]: inner dimension d; single-row boxes for the gather, 64-row boxes for the dense walk
@@ -1406,6 +1666,10 @@ cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s) {
   // HmT [terms * h_cols][hm_stride]: inner dimension u; one box of `cols` token rows per term
   if (!make_map(&map_hm, p.hmT, p.hm_stride, p.terms * p.h_cols, (size_t)p.hm_stride, p.cols)) return cudaErrorNotSupported;
   const int g = grid;
+  if (p.exact)
+    return p.qbits == 8   ? launch_down_q<8, true>(p, g, smem, s, map_wg, map_wt, map_hm)
+           : p.qbits == 4 ? launch_down_q<4, true>(p, g, smem, s, map_wg, map_wt, map_hm)
+                          : launch_down_q<0, true>(p, g, smem, s, map_wg, map_wt, map_hm);
   return p.qbits == 8   ? launch_down_q<8>(p, g, smem, s, map_wg, map_wt, map_hm)
          : p.qbits == 4 ? launch_down_q<4>(p, g, smem, s, map_wg, map_wt, map_hm)
                         : launch_down_q<0>(p, g, smem, s, map_wg, map_wt, map_hm);
@@ -1423,8 +1687,8 @@ cudaError_t launch_rmsnorm_limbs(const float* v, int B, int r, int v_stride, con
 }
 
 cudaError_t launch_rmsnorm_split(const float* v, int B, int r, int v_stride, const float* gain, float eps,
-                                 bool use_rms, int cols, void* x2, cudaStream_t s) {
-  return launch_pdl(rmsnorm_split_kernel, dim3(B), dim3(256), 0, s, v, r, v_stride, gain, eps, use_rms ? 1 : 0, cols,
+                                 bool use_rms, int cols, bool exact, void* x2, cudaStream_t s) {
+  return launch_pdl(rmsnorm_split_kernel, dim3(B), dim3(256), 0, s, v, r, v_stride, gain, eps, use_rms ? 1 : 0, cols, exact ? 1 : 0,
                     static_cast<__nv_bfloat16*>(x2));
 }
 

@@ -11,6 +11,8 @@ constexpr int kUmmaActIdentity = 3;
 
 // Token columns one pass of these kernels takes (the N of their MMAs).
 constexpr int kUmmaMaxCols = 256;
+constexpr int kUmmaExactTokens = 64;  // tokens of a pass with exact sums (see umma_kernels.cu) ...
+constexpr int kUmmaExactCols = 128;   // ... and token columns, terms included, of one launch of it
 
 struct UmmaRowsParams {
   const void* W;         // [*, K] bf16 (or int8 / packed int4 codes, see qbits), rows selected by idx (or 0..R-1)
@@ -36,6 +38,8 @@ struct UmmaRowsParams {
   int ncols_valid;
   int B;                 // tokens
   int x_cols;            // GATE: nonzero (a multiple of 8) = token b's vector is the sum of columns b and x_cols + b
+                         //   (exact: and 2 x_cols + b)
+  int exact;             // sums that round as fp32 does: chains of few MMAs added in registers; h in three terms
   const float* b_g;
   const int32_t* g_idx;
   const int8_t* g_sign;
@@ -49,7 +53,7 @@ struct UmmaRowsParams {
   int a_stride;
   void* hmT;             // UP: bf16 [h_terms * h_cols][hm_stride]: h of token b is the sum of rows b and (2 terms) h_cols + b
   int hm_stride;
-  int h_terms, h_cols;   //   2 terms: quantised rows only (0: 1)
+  int h_terms, h_cols;   //   2 terms: quantised rows only (0: 1); exact: 3
   int act_up;            // UP: activation on the up projection (double activation), kUmmaActIdentity = none
   int32_t* status;       // device status word
   int npad, ring_bytes;  // filled by the launcher
@@ -67,6 +71,7 @@ struct UmmaDownParams {
                          // multiple of 64 are zero
   int hm_stride;         // multiple of 64
   int terms, h_cols;     // terms of h (0: 1) and the rows between them
+  int exact;             // see UmmaRowsParams
   int tok0, B;           // tokens [tok0, tok0 + B) of those rows
   int cols;              // B rounded up to a multiple of 8 (token columns of one term)
   int splits;            // the list is cut into this many runs of 64-row blocks
@@ -93,6 +98,6 @@ cudaError_t launch_token_limbs(const void* x, int B, int K, int x_stride, void* 
 cudaError_t launch_rmsnorm_limbs(const float* v, int B, int r, int v_stride, const float* gain, float eps, bool use_rms,
                                  void* limbs, float* scale, cudaStream_t s);
 cudaError_t launch_rmsnorm_split(const float* v, int B, int r, int v_stride, const float* gain, float eps,
-                                 bool use_rms, int cols, void* x2, cudaStream_t s);
+                                 bool use_rms, int cols, bool exact, void* x2, cudaStream_t s);
 
 }  // namespace sffn

@@ -170,3 +170,17 @@ def test_int4_ring_slots_of_short_and_long_shares(mod, D, H):
     check(ffn, x, gate, w, "relu", ("fused", "general"), f"q4 slots {D}x{H}")
     gate, w = make_lopa(mod, D, H, 64, 61, 0.8)
     check(ffn, x, gate, w, "sqrelu", ("auto", "general"), f"q4 lopa slots {D}x{H}")
+
+
+@pytest.mark.parametrize("B,r", [(5, 0), (6, 64), (40, 128)])
+def test_int4_batches_of_odd_row_widths(mod, B, r):
+    D, H = 640, 1500
+    ffn = mod.SparseFFN(D, H, torch.bfloat16, r_max=r, B_max=B)
+    gate, w = make_lopa(mod, D, H, r, 62, 0.85) if r else make_std(D, H, 62, 0.85)
+    x = syn.tokens(B, D, torch.bfloat16, 62, DEV)
+    ref = run_oracle_q4(x, gate, w, "relu")
+    y = ffn.sparse_ffn_forward_q4(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0, ffn.status_words()
+    assert_y_close(y, ref["y"], rel_l2=1e-5, max_abs=5e-5, what=f"B={B} r={r}")  # h to 2^-17 (standard gate) or 2^-24
+    assert_active_set(ffn.last_active(), ref, what=f"B={B} r={r}")

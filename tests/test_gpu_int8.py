@@ -162,6 +162,7 @@ def test_int8_batches_tcgen05_edge_shapes(mod, D, H, B, s):
     (512, 1201, 256, "standard"),   # a full pass
     (512, 1201, 257, "standard"),   # and one token more
     (512, 1201, 129, "lopa"),       # the same for the LoPA gate, whose vector takes two columns a token
+    (384, 1001, 41, "lopa"),        # an odd multiple of 128, LoPA gate: exact sums, a full pass of 40 tokens and one more
 ])
 def test_int8_wide_batches_and_odd_row_widths(mod, D, H, B, kind):
     r = 128

@@ -239,6 +239,27 @@ def test_one_pass_takes_up_to_256_tokens(mod, kind, B):
     assert torch.equal(y, ffn.sparse_ffn_forward(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu"))
 
 
+@pytest.mark.parametrize("D,H,B,r", [(128, 300, 6, 0), (384, 1001, 64, 0), (384, 1001, 65, 0), (1152, 20000, 17, 0), (640, 700, 33, 0),
+                                     (384, 1001, 40, 64), (1408, 900, 41, 192), (640, 19500, 7, 64)])
+def test_batches_of_odd_row_widths_keep_fp32_sums_on_the_tensor_cores(mod, D, H, B, r):
+    # one K block, full passes (64 tokens, LoPA 40) and one more, token columns of every accumulator layout, several tiles a CTA
+    ffn = mod.SparseFFN(D, H, torch.bfloat16, r_max=r, B_max=B)
+    gate, w = make_lopa(mod, D, H, r, torch.bfloat16, 48, 0.9, "diag", True, True, True) if r else make_std(D, H, torch.bfloat16, 48, 0.9)
+    w["b_g"] = syn.bias_from_firing_profile(syn.zipf_firing_profile(H, 1.1, 0.02, 0.9, seed=5)).to(DEV)
+    x = syn.tokens(B, D, torch.bfloat16, 48, DEV)
+    launches0 = ffn.launch_count()
+    y = ffn.sparse_ffn_forward(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+    assert ffn.launch_count() - launches0 != B                   # not once per token
+    # fp32 sums of up to 20000 terms in another order: the tolerance of the fp32 routes
+    run_both_paths(mod, ffn, x, gate, w, "relu", ("auto",), tol=1e-5, what=f"{D}x{H} B={B} r={r}")
+    assert torch.equal(y, ffn.sparse_ffn_forward(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu"))
+    yd = ffn.dense_ffn_forward(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+    assert_y_close(yd, run_oracle(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu", route="dense")["y"], rel_l2=1e-5, max_abs=1e-5)
+    ffn.set_up_activation("silu")
+    ref = run_oracle(x, gate, w["b_g"], w["W_up"], w["W_down"], "sqrelu", act_up="silu")
+    assert_y_close(ffn.sparse_ffn_forward(x, gate, w["b_g"], w["W_up"], w["W_down"], "sqrelu"), ref["y"], rel_l2=1e-5, max_abs=1e-5)
+
+
 @pytest.mark.parametrize("dtype,D", [(torch.float32, 512), (torch.bfloat16, 520), (torch.float32, 776)])
 @pytest.mark.parametrize("kind", ["standard", "lopa"])
 @pytest.mark.parametrize("B", [2, 5, 70])
