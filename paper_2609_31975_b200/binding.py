@@ -45,6 +45,7 @@ def lib_path() -> Path:
     return _PKG / os.environ.get("SFFN_LIBRARY", "libsparse_ffn.so")
 
 
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda i: torch.cuda.current_stream(i).cuda_stream)
 _lib = None
 
 
@@ -104,6 +105,10 @@ def test_set_knob(name: str, value: int):
 
 def _ptr(t):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
+
+
+def _addr(t):
+    return None if t is None else t.data_ptr()
 
 
 def _codes(m):
@@ -241,40 +246,37 @@ class SparseFFN:
         _check("sffn_set_gate_engine", self.lib.sffn_set_gate_engine(self._h, GATE_ENGINE[engine]))
 
     def _gate(self, gate: dict) -> _Gate:
-        g = _Gate()
         if "W_g" in gate:
-            g.kind, g.W_g = 0, _codes(gate["W_g"]).data_ptr()
-        else:
-            g.kind, g.r = 1, _codes(gate["V"]).shape[0]
-            g.V, g.U = _codes(gate["V"]).data_ptr(), _codes(gate["U"]).data_ptr()
-            for k in ("g_idx", "g_sign", "rms_gain"):
-                t = gate.get(k)
-                setattr(g, k, None if t is None else t.data_ptr())
-            g.use_rmsnorm = int(gate.get("use_rmsnorm", True))
-            g.rms_eps = float(gate.get("rms_eps", 1e-5))
-        return g
+            return _Gate(0, 0, _codes(gate["W_g"]).data_ptr())
+        V, get = _codes(gate["V"]), gate.get
+        return _Gate(1, V.shape[0], None, V.data_ptr(), _codes(gate["U"]).data_ptr(), _addr(get("g_idx")), _addr(get("g_sign")),
+                     _addr(get("rms_gain")), int(get("use_rmsnorm", True)), float(get("rms_eps", 1e-5)))
 
     @staticmethod
     def _scales(gate: dict, W_up, W_down) -> _Q8Scales:
-        sc = _Q8Scales()
-        if "W_g" in gate:
-            sc.s_gate = gate["W_g"]["s"].data_ptr()
-        else:
-            sc.s_gate, sc.s_V = gate["U"]["s"].data_ptr(), gate["V"]["s"].data_ptr()
-        sc.s_up, sc.s_down = W_up["s"].data_ptr(), W_down["s"].data_ptr()
-        return sc
+        standard = "W_g" in gate
+        return _Q8Scales(gate["W_g" if standard else "U"]["s"].data_ptr(), None if standard else gate["V"]["s"].data_ptr(),
+                         W_up["s"].data_ptr(), W_down["s"].data_ptr())
+
+    def _out(self, x):
+        return x.new_empty(self.D if x.dim() == 1 else (*x.shape[:-1], self.D), dtype=torch.float32)
 
     def _stream(self, stream):
-        s = torch.cuda.current_stream(self.device) if stream is None else stream
-        return ctypes.c_void_p(s.cuda_stream)
+        if stream is not None:
+            return stream.cuda_stream
+        i = self.device.index
+        return _raw_stream(torch.cuda.current_device() if i is None else i)  # no Stream object for its handle
 
     def _call(self, fn, name, x, gate, b_g, W_up, W_down, act, y, stream):
         B = 1 if x.dim() == 1 else x.shape[0]
-        g = self._gate(gate)
         self._keep = (x, gate, b_g, W_up, W_down, y)
-        _check(name, fn(self._h, _ptr(x), B, ctypes.byref(g), _ptr(b_g), _ptr(W_up), _ptr(W_down),
-                        ACT[act] if isinstance(act, str) else int(act), _ptr(y), self._stream(stream)))
-        self._sync_check(name, B, gate)
+        # plain integers for addresses, and the structure for its pointer: ctypes converts both by itself
+        rc = fn(self._h, x.data_ptr(), B, self._gate(gate), _addr(b_g), _addr(W_up), _addr(W_down),
+                ACT[act] if isinstance(act, str) else int(act), _addr(y), self._stream(stream))
+        if rc:
+            raise SFFNError(name, rc)
+        if os.environ.get("SFFN_SYNC_CHECK") == "1":
+            self._sync_check(name, B, gate)
         return y
 
     def status_words(self, n: int = 8):
@@ -287,7 +289,7 @@ class SparseFFN:
     def _sync_check(self, name, B, gate):
         """With SFFN_SYNC_CHECK=1 in the environment every call is followed by a synchronisation and a look at the
         status word, so that the call that set it is the one that raises (diagnostics; slow)."""
-        if os.environ.get("SFFN_SYNC_CHECK") != "1" or torch.cuda.is_current_stream_capturing():
+        if torch.cuda.is_current_stream_capturing():
             return
         w = self.status_words()
         if w[0] != 0:
@@ -296,11 +298,12 @@ class SparseFFN:
 
     def _call_q8(self, fn, name, x, gate, b_g, W_up, W_down, act, y, stream):
         B = 1 if x.dim() == 1 else x.shape[0]
-        g, sc = self._gate(gate), self._scales(gate, W_up, W_down)
         self._keep = (x, gate, b_g, W_up, W_down, y)
-        _check(name, fn(self._h, _ptr(x), B, ctypes.byref(g), _ptr(b_g), _ptr(_codes(W_up)), _ptr(_codes(W_down)),
-                        ctypes.byref(sc), ACT[act] if isinstance(act, str) else int(act), _ptr(y),
-                        self._stream(stream)))
+        rc = fn(self._h, x.data_ptr(), B, self._gate(gate), _addr(b_g), _addr(_codes(W_up)), _addr(_codes(W_down)),
+                self._scales(gate, W_up, W_down), ACT[act] if isinstance(act, str) else int(act), _addr(y),
+                self._stream(stream))
+        if rc:
+            raise SFFNError(name, rc)
         return y
 
     def prepared(self, x, gate, b_g, W_up, W_down, act, y, *, dense=False, host=False, stream=None):
@@ -337,26 +340,26 @@ class SparseFFN:
     def sparse_ffn_forward(self, x, gate, b_g, W_up, W_down, act="relu", y=None, stream=None):
         """y = W_down^T (A(gate(x) + b_g) * (W_up x)) touching only the rows of fired neurons."""
         if y is None:
-            y = torch.empty((*x.shape[:-1], self.D), dtype=torch.float32, device=x.device)
+            y = self._out(x)
         return self._call(self.lib.sparse_ffn_forward, "sparse_ffn_forward", x, gate, b_g, W_up, W_down, act, y, stream)
 
     def dense_ffn_forward(self, x, gate, b_g, W_up, W_down, act="relu", y=None, stream=None):
         """The dense comparator: same function, all H rows read."""
         if y is None:
-            y = torch.empty((*x.shape[:-1], self.D), dtype=torch.float32, device=x.device)
+            y = self._out(x)
         return self._call(self.lib.dense_ffn_forward, "dense_ffn_forward", x, gate, b_g, W_up, W_down, act, y, stream)
 
     def sparse_ffn_forward_q8(self, x, gate, b_g, W_up, W_down, act="relu", y=None, stream=None):
         """:meth:`sparse_ffn_forward` on int8 weights with one fp32 scale per row (see the class docstring)."""
         if y is None:
-            y = torch.empty((*x.shape[:-1], self.D), dtype=torch.float32, device=x.device)
+            y = self._out(x)
         return self._call_q8(self.lib.sparse_ffn_forward_q8, "sparse_ffn_forward_q8", x, gate, b_g, W_up, W_down,
                              act, y, stream)
 
     def dense_ffn_forward_q8(self, x, gate, b_g, W_up, W_down, act="relu", y=None, stream=None):
         """The dense comparator on int8 weights."""
         if y is None:
-            y = torch.empty((*x.shape[:-1], self.D), dtype=torch.float32, device=x.device)
+            y = self._out(x)
         return self._call_q8(self.lib.dense_ffn_forward_q8, "dense_ffn_forward_q8", x, gate, b_g, W_up, W_down,
                              act, y, stream)
 
@@ -364,14 +367,14 @@ class SparseFFN:
         """:meth:`sparse_ffn_forward` on 4-bit weights: every matrix is ``dict(q=uint8 [rows, cols / 2], s=float32
         [rows])``, two's-complement codes, even column in the low nibble (sparse_ffn_forward_q4 of the header)."""
         if y is None:
-            y = torch.empty((*x.shape[:-1], self.D), dtype=torch.float32, device=x.device)
+            y = self._out(x)
         return self._call_q8(self.lib.sparse_ffn_forward_q4, "sparse_ffn_forward_q4", x, gate, b_g, W_up, W_down,
                              act, y, stream)
 
     def dense_ffn_forward_q4(self, x, gate, b_g, W_up, W_down, act="relu", y=None, stream=None):
         """The dense comparator on 4-bit weights."""
         if y is None:
-            y = torch.empty((*x.shape[:-1], self.D), dtype=torch.float32, device=x.device)
+            y = self._out(x)
         return self._call_q8(self.lib.dense_ffn_forward_q4, "dense_ffn_forward_q4", x, gate, b_g, W_up, W_down,
                              act, y, stream)
 
