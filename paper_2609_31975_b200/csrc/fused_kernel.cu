@@ -120,7 +120,7 @@ struct SmemLayout {
     aval = take(slab_max * 4);
     slot_a = take((n_act_slots + act_extra) * 4);
     red = take(6 * kRedStride * 4);  // two buffers per act group (four warps each), up to three groups
-    ctl = take(8 * 4);
+    ctl = take((8 + 16) * 4);  // control words, then one sum of squares per staging warp (LoPA)
     bars = take(2 * (n_gate_slots + n_act_slots + act_extra) * 8 + 8);  // + one for the CTA's rows of V (LoPA)
     row_params = take((lopa || scaled) ? (1 + (lopa ? 2 : 0) + (scaled ? 1 : 0)) * slab_max * 4 : 0);  // per-neuron gate parameters
     row_scales = take(scaled ? 2 * slab_max * 4 : 0);     // int8 rows: scales of the slab's W_up / W_down rows
@@ -413,6 +413,8 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
   const float* xsc = reinterpret_cast<const float*>(smem + L.xlimb + 128 + kTokenLimbs * D);  // scale of the limbs of chunk c
   const uint4* xl = reinterpret_cast<const uint4*>(smem + L.xlimb + 128);  // limb l of chunk c: xl[l * nvecD + c]
   volatile int* ctl = reinterpret_cast<volatile int*>(smem + L.ctl);
+  float* wss = reinterpret_cast<float*>(smem + L.ctl) + 8;
+  static_assert(kStageThreads / 32 <= 16, "one sum of squares per staging warp");
   const uint32_t bars = smem_u32(smem + L.bars);
   const uint32_t full_gate = bars, empty_gate = bars + 8 * NG;
   const uint32_t full_act = bars + 16 * NG, empty_act = bars + 16 * NG + 8 * NA;
@@ -540,6 +542,9 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
     }
   }
 
+  const bool use_rms = LOPA && p.use_rmsnorm;
+  const float* gain = use_rms ? p.gain : nullptr;
+  const float inv_r = LOPA ? 1.f / (float)K : 0.f, eps = p.eps;
   // ---- everyone else: wait for the predecessor in the stream, then stage the token ------------
   pdl_wait();
   if (tid == kStageBase) SFFN_GSTAMP(11);
@@ -555,12 +560,25 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
   constexpr int kGroup = EPV / XEPV;  // threads that share a chunk of the token (2 or 4; 1 where not used)
   int8_t* planes = reinterpret_cast<int8_t*>(smem + L.xlimb + 128);
   float* xsc_w = reinterpret_cast<float*>(smem + L.xlimb + 128 + kTokenLimbs * D);
-  for (int cx0 = warp * 32 - kStageBase; cx0 < D / XEPV; cx0 += kStageThreads) {  // warp-uniform trip count (shuffles)
+  // A thread's chunks of the token are all requested before the first is used: one at a time, the second and third of a
+  // wide token (512 chunks of 4096 bf16 entries for 448 threads) each cost another round trip to L2.
+  constexpr int kTokBatch = 3;
+  for (int cb = warp * 32 - kStageBase; cb < D / XEPV; cb += kTokBatch * kStageThreads) {  // warp-uniform trip counts (shuffles)
+  uint4 tok[kTokBatch];
+#pragma unroll
+  for (int i = 0; i < kTokBatch; ++i) {
+    const int cx = cb + i * kStageThreads + lane;
+    tok[i] = cx < D / XEPV ? __ldg(reinterpret_cast<const uint4*>(p.x) + cx) : make_uint4(0u, 0u, 0u, 0u);
+  }
+#pragma unroll
+  for (int i = 0; i < kTokBatch; ++i) {
+    const int cx0 = cb + i * kStageThreads;
+    if (cx0 >= D / XEPV) break;
     const int cx = cx0 + lane;
     const bool on = cx < D / XEPV;
     float f[XEPV];
     if (on) {
-      Elem<X>::unpack(__ldg(reinterpret_cast<const uint4*>(p.x) + cx), f);
+      Elem<X>::unpack(tok[i], f);
 #pragma unroll
       for (int g4 = 0; g4 < XEPV / 4; ++g4) {
         const int k0 = cx * XEPV + 4 * g4;  // first of four consecutive elements: quarter (k0 % EPV) / 4 of chunk k0 / EPV
@@ -606,6 +624,8 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
       }
     }
   }
+  }
+  float gscale = 1.f;  // LoPA: 1 / RMS of the gate vector, applied to the finished dot products
   if (LOPA) {
     // Rank-r stage of the LoPA gate, v = V x, spread over the grid: this CTA computes its share of the rows of V,
     // publishes them, and collects everybody's.  All CTAs of the call become resident without waiting for this one
@@ -622,8 +642,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
     // where they do not fit beside the sums (wide rows, high rank) they are read from global memory instead
     const uint4* vsm = p.v_in_smem ? reinterpret_cast<const uint4*>(act_ring)
                                    : reinterpret_cast<const uint4*>(static_cast<const char*>(p.V) + (size_t)vlo * row_bytes);
-    float* wss = reinterpret_cast<float*>(act_ring + (p.v_in_smem ? (size_t)v_max * row_bytes : 0));
-    float* vpart = wss + 32;
+    float* vpart = reinterpret_cast<float*>(act_ring + (p.v_in_smem ? (size_t)v_max * row_bytes : 0)) + 32;
     named_bar_sync(5, kStageThreads);  // the token is staged
     mbar_wait(v_bar, 0, ctl, p.status, p.wait_cycles, 50);
     // the warps share the CTA's rows: wpr warps per row (one when there are more rows than warps), each lane sums its
@@ -632,9 +651,15 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
     const int wpr = nrows > 0 && nrows < kSW ? kSW / nrows : 1;
     for (int row = sw / wpr; row < nrows; row += kSW / wpr) {
       const int part = sw % wpr;
-      float a = 0.f;
-      for (int c = part * 32 + lane; c < nvecD; c += wpr * 32) a = chunk_dot<T>(vsm[(size_t)row * nvecD + c], sx, c, nvecD, a);
-      a = warp_sum(a);
+      float a0 = 0.f, a1 = 0.f;
+      int c = part * 32 + lane;
+      for (; c + wpr * 32 < nvecD; c += wpr * 64) {
+        const uint4 w0 = vsm[(size_t)row * nvecD + c], w1 = vsm[(size_t)row * nvecD + c + wpr * 32];
+        a0 = chunk_dot<T>(w0, sx, c, nvecD, a0);
+        a1 = chunk_dot<T>(w1, sx, c + wpr * 32, nvecD, a1);
+      }
+      if (c < nvecD) a0 = chunk_dot<T>(vsm[(size_t)row * nvecD + c], sx, c, nvecD, a0);
+      const float a = warp_sum(a0 + a1);
       if (lane == 0) vpart[row * wpr + part] = a;
     }
     named_bar_sync(5, kStageThreads);
@@ -652,6 +677,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
       const int k1 = k + kStageThreads;
       unsigned long long w0 = 0, w1 = 0;
       bool have0 = false, have1 = k1 >= r;
+      const float g0 = gain ? __ldg(gain + k) : 1.f, g1 = gain && k1 < r ? __ldg(gain + k1) : 1.f;  // parameters: under way meanwhile
       for (;;) {
         if (!have0) asm volatile("ld.global.cg.b64 %0, [%1];" : "=l"(w0) : "l"(p.vtag + k) : "memory");
         if (!have1) asm volatile("ld.global.cg.b64 %0, [%1];" : "=l"(w1) : "l"(p.vtag + k1) : "memory");
@@ -663,21 +689,22 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
       const float v0 = __uint_as_float((uint32_t)w0), v1 = k1 < r ? __uint_as_float((uint32_t)w1) : 0.f;
       ss = fmaf(v0, v0, ss);
       ss = fmaf(v1, v1, ss);
-      sn[vec_pos<EPV>(k, r)] = v0;
-      if (k1 < r) sn[vec_pos<EPV>(k1, r)] = v1;
+      sn[vec_pos<EPV>(k, r)] = v0 * g0;
+      if (k1 < r) sn[vec_pos<EPV>(k1, r)] = v1 * g1;
     }
-    // n = RMSNorm(v) (or v): the warps' sums of squares are added in a fixed order by everyone
+    // n = RMSNorm(v) (or v): 1 / RMS is left to the finished dot products, so that no second pass over the vector and no
+    // second barrier stand between the values' arrival and the gate (1 us of 5.4 at r = 512)
     ss = warp_sum(ss);
     if (lane == 0) wss[sw] = ss;
-    named_bar_sync(5, kStageThreads);
-    float tot = 0.f;
-#pragma unroll
-    for (int i = 0; i < kSW; ++i) tot += wss[i];
-    const float inv = p.use_rmsnorm ? rsqrtf(tot / (float)r + p.eps) : 1.f;
-    for (int k = st; k < r; k += kStageThreads)
-      sn[vec_pos<EPV>(k, r)] *= ((p.use_rmsnorm && p.gain) ? p.gain[k] : 1.f) * inv;
   }
   named_bar_sync(3, kThreads);
+  if (LOPA && use_rms) {
+    // the warps' sums of squares, added in a fixed order by everyone
+    float tot = 0.f;
+#pragma unroll
+    for (int i = 0; i < kStageThreads / 32; ++i) tot += wss[i];
+    gscale = rsqrtf(tot * inv_r + eps);
+  }
   if (tid == kStageBase) SFFN_STAMP(0);
 
   const float* gvec = LOPA ? sn : sx;  // the vector every gate row is dotted with
@@ -901,7 +928,8 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
       if (lane == rr) mine = z;
     }
     if (lane < rows) {
-      const float z = kScaled ? fmaf(mine, scale, add) : mine + add;
+      if (LOPA) scale *= gscale;
+      const float z = kScaled || LOPA ? fmaf(mine, scale, add) : mine + add;
       const bool fired = z > 0.f;
       if (!p.dense && (fired || !p.flag_or) && SFFN_IN_BOUNDS(j0 + lane < p.H && r0 + lane < p.slab_max, p.status, 3))
         p.flag[j0 + lane] = fired ? 1 : 0;
