@@ -82,9 +82,9 @@ typedef enum { SFFN_GATE_STANDARD = 0, SFFN_GATE_LOPA = 1 } sffn_gate_kind;
 /* Which kernels serve a call.  AUTO picks the fused kernels for B = 1 when the shape allows it and the
  * tcgen05 tensor-core kernels for batches (B >= 2) of bf16 tokens with bf16, int8 or int4 rows (int8 rows are
  * multiplied as int8 against the tokens split into int8 limbs, or, like int4 rows, expanded to bf16 in shared
- * memory on their way to the tensor cores; more than 256 tokens (LoPA gate: 128; rows of
- * an odd multiple of 128 elements: 64, LoPA 40) run in passes of as many, the list of fired neurons being the union over
- * all passes).  A batch those kernels do not take (fp32
+ * memory on their way to the tensor cores; more than 256 tokens (LoPA gate: 128; int8 / int4 rows multiplied as int8: 64;
+ * bf16 rows of an odd multiple of 128 elements: 64; any such rows under a LoPA gate: 40) run in passes of as many, the list
+ * of fired neurons being the union over all passes).  A batch those kernels do not take (fp32
  * operands, a row width they do not tile) runs the fused kernel once per token with the fired flags OR-ed,
  * which is faster than the CUDA-core batch kernels; what is left goes to the general CUDA-core kernels.
  * The others force one family (SFFN_ERR_UNSUPPORTED if it cannot serve the call): GENERAL = CUDA-core
@@ -184,10 +184,10 @@ int dense_ffn_forward(sffn_handle* handle, const void* x, int B, const sffn_gate
  * as the bytes 16 x code), all sums in fp32 beyond a chunk; LoPA gates use fp32 arithmetic throughout.  A batch runs
  * the tcgen05 batch kernels (D a multiple of 256 -- five tokens or more, LoPA six: of 128 -- and r of 64; otherwise, or under
  * SFFN_PATH_FUSED, the fused kernel once per token; the list of fired neurons is the union over the tokens).  There the
- * gate and up products of up to 64 tokens with int8 rows are int8 x int8 with int32 accumulators, each token entering as
- * four int8 limbs and a scale (x = s (q0 + q1/128 + q2/128^2 + q3/128^3) up to 2^-22 max|x|; D a multiple of 256, r of
- * 128; int4 rows take the same route, their nibbles expanded to int8 in shared memory); the down product, larger batches
- * and other widths expand the codes to bf16 in shared memory; row scales are applied to the accumulator rows.  The CUDA-core kernels (fp32 arithmetic on the decoded codes) serve
+ * gate and up products of int8 rows are int8 x int8 with int32 accumulators, each token entering as four int8 limbs and a
+ * scale (x = s (q0 + q1/128 + q2/128^2 + q3/128^3) up to 2^-22 max|x|; D a multiple of 256, r of 128; int4 rows take the
+ * same route, their nibbles expanded to int8 in shared memory); the down product and other widths expand the codes to bf16
+ * in shared memory; row scales are applied to the accumulator rows.  The CUDA-core kernels (fp32 arithmetic on the decoded codes) serve
  * SFFN_PATH_GENERAL (SFFN_PATH_MMA_SYNC: SFFN_ERR_UNSUPPORTED).  Converting a trained model to this format is
  * an offline step outside this library. */
 typedef struct {

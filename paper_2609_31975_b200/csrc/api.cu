@@ -285,9 +285,19 @@ thread_local int g_last_cuda_line = 0;
 // Whether a batch takes the tcgen05 kernels with exact sums (see h_terms_for).
 bool exact_batch(int D, bool quantised, bool lopa) { return D % 256 != 0 && (!quantised || lopa); }
 
+// Whether a quantised batch multiplies its codes as int8 against the tokens' int8 limbs.
+bool limb_batch(int D, int gate_k) {
+  return D % 256 == 0 && sffn::umma_rows_native_i8_supported(D, 1) && sffn::umma_rows_native_i8_supported(gate_k, 1);
+}
+
 // Tokens that one pass of the tcgen05 kernels takes: 256 columns of the gate GEMM's token operand, which the LoPA
-// vector's high and low parts share; with exact sums 64, or what fits 128 columns at three terms each.
-int umma_pass_tokens(int D, bool quantised, bool lopa) {
+// vector's high and low parts share; with exact sums 64, or what fits 128 columns at three terms each.  Quantised rows
+// that go against limbs: 64 tokens, four limbs each, in larger batches too.  Codes expanded to bf16 would let 256 go at
+// once, but their sums are fp32 ones that truncate, and the LoPA vector enters with 16 bits, where limbs have exact int32
+// sums and 2^-22: a neuron near zero would fire or not by the size of the batch (int8, 4096 x 14336, 200 tokens: 366 us
+// in passes of 64, 152 in one).
+int umma_pass_tokens(int D, int gate_k, bool quantised, bool lopa) {
+  if (quantised && limb_batch(D, gate_k)) return kMaxMmaTokens;
   if (exact_batch(D, quantised, lopa)) return lopa ? sffn::kUmmaExactCols / 3 / 8 * 8 : sffn::kUmmaExactTokens;
   return lopa ? kMaxUmmaTokens / 2 : kMaxUmmaTokens;
 }
@@ -305,11 +315,9 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
   // int8 rows whose K blocks are whole (128 codes): multiplied as int8 against the tokens' int8 limbs, nothing to expand
   // (the down projection keeps the expansion: its B operand, Hm, has no scale known before the whole of it exists)
   // (int4 rows: the nibbles expanded to int8 on the way, for the same MMAs)
-  // More than 64 tokens (four limbs each: 256 columns) take the expansion to bf16 in all three GEMMs.
-  // Odd multiples of 128 expand as well: bf16 tokens enter exactly, where limbs with one scale per token would cost a token
-  // with an outlier some of what the single-token route, which has a scale per chunk, keeps.
-  const bool native = q8 && D % 256 == 0 && B <= kMaxMmaTokens && umma_rows_native_i8_supported(D, B) &&
-                      umma_rows_native_i8_supported(g->kind == SFFN_GATE_LOPA ? g->r : D, B);
+  // Odd multiples of 128 expand to bf16: bf16 tokens enter exactly, where limbs with one scale per token would cost a
+  // token with an outlier some of what the single-token route, which has a scale per chunk, keeps.
+  const bool native = q8 && limb_batch(D, g->kind == SFFN_GATE_LOPA ? g->r : D);
   const int wq_rows = native ? (qbits == 8 ? 1 : 2) : wq;
   void* xlimb = h->ws + h->L.xlimb;
   void* nlimb = h->ws + h->L.nlimb;
@@ -616,7 +624,7 @@ int run(sffn_handle* h, const void* x, int B, const sffn_gate* g, const float* b
   const bool umma_ok = h->path != SFFN_PATH_MMA_SYNC && sffn::umma_rows_supported(gate_k, 1) &&
                        sffn::umma_rows_supported(h->D, 1) && sffn::umma_down_supported(h->D, 1) &&
                        (h->D % 256 == 0 || B >= (exact_batch(h->D, q8 != nullptr, lopa_gate) ? kExactMinTokens : kOddWidthMinTokens));
-  const int pass_max = umma_ok ? umma_pass_tokens(h->D, q8 != nullptr, lopa_gate) : kMaxMmaTokens;
+  const int pass_max = umma_ok ? umma_pass_tokens(h->D, gate_k, q8 != nullptr, lopa_gate) : kMaxMmaTokens;
   const bool tensor_batch = h->dtype == SFFN_BF16 && B >= 2 && h->path != SFFN_PATH_GENERAL && h->path != SFFN_PATH_FUSED &&
                             (umma_ok || (!q8 && sffn::batched_mma_supported(h->D, gate_k, 1)));
   // Any other batch (fp32 operands, a row width the tensor-core kernels do not tile, SFFN_PATH_FUSED): the single-token

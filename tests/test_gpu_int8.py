@@ -157,15 +157,16 @@ def test_int8_batches_tcgen05_edge_shapes(mod, D, H, B, s):
 @pytest.mark.parametrize("D,H,B,kind", [
     (128, 300, 5, "standard"),      # one column tile of the down projection, one K block
     (384, 1001, 130, "standard"),   # an odd multiple of 128: h in two bf16 values, the down projection in two passes
-    (640, 2000, 64, "standard"),    # the most tokens that run on int8 limbs
-    (512, 2000, 65, "standard"),    # one more: codes expanded to bf16 in all three GEMMs
-    (512, 1201, 256, "standard"),   # a full pass
+    (640, 2000, 64, "standard"),    # an odd multiple of 128, the down projection in one pass
+    (512, 2000, 65, "standard"),    # int8 limbs: a full pass of 64 tokens and one more
+    (512, 1201, 256, "standard"),   # four full passes
     (512, 1201, 257, "standard"),   # and one token more
-    (512, 1201, 129, "lopa"),       # the same for the LoPA gate, whose vector takes two columns a token
+    (512, 1201, 129, "lopa"),       # the same for the LoPA gate
+    (512, 1201, 129, "lopa64"),     # a rank that limbs do not tile: codes expanded to bf16, 128 tokens and one more
     (384, 1001, 41, "lopa"),        # an odd multiple of 128, LoPA gate: exact sums, a full pass of 40 tokens and one more
 ])
 def test_int8_wide_batches_and_odd_row_widths(mod, D, H, B, kind):
-    r = 128
+    r = 64 if kind == "lopa64" else 128
     ffn = mod.SparseFFN(D, H, torch.bfloat16, r_max=r, B_max=B)
     gate, w = make_std(D, H, 16, 0.9) if kind == "standard" else make_lopa(mod, D, H, r, 16, 0.9)
     w["b_g"] = syn.bias_from_firing_profile(syn.zipf_firing_profile(H, 1.1, 0.02, 0.9, seed=5)).to(DEV)
@@ -180,6 +181,46 @@ def test_int8_wide_batches_and_odd_row_widths(mod, D, H, B, kind):
     assert_y_close(y, ref["y"], what=f"q8 wide {kind} {D}x{H} B={B}", **tol)
     assert_active_set(ffn.last_active(), ref, what=f"q8 wide {kind} {D}x{H} B={B}")
     assert torch.equal(y, ffn.sparse_ffn_forward_q8(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu"))
+
+
+def pack(q, qbits):
+    """Codes as the entry points take them: int8, or two 4-bit codes a byte."""
+    if qbits == 8:
+        return q.to(DEV)
+    n = q.bitwise_and(15).view(torch.uint8)
+    return (n[:, 0::2] | (n[:, 1::2] << 4)).to(DEV)
+
+
+@pytest.mark.parametrize("qbits", [8, 4])
+@pytest.mark.parametrize("kind", ["standard", "lopa"])
+@pytest.mark.parametrize("B", [5, 64, 65, 200])
+def test_quantised_batches_of_any_size_keep_int32_sums_and_22_bits_of_the_token(mod, qbits, kind, B):
+    # Pre-activations that are what is left when large terms cancel, below 2^-24 of those terms (standard) or 2^-16 of the
+    # vector's largest entry (LoPA): int32 sums against limbs of 2^-22 keep them, sums or vectors of fewer bits give zero.
+    D, H, r, top = 512, 600, 128, 2 ** (qbits - 1) - 1
+    ones = lambda n: torch.ones(n, device=DEV)  # noqa: E731
+    ffn = mod.SparseFFN(D, H, torch.bfloat16, r_max=r, B_max=B)
+    x = torch.zeros((B, D))
+    sign = torch.where(torch.arange(H) % 3 == 1, 1, -1).to(torch.int8)  # every third neuron fires
+    x[:, 0] = 127.0
+    if kind == "standard":
+        x[:, 1], x[:, 2] = 127.0, 2.0 ** -18
+        q = torch.zeros((H, D), dtype=torch.int8)
+        q[:, 0], q[:, 1], q[:, 2] = top, -top, sign
+        gate = {"W_g": dict(q=pack(q, qbits), s=ones(H))}
+    else:
+        x[:, 1], x[:, 2] = 0.25, 2.0 ** -14
+        V, U = torch.zeros((r, D), dtype=torch.int8), torch.zeros((H, r), dtype=torch.int8)
+        V[0, 0] = V[0, 1] = V[0, 2] = V[1, 0] = V[1, 1] = 1   # v0 = 127.25 + 2^-14, v1 = 127.25
+        U[:, 0], U[:, 1] = sign, -sign
+        gate = dict(V=dict(q=pack(V, qbits), s=ones(r)), U=dict(q=pack(U, qbits), s=ones(H)), use_rmsnorm=False)
+    up = torch.randint(-top, top + 1, (H, D), generator=torch.Generator().manual_seed(3)).to(torch.int8)
+    w = dict(q=pack(up, qbits), s=torch.full((H,), 0.01, device=DEV))
+    call = ffn.sparse_ffn_forward_q8 if qbits == 8 else ffn.sparse_ffn_forward_q4
+    call(x.bfloat16().to(DEV), gate, None, w, w, "relu")
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0
+    assert torch.equal(ffn.last_active().cpu().long(), torch.nonzero(sign > 0)[:, 0])
 
 
 @pytest.mark.parametrize("path", ["general", "fused"])
