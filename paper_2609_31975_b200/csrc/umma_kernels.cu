@@ -345,6 +345,16 @@ struct WalkMap<false> {
   __device__ const CUtensorMap* get() const { return nullptr; }
 };
 
+// The leading 8 bits of v as bf16; v keeps the rest.  Nothing is left of an infinite value or NaN, and a finite one beyond the
+// largest bf16 leaves what is above that.
+__device__ __forceinline__ __nv_bfloat16 take_bf16(float& v) {
+  __nv_bfloat16 t = __float2bfloat16(v);
+  if (!(fabsf(__bfloat162float(t)) < INFINITY)) t = __float2bfloat16_rz(v);
+  const float f = __bfloat162float(t);
+  v = fabsf(f) < INFINITY ? v - f : 0.f;
+  return t;
+}
+
 // Exact sums (EX): the tensor cores truncate when they add onto an accumulator, so a sum over K = 2688 comes out low by
 // 1e-6 of its typical size, ten times what fp32 rounding leaves.  Here every two MMAs (K = 32) start an accumulator of
 // their own; the epilogue warps add a stage's accumulators in fp32 registers, which round to nearest.  An issuer has one
@@ -395,7 +405,7 @@ __device__ __forceinline__ void add_stage(uint32_t taddr, int accs, int npad, in
       for (int q = 0; q < 16; ++q)
         if (g + q < HALF) {  // (the upper eight are not used where there are none)
           const float y = part[q] - low[g + q], t = sum[g + q] + y;
-          low[g + q] = (t - sum[g + q]) - y;
+          low[g + q] = fabsf(t) < INFINITY ? (t - sum[g + q]) - y : 0.f;  // an infinite sum stays one
           sum[g + q] = t;
         }
     }
@@ -689,9 +699,12 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
     tc_fence_after();
     // h of one (neuron, token): one bf16 value, or (quantised rows of some widths) two that add up to 16 bits of it
     auto store_h = [&](__nv_bfloat16* dst, float h) {
-      const __nv_bfloat16 t = __float2bfloat16(h);
-      *dst = t;
-      if (kQ && p.h_terms == 2) dst[(size_t)p.h_cols * p.hm_stride] = __float2bfloat16(h - __bfloat162float(t));
+      if (kQ && p.h_terms == 2) {
+        *dst = take_bf16(h);
+        dst[(size_t)p.h_cols * p.hm_stride] = __float2bfloat16(h);
+      } else {
+        *dst = __float2bfloat16(h);
+      }
     };
     if constexpr (kNat) {
       // int32 accumulators, four columns per token (its limbs, most significant first, 7 bits apart):
@@ -738,8 +751,9 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
 #pragma unroll
         for (int q = 0; q < 8; ++q)
           if (row_ok && c0 + q < B)
+            // (a neuron that did not fire for this token adds zero whatever its W_up row holds)
             store_h(hm + (size_t)(c0 + q) * p.hm_stride,
-                    kQ ? av[q] * activation(act_up, v[q] * sc) * osc : av[q] * activation(act_up, v[q]));
+                    av[q] == 0.f ? 0.f : kQ ? av[q] * activation(act_up, v[q] * sc) * osc : av[q] * activation(act_up, v[q]));
       }
     } else {
       const int act = p.act;
@@ -813,16 +827,15 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
       for (int i = 0; i < kHalf; ++i) {
         const int b = c0 + i;
         if (b < B) {
-          float h = p.a[(size_t)b * p.a_stride + j] * activation(p.act_up, kQ ? sum[i] * sc : sum[i]);
+          const float av = p.a[(size_t)b * p.a_stride + j];
+          // a neuron that did not fire for this token adds zero whatever its W_up row holds
+          float h = av == 0.f ? 0.f : av * activation(p.act_up, kQ ? sum[i] * sc : sum[i]);
           if (kQ) h *= osc;
           // 24 bits of h as three bf16 values
-          const __nv_bfloat16 h0 = __float2bfloat16(h);
-          h -= __bfloat162float(h0);
-          const __nv_bfloat16 h1 = __float2bfloat16(h);
           __nv_bfloat16* dst = hm + (size_t)b * p.hm_stride;
-          dst[0] = h0;
-          dst[term] = h1;
-          dst[2 * term] = __float2bfloat16(h - __bfloat162float(h1));
+          dst[0] = take_bf16(h);
+          dst[term] = take_bf16(h);
+          dst[2 * term] = __float2bfloat16(h);
         }
       }
     } else {
@@ -1382,13 +1395,10 @@ __global__ void __launch_bounds__(256) rmsnorm_split_kernel(const float* v, int 
     inv = rsqrtf(tot / (float)r + eps);
   }
   for (int k = threadIdx.x; k < r; k += blockDim.x) {
-    const float n = use_rms ? (gain ? gain[k] : 1.f) * vb[k] * inv : vb[k];
-    const __nv_bfloat16 hi = __float2bfloat16(n);
-    x2[(size_t)b * r + k] = hi;
-    const float low = n - __bfloat162float(hi);
-    const __nv_bfloat16 mid = __float2bfloat16(low);
-    x2[(size_t)(cols + b) * r + k] = mid;
-    if (exact) x2[(size_t)(2 * cols + b) * r + k] = __float2bfloat16(low - __bfloat162float(mid));
+    float n = use_rms ? (gain ? gain[k] : 1.f) * vb[k] * inv : vb[k];
+    x2[(size_t)b * r + k] = take_bf16(n);
+    x2[(size_t)(cols + b) * r + k] = take_bf16(n);
+    if (exact) x2[(size_t)(2 * cols + b) * r + k] = __float2bfloat16(n);
   }
 }
 

@@ -260,6 +260,51 @@ def test_batches_of_odd_row_widths_keep_fp32_sums_on_the_tensor_cores(mod, D, H,
     assert_y_close(ffn.sparse_ffn_forward(x, gate, w["b_g"], w["W_up"], w["W_down"], "sqrelu"), ref["y"], rel_l2=1e-5, max_abs=1e-5)
 
 
+@pytest.mark.parametrize("kind,D", [("standard", 384), ("lopa", 384), ("int8", 384), ("int8_lopa", 384)])
+def test_odd_width_batches_treat_infinities_as_the_single_token_kernel_does(mod, kind, D):
+    # one token overflows its sums, one row of W_up is infinite and fires for one other token: only these two tokens' y may
+    # be non-finite, and the same neurons fire as token by token
+    H, r, B = 1000, 64, 8
+    ffn = mod.SparseFFN(D, H, torch.bfloat16, r_max=r, B_max=B)
+    x = syn.tokens(B, D, torch.bfloat16, 49, DEV)
+    call = ffn.sparse_ffn_forward_q8 if kind.startswith("int8") else ffn.sparse_ffn_forward
+    if kind == "standard":
+        gate, w = make_std(D, H, torch.bfloat16, 49, 0.9)
+        x[3, 0] = float("inf")                       # z = +-Inf
+    elif kind == "lopa":
+        gate, w = make_lopa(mod, D, H, r, torch.bfloat16, 49, 0.9, "diag", True, True, False)
+        gate["V"][0, 0] = 1e3
+        x[:, 0] = 0
+        x[3, 0] = 1e36                               # one entry of V x overflows, the others do not
+    else:
+        lopa = kind == "int8_lopa"
+        w = syn.lopa_ffn_q8(D, H, r, 49, DEV, sparsity=0.9) if lopa else syn.standard_ffn_q8(D, H, 49, DEV, sparsity=0.9)
+        gate = {"V": w["V"], "U": w["U"], "use_rmsnorm": False} if lopa else {"W_g": w["W_g"]}
+        x[3, 0] = 1e35 if lopa else 1e37             # finite sums, h = a u overflows
+    codes = isinstance(w["W_up"], dict)
+    if not codes:
+        ffn.set_path("fused")
+        fires = []
+        for t in range(B):
+            call(x[t], gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+            fires.append(set(ffn.last_active().tolist()))
+        alone = sorted(fires[5] - set().union(*(fires[t] for t in range(B) if t != 5)))
+        w["W_up"][alone[0]] = float("inf")
+    out = {}
+    for path in ("fused", "auto"):
+        ffn.set_path(path)
+        y = call(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+        torch.cuda.synchronize()
+        assert ffn.device_status() == 0
+        out[path] = (y, ffn.last_active())
+    assert torch.equal(out["auto"][1], out["fused"][1])
+    good = torch.isfinite(out["fused"][0]).all(dim=1)
+    assert not good[3] and good.sum() == (B - 1 if codes else B - 2)
+    assert torch.equal(torch.isfinite(out["auto"][0]).all(dim=1), good)
+    for t in good.nonzero()[:, 0].tolist():
+        assert_y_close(out["auto"][0][t], out["fused"][0][t].double().cpu().numpy(), rel_l2=1e-3, max_abs=1e-3)  # int8: limbs of 3e-5
+
+
 @pytest.mark.parametrize("dtype,D", [(torch.float32, 512), (torch.bfloat16, 520), (torch.float32, 776)])
 @pytest.mark.parametrize("kind", ["standard", "lopa"])
 @pytest.mark.parametrize("B", [2, 5, 70])
