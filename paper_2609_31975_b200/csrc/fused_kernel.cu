@@ -210,6 +210,7 @@ template <bool kBackoff = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* ctl, int32_t* status,
                                           long long budget, int site) {
   if (mbar_try(bar, parity)) return true;
+  if (ctl[kAbort]) return false;
   const long long t0 = clock64();
   for (;;) {
 #pragma unroll 1
@@ -220,6 +221,25 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     if (ctl[kAbort]) return false;
     if (clock64() - t0 > budget) {
       raise_timeout(ctl, status, site);
+      return false;
+    }
+  }
+}
+
+// The same for a whole warp, which leaves together.  Each lane has a clock of its own: where lanes wait by themselves, the
+// budget can run out for some and not for others, and they must not part ways before a shuffle or a barrier.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* ctl, int32_t* status,
+                                               long long budget, int site) {
+  if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+  if (__any_sync(0xffffffffu, ctl[kAbort] != 0)) return false;
+  const long long t0 = clock64();
+  for (;;) {
+#pragma unroll 1
+    for (int i = 0; i < 64; ++i)
+      if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+    const bool late = clock64() - t0 > budget;
+    if (__any_sync(0xffffffffu, ctl[kAbort] != 0 || late)) {
+      if (late) raise_timeout(ctl, status, site);
       return false;
     }
   }
@@ -709,8 +729,11 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
 
   const float* gvec = LOPA ? sn : sx;  // the vector every gate row is dotted with
 
-  // One ring slot of gate rows: dot every row with the gate vector, publish the results, give the slot back.  False
-  // when the wait for the slot's rows ran out.
+  // One ring slot of gate rows: dot every row with the gate vector, publish the results, give the slot back.  When the wait
+  // for the slot's rows runs out, which it can for some lanes of the warp and not for others, the warp stays together:
+  // quantised rows under a standard gate wait as a warp and leave (false), the others go through the motions on whatever is
+  // there (the call has failed; the slot is not given back).  The vote of a warp's wait costs the fp32 LoPA gate 1 us a call
+  // (3840 x 14230, r = 480: 25.2 -> 26.2), going on costs the int4 gate 0.3 (3840 x 10240: 12.9 -> 13.2).
   const int gw = warp - kFirstGateWarp;
   auto gate_slot = [&](int s) -> bool {
     const int slot = s % NG;
@@ -730,7 +753,11 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
         if (gi >= 0) add += row_sg[r0 + lane] * sx[vec_pos<EPV>(gi, D)];
       }
     }
-    if (!mbar_wait(full_gate + 8 * slot, (s / NG) & 1, ctl, p.status, p.wait_cycles, 44)) return false;
+    if constexpr (kLimbs || kLimbs4) {
+      if (!mbar_wait_warp(full_gate + 8 * slot, (s / NG) & 1, ctl, p.status, p.wait_cycles, 44)) return false;
+    } else {
+      mbar_wait(full_gate + 8 * slot, (s / NG) & 1, ctl, p.status, p.wait_cycles, 44);
+    }
     const unsigned char* base = gate_ring + (size_t)slot * p.gate_slot_bytes;
     float mine = 0.f;
     // Short gate rows (LoPA: r elements): a row is a few chunks per lane, and with one warp per scheduler the cost is
@@ -936,7 +963,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
       row_state[r0 + lane] = fired ? __float_as_uint(fmaxf(activation(p.act, z), 0.f)) : 0x80000000u;
     }
     __syncwarp();
-    if (lane == 0) {
+    if (lane == 0 && (kLimbs || kLimbs4 || !ctl[kAbort])) {
       mbar_arrive(empty_gate + 8 * slot);
       if (p.act_extra) atomicAdd(const_cast<int*>(ctl) + kGateDone, 1);  // this slot's rows have been read
     }
@@ -1168,7 +1195,8 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
     // Two ring slots per round when the second one exists: both rows are dotted before the one
     // four-warp barrier, which halves the serial latency per fired row.  The stop marker always
     // arrives, so waiting for the second slot of a round cannot block for good.  A thread whose
-    // wait ran out still joins the barrier and raises the group's stop flag, so the four warps
+    // wait ran out (a budget can run out for some lanes of a warp and not for others) still goes through
+    // the round's shuffles, joins the barrier and raises the group's stop flag, so the four warps
     // always leave the loop together.
     if constexpr (GATED) {
       // Two W_up rows per round; the W_down rows that the previous round asked for are added after this round's h
@@ -1178,14 +1206,14 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
       int pend = 0;         // W_down rows requested by the previous round
       bool failed = false;  // a wait ran out
       auto add_down = [&](int n) {
-        for (int k = 0; k < n && !failed; ++k) {
-          if (!mbar_wait(full_dn + 8 * ds, dpar, ctl, p.status, p.wait_cycles, 54)) { failed = true; break; }
+        for (int k = 0; k < n; ++k) {
+          if (!failed) failed = !mbar_wait(full_dn + 8 * ds, dpar, ctl, p.status, p.wait_cycles, 54);
           const float h = dn_h[ds];
           const uint4* wd = reinterpret_cast<const uint4*>(act_ring + (size_t)(NU + ds) * row_bytes);
 #pragma unroll
           for (int i = 0; i < CPT; ++i) {
             const int c = gat + i * kGT;
-            if (c < nvecD) {
+            if (c < nvecD && !failed) {
               float f[EPV];
               Elem<T>::unpack(wd[c], f);
 #pragma unroll
@@ -1197,7 +1225,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
             }
           }
           __syncwarp();
-          if (lane == 0) mbar_arrive(empty_dn + 8 * ds);
+          if (lane == 0 && !failed) mbar_arrive(empty_dn + 8 * ds);
           if (++ds == ND) { ds = 0; dpar ^= 1; }
         }
       };
@@ -1206,9 +1234,10 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
         const int us1 = us + 1 == NU ? 0 : us + 1;
         const uint32_t upar1 = us + 1 == NU ? upar ^ 1 : upar;
         const bool got0 = mbar_wait(full_up + 8 * us, upar, ctl, p.status, p.wait_cycles, 45);
-        const float a0 = got0 ? up_a[us] : -1.f;
+        const float a0 = got0 && !failed ? up_a[us] : -1.f;
         bool got1 = true;
         float a1 = -1.f;
+        float part0 = 0.f, part1 = 0.f;
         if (a0 >= 0.f) {
           got1 = mbar_wait(full_up + 8 * us1, upar1, ctl, p.status, p.wait_cycles, 46);
           a1 = got1 ? up_a[us1] : -1.f;
@@ -1216,7 +1245,6 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
         if (a0 >= 0.f) {
           const uint4* wu0 = reinterpret_cast<const uint4*>(act_ring + (size_t)us * row_bytes);
           const uint4* wu1 = reinterpret_cast<const uint4*>(act_ring + (size_t)us1 * row_bytes);
-          float part0 = 0.f, part1 = 0.f;
           float2 pk0 = make_float2(0.f, 0.f), pk1 = pk0, pk0b = pk0, pk1b = pk0;
 #pragma unroll
           for (int i = 0; i < CPT; ++i) {
@@ -1248,12 +1276,12 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
             part0 = (pk0.x + pk0.y) + (pk0b.x + pk0b.y);
             part1 = (pk1.x + pk1.y) + (pk1b.x + pk1b.y);
           }
-          part0 = warp_sum(part0);
-          part1 = warp_sum(part1);
-          if (lane == 0) {
-            rp[gaw] = part0;
-            rp[kGAW + gaw] = part1;
-          }
+        }
+        part0 = warp_sum(part0);
+        part1 = warp_sum(part1);
+        if (lane == 0) {
+          rp[gaw] = part0;
+          rp[kGAW + gaw] = part1;
         }
         if (a0 < 0.f || !got1) rp[2 * kGAW] = 1.f;  // stop marker first in the round, or a failed wait
         named_bar_sync(2, kGT);
@@ -1280,7 +1308,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
         }
         add_down(pend);
         pend = asked;
-        if (stop || a1 < 0.f || failed) {
+        if (stop || a1 < 0.f) {
           add_down(pend);
           break;
         }
@@ -1406,10 +1434,10 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
       const uint4* wd0 = reinterpret_cast<const uint4*>(s0 + row_bytes);
       const uint4* wd1 = reinterpret_cast<const uint4*>(s1 + row_bytes);
       uint4 d0[kEarlyDown ? CPT : 1], d1[kEarlyDown ? CPT : 1];
+      float part0 = 0.f, part1 = 0.f;
       if (a0 >= 0.f) {
         const uint4* wu0 = reinterpret_cast<const uint4*>(s0);
         const uint4* wu1 = reinterpret_cast<const uint4*>(s1);
-        float part0 = 0.f, part1 = 0.f;
         float2 pk0 = make_float2(0.f, 0.f), pk1 = pk0, pk0b = pk0, pk1b = pk0;  // packed partial sums
         if (a1 >= 0.f) {
 #pragma unroll
@@ -1429,8 +1457,6 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
 #pragma unroll
             for (int i = 0; i < CPT; ++i) { d0[i] = row_chunk(wd0, i); d1[i] = row_chunk(wd1, i); }
           }
-          part0 = warp_sum(part0);
-          part1 = warp_sum(part1);
         } else {
 #pragma unroll
           for (int i0 = 0; i0 < CPT; i0 += kBatch) {
@@ -1445,8 +1471,11 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
 #pragma unroll
             for (int i = 0; i < CPT; ++i) d0[i] = row_chunk(wd0, i);
           }
-          part0 = warp_sum(part0);
         }
+      }
+      if (__any_sync(0xffffffffu, a0 >= 0.f)) {
+        part0 = warp_sum(part0);
+        part1 = warp_sum(part1);
         if (lane == 0) {
           rp[gaw] = part0;
           rp[kGAW + gaw] = part1;
@@ -1553,7 +1582,9 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
   const int rank = ctl[kRank];
   const int slice = rank >= 0 && rank < R ? rank : -1;
   if (rank == G - 1 && tt == 0 && !ctl[kAbort]) *p.epoch_word = ep;  // every CTA has its number: the next call tags with ep + 1
-  if (slice < 0 || ctl[kAbort]) {
+  // (an aborting CTA that has a slice goes through its barriers like any other and stores nothing: the flag may be raised
+  // between two threads' looks at it)
+  if (slice < 0) {
     abort_grace(ctl);
     return;
   }

@@ -634,7 +634,8 @@ __global__ void __launch_bounds__(kThreads, 1) fused_tc_kernel(const TcParams p,
       for (int e = 0; e < 4; ++e) acc[i][e] = make_float2(0.f, 0.f);
     // Two ring slots per round when the second one exists (both rows are dotted before the one barrier of the
     // round).  The stop marker always arrives, so waiting for the second slot cannot block for good; a thread
-    // whose wait ran out still joins the barrier and raises the group's stop flag.
+    // whose wait ran out (a budget can run out for some lanes of a warp and not for others) still goes through the
+    // round's shuffles, joins the barrier and raises the group's stop flag.
     int slot = 0;
     uint32_t par = 0;
     const bool pair = NA >= 4;
@@ -652,10 +653,10 @@ __global__ void __launch_bounds__(kThreads, 1) fused_tc_kernel(const TcParams p,
       }
       const unsigned char* s0 = act_ring + (size_t)slot * p.act_slot_bytes;
       const unsigned char* s1 = act_ring + (size_t)slot1 * p.act_slot_bytes;
+      float2 pk0 = make_float2(0.f, 0.f), pk1 = pk0;
       if (a0 >= 0.f) {
         const uint4* wu0 = reinterpret_cast<const uint4*>(s0);
         const uint4* wu1 = reinterpret_cast<const uint4*>(s1);
-        float2 pk0 = make_float2(0.f, 0.f), pk1 = pk0;
 #pragma unroll
         for (int i = 0; i < CPT; ++i) {
           const int c = at + i * kAT;
@@ -671,6 +672,8 @@ __global__ void __launch_bounds__(kThreads, 1) fused_tc_kernel(const TcParams p,
             }
           }
         }
+      }
+      if (__any_sync(0xffffffffu, a0 >= 0.f)) {
         const float part0 = warp_sum(pk0.x + pk0.y), part1 = warp_sum(pk1.x + pk1.y);
         if (lane == 0) {
           rp[aw] = part0;
@@ -744,7 +747,9 @@ __global__ void __launch_bounds__(kThreads, 1) fused_tc_kernel(const TcParams p,
   const int rank = ctl[kRank];
   const int slice = rank >= 0 && rank < R ? rank : -1;
   if (rank == G - 1 && tt == 0 && !ctl[kAbort]) *p.epoch_word = ep;  // every CTA has its number: the next call tags with ep + 1
-  if (slice < 0 || ctl[kAbort]) {
+  // (an aborting CTA that has a slice goes through its barriers like any other and stores nothing: the flag may be raised
+  // between two threads' looks at it)
+  if (slice < 0) {
     abort_grace(ctl);
     return;
   }

@@ -57,6 +57,44 @@ def test_single_token_call_times_out_reports_and_recovers(mod, D, H, dtype, tens
     assert other.device_status() == 0
 
 
+@pytest.mark.parametrize("kind", ["bf16", "f32", "lopa", "int8", "gated", "tensor_gate"])
+@pytest.mark.parametrize("cycles", [500, 4000, 12000])
+def test_waits_of_every_role_run_out_and_the_call_still_comes_back(mod, kind, cycles):
+    """Budgets of 0.3 to 6 us, shorter than what most roles of a 10 to 30 us call wait for: producers, gate warps, act warps
+    and summing CTAs give up at moments of their own, lanes of one warp not all in the same clock cycle."""
+    D, H, r = 2048, 12000, 256
+    dtype = torch.float32 if kind == "f32" else torch.bfloat16
+    ffn = mod.SparseFFN(D, H, dtype, r_max=r, B_max=1)
+    x = syn.tokens(1, D, dtype, 13, DEV)[0]
+    call = ffn.sparse_ffn_forward_q8 if kind == "int8" else ffn.sparse_ffn_forward
+    if kind == "lopa":
+        w = syn.lopa_ffn(D, H, r, dtype, 13, DEV, sparsity=0.8)
+        gate = {"V": w["V"], "U": w["U"], "g_idx": mod.g_diagonal(H, D, DEV)}
+    else:
+        w = syn.standard_ffn_q8(D, H, 13, DEV, sparsity=0.8) if kind == "int8" else syn.standard_ffn(D, H, dtype, 13, DEV, sparsity=0.8)
+        gate = {"W_g": w["W_g"]}
+    if kind == "gated":
+        ffn.set_up_activation("relu")
+        ffn.set_gated_skip(True)
+    if kind == "tensor_gate":
+        ffn.set_gate_engine("tensor_core")
+    want = call(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu").clone()
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0
+    mod.test_set_knob("wait_cycles", cycles)
+    for _ in range(5):
+        call(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+        torch.cuda.synchronize()
+        assert ffn.device_status() in ((5,) if cycles == 500 else (0, 5))
+        ffn.reset()
+    mod.test_set_knob("wait_cycles", 0)
+    for _ in range(2):
+        y = call(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+        torch.cuda.synchronize()
+        assert ffn.device_status() == 0
+        assert torch.equal(y, want)
+
+
 def test_batched_tcgen05_gate_times_out_releases_tmem_and_recovers(mod):
     D, H, B = 512, 4000, 8
     w = syn.standard_ffn(D, H, torch.bfloat16, 12, DEV, sparsity=0.9)
