@@ -1053,7 +1053,18 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
         }
     }
     int tcount = 0, it = 0, s = 0;
-    for (int tile = blockIdx.x; tile + (share_last ? (int)gridDim.x : 0) < n_tiles; tile += gridDim.x, ++tcount) {
+    int tile = blockIdx.x;
+    // which rows of the tile fired, as the up kernel or the compaction reads it
+    auto publish = [&](bool fired) {
+      const int li = tile * tile_rows + row_thr;
+      const bool valid = row_thr >= 0 && row_thr < tile_rows && li < n_rows;
+      if (p.flag && valid) p.flag[li] = fired ? 1 : 0;
+      if (p.words_out) {
+        const unsigned m = __ballot_sync(0xffffffffu, fired && valid);
+        if (lane == 0) p.words_out[4 * tile + (warp & 3)] = m;
+      }
+    };
+    for (; tile + (share_last ? (int)gridDim.x : 0) < n_tiles; tile += gridDim.x, ++tcount) {
       bool fired = false;
       if constexpr (EX) {
         const bool done = exact_epilogue(tile, tcount, set, it, s, fired);
@@ -1071,18 +1082,18 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
       } else {
         if (!epilogue(tile, tcount, 0, 1, false, fired)) break;
       }
-      const int row_in_tile = row_thr;
-      const int li = tile * tile_rows + row_in_tile;
-      const bool valid = row_in_tile >= 0 && row_in_tile < tile_rows && li < n_rows;
-      if (!UP && p.flag && valid) p.flag[li] = fired ? 1 : 0;
-      if (!UP && p.words_out) {
-        const unsigned m = __ballot_sync(0xffffffffu, fired && valid);
-        if (lane == 0) p.words_out[4 * tile + (warp & 3)] = m;
-      }
+      if (!UP) publish(fired);
       if (EX) continue;
       tc_fence_before();
       mbar_arrive(acc_empty);
     }
+    // after a wait that ran out: nothing fired in the tiles that are left (the masks there are an earlier call's, or
+    // the bytes of another route, whose bits need not stand for rows at all)
+    if (!UP && set == 0)
+      for (; tile + (share_last ? (int)gridDim.x : 0) < n_tiles; tile += gridDim.x) {
+        pdl_wait();
+        publish(false);
+      }
   }
 
   // ---- the CTA's last tile (wide batches): by now the producer and issuer warps have nothing left to do, so

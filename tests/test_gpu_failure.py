@@ -116,3 +116,39 @@ def test_batched_tcgen05_gate_times_out_releases_tmem_and_recovers(mod):
         torch.cuda.synchronize()
         assert ffn.device_status() == 0
         assert_y_close(y, ref["y"], what="batched call after a timeout")
+
+
+@pytest.mark.parametrize("D,B,r,q8", [
+    (512, 8, 0, False),     # bf16 accumulators
+    (384, 8, 0, False),     # sums in registers, two sets of epilogue warps
+    (384, 40, 64, False),   # the same, LoPA: the vector's kernel loses a copy as well
+    (384, 6, 64, True),     # expanders in front of it
+    (384, 12, 0, True),     # h in two terms
+    (512, 200, 0, False),   # two accumulators, the last tile shared by all warps
+])
+def test_batched_gate_that_times_out_leaves_no_fired_rows_and_recovers(mod, D, B, r, q8):
+    H = 4000
+    make = {(False, 0): syn.standard_ffn, (False, 1): syn.lopa_ffn, (True, 0): syn.standard_ffn_q8, (True, 1): syn.lopa_ffn_q8}[q8, r > 0]
+    w = make(*((D, H, r) if r else (D, H)), *(() if q8 else (torch.bfloat16,)), 14, DEV, sparsity=0.9)
+    gate = {"V": w["V"], "U": w["U"], "g_idx": mod.g_diagonal(H, D, DEV)} if r else {"W_g": w["W_g"]}
+    x = syn.tokens(B, D, torch.bfloat16, 14, DEV)
+    ffn = mod.SparseFFN(D, H, torch.bfloat16, r_max=r, B_max=B)
+    call = ffn.sparse_ffn_forward_q8 if q8 else ffn.sparse_ffn_forward
+    want = call(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu").clone()
+    all_fire = torch.full((H,), 1e4, device=DEV)
+    call(x, gate, all_fire, w["W_up"], w["W_down"], "relu")
+    assert ffn.last_active().numel() == H and ffn.device_status() == 0
+    mod.test_set_knob("wait_cycles", SHORT)
+    mod.test_set_knob("drop_stage", 0)                     # CTA 0 of the gate GEMMs never copies its first stage
+    call(x, gate, -all_fire, w["W_up"], w["W_down"], "relu")
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 5
+    assert ffn.last_active().numel() == 0                  # not the rows that the call before left in the masks
+    mod.test_set_knob("drop_stage", -1)
+    mod.test_set_knob("wait_cycles", 0)
+    ffn.reset()
+    for _ in range(3):
+        y = call(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+        torch.cuda.synchronize()
+        assert ffn.device_status() == 0
+        assert torch.equal(y, want)
