@@ -484,7 +484,7 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
       d.tok0 = b0; d.B = nb; d.cols = round8(nb);
       // (the workspace holds most_splits() partials of nb tokens; the first argument bounds what the SMs can use)
       const int cap = nb <= kMaxMmaTokens ? kMaxSplits : most_splits(D, nb);
-      d.splits = splits = umma_down_splits(D, h_terms * d.cols, h->sm_count, cap);
+      d.splits = splits = umma_down_splits(D, h_terms * d.cols, exact, h->sm_count, cap);
       d.walk_all = (own_list && may_walk) ? count + 1 : nullptr;
       d.partial = partial; d.status = h->at<int32_t>(h->L.status);
       SFFN_CUDA(launch_umma_down(d, s));

@@ -1650,13 +1650,23 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
 }
 
 // Token columns up to which two CTAs of the down kernel share an SM (each with two accumulators in half of the TMEM, and
-// at least four ring stages); wider batches give one CTA the whole SM.
+// at least four ring stages); wider batches give one CTA the whole SM, and so do exact sums, whose accumulators fill
+// the TMEM.
 constexpr int kDownPairCols = 64;
+static bool down_pairs(int cols, bool exact) { return cols <= kDownPairCols && !exact; }
 
-int umma_down_splits(int D, int cols, int sm_count, int max_splits) {
-  const int d_tiles = D / kTileRows;
-  int splits = (cols <= kDownPairCols ? 2 : 1) * sm_count / (d_tiles > 0 ? d_tiles : 1);
-  return splits < 1 ? 1 : splits > max_splits ? max_splits : splits;
+int umma_down_splits(int D, int cols, bool exact, int sm_count, int max_splits) {
+  const int tiles = D >= kTileRows ? D / kTileRows : 1;
+  auto splits_of = [&](int ctas) {
+    const int n = ctas / tiles;
+    return n < 1 ? 1 : n > max_splits ? max_splits : n;
+  };
+  if (down_pairs(cols, exact)) return splits_of(2 * sm_count);
+  const int one = splits_of(sm_count), two = splits_of(2 * sm_count);
+  // Exact sums: two waves of CTAs, each with a set-up of its own (about 6 us), only where they shorten the contraction by a
+  // tenth: wide rows, whose tiles leave SMs idle in one wave.  16 tokens, one wave / two: 2688 x 8000 67 / 74 us, 6528 x
+  // 20000 (102 and 255 CTAs) 312 / 301.
+  return exact && 10 * (two - 2 * one) >= one * two ? two : one;
 }
 
 bool umma_down_supported(int D, int cols) { return D % kTileRows == 0 && cols >= 1 && cols <= kUmmaMaxCols; }
@@ -1682,7 +1692,7 @@ cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s) {
   if (p.cols % 8 || p.cols < p.B || p.npad > kUmmaMaxCols) return cudaErrorInvalidValue;
   p.wait_cycles = fused_test_knobs().wait_cycles;
   const int stage_bytes = kAAtomBytes + p.npad * 128 + p.qbits * kTileRows * kAtomK / 8;
-  int stages = ((own <= kDownPairCols && !p.exact ? 111 : 225) * 1024 - 1024 - 1024) / stage_bytes;
+  int stages = ((down_pairs(own, p.exact) ? 111 : 225) * 1024 - 1024 - 1024) / stage_bytes;
   if (stages > 12) stages = 12;
   stages &= p.exact ? ~3 : ~1;
   if (stages < 2) return cudaErrorInvalidValue;

@@ -82,7 +82,7 @@ struct UmmaDownParams {
   long long wait_cycles; // budget of every device-side wait (filled by the launcher)
 };
 
-int umma_down_splits(int D, int cols, int sm_count, int max_splits);  // cols: token columns of all terms
+int umma_down_splits(int D, int cols, bool exact, int sm_count, int max_splits);  // cols: token columns of all terms
 bool umma_down_supported(int D, int cols);
 cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s);
 bool umma_rows_supported(int K, int cols);
