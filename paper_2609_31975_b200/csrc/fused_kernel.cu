@@ -1685,7 +1685,10 @@ Geometry plan(int wkind, int D, int H, int K, bool lopa, int grid) {
   nr = nr < 1 ? 1 : nr > 32 ? 32 : nr;
   // Short rows: 8 KB of them would leave CTAs without a slot, or warps of a CTA.  A share of up to eight rows gives every
   // gate warp its own (int4, 384 x 1024: 32 rows a slot took 12.4 us, one 7.1).  Beyond that, as measured per storage
-  // type: int8 rows are dotted two at a time (1408 x 3072: 5 rows a slot 10.5 us, 2 rows 9.3), int4 rows by three (2944 x
+  // type: int8 rows are dotted two at a time (1408 x 3072: 5 rows a slot 10.5 us, 2 rows 9.3) while a CTA's share is short;
+  // a longer share of rows up to 2048 wide takes eight, or two rows a slot would be all that is in flight (32 rows a CTA and
+  // more: 1024 x 28672, 194 rows a CTA, 2 / 4 / 8 / 16 rows a slot 21.1 / 20.7 / 17.1 / 18.3 us, 1280 x 5120, 35 rows, 2 / 8
+  // rows 10.1 / 9.2; 28 rows, 1024 x 4096: 8.1 / 8.2; wider rows, 3072 x 14336: 15.3 / 20.6).  int4 rows by three (2944 x
   // 6272: 5 rows 13.0 us, 3 rows 11.6; four, which share more reads of the limbs, where they still make two slots a gate
   // warp: 3840 x 10240 12.9 us, 3 rows 13.2), fp32 / bf16 rows up to
   // eight at a time but in three slots or more (704 x 2048: 2 rows 7.2 us, 5 rows 6.8).  LoPA: at most eight
@@ -1694,6 +1697,7 @@ Geometry plan(int wkind, int D, int H, int K, bool lopa, int grid) {
   const int cap = lopa ? (wkind == kWQ4 ? 4 : gate_row_bytes <= 1024 ? 8 : nr) : wkind == kWQ8 ? 2 : wkind == kWQ4 ? (rows_of_cta >= 64 ? 4 : 3) : nr;
   const int least = lopa ? 4 : 3;  // slots
   if (nr > cap) nr = cap;
+  if (wkind == kWQ8 && !lopa && rows_of_cta >= 32 && gate_row_bytes <= 2048) nr = 8;
   if (rows_of_cta <= 8 && !lopa) nr = 1;
   else if (nr > (rows_of_cta + least - 1) / least) nr = (rows_of_cta + least - 1) / least;
   if (lopa) {

@@ -223,6 +223,15 @@ def test_quantised_batches_of_any_size_keep_int32_sums_and_22_bits_of_the_token(
     assert torch.equal(ffn.last_active().cpu().long(), torch.nonzero(sign > 0)[:, 0])
 
 
+@pytest.mark.parametrize("D,H", [(512, 4588), (512, 4736), (2048, 4737), (256, 9000), (2064, 4737)])
+def test_int8_ring_slots_of_short_and_long_shares(mod, D, H):
+    # 31 rows a CTA (slots of two), 32 and 33 (slots of eight, the widest row), 61 (ragged last slots), a row too wide for eight
+    ffn = mod.SparseFFN(D, H, torch.bfloat16, B_max=1)
+    gate, w = make_std(D, H, 63, 0.8)
+    x = syn.tokens(1, D, torch.bfloat16, 63, DEV)[0]
+    check(mod, ffn, x, gate, w, "relu", ("fused", "general"), f"q8 slots {D}x{H}")
+
+
 @pytest.mark.parametrize("path", ["general", "fused"])
 def test_int8_full_and_zero_sparsity_and_double_activation(mod, path):
     D, H = 768, 1500

@@ -78,6 +78,25 @@ def test_kernel_geometry_invariants_on_the_host():
                     act_threads = 256 if lopa else 128
                     assert cpt in (1, 2, 4, 8) and cpt * act_threads * (16 // esz) >= D
     assert n_ok > 300                                          # the benchmark shapes and most others are served
+    for wkind, per_byte in ((2, 1), (3, 2)):                   # int8 and int4 rows
+        for D in (256, 384, 512, 1024, 1408, 2048, 3072, 4096, 8192):
+            for H in (64, 1184, 1185, 4096, 8192, 28672):
+                for lopa, K in ((0, D), (1, 64), (1, 480), (1, 1024)):
+                    lib.sffn_test_fused_plan(wkind, D, H, K, lopa, 148, out)
+                    ok, nr, gsb, ng, gw, asb, na, cpt, smem = list(out)
+                    if not ok:
+                        continue
+                    n_ok += 1
+                    row, share = K // per_byte, -(-H // 148)
+                    assert smem <= 227 * 1024 and 1 <= nr <= 32 and nr * row <= gsb and gsb % 128 == 0
+                    assert gw >= 2 and gw % 2 == 0 and gw <= (4 if lopa else 8) and ng % gw == 0 and ng >= gw
+                    assert na >= 2 and asb >= 2 * D // per_byte
+                    assert cpt * (256 if lopa else 128) * 16 * per_byte >= D
+                    if share <= 8 and not lopa:
+                        assert nr == 1                         # a slot, and so a warp, for every row
+                    if wkind == 2 and not lopa and D <= 2048:
+                        assert ng * nr >= min(share, 64)       # rows in flight: 64 or the CTA's whole share
+    assert n_ok > 500
     lib.sffn_test_fused_plan(1, 4096, 14336, 4096, 0, 148, out)
     assert list(out)[0] == 1 and list(out)[3] == 16            # the graded shape: 16 gate slots of one 8 KB row
     tr, nt, own = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
