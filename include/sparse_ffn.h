@@ -84,7 +84,9 @@ typedef enum { SFFN_GATE_STANDARD = 0, SFFN_GATE_LOPA = 1 } sffn_gate_kind;
  * multiplied as int8 against the tokens split into int8 limbs, or, like int4 rows, expanded to bf16 in shared
  * memory on their way to the tensor cores; more than 256 tokens (LoPA gate: 128; int8 / int4 rows multiplied as int8: 64;
  * bf16 rows of an odd multiple of 128 elements: 64; any such rows under a LoPA gate: 40) run in passes of as many, the list
- * of fired neurons being the union over all passes).  A batch those kernels do not take (fp32
+ * of fired neurons being the union over all passes).  Precision by row width: at multiples of 256, h enters the down
+ * projection of a batch as one bf16 value (relative error of y about 1.7e-3); at odd multiples of 128 as three, with sums
+ * that round as fp32 does (1e-7), under a standard gate on quantised rows as two (3e-6).  A batch those kernels do not take (fp32
  * operands, a row width they do not tile) runs the fused kernel once per token with the fired flags OR-ed,
  * which is faster than the CUDA-core batch kernels; what is left goes to the general CUDA-core kernels.
  * The others force one family (SFFN_ERR_UNSUPPORTED if it cannot serve the call): GENERAL = CUDA-core
@@ -182,7 +184,7 @@ int dense_ffn_forward(sffn_handle* handle, const void* x, int B, const sffn_gate
  * dot products are integer ones (dp4a) against the token split, 16 entries at a time, into two int8 limbs and a
  * scale (x = s_c (q0 + q1/128) up to 3e-5 of the largest |x| among those 16 entries; int4: 32 entries, nibbles used
  * as the bytes 16 x code), all sums in fp32 beyond a chunk; LoPA gates use fp32 arithmetic throughout.  A batch runs
- * the tcgen05 batch kernels (D a multiple of 256 -- five tokens or more, LoPA six: of 128 -- and r of 64; otherwise, or under
+ * the tcgen05 batch kernels (D a multiple of 256 -- five tokens or more, LoPA six, wider than 4224 eight: of 128 -- and r of 64; otherwise, or under
  * SFFN_PATH_FUSED, the fused kernel once per token; the list of fired neurons is the union over the tokens).  There the
  * gate and up products of int8 rows are int8 x int8 with int32 accumulators, each token entering as four int8 limbs and a
  * scale (x = s (q0 + q1/128 + q2/128^2 + q3/128^3) up to 2^-22 max|x|; D a multiple of 256, r of 128; int4 rows take the

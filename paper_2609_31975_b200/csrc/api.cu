@@ -22,8 +22,6 @@ constexpr int kMaxChunk = 4;         // tokens per pass of the general kernels
 constexpr int kMaxSplits = 16;       // union-row splits of the batched down projection
 constexpr int kMaxMmaTokens = 64;    // tokens per pass of the mma.sync kernels, and of the tcgen05 ones on int8 limbs
 constexpr int kMaxUmmaTokens = sffn::kUmmaMaxCols;  // tokens per pass of the tcgen05 kernels
-constexpr int kOddWidthMinTokens = 5;  // rows of an odd multiple of 128: batches from here on the tcgen05 kernels ...
-constexpr int kExactMinTokens = 6;     // ... and where those have to form exact sums
 
 inline int round8(int v) { return (v + 7) & ~7; }
 
@@ -284,6 +282,17 @@ thread_local int g_last_cuda_line = 0;
 
 // Whether a batch takes the tcgen05 kernels with exact sums (see h_terms_for).
 bool exact_batch(int D, bool quantised, bool lopa) { return D % 256 != 0 && (!quantised || lopa); }
+
+// Fewest tokens of a batch over rows of an odd multiple of 128 for the tcgen05 kernels; fewer run token by token.  The lines
+// lie where every width measured (384 to 6528 columns) is faster from there on: quantised rows, standard gate, 5 (int4, 6528
+// x 20000, 4 / 5 tokens: 150 / 153 us against 134 / 167 token by token; 384 x 1200: 24 / 24 against 27 / 33); with exact
+// sums 6 (bf16, 384 x 1200, 5 / 6 tokens: 30 / 30 us against 27 / 32; 6528 x 20000: 238 / 249 against 287 / 344), but
+// quantised rows wider than 4224, LoPA gate, 8 (int8, 6528 x 20000, r = 768, 6 / 8 tokens: 188 / 196 us against 170 / 227;
+// 4224 x 12900, r = 512, 6 tokens: 105 against 130).
+int odd_width_tokens(int D, bool quantised, bool lopa) {
+  if (!exact_batch(D, quantised, lopa)) return 5;
+  return quantised && D > 4224 ? 8 : 6;
+}
 
 // Whether a quantised batch multiplies its codes as int8 against the tokens' int8 limbs.
 bool limb_batch(int D, int gate_k) {
@@ -613,17 +622,14 @@ int run(sffn_handle* h, const void* x, int B, const sffn_gate* g, const float* b
   const bool lopa_gate = g->kind == SFFN_GATE_LOPA;
   const int gate_k = lopa_gate ? g->r : h->D;
   // A batch the tensor-core kernels can take: bf16 tokens; bf16, int8 or int4 rows of a multiple of 256 elements, or of
-  // 128 from a few tokens on (see h_terms_for); a LoPA rank of a multiple of 64.  At the odd multiples of 128 the other
-  // route is the single-token kernel once per token: int8, standard gate, 1152 x 3500, B = 3 / 4 / 8: 27 / 28 / 28 us
-  // against 28 / 37 / 73 token by token, 6528 x 20000: 151 / 157 / 184 against 131 / 175 / 348; with exact sums (bf16 rows,
-  // LoPA gates), bf16, 1152 x 3500, B = 6 / 16: 37 / 41 us against 52 / 137, 6528 x 20000: 260 / 318 against 370 / 985.
+  // 128 from a few tokens on (see h_terms_for and odd_width_tokens); a LoPA rank of a multiple of 64.
   // Larger batches are cut into passes of as many tokens as one launch chain holds: a pass reads every gate row and the
   // rows of its own union, so fewer passes read fewer bytes (bf16, 4096 x 14336, 200 tokens: 4 passes of 64 took 333 us, one
   // takes 137).  The mma.sync kernels (selected, or a bf16 LoPA rank that is no multiple of 64) take passes of 64 and rows
   // of a multiple of 256 elements.
   const bool umma_ok = h->path != SFFN_PATH_MMA_SYNC && sffn::umma_rows_supported(gate_k, 1) &&
                        sffn::umma_rows_supported(h->D, 1) && sffn::umma_down_supported(h->D, 1) &&
-                       (h->D % 256 == 0 || B >= (exact_batch(h->D, q8 != nullptr, lopa_gate) ? kExactMinTokens : kOddWidthMinTokens));
+                       (h->D % 256 == 0 || B >= odd_width_tokens(h->D, q8 != nullptr, lopa_gate));
   const int pass_max = umma_ok ? umma_pass_tokens(h->D, gate_k, q8 != nullptr, lopa_gate) : kMaxMmaTokens;
   const bool tensor_batch = h->dtype == SFFN_BF16 && B >= 2 && h->path != SFFN_PATH_GENERAL && h->path != SFFN_PATH_FUSED &&
                             (umma_ok || (!q8 && sffn::batched_mma_supported(h->D, gate_k, 1)));

@@ -232,6 +232,19 @@ def test_int8_ring_slots_of_short_and_long_shares(mod, D, H):
     check(mod, ffn, x, gate, w, "relu", ("fused", "general"), f"q8 slots {D}x{H}")
 
 
+@pytest.mark.parametrize("D,r,least", [(384, 0, 5), (6528, 0, 5), (4224, 64, 6), (4480, 64, 8), (6528, 64, 8)])
+def test_int8_batches_of_odd_row_widths_run_token_by_token_below_the_measured_line(mod, D, r, least):
+    H = 300
+    ffn = mod.SparseFFN(D, H, torch.bfloat16, r_max=r, B_max=least)
+    gate, w = make_lopa(mod, D, H, r, 64, 0.9) if r else make_std(D, H, 64, 0.9)
+    for B in (least - 1, least):
+        x = syn.tokens(B, D, torch.bfloat16, 64, DEV)
+        y = ffn.sparse_ffn_forward_q8(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+        one_by_one = torch.stack([ffn.sparse_ffn_forward_q8(t, gate, w["b_g"], w["W_up"], w["W_down"], "relu") for t in x])
+        assert torch.equal(y, one_by_one) == (B < least)
+        assert_y_close(y, run_oracle_q8(x, gate, w, "relu")["y"], rel_l2=TOL, max_abs=TOL, what=f"{D} r={r} B={B}")
+
+
 @pytest.mark.parametrize("path", ["general", "fused"])
 def test_int8_full_and_zero_sparsity_and_double_activation(mod, path):
     D, H = 768, 1500
