@@ -33,9 +33,9 @@
 // bf16 per cycle and SM whatever the token count, i.e. 16 codes per cycle: quantised batches are bound by that
 // rate, not by their bytes.
 // Up to 256 token columns go through in one pass.  Wide batches (npad > 128) leave room for two accumulators and a ring
-// of four stages of ~40 KB; they are bound by the token rows every CTA reads again (200 tokens x 4096: 1.6 MB a CTA
+// of four stages of ~40 KB (two with expanded codes and 241 columns or more); they are bound by the token rows every CTA reads again (200 tokens x 4096: 1.6 MB a CTA
 // through L2 beside 0.8 MB of weights), still far cheaper than further passes over the weights (200 tokens, 4096 x
-// 14336, bf16: 135 us in one pass against 333 us in four of at most 64).
+// 14336, bf16: 137 us in one pass against 333 us in four of at most 64).
 // Every wait is bounded by a cycle budget; on expiry the status word is set, all roles wind down and the TMEM
 // columns are released before the CTA exits.
 #include "umma_kernels.cuh"
