@@ -1391,99 +1391,163 @@ __global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarp
   }
 }
 
+// The vector of a token for the small kernels below: entry k = threadIdx.x + i * blockDim.x of a row of up to kKept *
+// blockDim.x entries stays in register i from the first look at it; the rest of a longer row is read again.
+constexpr int kVecThreads = 256, kKept = 8;
+struct KeptVec {
+  const float* v;
+  int r;
+  float kept[kKept];
+  __device__ __forceinline__ KeptVec(const float* v_, int r_) : v(v_), r(r_) {
+#pragma unroll
+    for (int i = 0; i < kKept; ++i) {
+      const int k = threadIdx.x + i * kVecThreads;
+      kept[i] = k < r ? v[k] : 0.f;
+    }
+  }
+  template <typename F>
+  __device__ __forceinline__ void each(F f) const {  // f(k, entry) in ascending order of k
+#pragma unroll
+    for (int i = 0; i < kKept; ++i) {
+      const int k = threadIdx.x + i * kVecThreads;
+      if (k < r) f(k, kept[i]);
+    }
+    for (int k = threadIdx.x + kKept * kVecThreads; k < r; k += kVecThreads) f(k, v[k]);
+  }
+};
+// 1 / rms of the vector.
+__device__ __forceinline__ float inverse_rms(const KeptVec& vec, float eps, float* red) {
+  float ss = 0.f;
+  vec.each([&](int, float e) { ss = fmaf(e, e, ss); });
+  ss = warp_sum(ss);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  float tot = 0.f;
+#pragma unroll
+  for (int w = 0; w < kVecThreads / 32; ++w) tot += red[w];
+  return rsqrtf(tot / (float)vec.r + eps);
+}
+
 // LoPA gate, batched: n = RMSNorm(v) (or v itself) as a sum of two bf16 vectors for the tensor cores: row b of
 // x2 holds the high part of token b's vector, row cols + b the low part (v - bf16(v)), so that the gate's U n keeps
 // close to fp32 accuracy.  `exact`: row 2 cols + b holds what those two leave (24 bits in all).  One CTA per token.
-__global__ void __launch_bounds__(256) rmsnorm_split_kernel(const float* v, int r, int v_stride, const float* gain,
-                                                            float eps, int use_rms, int cols, int exact,
-                                                            __nv_bfloat16* x2) {
-  __shared__ float red[8];
+__global__ void __launch_bounds__(kVecThreads) rmsnorm_split_kernel(const float* v, int r, int v_stride, const float* gain,
+                                                                    float eps, int use_rms, int cols, int exact,
+                                                                    __nv_bfloat16* x2) {
+  __shared__ float red[kVecThreads / 32];
   pdl_launch_dependents();
   pdl_wait();
   const int b = blockIdx.x;
-  const float* vb = v + (size_t)b * v_stride;
-  float inv = 1.f;
-  if (use_rms) {
-    float ss = 0.f;
-    for (int k = threadIdx.x; k < r; k += blockDim.x) ss = fmaf(vb[k], vb[k], ss);
-    ss = warp_sum(ss);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-    __syncthreads();
-    float tot = 0.f;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) tot += red[w];
-    inv = rsqrtf(tot / (float)r + eps);
-  }
-  for (int k = threadIdx.x; k < r; k += blockDim.x) {
-    float n = use_rms ? (gain ? gain[k] : 1.f) * vb[k] * inv : vb[k];
+  const KeptVec vec(v + (size_t)b * v_stride, r);
+  const float inv = use_rms ? inverse_rms(vec, eps, red) : 1.f;
+  vec.each([&](int k, float e) {
+    float n = use_rms ? (gain ? gain[k] : 1.f) * e * inv : e;
     x2[(size_t)b * r + k] = take_bf16(n);
     x2[(size_t)(cols + b) * r + k] = take_bf16(n);
     if (exact) x2[(size_t)(2 * cols + b) * r + k] = __float2bfloat16(n);
-  }
+  });
 }
 
 // Tokens as int8 limbs for the kind::i8 MMAs: t[k] = scale * (q0 + q1 / 128 + q2 / 128^2 + q3 / 128^3) up to
 // scale * 2^-22, with scale = max |t| / 127, |q0| <= 127 and the other limbs <= 64 in magnitude.  Row 4 b + l of
-// `limbs` holds limb l of token b.  One CTA per token; `val(k)` yields the token's entries.
-template <typename F>
-__device__ __forceinline__ void write_limbs(F val, int K, int8_t* limbs, float* scale_out, float* red) {
-  float m = 0.f;
-  for (int k = threadIdx.x; k < K; k += blockDim.x) m = fmaxf(m, fabsf(val(k)));
+// `limbs` holds limb l of token b.  One CTA per token.
+// scale of a token whose threads have seen entries of at most m
+__device__ __forceinline__ float limb_scale(float m, float* red, int warps) {
 #pragma unroll
   for (int d = 16; d >= 1; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
-  __syncthreads();  // `red` may still be read by the caller
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
   float mx = 0.f;
+  for (int w = 0; w < warps; ++w) mx = fmaxf(mx, red[w]);
+  return mx > 0.f ? mx / 127.f : 1.f;
+}
+// the limbs of one entry
+__device__ __forceinline__ void limbs_of(float e, float inv, int* q4) {
+  float t = fminf(fmaxf(e * inv, -127.f), 127.f);
 #pragma unroll
-  for (int w = 0; w < 8; ++w) mx = fmaxf(mx, red[w]);
-  const float scale = mx > 0.f ? mx / 127.f : 1.f;
-  if (threadIdx.x == 0) *scale_out = scale;
-  const float inv = 1.f / scale;
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    float t = val(k) * inv;
-    t = fminf(fmaxf(t, -127.f), 127.f);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      const float q = rintf(t);
-      limbs[(size_t)l * K + k] = (int8_t)(int)q;
-      t = (t - q) * 128.f;
-    }
+  for (int l = 0; l < 4; ++l) {
+    const float q = rintf(t);
+    q4[l] = (int)q;
+    t = (t - q) * 128.f;
   }
 }
 
-__global__ void __launch_bounds__(256) token_limbs_kernel(const __nv_bfloat16* x, int K, int x_stride, int8_t* limbs,
-                                                          float* scale) {
-  __shared__ float red[8];
+// A thread takes eight consecutive entries (16 bytes) at a time and keeps those of its first two rounds; it stores eight
+// limbs at a time.  Bound by its own latency, which stands between the predecessor and the first gate MMA: one round trip to
+// the token instead of two dozen (4096 entries by 256 threads, an entry at a time, twice: batches of int4 and int8 rows
+// 4 to 5 us longer).
+constexpr int kLimbThreads = 512, kLimbRounds = 2;
+__global__ void __launch_bounds__(kLimbThreads) token_limbs_kernel(const __nv_bfloat16* x, int K, int x_stride, int8_t* limbs,
+                                                                   float* scale) {
+  __shared__ float red[kLimbThreads / 32];
   pdl_launch_dependents();
   pdl_wait();
   const int b = blockIdx.x;
-  const __nv_bfloat16* xb = x + (size_t)b * x_stride;
-  write_limbs([&](int k) { return __bfloat162float(xb[k]); }, K, limbs + (size_t)4 * b * K, scale + b, red);
+  const uint4* xb = reinterpret_cast<const uint4*>(x + (size_t)b * x_stride);
+  const int n8 = K / 8;
+  uint4 kept[kLimbRounds];
+  float m = 0.f;
+  auto largest = [&](const uint4& w) {
+    float e[8];
+    Elem<__nv_bfloat16>::unpack(w, e);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) m = fmaxf(m, fabsf(e[q]));
+  };
+#pragma unroll
+  for (int i = 0; i < kLimbRounds; ++i) {
+    const int k = threadIdx.x + i * kLimbThreads;
+    kept[i] = k < n8 ? xb[k] : make_uint4(0, 0, 0, 0);
+  }
+#pragma unroll
+  for (int i = 0; i < kLimbRounds; ++i) largest(kept[i]);
+  for (int k = threadIdx.x + kLimbRounds * kLimbThreads; k < n8; k += kLimbThreads) largest(xb[k]);
+  const float s = limb_scale(m, red, kLimbThreads / 32);
+  if (threadIdx.x == 0) scale[b] = s;
+  const float inv = 1.f / s;
+  int8_t* out = limbs + (size_t)4 * b * K;
+  auto put = [&](int k, const uint4& w) {
+    float e[8];
+    Elem<__nv_bfloat16>::unpack(w, e);
+    uint2 o[4] = {};
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      int l4[4];
+      limbs_of(e[q], inv, l4);
+#pragma unroll
+      for (int l = 0; l < 4; ++l) (q < 4 ? o[l].x : o[l].y) |= (uint32_t)(l4[l] & 0xff) << (8 * (q & 3));
+    }
+#pragma unroll
+    for (int l = 0; l < 4; ++l) *reinterpret_cast<uint2*>(out + (size_t)l * K + 8 * k) = o[l];
+  };
+#pragma unroll
+  for (int i = 0; i < kLimbRounds; ++i) {
+    const int k = threadIdx.x + i * kLimbThreads;
+    if (k < n8) put(k, kept[i]);
+  }
+  for (int k = threadIdx.x + kLimbRounds * kLimbThreads; k < n8; k += kLimbThreads) put(k, xb[k]);
 }
 
 // LoPA gate with int8 rows: n = RMSNorm(v) (or v itself) as limbs.  One CTA per token.
-__global__ void __launch_bounds__(256) rmsnorm_limbs_kernel(const float* v, int r, int v_stride, const float* gain,
-                                                            float eps, int use_rms, int8_t* limbs, float* scale) {
-  __shared__ float red[8];
+__global__ void __launch_bounds__(kVecThreads) rmsnorm_limbs_kernel(const float* v, int r, int v_stride, const float* gain,
+                                                                    float eps, int use_rms, int8_t* limbs, float* scale) {
+  __shared__ float red[kVecThreads / 32], red2[kVecThreads / 32];
   pdl_launch_dependents();
   pdl_wait();
   const int b = blockIdx.x;
-  const float* vb = v + (size_t)b * v_stride;
-  float inv = 1.f;
-  if (use_rms) {
-    float ss = 0.f;
-    for (int k = threadIdx.x; k < r; k += blockDim.x) ss = fmaf(vb[k], vb[k], ss);
-    ss = warp_sum(ss);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-    __syncthreads();
-    float tot = 0.f;
+  const KeptVec vec(v + (size_t)b * v_stride, r);
+  const float inv_rms = use_rms ? inverse_rms(vec, eps, red) : 1.f;
+  auto n_of = [&](int k, float e) { return use_rms ? (gain ? gain[k] : 1.f) * e * inv_rms : e; };
+  float m = 0.f;
+  vec.each([&](int k, float e) { m = fmaxf(m, fabsf(n_of(k, e))); });
+  const float s = limb_scale(m, red2, kVecThreads / 32);
+  if (threadIdx.x == 0) scale[b] = s;
+  const float inv = 1.f / s;
+  vec.each([&](int k, float e) {
+    int q4[4];
+    limbs_of(n_of(k, e), inv, q4);
 #pragma unroll
-    for (int w = 0; w < 8; ++w) tot += red[w];
-    inv = rsqrtf(tot / (float)r + eps);
-  }
-  write_limbs([&](int k) { return use_rms ? (gain ? gain[k] : 1.f) * vb[k] * inv : vb[k]; }, r, limbs + (size_t)4 * b * r,
-              scale + b, red);
+    for (int l = 0; l < 4; ++l) limbs[((size_t)4 * b + l) * r + k] = (int8_t)q4[l];
+  });
 }
 
 }  // namespace
@@ -1716,19 +1780,19 @@ cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s) {
 }
 
 cudaError_t launch_token_limbs(const void* x, int B, int K, int x_stride, void* limbs, float* scale, cudaStream_t s) {
-  return launch_pdl(token_limbs_kernel, dim3(B), dim3(256), 0, s, static_cast<const __nv_bfloat16*>(x), K, x_stride,
+  return launch_pdl(token_limbs_kernel, dim3(B), dim3(kLimbThreads), 0, s, static_cast<const __nv_bfloat16*>(x), K, x_stride,
                     static_cast<int8_t*>(limbs), scale);
 }
 
 cudaError_t launch_rmsnorm_limbs(const float* v, int B, int r, int v_stride, const float* gain, float eps, bool use_rms,
                                  void* limbs, float* scale, cudaStream_t s) {
-  return launch_pdl(rmsnorm_limbs_kernel, dim3(B), dim3(256), 0, s, v, r, v_stride, gain, eps, use_rms ? 1 : 0,
+  return launch_pdl(rmsnorm_limbs_kernel, dim3(B), dim3(kVecThreads), 0, s, v, r, v_stride, gain, eps, use_rms ? 1 : 0,
                     static_cast<int8_t*>(limbs), scale);
 }
 
 cudaError_t launch_rmsnorm_split(const float* v, int B, int r, int v_stride, const float* gain, float eps,
                                  bool use_rms, int cols, bool exact, void* x2, cudaStream_t s) {
-  return launch_pdl(rmsnorm_split_kernel, dim3(B), dim3(256), 0, s, v, r, v_stride, gain, eps, use_rms ? 1 : 0, cols, exact ? 1 : 0,
+  return launch_pdl(rmsnorm_split_kernel, dim3(B), dim3(kVecThreads), 0, s, v, r, v_stride, gain, eps, use_rms ? 1 : 0, cols, exact ? 1 : 0,
                     static_cast<__nv_bfloat16*>(x2));
 }
 
