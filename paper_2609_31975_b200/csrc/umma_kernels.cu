@@ -20,7 +20,7 @@
 //              lets the copies run at memory speed; warp 8 allocates and frees the TMEM columns
 //   warps 4-7  epilogue: tcgen05.ld the accumulator row of "their" neuron (all accumulators added), apply the
 //              gate / scale epilogue; for wide batches all twelve warps share the epilogue of the CTA's last tile
-// A tile has 128 rows when a CTA owns several tiles; a smaller problem is cut into one tile per SM.  The ring of
+// A problem of up to 256 rows per SM is cut into one or two tiles per SM, all of one height (see tile_rows_for).  The ring of
 // stages (up to 12) is cut out of the dynamic shared memory on the device, once the tile height is known.
 // Every kernel here is launched with programmatic dependent launch: set-up first, griddepcontrol.wait before the
 // first dependent read or global write.
@@ -321,11 +321,17 @@ __device__ __forceinline__ void expand_block_q4_i8(uint32_t raw, uint32_t dst, i
 // Makes this thread's shared-memory stores visible to the tensor core's reads.
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// Rows per tile: 128 when there is more than one tile per CTA, otherwise the row count spread over
-// the whole grid (a multiple of 8, the swizzle period), so that every SM streams a share.
-__host__ __device__ inline int tile_rows_for(int n_rows, int grid) {
-  if (n_rows >= kTileRows * grid) return kTileRows;
-  int t = ((n_rows + grid - 1) / grid + 7) & ~7;
+// Rows per tile of a GEMM over rows of K elements: the row count spread over the whole grid, one tile or two for each CTA (a
+// multiple of 8, the swizzle period), so that every SM streams a share.  Two tiles of equal height, not tiles of 128 rows
+// whose second wave leaves most SMs idle: 24000 rows are 273 tiles of 88 rows, where 188 of 128 kept 40 of 148 SMs busy in the
+// second half (bf16, 5120 x 20000, 2 / 32 tokens: 80.7 / 155 -> 70.5 / 127 us; int4, 8192 x 24000, 64: 484 -> 339).  128
+// where a CTA owns more than two, and for short rows (the LoPA gate), whose tiles are gone before the imbalance shows (r =
+// 512 / 1024: 0 to 1 % faster; r = 1536: equal tiles 1 to 3 % faster).
+constexpr int kShortRow = 1024;
+__host__ __device__ inline int tile_rows_for(int n_rows, int grid, int K) {
+  const int per_cta = n_rows > kTileRows * grid ? 2 : 1;
+  if (n_rows > 2 * kTileRows * grid || (per_cta == 2 && K <= kShortRow)) return kTileRows;
+  int t = ((n_rows + per_cta * grid - 1) / (per_cta * grid) + 7) & ~7;
   return t < 8 ? 8 : t > kTileRows ? kTileRows : t;
 }
 
@@ -555,7 +561,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
   const bool walk_all = MODE == kUpMayWalk && own_list && p.walk_all &&
                         (long long)n_listed * 100 >= (long long)p.R * kWalkAllPercent;
   if (walk_all) n_rows = p.R;
-  const int tile_rows = tile_rows_for(n_rows, gridDim.x);
+  const int tile_rows = tile_rows_for(n_rows, gridDim.x, p.K);
   const int n_tiles = (n_rows + tile_rows - 1) / tile_rows;
   if (own_list && walk_all) {
     // publish the list only: word w is written out by CTA w mod grid
@@ -1554,15 +1560,15 @@ __global__ void __launch_bounds__(kVecThreads) rmsnorm_limbs_kernel(const float*
 
 
 // Tiling of the gate GEMM over R rows (the up kernel needs it to read the gate's bit masks).
-void umma_gate_tiling(int R, int sm_count, int* tile_rows, int* n_tiles) {
+void umma_gate_tiling(int R, int K, int sm_count, int* tile_rows, int* n_tiles) {
   const int grid = R < 8 * sm_count ? (R + 7) / 8 : sm_count;
-  *tile_rows = tile_rows_for(R, grid);
+  *tile_rows = tile_rows_for(R, grid, K);
   *n_tiles = (R + *tile_rows - 1) / *tile_rows;
 }
 
-bool umma_own_list_supported(int R, int sm_count) {
+bool umma_own_list_supported(int R, int K, int sm_count) {
   int tr, nt;
-  umma_gate_tiling(R, sm_count, &tr, &nt);
+  umma_gate_tiling(R, K, sm_count, &tr, &nt);
   return 4 * nt <= kScanChunks * kThreadsRows && R <= (long long)kMaxOwnTiles * kTileRows * sm_count;
 }
 
@@ -1697,7 +1703,7 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
   if (p.npad > kUmmaMaxCols) return cudaErrorInvalidValue;
   if (i8 && (p.K % 128 || !p.tok_scale)) return cudaErrorInvalidValue;
   // weights: all R rows; boxes of one tile's rows for the gate, single-row boxes for the gather
-  if (!make_weight_map(&map_w, p.W, p.K, p.R, up ? 1 : tile_rows_for(p.R, grid), p.qbits)) return cudaErrorNotSupported;
+  if (!make_weight_map(&map_w, p.W, p.K, p.R, up ? 1 : tile_rows_for(p.R, grid, p.K), p.qbits)) return cudaErrorNotSupported;
   // tokens: only the rows that exist; the box covers npad rows and the rest reads as zero
   if (i8 ? !make_map_i8(&map_x, p.X, p.K, p.ncols_valid, (size_t)p.x_stride, p.npad)
                    : !make_map(&map_x, p.X, p.K, p.ncols_valid, (size_t)p.x_stride, p.npad))
@@ -1707,7 +1713,7 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
     // wide batches: the union may cover most rows; the kernel then walks every row with tiled boxes of the tile
     // height of R rows (decided on the device from the union's size, so it depends on this call's inputs only)
     WalkMap<true> map_t;
-    if (!make_weight_map(&map_t.m, p.W, p.K, p.R, tile_rows_for(p.R, grid), p.qbits)) return cudaErrorNotSupported;
+    if (!make_weight_map(&map_t.m, p.W, p.K, p.R, tile_rows_for(p.R, grid, p.K), p.qbits)) return cudaErrorNotSupported;
     return launch_rows_mode<kUpMayWalk>(p, grid, smem, s, map_w, map_x, map_t);
   }
   return launch_rows_mode<kUp>(p, grid, smem, s, map_w, map_x, WalkMap<false>{});

@@ -1,0 +1,74 @@
+"""Tiles of the batched gate and up GEMMs where the rows are more than 128 per SM: two of equal height for each CTA."""
+import ctypes
+
+import pytest
+import torch
+
+import synthetic_inputs as syn
+from parity import assert_active_set, assert_y_close, run_oracle
+
+DEV = "cuda:0"
+
+
+def tiling(lib, R, K, sms=148):
+    tr, nt, own = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
+    lib.sffn_test_umma_row_tiling(R, K, sms, ctypes.byref(tr), ctypes.byref(nt), ctypes.byref(own))
+    return tr.value, nt.value, own.value
+
+
+@pytest.mark.parametrize("sms", [132, 148, 160])
+def test_two_equal_tiles_for_each_cta(sms):
+    import paper_2609_31975_b200 as m
+
+    lib = m.load_library()
+    for R in (8, 1200, 14336, 128 * sms - 1, 128 * sms, 128 * sms + 1, 20000, 24000, 28672, 256 * sms - 7, 256 * sms, 256 * sms + 1, 60000):
+        for K in (64, 1024, 1088, 4096, 8192):
+            tr, nt, own = tiling(lib, R, K, sms)
+            assert tr % 8 == 0 and 8 <= tr <= 128 and (nt - 1) * tr < R <= nt * tr
+            if R <= 128 * sms:
+                assert nt <= sms
+            elif R <= 256 * sms and K > 1024:
+                assert nt <= 2 * sms and tr <= (R + 2 * sms - 1) // (2 * sms) + 7   # no taller than a share, rounded up
+            else:
+                assert tr == 128
+            assert not own or 4 * nt <= 4 * 384                                     # mask words fit the in-kernel scan
+    assert tiling(lib, 24000, 8192) == (88, 273, 1)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("D,H,B,s", [
+    (1280, 18945, 3, 0.9),    # one row more than one tile per CTA holds; the union is one tile per CTA
+    (1280, 24001, 40, 0.5),   # a ragged last tile; the union is (nearly) every row, walked in the same tiles
+    (1280, 20000, 20, 0.3),   # the union is most rows, listed: two tiles per CTA
+])
+def test_batches_over_two_equal_tiles(D, H, B, s):
+    import paper_2609_31975_b200 as m
+
+    ffn = m.SparseFFN(D, H, torch.bfloat16, B_max=B)
+    w = syn.standard_ffn(D, H, torch.bfloat16, 71, DEV, sparsity=s)
+    gate = {"W_g": w["W_g"]}
+    x = syn.tokens(B, D, torch.bfloat16, 71, DEV)
+    ref = run_oracle(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu", threads=16)
+    y = ffn.sparse_ffn_forward(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0
+    assert_y_close(y, ref["y"], what=f"{D}x{H} B={B}")
+    assert_active_set(ffn.last_active(), ref, what=f"{D}x{H} B={B}")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("D", [256, 1280, 4096, 8192, 8448])
+def test_token_limbs_of_every_width(D):
+    """Widths below, at and above what the limb kernel's threads keep in registers: the batch against the single-token calls,
+    whose tokens go through other code (their error is 3e-5 of a group's largest entry, the batch's a bf16 h: 1e-2)."""
+    import paper_2609_31975_b200 as m
+
+    w = syn.standard_ffn_q8(D, 300, 72, DEV, sparsity=0.5)
+    ffn = m.SparseFFN(D, 300, torch.bfloat16, B_max=3)
+    x = syn.tokens(3, D, torch.bfloat16, 72, DEV)
+    args = ({"W_g": w["W_g"]}, w["b_g"], w["W_up"], w["W_down"], "relu")
+    y = ffn.sparse_ffn_forward_q8(x, *args)
+    one = torch.stack([ffn.sparse_ffn_forward_q8(x[b], *args) for b in range(3)])
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0
+    assert ((y - one).norm() / one.norm()).item() < 1e-2
