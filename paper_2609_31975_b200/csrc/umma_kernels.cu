@@ -61,6 +61,7 @@ constexpr int kProducerWarps = 4;
 constexpr int kMaxStages = 16;                       // barrier slots; bf16 rows use up to 12
 constexpr int kMaxStagesBf16 = 12;
 constexpr int kExpandSlots = 4;                      // quantised rows: ring of expanded bf16 blocks
+constexpr int kDownExpand = 4;                       // the same in the down kernel, at most (2 or 4, see launch_umma_down)
 constexpr int kWalkMinTokens = 32;                   // batches from which the up kernel may walk every row
 constexpr int kWalkAllPercent = 70;                  // union share of the rows from which "every row" is walked
 constexpr int kMaxIssuers = 4;
@@ -1158,17 +1159,25 @@ __global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarp
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const int npad = p.npad;
   constexpr int kRawBytes = QB * kTileRows * kAtomK / 8;  // quantised rows: the codes of a stage's 64 rows x 128 columns
-  const int raw_off = kAAtomBytes + npad * 128;
+  // Quantised rows: a ring slot holds what the copies bring (h, then the codes); the expanded blocks have a short ring of
+  // their own in front of it (stage kb uses block kb mod E), as in the rows kernels.  One ring of slots with room for both was
+  // two slots deep from 24 tokens of int8 rows on (whole calls, 4096 x 14336, 24 / 64 tokens: 70.6 / 96.8 -> 62.5 / 88.6 us;
+  // 8192 x 24000, 24 tokens: 178 -> 145).  Exact sums keep the one ring.
+  constexpr bool kTwo = QB != 0 && !EX;
+  const int E = p.expand, expand_bytes = kTwo ? E * kAAtomBytes : 0;
+  const int b_off = kTwo ? 0 : kAAtomBytes;               // h within a slot
+  const int raw_off = b_off + npad * 128;
   const int stage_bytes = raw_off + kRawBytes;
   const int S = p.stages;
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)S * stage_bytes);
-  const uint32_t stage0 = smem_u32(smem);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + expand_bytes + (size_t)S * stage_bytes);
+  const uint32_t expand0 = smem_u32(smem), stage0 = expand0 + expand_bytes;
   const uint32_t full = smem_u32(bars), empty = smem_u32(bars + S);
   const uint32_t acc_full = smem_u32(bars + 2 * S);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  const uint32_t ready = smem_u32(bars + 2 * S + 4);
+  const uint32_t ready = smem_u32(bars + 2 * S + 4);  // expanded block written (kTwo: one per block, else one per slot) ...
+  const uint32_t afree = ready + 8 * kDownExpand;     // ... kTwo: and read by its MMAs
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int d_tiles = p.D / kTileRows;
@@ -1185,8 +1194,13 @@ __global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarp
     for (int s = 0; s < S; ++s) {
       mbar_init(full + 8 * s, 1);
       mbar_init(empty + 8 * s, 1);
-      if (QB) mbar_init(ready + 8 * s, kExpandWarps / 2);
+      if (QB && !kTwo) mbar_init(ready + 8 * s, kExpandWarps / 2);
     }
+    if (kTwo)
+      for (int e = 0; e < E; ++e) {
+        mbar_init(ready + 8 * e, kExpandWarps / 2);
+        mbar_init(afree + 8 * e, 1);
+      }
     if (EX)
       for (int q = 0; q < kMaxIssuers; ++q) {
         mbar_init(place_full + 8 * q, 1);
@@ -1268,7 +1282,7 @@ __global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarp
         tma_tile_2d(wdst + lane * kHalfBytes, &map_wt, (d0 + lane * kAtomK) / kColDiv, u0, full + 8 * s);
       }
       if (lane < terms)
-        tma_tile_2d(abase + kAAtomBytes + lane * p.cols * 128, &map_hm, u0, lane * p.h_cols + p.tok0, full + 8 * s);
+        tma_tile_2d(abase + b_off + lane * p.cols * 128, &map_hm, u0, lane * p.h_cols + p.tok0, full + 8 * s);
     }
   } else if (QB && warp >= kExpand0 / 32) {
     // ======================= expanders (quantised rows): the stage's codes -> its two bf16 blocks =
@@ -1279,14 +1293,17 @@ __global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarp
     for (int kb = 0; kb < kblocks; ++kb, ++s) {
       if (s == S) { s = 0; ph ^= 1; }
       if ((s & 1) != pair) continue;
-      const bool ok = mbar_wait(full + 8 * s, ph, abort_flag, p.status, p.wait_cycles);
+      const int e = kb & (E - 1);  // (of the parity of s, as S is even)
+      const bool ok = mbar_wait(full + 8 * s, ph, abort_flag, p.status, p.wait_cycles) &&
+                      (!kTwo || mbar_wait(afree + 8 * e, (kb & E) ? 0u : 1u, abort_flag, p.status, p.wait_cycles));
       if (!__all_sync(0xffffffffu, ok)) break;
-      const uint32_t sbase = stage0 + s * stage_bytes;
-      expand_block<QB ? QB : 8>(sbase + raw_off, sbase, kAtomK, et, 16 * kExpandWarps);
-      expand_block<QB ? QB : 8>(sbase + raw_off + kRawBytes / 2, sbase + kAAtomBytes / 2, kAtomK, et, 16 * kExpandWarps);
+      const uint32_t raw = stage0 + s * stage_bytes + raw_off;
+      const uint32_t dst = kTwo ? expand0 + e * kAAtomBytes : stage0 + s * stage_bytes;
+      expand_block<QB ? QB : 8>(raw, dst, kAtomK, et, 16 * kExpandWarps);
+      expand_block<QB ? QB : 8>(raw + kRawBytes / 2, dst + kAAtomBytes / 2, kAtomK, et, 16 * kExpandWarps);
       fence_proxy_async();
       __syncwarp();
-      if (lane == 0) mbar_arrive(ready + 8 * s);
+      if (lane == 0) mbar_arrive(ready + 8 * (kTwo ? e : s));
     }
   } else if (warp >= 8 && warp < 12) {
     // ======================= MMA issuers (slot s belongs to issuer s mod 2) =====================
@@ -1318,14 +1335,18 @@ __global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarp
       for (int kb = 0; kb < kblocks; ++kb, ++s) {
         if (s == S) { s = 0; ph ^= 1; }
         if (nacc == 2 && (s & 1) != m) continue;
-        if (!mbar_wait((QB ? ready : full) + 8 * s, ph, abort_flag, p.status, p.wait_cycles)) { ok = false; break; }
+        const int e = kb & (E - 1);
+        if (!(kTwo ? mbar_wait(ready + 8 * e, (kb & E) ? 1u : 0u, abort_flag, p.status, p.wait_cycles)
+                   : mbar_wait(full + 8 * s, ph, abort_flag, p.status, p.wait_cycles))) { ok = false; break; }
         tc_fence_after();
         const uint32_t sbase = stage0 + s * stage_bytes;
-        const uint64_t bdesc = make_desc(sbase + kAAtomBytes);
+        const uint32_t abase = kTwo ? expand0 + e * kAAtomBytes : sbase;
+        const uint64_t bdesc = make_desc(sbase + b_off);
 #pragma unroll
         for (int k = 0; k < kAtomK / 16; ++k)  // 16 list rows = two groups of eight swizzle rows
-          umma(acc, make_desc_mn(sbase + k * 2048, 8192, 1024), bdesc + 2 * k, idesc, (kb >= nacc || k > 0) ? 1u : 0u);
+          umma(acc, make_desc_mn(abase + k * 2048, 8192, 1024), bdesc + 2 * k, idesc, (kb >= nacc || k > 0) ? 1u : 0u);
         umma_commit(empty + 8 * s);
+        if (kTwo) umma_commit(afree + 8 * e);
       }
       if (ok && kblocks > 0) umma_commit(acc_full);
     }
@@ -1761,13 +1782,20 @@ cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s) {
   p.npad = (own + 15) / 16 * 16;
   if (p.cols % 8 || p.cols < p.B || p.npad > kUmmaMaxCols) return cudaErrorInvalidValue;
   p.wait_cycles = fused_test_knobs().wait_cycles;
-  const int stage_bytes = kAAtomBytes + p.npad * 128 + p.qbits * kTileRows * kAtomK / 8;
-  int stages = ((down_pairs(own, p.exact) ? 111 : 225) * 1024 - 1024 - 1024) / stage_bytes;
+  const bool two = p.qbits && !p.exact;  // rings of copies and of expanded blocks
+  const int stage_bytes = (two ? 0 : kAAtomBytes) + p.npad * 128 + p.qbits * kTileRows * kAtomK / 8;
+  // Expanded blocks: two leave more slots for the copies, which is worth more (int8, 4096 x 14336, 16 tokens, 2 / 4: 56.9 /
+  // 58.1 us; int4, 8192 x 24000, 24: 155 / 165), but four where a CTA has the SM to itself (int4, 2688 x 8000, 64: 67.2 /
+  // 65.7) and for 4-bit codes from 32 columns on, while four slots remain (8192 x 24000, 32: 255 / 252).
+  const int room = (down_pairs(own, p.exact) ? 111 : 225) * 1024 - 1024 - 1024;
+  p.expand = !down_pairs(own, p.exact) || (p.qbits == 4 && own >= 32 && room - 4 * kAAtomBytes >= 4 * stage_bytes) ? kDownExpand : 2;
+  const int expanded = two ? p.expand * kAAtomBytes : 0;
+  int stages = (room - expanded) / stage_bytes;
   if (stages > 12) stages = 12;
   stages &= p.exact ? ~3 : ~1;
   if (stages < 2) return cudaErrorInvalidValue;
   p.stages = stages;
-  const size_t smem = 1024 + (size_t)stages * stage_bytes + (3 * stages + 4 + 2 * kMaxIssuers) * 8 + 64;
+  const size_t smem = 1024 + expanded + (size_t)stages * stage_bytes + (3 * stages + 4 + 2 * kMaxIssuers + 2 * kDownExpand) * 8 + 64;
   const int grid = (p.D / kTileRows) * p.splits;
   alignas(64) CUtensorMap map_wg, map_wt, map_hm;
   // W_down [H, D]: inner dimension d; single-row boxes for the gather, 64-row boxes for the dense walk

@@ -78,7 +78,7 @@ struct UmmaDownParams {
   const int32_t* walk_all;  // device word: nonzero = walk every row of W_down instead of the list (set by the up kernel), or null
   float* partial;        // [splits][B][D]
   int32_t* status;
-  int npad, stages;      // filled by the launcher
+  int npad, stages, expand;  // filled by the launcher
   long long wait_cycles; // budget of every device-side wait (filled by the launcher)
 };
 
