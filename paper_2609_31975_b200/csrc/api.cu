@@ -352,6 +352,9 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
 
   const bool exact = umma && exact_batch(D, q8 != nullptr, g->kind == SFFN_GATE_LOPA);
   const int h_terms = h_terms_for(D, exact, q8 != nullptr);
+  const float* v = vbuf;  // v, or the runs of K that add up to it
+  int v_runs = 1;
+  size_t v_step = 0;
   if (lopa && umma) {  // v = V x on the tensor cores: the rows kernel with the identity as its epilogue
     UmmaRowsParams p{};
     p.W = g->V; p.R = g->r; p.K = D;
@@ -359,6 +362,14 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
     p.X = xb; p.x_stride = D; p.ncols_valid = B; p.B = B;
     if (native) { p.X = xlimb; p.ncols_valid = 4 * B; p.tok_scale = xscale; }
     p.act = kUmmaActIdentity; p.a_out = vbuf; p.a_stride = rs;
+    // (sums of runs of K lie where the down projection's go later: at least kMaxUpDownGrid * kMaxChunk * D floats)
+    if (!exact)
+      umma_k_splits(g->r, D, native, h->sm_count, (int)((long long)kMaxUpDownGrid * kMaxChunk * D / ((long long)B * rs)), &p.k_tiles, &p.k_splits);
+    if (p.k_splits > 1) {
+      v_runs = p.k_splits;
+      p.split_stride = v_step = (size_t)B * rs;
+      v = p.a_out = h->at<float>(h->L.partial);
+    }
     p.exact = exact;
     p.status = h->at<int32_t>(h->L.status);
     SFFN_CUDA(launch_umma_rows(false, p, native ? 4 * B : B, h->sm_count, s));
@@ -398,7 +409,7 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
     int cols = B;
     if (lopa && native) {
       // RMSNorm (or none) and the split into int8 limbs in one launch
-      SFFN_CUDA(launch_rmsnorm_limbs(vbuf, B, g->r, rs, g->rms_gain, g->rms_eps, g->use_rmsnorm != 0, nlimb, nscale, s));
+      SFFN_CUDA(launch_rmsnorm_limbs(v, B, g->r, rs, v_runs, v_step, g->rms_gain, g->rms_eps, g->use_rmsnorm != 0, nlimb, nscale, s));
       ++h->launches;
       p.W = g->U; p.K = g->r; p.X = nlimb; p.x_stride = g->r; p.tok_scale = nscale;
       p.g_idx = g->g_idx; p.g_sign = g->g_sign;
@@ -406,7 +417,7 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
     } else if (lopa) {
       // RMSNorm (or none) and the split into bf16 pairs (exact sums: triples) in one launch
       p.x_cols = round8(B);
-      SFFN_CUDA(launch_rmsnorm_split(vbuf, B, g->r, rs, g->rms_gain, g->rms_eps, g->use_rmsnorm != 0, p.x_cols, exact, x2, s));
+      SFFN_CUDA(launch_rmsnorm_split(v, B, g->r, rs, v_runs, v_step, g->rms_gain, g->rms_eps, g->use_rmsnorm != 0, p.x_cols, exact, x2, s));
       ++h->launches;
       p.W = g->U; p.K = g->r; p.X = x2; p.x_stride = g->r;
       p.g_idx = g->g_idx; p.g_sign = g->g_sign;

@@ -467,7 +467,12 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
   constexpr int kAtomElems = kNat ? 128 : kAtomK;              // elements of one 128-byte swizzle row
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int kblocks = p.K / kAtomElems;
+  // Gate mode: a second grid dimension cuts K into runs of blocks (see umma_k_splits); each writes sums of its own.
+  constexpr bool kSplits = MODE == kGate && !EX;
+  const int k_run = kSplits ? (p.K / kAtomElems + (int)gridDim.y - 1) / (int)gridDim.y : p.K / kAtomElems;
+  const int kb_first = kSplits ? (int)blockIdx.y * k_run : 0;
+  const int kblocks = min(k_run, p.K / kAtomElems - kb_first);
+  float* const a_out = p.a_out + (kSplits ? (size_t)blockIdx.y * p.split_stride : 0);
 
   // Set-up that needs nothing from earlier kernels runs while the predecessor in the stream finishes.
   pdl_launch_dependents();
@@ -725,7 +730,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
       // int32 accumulators, four columns per token (its limbs, most significant first, 7 bits apart):
       // value = token scale * row scale * (i0 + i1 / 128 + i2 / 128^2 + i3 / 128^3)
       __nv_bfloat16* hm = static_cast<__nv_bfloat16*>(p.hmT) + li;
-      float* arow = p.a_out + j;
+      float* arow = a_out + j;
       const __nv_bfloat16* xg = static_cast<const __nv_bfloat16*>(p.xtok) + (gi >= 0 ? gi : 0);
       for (int c0 = 8 * part; c0 < npad; c0 += 8 * nparts) {
         int iv[8];
@@ -771,7 +776,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
       }
     } else {
       const int act = p.act;
-      float* arow = p.a_out + j;
+      float* arow = a_out + j;
       const __nv_bfloat16* xg = static_cast<const __nv_bfloat16*>(p.xtok) + (gi >= 0 ? gi : 0);
       // LoPA: a token's vector is the sum of two bf16 vectors (columns b and x_cols + b), whose products are added here
       const int cols = p.x_cols ? p.x_cols : npad;
@@ -865,7 +870,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
           float z = kQ ? sum[i] * sc + bias : sum[i] + bias;
           if (gi >= 0) z += sg * __bfloat162float(xg[(size_t)b * p.xtok_stride]);
           fired |= z > 0.f;
-          p.a_out[(size_t)b * p.a_stride + j] = activation(p.act, z);
+          a_out[(size_t)b * p.a_stride + j] = activation(p.act, z);
         }
       }
     }
@@ -917,7 +922,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
         }
         const uint32_t abase = ring0 + s * stage_bytes;
         for (int a = 0; a < na; ++a) {
-          const int k0 = (kb * atoms + a) * kAtomElems;
+          const int k0 = (kb_first + kb * atoms + a) * kAtomElems;
           // where the weight block lands, the byte column it starts at, and the bytes of one landed row
           const uint32_t wdst = abase + w_off + a * (kExp ? raw_block_bytes : a_block_bytes);
           const int wc0 = QB == 2 ? k0 / 2 : kExp ? k0 * QB / 8 : k0;
@@ -1421,16 +1426,29 @@ __global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarp
 // The vector of a token for the small kernels below: entry k = threadIdx.x + i * blockDim.x of a row of up to kKept *
 // blockDim.x entries stays in register i from the first look at it; the rest of a longer row is read again.
 constexpr int kVecThreads = 256, kKept = 8;
+// An entry is the sum of `runs` values, `step` apart (see umma_k_splits).
 struct KeptVec {
   const float* v;
-  int r;
+  int r, runs;
+  size_t step;
   float kept[kKept];
-  __device__ __forceinline__ KeptVec(const float* v_, int r_) : v(v_), r(r_) {
+  __device__ __forceinline__ float at(int k) const {
+    float e = v[k];
+#pragma unroll 4
+    for (int i = 1; i < runs; ++i) e += v[i * step + k];
+    return e;
+  }
+  __device__ __forceinline__ KeptVec(const float* v_, int r_, int runs_, size_t step_) : v(v_), r(r_), runs(runs_), step(step_) {
 #pragma unroll
-    for (int i = 0; i < kKept; ++i) {
-      const int k = threadIdx.x + i * kVecThreads;
-      kept[i] = k < r ? v[k] : 0.f;
-    }
+    for (int i = 0; i < kKept; ++i) kept[i] = 0.f;
+    // four runs of all entries in flight, each entry added up in the order of the runs
+#pragma unroll 4
+    for (int run = 0; run < runs; ++run)
+#pragma unroll
+      for (int i = 0; i < kKept; ++i) {
+        const int k = threadIdx.x + i * kVecThreads;
+        if (k < r) kept[i] += v[run * step + k];
+      }
   }
   template <typename F>
   __device__ __forceinline__ void each(F f) const {  // f(k, entry) in ascending order of k
@@ -1439,7 +1457,7 @@ struct KeptVec {
       const int k = threadIdx.x + i * kVecThreads;
       if (k < r) f(k, kept[i]);
     }
-    for (int k = threadIdx.x + kKept * kVecThreads; k < r; k += kVecThreads) f(k, v[k]);
+    for (int k = threadIdx.x + kKept * kVecThreads; k < r; k += kVecThreads) f(k, at(k));
   }
 };
 // 1 / rms of the vector.
@@ -1458,14 +1476,14 @@ __device__ __forceinline__ float inverse_rms(const KeptVec& vec, float eps, floa
 // LoPA gate, batched: n = RMSNorm(v) (or v itself) as a sum of two bf16 vectors for the tensor cores: row b of
 // x2 holds the high part of token b's vector, row cols + b the low part (v - bf16(v)), so that the gate's U n keeps
 // close to fp32 accuracy.  `exact`: row 2 cols + b holds what those two leave (24 bits in all).  One CTA per token.
-__global__ void __launch_bounds__(kVecThreads) rmsnorm_split_kernel(const float* v, int r, int v_stride, const float* gain,
+__global__ void __launch_bounds__(kVecThreads) rmsnorm_split_kernel(const float* v, int r, int v_stride, int runs, size_t step, const float* gain,
                                                                     float eps, int use_rms, int cols, int exact,
                                                                     __nv_bfloat16* x2) {
   __shared__ float red[kVecThreads / 32];
   pdl_launch_dependents();
   pdl_wait();
   const int b = blockIdx.x;
-  const KeptVec vec(v + (size_t)b * v_stride, r);
+  const KeptVec vec(v + (size_t)b * v_stride, r, runs, step);
   const float inv = use_rms ? inverse_rms(vec, eps, red) : 1.f;
   vec.each([&](int k, float e) {
     float n = use_rms ? (gain ? gain[k] : 1.f) * e * inv : e;
@@ -1555,13 +1573,13 @@ __global__ void __launch_bounds__(kLimbThreads) token_limbs_kernel(const __nv_bf
 }
 
 // LoPA gate with int8 rows: n = RMSNorm(v) (or v itself) as limbs.  One CTA per token.
-__global__ void __launch_bounds__(kVecThreads) rmsnorm_limbs_kernel(const float* v, int r, int v_stride, const float* gain,
+__global__ void __launch_bounds__(kVecThreads) rmsnorm_limbs_kernel(const float* v, int r, int v_stride, int runs, size_t step, const float* gain,
                                                                     float eps, int use_rms, int8_t* limbs, float* scale) {
   __shared__ float red[kVecThreads / 32], red2[kVecThreads / 32];
   pdl_launch_dependents();
   pdl_wait();
   const int b = blockIdx.x;
-  const KeptVec vec(v + (size_t)b * v_stride, r);
+  const KeptVec vec(v + (size_t)b * v_stride, r, runs, step);
   const float inv_rms = use_rms ? inverse_rms(vec, eps, red) : 1.f;
   auto n_of = [&](int k, float e) { return use_rms ? (gain ? gain[k] : 1.f) * e * inv_rms : e; };
   float m = 0.f;
@@ -1667,7 +1685,7 @@ bool make_weight_map(CUtensorMap* m, const void* base, int K, int rows, int box_
 }
 
 template <int MODE, typename Map>
-cudaError_t launch_rows_mode(const UmmaRowsParams& p, int grid, size_t smem, cudaStream_t s, const CUtensorMap& map_w,
+cudaError_t launch_rows_mode(const UmmaRowsParams& p, dim3 grid, size_t smem, cudaStream_t s, const CUtensorMap& map_w,
                              const CUtensorMap& map_x, const Map& map_t) {
   static unsigned long long configured[4] = {0, 0, 0, 0};
   cudaError_t e;
@@ -1676,36 +1694,53 @@ cudaError_t launch_rows_mode(const UmmaRowsParams& p, int grid, size_t smem, cud
       static unsigned long long configured_ex[3] = {0, 0, 0};
       auto k = p.qbits == 8 ? umma_rows_kernel<MODE, 8, true> : p.qbits == 4 ? umma_rows_kernel<MODE, 4, true> : umma_rows_kernel<MODE, 0, true>;
       if ((e = allow_dynamic_smem(k, 227 * 1024, configured_ex[p.qbits == 8 ? 1 : p.qbits == 4 ? 2 : 0])) != cudaSuccess) return e;
-      return launch_pdl(k, dim3(grid), dim3(kThreadsRows + 128 + (p.qbits ? 32 * kExpandWarps : 0)), smem, s, p, map_w, map_x, map_t);
+      return launch_pdl(k, grid, dim3(kThreadsRows + 128 + (p.qbits ? 32 * kExpandWarps : 0)), smem, s, p, map_w, map_x, map_t);
     }
   }
   if (p.qbits == 1) {
     auto k = umma_rows_kernel<MODE, 1>;
     if ((e = allow_dynamic_smem(k, 227 * 1024, configured[3])) != cudaSuccess) return e;
-    return launch_pdl(k, dim3(grid), dim3(kThreadsRows), smem, s, p, map_w, map_x, map_t);
+    return launch_pdl(k, grid, dim3(kThreadsRows), smem, s, p, map_w, map_x, map_t);
   }
   if (p.qbits == 2) {
     static unsigned long long configured2 = 0;
     auto k = umma_rows_kernel<MODE, 2>;
     if ((e = allow_dynamic_smem(k, 227 * 1024, configured2)) != cudaSuccess) return e;
-    return launch_pdl(k, dim3(grid), dim3(kThreadsRows + 32 * kExpandWarps), smem, s, p, map_w, map_x, map_t);
+    return launch_pdl(k, grid, dim3(kThreadsRows + 32 * kExpandWarps), smem, s, p, map_w, map_x, map_t);
   }
   if (p.qbits == 8) {
     auto k = umma_rows_kernel<MODE, 8>;
     if ((e = allow_dynamic_smem(k, 227 * 1024, configured[0])) != cudaSuccess) return e;
-    return launch_pdl(k, dim3(grid), dim3(kThreadsRows + 32 * kExpandWarps), smem, s, p, map_w, map_x, map_t);
+    return launch_pdl(k, grid, dim3(kThreadsRows + 32 * kExpandWarps), smem, s, p, map_w, map_x, map_t);
   }
   if (p.qbits == 4) {
     auto k = umma_rows_kernel<MODE, 4>;
     if ((e = allow_dynamic_smem(k, 227 * 1024, configured[1])) != cudaSuccess) return e;
-    return launch_pdl(k, dim3(grid), dim3(kThreadsRows + 32 * kExpandWarps), smem, s, p, map_w, map_x, map_t);
+    return launch_pdl(k, grid, dim3(kThreadsRows + 32 * kExpandWarps), smem, s, p, map_w, map_x, map_t);
   }
   auto k = umma_rows_kernel<MODE, 0>;
   if ((e = allow_dynamic_smem(k, 227 * 1024, configured[2])) != cudaSuccess) return e;
-  return launch_pdl(k, dim3(grid), dim3(kThreadsRows), smem, s, p, map_w, map_x, map_t);
+  return launch_pdl(k, grid, dim3(kThreadsRows), smem, s, p, map_w, map_x, map_t);
 }
 
 }  // namespace
+
+// The LoPA stage v = V x has few rows (the rank) of many columns.  A tile of eight rows for each SM reads all token columns for
+// them: with tiles of up to 64 rows and K cut into runs, whose sums the next kernel adds in their order, a CTA reads an eighth
+// of that, and ranks below 8 rows per SM fill the SMs too.  A run has at least four K blocks.  Whole calls, 4096 x 14336, r =
+// 512, 5 / 64 tokens: 47.8 / 93.8 -> 47.1 / 87.6 us (bf16), 46.2 / 108 -> 43.9 / 98.2 (int4); 8192 x 28672, r = 1024, 8:
+// 117 -> 114 (bf16), 102 -> 97.9 (int8).
+void umma_k_splits(int R, int K, bool codes, int sm_count, int max_splits, int* tiles, int* splits) {
+  const int kb = K / (codes ? 128 : kAtomK);
+  auto least = [](int a, int b) { return a < b ? a : b; };
+  int t = (R + 63) / 64, n = least(least(max_splits, 16), least(sm_count / t, kb / 4));
+  *tiles = *splits = 1;
+  if (n < 2) return;
+  if (4 * t * n < 3 * sm_count) t = least((R + 7) / 8, sm_count / n);
+  const int rows = ((R + t - 1) / t + 7) & ~7, run = (kb + n - 1) / n;
+  *tiles = (R + rows - 1) / rows;
+  *splits = (kb + run - 1) / run;
+}
 
 cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, cudaStream_t s) {
   p.npad = (cols + 15) / 16 * 16;
@@ -1714,7 +1749,9 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
   if (p.x_cols && (p.x_cols % 8 || cols != (p.exact ? 3 : 2) * p.x_cols)) return cudaErrorInvalidValue;
   p.wait_cycles = fused_test_knobs().wait_cycles;
   p.drop_stage = fused_test_knobs().drop_stage;
-  const int grid = p.R < 8 * sm_count ? (p.R + 7) / 8 : sm_count;
+  const int splits = p.k_splits > 1 ? p.k_splits : 1;
+  if (splits > 1 && (up || p.exact || p.b_g || p.g_idx || p.flag || p.words_out || p.act != kUmmaActIdentity)) return cudaErrorInvalidValue;
+  const int grid = splits > 1 ? p.k_tiles : p.R < 8 * sm_count ? (p.R + 7) / 8 : sm_count;
   // all the dynamic shared memory a CTA can have; the kernel cuts its ring out of it once it knows its tiles
   const size_t smem = 226 * 1024;
   p.ring_bytes = (int)smem - 1024 - kHeaderBytes;
@@ -1729,15 +1766,15 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
   if (i8 ? !make_map_i8(&map_x, p.X, p.K, p.ncols_valid, (size_t)p.x_stride, p.npad)
                    : !make_map(&map_x, p.X, p.K, p.ncols_valid, (size_t)p.x_stride, p.npad))
     return cudaErrorNotSupported;
-  if (!up) return launch_rows_mode<kGate>(p, grid, smem, s, map_w, map_x, WalkMap<false>{});
+  if (!up) return launch_rows_mode<kGate>(p, dim3(grid, splits), smem, s, map_w, map_x, WalkMap<false>{});
   if (p.walk_all && umma_may_walk(p.B) && !p.exact) {
     // wide batches: the union may cover most rows; the kernel then walks every row with tiled boxes of the tile
     // height of R rows (decided on the device from the union's size, so it depends on this call's inputs only)
     WalkMap<true> map_t;
     if (!make_weight_map(&map_t.m, p.W, p.K, p.R, tile_rows_for(p.R, grid, p.K), p.qbits)) return cudaErrorNotSupported;
-    return launch_rows_mode<kUpMayWalk>(p, grid, smem, s, map_w, map_x, map_t);
+    return launch_rows_mode<kUpMayWalk>(p, dim3(grid), smem, s, map_w, map_x, map_t);
   }
-  return launch_rows_mode<kUp>(p, grid, smem, s, map_w, map_x, WalkMap<false>{});
+  return launch_rows_mode<kUp>(p, dim3(grid), smem, s, map_w, map_x, WalkMap<false>{});
 }
 
 // Token columns up to which two CTAs of the down kernel share an SM (each with two accumulators in half of the TMEM, and
@@ -1818,16 +1855,16 @@ cudaError_t launch_token_limbs(const void* x, int B, int K, int x_stride, void* 
                     static_cast<int8_t*>(limbs), scale);
 }
 
-cudaError_t launch_rmsnorm_limbs(const float* v, int B, int r, int v_stride, const float* gain, float eps, bool use_rms,
-                                 void* limbs, float* scale, cudaStream_t s) {
-  return launch_pdl(rmsnorm_limbs_kernel, dim3(B), dim3(kVecThreads), 0, s, v, r, v_stride, gain, eps, use_rms ? 1 : 0,
+cudaError_t launch_rmsnorm_limbs(const float* v, int B, int r, int v_stride, int runs, size_t step, const float* gain, float eps,
+                                 bool use_rms, void* limbs, float* scale, cudaStream_t s) {
+  return launch_pdl(rmsnorm_limbs_kernel, dim3(B), dim3(kVecThreads), 0, s, v, r, v_stride, runs, step, gain, eps, use_rms ? 1 : 0,
                     static_cast<int8_t*>(limbs), scale);
 }
 
-cudaError_t launch_rmsnorm_split(const float* v, int B, int r, int v_stride, const float* gain, float eps,
+cudaError_t launch_rmsnorm_split(const float* v, int B, int r, int v_stride, int runs, size_t step, const float* gain, float eps,
                                  bool use_rms, int cols, bool exact, void* x2, cudaStream_t s) {
-  return launch_pdl(rmsnorm_split_kernel, dim3(B), dim3(kVecThreads), 0, s, v, r, v_stride, gain, eps, use_rms ? 1 : 0, cols, exact ? 1 : 0,
-                    static_cast<__nv_bfloat16*>(x2));
+  return launch_pdl(rmsnorm_split_kernel, dim3(B), dim3(kVecThreads), 0, s, v, r, v_stride, runs, step, gain, eps, use_rms ? 1 : 0,
+                    cols, exact ? 1 : 0, static_cast<__nv_bfloat16*>(x2));
 }
 
 }  // namespace sffn

@@ -72,3 +72,36 @@ def test_token_limbs_of_every_width(D):
     torch.cuda.synchronize()
     assert ffn.device_status() == 0
     assert ((y - one).norm() / one.norm()).item() < 1e-2
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("D,r,B", [
+    (256, 64, 2),       # too few columns to cut
+    (512, 128, 3),      # two runs
+    (4096, 64, 5),      # sixteen runs of one tile's rows
+    (3840, 448, 16),    # runs of unequal length
+    (4352, 1088, 70),   # unequal runs, a ragged last tile of rows
+    (2304, 2112, 4),    # a vector longer than what the norm kernel's threads keep
+])
+@pytest.mark.parametrize("q8", [False, True])
+def test_lopa_batches_with_v_from_several_runs_of_columns(D, r, B, q8):
+    """bf16: against the oracle.  int8: against the single-token calls, whose gate vector is summed elsewhere (fp32 sums on both
+    sides, a bf16 h in the batch: 1e-2)."""
+    import paper_2609_31975_b200 as m
+
+    H = 600
+    r = r // 128 * 128 or 128 if q8 else r
+    w = syn.lopa_ffn_q8(D, H, r, 73, DEV, sparsity=0.7) if q8 else syn.lopa_ffn(D, H, r, torch.bfloat16, 73, DEV, sparsity=0.7)
+    gate = {"V": w["V"], "U": w["U"], "g_idx": m.g_diagonal(H, D, DEV)}
+    ffn = m.SparseFFN(D, H, torch.bfloat16, r_max=r, B_max=B)
+    x = syn.tokens(B, D, torch.bfloat16, 73, DEV)
+    args = (gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+    y = (ffn.sparse_ffn_forward_q8 if q8 else ffn.sparse_ffn_forward)(x, *args)
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0
+    if q8:
+        one = torch.stack([ffn.sparse_ffn_forward_q8(x[b], *args) for b in range(B)])
+        assert ((y - one).norm() / one.norm()).item() < 1e-2
+    else:
+        ref = run_oracle(x, *args)
+        assert_y_close(y, ref["y"], what=f"{D} r={r} B={B}")
