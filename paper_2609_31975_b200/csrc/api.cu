@@ -335,10 +335,6 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
   void* nlimb = h->ws + h->L.nlimb;
   float* xscale = h->at<float>(h->L.tscale);
   float* nscale = xscale + kMaxMmaTokens;
-  if (native) {
-    SFFN_CUDA(launch_token_limbs(x, B, D, D, xlimb, xscale, s));
-    ++h->launches;
-  }
   float* actbuf = h->at<float>(h->L.act);
   uint8_t* flag = h->at<uint8_t>(h->L.flag);
   int32_t* idx = h->at<int32_t>(h->L.idx);
@@ -352,24 +348,32 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
 
   const bool exact = umma && exact_batch(D, q8 != nullptr, g->kind == SFFN_GATE_LOPA);
   const int h_terms = h_terms_for(D, exact, q8 != nullptr);
-  const float* v = vbuf;  // v, or the runs of K that add up to it
-  int v_runs = 1;
-  size_t v_step = 0;
+  // v = V x can be cut into runs of K, whose sums lie where the down projection's go later (at least kMaxUpDownGrid * kMaxChunk
+  // * D floats): fp32 sums of each run, which the norm adds in their order, or (limbs) one integer sum of all, the same
+  // bits as without runs.  (The room bounds the fp32 runs of wide vectors of many tokens, so that their number, and with it the
+  // order of the sums, can depend on the size of the batch, as the number of accumulators does.)
+  float* v = vbuf;
+  int v_tiles = 1, v_runs = 1, vs = rs;
+  if (lopa && umma && !exact) {
+    const long long room = (long long)kMaxUpDownGrid * kMaxChunk * D / B;
+    umma_k_splits(g->r, D, native, h->sm_count, !native ? (int)(room / rs) : room / g->r >= 4 ? 16 : 1, &v_tiles, &v_runs);
+    if (v_runs > 1) {
+      v = h->at<float>(h->L.partial);
+      if (native) vs = g->r;
+    }
+  }
+  if (native) {
+    SFFN_CUDA(launch_token_limbs(x, B, D, D, xlimb, xscale, v, v_runs > 1 ? 16 * vs : 0, s));
+    ++h->launches;
+  }
   if (lopa && umma) {  // v = V x on the tensor cores: the rows kernel with the identity as its epilogue
     UmmaRowsParams p{};
     p.W = g->V; p.R = g->r; p.K = D;
     p.qbits = wq_rows; p.w_scale = q8 ? q8->s_V : nullptr;
     p.X = xb; p.x_stride = D; p.ncols_valid = B; p.B = B;
     if (native) { p.X = xlimb; p.ncols_valid = 4 * B; p.tok_scale = xscale; }
-    p.act = kUmmaActIdentity; p.a_out = vbuf; p.a_stride = rs;
-    // (sums of runs of K lie where the down projection's go later: at least kMaxUpDownGrid * kMaxChunk * D floats)
-    if (!exact)
-      umma_k_splits(g->r, D, native, h->sm_count, (int)((long long)kMaxUpDownGrid * kMaxChunk * D / ((long long)B * rs)), &p.k_tiles, &p.k_splits);
-    if (p.k_splits > 1) {
-      v_runs = p.k_splits;
-      p.split_stride = v_step = (size_t)B * rs;
-      v = p.a_out = h->at<float>(h->L.partial);
-    }
+    p.act = kUmmaActIdentity; p.a_out = v; p.a_stride = vs;
+    p.k_tiles = v_tiles; p.k_splits = v_runs; p.split_stride = native ? 0 : (size_t)B * vs;
     p.exact = exact;
     p.status = h->at<int32_t>(h->L.status);
     SFFN_CUDA(launch_umma_rows(false, p, native ? 4 * B : B, h->sm_count, s));
@@ -409,7 +413,8 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
     int cols = B;
     if (lopa && native) {
       // RMSNorm (or none) and the split into int8 limbs in one launch
-      SFFN_CUDA(launch_rmsnorm_limbs(v, B, g->r, rs, v_runs, v_step, g->rms_gain, g->rms_eps, g->use_rmsnorm != 0, nlimb, nscale, s));
+      const UmmaLimbSums sums{q8->s_V, xscale, qbits == 8 ? 1.f : 0.0625f};
+      SFFN_CUDA(launch_rmsnorm_limbs(v, B, g->r, vs, v_runs > 1 ? &sums : nullptr, g->rms_gain, g->rms_eps, g->use_rmsnorm != 0, nlimb, nscale, s));
       ++h->launches;
       p.W = g->U; p.K = g->r; p.X = nlimb; p.x_stride = g->r; p.tok_scale = nscale;
       p.g_idx = g->g_idx; p.g_sign = g->g_sign;
@@ -417,7 +422,7 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
     } else if (lopa) {
       // RMSNorm (or none) and the split into bf16 pairs (exact sums: triples) in one launch
       p.x_cols = round8(B);
-      SFFN_CUDA(launch_rmsnorm_split(v, B, g->r, rs, v_runs, v_step, g->rms_gain, g->rms_eps, g->use_rmsnorm != 0, p.x_cols, exact, x2, s));
+      SFFN_CUDA(launch_rmsnorm_split(v, B, g->r, rs, v_runs, (size_t)B * rs, g->rms_gain, g->rms_eps, g->use_rmsnorm != 0, p.x_cols, exact, x2, s));
       ++h->launches;
       p.W = g->U; p.K = g->r; p.X = x2; p.x_stride = g->r;
       p.g_idx = g->g_idx; p.g_sign = g->g_sign;

@@ -206,6 +206,12 @@ __device__ __forceinline__ void tmem_ld8_int(uint32_t taddr, int nacc, int strid
   }
 }
 
+// What the products with a token's four limbs (most significant first, 7 bits apart) amount to: i0 + i1 / 128 + i2 / 128^2 +
+// i3 / 128^3.
+__device__ __forceinline__ float limb_sum(int i0, int i1, int i2, int i3) {
+  return ((float)i0 + (float)i1 * 0.0078125f) + ((float)i2 * 6.103515625e-05f + (float)i3 * 4.76837158203125e-07f);
+}
+
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
@@ -727,8 +733,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
       }
     };
     if constexpr (kNat) {
-      // int32 accumulators, four columns per token (its limbs, most significant first, 7 bits apart):
-      // value = token scale * row scale * (i0 + i1 / 128 + i2 / 128^2 + i3 / 128^3)
+      // int32 accumulators, four columns per token (its limbs): value = token scale * row scale * their sum
       __nv_bfloat16* hm = static_cast<__nv_bfloat16*>(p.hmT) + li;
       float* arow = a_out + j;
       const __nv_bfloat16* xg = static_cast<const __nv_bfloat16*>(p.xtok) + (gi >= 0 ? gi : 0);
@@ -739,9 +744,12 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
         for (int q = 0; q < 2; ++q) {
           const int b = c0 / 4 + q;
           if (row_ok && b < B) {
-            const float val = p.tok_scale[b] * sc *
-                              (((float)iv[4 * q] + (float)iv[4 * q + 1] * 0.0078125f) +
-                               ((float)iv[4 * q + 2] * 6.103515625e-05f + (float)iv[4 * q + 3] * 4.76837158203125e-07f));
+            if (kSplits && p.k_splits > 1) {  // a run of K: added to the integer sums of the others, in whatever order
+#pragma unroll
+              for (int l = 0; l < 4; ++l) atomicAdd(reinterpret_cast<int*>(a_out) + (size_t)(4 * b + l) * p.a_stride + j, iv[4 * q + l]);
+              continue;
+            }
+            const float val = p.tok_scale[b] * sc * limb_sum(iv[4 * q], iv[4 * q + 1], iv[4 * q + 2], iv[4 * q + 3]);
             if (UP) {
               const float av = p.a[(size_t)b * p.a_stride + j];
               hm[(size_t)b * p.hm_stride] = __float2bfloat16(av * activation(p.act_up, val) * osc);
@@ -1523,7 +1531,7 @@ __device__ __forceinline__ void limbs_of(float e, float inv, int* q4) {
 // 4096 x 14336 with 2 to 64 tokens 8 to 9 us longer, of 8192 x 24000 20 us).
 constexpr int kLimbThreads = 512, kLimbRounds = 2;
 __global__ void __launch_bounds__(kLimbThreads) token_limbs_kernel(const __nv_bfloat16* x, int K, int x_stride, int8_t* limbs,
-                                                                   float* scale) {
+                                                                   float* scale, int4* zero, int zero_n) {
   __shared__ float red[kLimbThreads / 32];
   pdl_launch_dependents();
   pdl_wait();
@@ -1543,6 +1551,7 @@ __global__ void __launch_bounds__(kLimbThreads) token_limbs_kernel(const __nv_bf
     const int k = threadIdx.x + i * kLimbThreads;
     kept[i] = k < n8 ? xb[k] : make_uint4(0, 0, 0, 0);
   }
+  for (int k = threadIdx.x; k < zero_n; k += kLimbThreads) zero[(size_t)b * zero_n + k] = make_int4(0, 0, 0, 0);
 #pragma unroll
   for (int i = 0; i < kLimbRounds; ++i) largest(kept[i]);
   for (int k = threadIdx.x + kLimbRounds * kLimbThreads; k < n8; k += kLimbThreads) largest(xb[k]);
@@ -1572,27 +1581,70 @@ __global__ void __launch_bounds__(kLimbThreads) token_limbs_kernel(const __nv_bf
   for (int k = threadIdx.x + kLimbRounds * kLimbThreads; k < n8; k += kLimbThreads) put(k, xb[k]);
 }
 
-// LoPA gate with int8 rows: n = RMSNorm(v) (or v itself) as limbs.  One CTA per token.
-__global__ void __launch_bounds__(kVecThreads) rmsnorm_limbs_kernel(const float* v, int r, int v_stride, int runs, size_t step, const float* gain,
-                                                                    float eps, int use_rms, int8_t* limbs, float* scale) {
-  __shared__ float red[kVecThreads / 32], red2[kVecThreads / 32];
+// The entries of v for the kernel below: fp32 values, or the four limbs' integer sums over all runs of K (see umma_k_splits), from
+// which v gets the bits that it has without runs.
+struct PlainVec {
+  float* v;
+  int stride;
+  __device__ __forceinline__ void token(int b) { v += (size_t)b * stride; }
+  __device__ __forceinline__ float entry(int k) const { return v[k]; }
+  __device__ __forceinline__ float& home(int k) const { return v[k]; }
+};
+struct LimbSumsVec {
+  int* v;
+  int stride;
+  const float *row_scale, *tok_scale;
+  float code_scale, tok;
+  __device__ __forceinline__ void token(int b) { v += (size_t)4 * b * stride, tok = tok_scale[b]; }
+  __device__ __forceinline__ float entry(int k) const {
+    return tok * (row_scale[k] * code_scale) * limb_sum(v[k], v[stride + k], v[2 * stride + k], v[3 * stride + k]);
+  }
+  __device__ __forceinline__ float& home(int k) const { return *reinterpret_cast<float*>(v + k); }
+};
+
+// LoPA gate with int8 rows: n = RMSNorm(v) (or v itself) as limbs.  One CTA per token.  An entry is fetched once, by a thread
+// that keeps it in shared memory (past kVecKept entries: at its home); the squares are added by the first kVecThreads threads
+// whatever the block, which fixes the order of that sum.
+constexpr int kVecMaxThreads = 1024, kVecKept = 4096;
+template <typename Vec>
+__global__ void __launch_bounds__(kVecMaxThreads) rmsnorm_limbs_kernel(Vec vec, int r, const float* gain, float eps, int use_rms,
+                                                                       int8_t* limbs, float* scale) {
+  __shared__ float kept[kVecKept], red[kVecMaxThreads / 32], red2[kVecMaxThreads / 32];
   pdl_launch_dependents();
   pdl_wait();
-  const int b = blockIdx.x;
-  const KeptVec vec(v + (size_t)b * v_stride, r, runs, step);
-  const float inv_rms = use_rms ? inverse_rms(vec, eps, red) : 1.f;
-  auto n_of = [&](int k, float e) { return use_rms ? (gain ? gain[k] : 1.f) * e * inv_rms : e; };
+  const int b = blockIdx.x, tid = threadIdx.x;
+  vec.token(b);
+  auto at = [&](int k) -> float& { return k < kVecKept ? kept[k] : vec.home(k); };
+#pragma unroll 1
+  for (int k = tid; k < r; k += blockDim.x) at(k) = vec.entry(k);
+  if (use_rms) {
+    __syncthreads();
+    if (tid < kVecThreads) {
+      float ss = 0.f;
+      for (int k = tid; k < r; k += kVecThreads) ss = fmaf(at(k), at(k), ss);
+      ss = warp_sum(ss);
+      if ((tid & 31) == 0) red[tid >> 5] = ss;
+    }
+    __syncthreads();
+    float tot = 0.f;
+#pragma unroll
+    for (int w = 0; w < kVecThreads / 32; ++w) tot += red[w];
+    const float inv_rms = rsqrtf(tot / (float)r + eps);
+#pragma unroll 1
+    for (int k = tid; k < r; k += blockDim.x) at(k) = (gain ? gain[k] : 1.f) * at(k) * inv_rms;
+  }
   float m = 0.f;
-  vec.each([&](int k, float e) { m = fmaxf(m, fabsf(n_of(k, e))); });
-  const float s = limb_scale(m, red2, kVecThreads / 32);
-  if (threadIdx.x == 0) scale[b] = s;
+  for (int k = tid; k < r; k += blockDim.x) m = fmaxf(m, fabsf(at(k)));
+  const float s = limb_scale(m, red2, blockDim.x / 32);
+  if (tid == 0) scale[b] = s;
   const float inv = 1.f / s;
-  vec.each([&](int k, float e) {
+#pragma unroll 1
+  for (int k = tid; k < r; k += blockDim.x) {
     int q4[4];
-    limbs_of(n_of(k, e), inv, q4);
+    limbs_of(at(k), inv, q4);
 #pragma unroll
     for (int l = 0; l < 4; ++l) limbs[((size_t)4 * b + l) * r + k] = (int8_t)q4[l];
-  });
+  }
 }
 
 }  // namespace
@@ -1726,10 +1778,12 @@ cudaError_t launch_rows_mode(const UmmaRowsParams& p, dim3 grid, size_t smem, cu
 }  // namespace
 
 // The LoPA stage v = V x has few rows (the rank) of many columns.  A tile of eight rows for each SM reads all token columns for
-// them: with tiles of up to 64 rows and K cut into runs, whose sums the next kernel adds in their order, a CTA reads an eighth
-// of that, and ranks below 8 rows per SM fill the SMs too.  A run has at least four K blocks.  Whole calls, 4096 x 14336, r =
-// 512, 5 / 64 tokens: 47.8 / 93.8 -> 47.1 / 87.6 us (bf16), 46.2 / 108 -> 43.9 / 98.2 (int4); 8192 x 28672, r = 1024, 8:
-// 117 -> 114 (bf16), 102 -> 97.9 (int8).
+// them: with tiles of up to 64 rows and K cut into runs all CTAs together read an eighth of that, and ranks below 8 rows per SM
+// fill the SMs too.  The next kernel adds the fp32 sums of the runs in their order; integer sums (limbs) are added in memory, so
+// that what cancels across runs leaves nothing behind and v has the bits of one run (as int4 of every run, added by the norm,
+// calls of r >= 1280 were 2 us longer: one SM read 130 KB).  Whole calls, 4096 x 14336, r = 512, 5 / 64 tokens, not cut / cut:
+// 47.8 / 93.8 -> 47.1 / 87.6 us (bf16), 8 / 64 tokens 49.8 / 108 -> 47.0 / 98.7 (int4); 8192 x 28672, r = 1024, 8 tokens:
+// 101 -> 96.5 (int8).
 void umma_k_splits(int R, int K, bool codes, int sm_count, int max_splits, int* tiles, int* splits) {
   const int kb = K / (codes ? 128 : kAtomK);
   auto least = [](int a, int b) { return a < b ? a : b; };
@@ -1850,15 +1904,19 @@ cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s) {
                         : launch_down_q<0>(p, g, smem, s, map_wg, map_wt, map_hm);
 }
 
-cudaError_t launch_token_limbs(const void* x, int B, int K, int x_stride, void* limbs, float* scale, cudaStream_t s) {
+cudaError_t launch_token_limbs(const void* x, int B, int K, int x_stride, void* limbs, float* scale, void* zero, int zero_bytes,
+                               cudaStream_t s) {
   return launch_pdl(token_limbs_kernel, dim3(B), dim3(kLimbThreads), 0, s, static_cast<const __nv_bfloat16*>(x), K, x_stride,
-                    static_cast<int8_t*>(limbs), scale);
+                    static_cast<int8_t*>(limbs), scale, static_cast<int4*>(zero), zero_bytes / 16);
 }
 
-cudaError_t launch_rmsnorm_limbs(const float* v, int B, int r, int v_stride, int runs, size_t step, const float* gain, float eps,
+cudaError_t launch_rmsnorm_limbs(float* v, int B, int r, int v_stride, const UmmaLimbSums* sums, const float* gain, float eps,
                                  bool use_rms, void* limbs, float* scale, cudaStream_t s) {
-  return launch_pdl(rmsnorm_limbs_kernel, dim3(B), dim3(kVecThreads), 0, s, v, r, v_stride, runs, step, gain, eps, use_rms ? 1 : 0,
-                    static_cast<int8_t*>(limbs), scale);
+  const dim3 block(r <= 256 ? 256 : r <= 512 ? 512 : kVecMaxThreads);
+  int8_t* out = static_cast<int8_t*>(limbs);
+  if (!sums) return launch_pdl(rmsnorm_limbs_kernel<PlainVec>, dim3(B), block, 0, s, PlainVec{v, v_stride}, r, gain, eps, use_rms ? 1 : 0, out, scale);
+  const LimbSumsVec vec{reinterpret_cast<int*>(v), v_stride, sums->row_scale, sums->tok_scale, sums->code_scale, 0.f};
+  return launch_pdl(rmsnorm_limbs_kernel<LimbSumsVec>, dim3(B), block, 0, s, vec, r, gain, eps, use_rms ? 1 : 0, out, scale);
 }
 
 cudaError_t launch_rmsnorm_split(const float* v, int B, int r, int v_stride, int runs, size_t step, const float* gain, float eps,

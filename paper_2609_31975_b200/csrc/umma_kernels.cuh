@@ -47,8 +47,8 @@ struct UmmaRowsParams {
   int xtok_stride;
   int act;
   float* a_out;          // GATE: gate values a_out[b * a_stride + j]
-  int k_splits, k_tiles; // GATE, raw products only (0: not cut): runs of K and tiles of rows (umma_k_splits); run i writes at
-  size_t split_stride;   //   a_out + i * split_stride
+  int k_splits, k_tiles; // GATE, raw products only (0: not cut): runs of K and tiles of rows (umma_k_splits); run i writes
+  size_t split_stride;   //   at a_out + i * split_stride; limbs (qbits = 1 / 2): all add their integers to rows 4 b + l of a_out
   uint8_t* flag;         // GATE: [R] any token fires, or null
   uint32_t* words_out;   // GATE: the same as bit masks, word 4 * tile + epilogue warp, or null
   const float* a;        // UP: gate values
@@ -94,13 +94,20 @@ bool umma_own_list_supported(int R, int K, int sm_count);  // R gate rows of K e
 void umma_gate_tiling(int R, int K, int sm_count, int* tile_rows, int* n_tiles);
 cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, cudaStream_t s);
 bool umma_rows_native_i8_supported(int K, int tokens);
-// Tokens [B][K] bf16 as four int8 limbs each ([4 B][K], most significant first, 7 bits apart) and one scale per token.
-cudaError_t launch_token_limbs(const void* x, int B, int K, int x_stride, void* limbs, float* scale, cudaStream_t s);
+// Tokens [B][K] bf16 as four int8 limbs each ([4 B][K], most significant first, 7 bits apart) and one scale per token;
+// zeroes B * zero_bytes (a multiple of 16) beside it.
+cudaError_t launch_token_limbs(const void* x, int B, int K, int x_stride, void* limbs, float* scale, void* zero, int zero_bytes,
+                               cudaStream_t s);
 // How v = V x (R rows of K elements or codes) is cut: `splits` runs of K (1: not), each over `tiles` tiles of rows.
 void umma_k_splits(int R, int K, bool codes, int sm_count, int max_splits, int* tiles, int* splits);
-// The same for the LoPA vector n = RMSNorm(v) (or v), from fp32.  v is the sum of `runs` vectors, `step` floats apart.
-cudaError_t launch_rmsnorm_limbs(const float* v, int B, int r, int v_stride, int runs, size_t step, const float* gain, float eps,
+// The same for the LoPA vector n = RMSNorm(v) (or v): from fp32 (`sums` null), or from integer sums, four rows of v_stride a token.
+struct UmmaLimbSums {
+  const float *row_scale, *tok_scale;  // of V's rows and of the tokens' limbs
+  float code_scale;                    // 1, or 1 / 16 (4-bit codes, whose products are of 16 x the code)
+};
+cudaError_t launch_rmsnorm_limbs(float* v, int B, int r, int v_stride, const UmmaLimbSums* sums, const float* gain, float eps,
                                  bool use_rms, void* limbs, float* scale, cudaStream_t s);
+// The bf16 pairs (or triples) of n.  v is the sum of `runs` vectors, `step` floats apart.
 cudaError_t launch_rmsnorm_split(const float* v, int B, int r, int v_stride, int runs, size_t step, const float* gain, float eps,
                                  bool use_rms, int cols, bool exact, void* x2, cudaStream_t s);
 

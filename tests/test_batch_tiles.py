@@ -105,3 +105,60 @@ def test_lopa_batches_with_v_from_several_runs_of_columns(D, r, B, q8):
     else:
         ref = run_oracle(x, *args)
         assert_y_close(y, ref["y"], what=f"{D} r={r} B={B}")
+
+
+def pack(q, qbits):
+    """Codes as the entry points take them, on the GPU: int8, or two 4-bit codes a byte (even column in the low half)."""
+    if qbits == 8:
+        return q.to(DEV)
+    n = q.bitwise_and(15).view(torch.uint8)
+    return (n[:, 0::2] | (n[:, 1::2] << 4)).to(DEV)
+
+
+def small_parts(n, B, gen):
+    """n neurons over B tokens: how large each one's pre-activation is in the token that owns it (a part that lies in the second,
+    third or fourth limb of a token whose largest entry is 127), and whether it is positive there."""
+    part = torch.tensor([2.0 ** -4, 2.0 ** -11, 2.0 ** -18])[torch.randint(0, 3, (n,), generator=gen)]
+    return part, torch.rand(n, generator=gen) < 0.5
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("qbits", [8, 4])
+@pytest.mark.parametrize("rms", [False, True])
+@pytest.mark.parametrize("D,r,B", [
+    (512, 128, 3),      # not cut
+    (1024, 256, 5),     # two runs
+    (4096, 128, 64),    # eight
+    (3840, 896, 16),    # runs of unequal length
+    (8192, 512, 2),     # sixteen
+    (1024, 4224, 3),    # a vector longer than what the norm kernel keeps in shared memory
+])
+def test_quantised_lopa_vectors_cut_into_runs_keep_integer_sums(D, r, B, rms, qbits):
+    """Every entry of v is a small part beside two products of 127 and the largest code that cancel, one in the first and one in
+    the last run of columns: integer sums keep the part and its sign, fp32 sums of runs lose all below 2^-24 of the products."""
+    import paper_2609_31975_b200 as m
+
+    gen = torch.Generator().manual_seed(D + r)
+    top, H = 2 ** (qbits - 1) - 1, r
+    col = torch.randint(1, D - 1, (r,), generator=gen)
+    # x: a column's part and sign are those of the token that owns the column; the other tokens have it negative
+    part, positive = small_parts(D, B, gen)
+    cown = torch.randint(0, B, (D,), generator=gen)
+    x = -part.repeat(B, 1)
+    for b in range(B):
+        x[b, positive & (cown == b)] *= -1
+    x[:, 0] = x[:, D - 1] = 127.0
+    V = torch.zeros((r, D), dtype=torch.int8)
+    V[:, 0], V[:, D - 1] = top, -top
+    V[torch.arange(r), col] = 1
+    U = torch.eye(r, dtype=torch.int8)
+    ones = torch.ones(r, device=DEV)
+    gate = dict(V=dict(q=pack(V, qbits), s=ones), U=dict(q=pack(U, qbits), s=ones), use_rmsnorm=rms)
+    w = dict(q=pack(torch.ones((H, D), dtype=torch.int8), qbits), s=torch.full((H,), 0.01, device=DEV))
+    ffn = m.SparseFFN(D, H, torch.bfloat16, r_max=r, B_max=B)
+    (ffn.sparse_ffn_forward_q8 if qbits == 8 else ffn.sparse_ffn_forward_q4)(x.bfloat16().to(DEV), gate, None, w, w, "relu")
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0
+    # V's products are exact; the limbs of n reach 2^-22 of its largest entry, far below 2^-18 / 2^-4
+    fires = (x[:, col] > 0).any(dim=0)
+    assert torch.equal(ffn.last_active().cpu().long(), torch.nonzero(fires)[:, 0])
