@@ -351,15 +351,15 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
   // v = V x can be cut into runs of K, whose sums lie where the down projection's go later (at least kMaxUpDownGrid * kMaxChunk
   // * D floats): fp32 sums of each run, which the norm adds in their order, or (limbs) one integer sum of all, the same
   // bits as without runs.  (The room bounds the fp32 runs of wide vectors of many tokens, so that their number, and with it the
-  // order of the sums, can depend on the size of the batch, as the number of accumulators does.)
+  // order of the sums, can depend on the size of the batch, as the number of accumulators does; not on the handle's r_max.)
   float* v = vbuf;
   int v_tiles = 1, v_runs = 1, vs = rs;
   if (lopa && umma && !exact) {
-    const long long room = (long long)kMaxUpDownGrid * kMaxChunk * D / B;
-    umma_k_splits(g->r, D, native, h->sm_count, !native ? (int)(room / rs) : room / g->r >= 4 ? 16 : 1, &v_tiles, &v_runs);
+    const long long room = (long long)kMaxUpDownGrid * kMaxChunk * D / ((long long)B * g->r);
+    umma_k_splits(g->r, D, native, h->sm_count, !native ? (int)room : room >= 4 ? 16 : 1, &v_tiles, &v_runs);
     if (v_runs > 1) {
       v = h->at<float>(h->L.partial);
-      if (native) vs = g->r;
+      vs = g->r;
     }
   }
   if (native) {
@@ -422,7 +422,7 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
     } else if (lopa) {
       // RMSNorm (or none) and the split into bf16 pairs (exact sums: triples) in one launch
       p.x_cols = round8(B);
-      SFFN_CUDA(launch_rmsnorm_split(v, B, g->r, rs, v_runs, (size_t)B * rs, g->rms_gain, g->rms_eps, g->use_rmsnorm != 0, p.x_cols, exact, x2, s));
+      SFFN_CUDA(launch_rmsnorm_split(v, B, g->r, vs, v_runs, (size_t)B * vs, g->rms_gain, g->rms_eps, g->use_rmsnorm != 0, p.x_cols, exact, x2, s));
       ++h->launches;
       p.W = g->U; p.K = g->r; p.X = x2; p.x_stride = g->r;
       p.g_idx = g->g_idx; p.g_sign = g->g_sign;

@@ -162,3 +162,23 @@ def test_quantised_lopa_vectors_cut_into_runs_keep_integer_sums(D, r, B, rms, qb
     # V's products are exact; the limbs of n reach 2^-22 of its largest entry, far below 2^-18 / 2^-4
     fires = (x[:, col] > 0).any(dim=0)
     assert torch.equal(ffn.last_active().cpu().long(), torch.nonzero(fires)[:, 0])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("q8", [False, True])
+def test_lopa_batches_are_the_same_bits_whatever_rank_the_handle_allows(q8):
+    """128 tokens of rank 256: V is cut into four runs of columns, whose sums are laid out by the rank in use."""
+    import paper_2609_31975_b200 as m
+
+    D, H, r, B = 1024, 600, 256, 128
+    w = syn.lopa_ffn_q8(D, H, r, 74, DEV, sparsity=0.7) if q8 else syn.lopa_ffn(D, H, r, torch.bfloat16, 74, DEV, sparsity=0.7)
+    gate = {"V": w["V"], "U": w["U"], "g_idx": m.g_diagonal(H, D, DEV)}
+    x = syn.tokens(B, D, torch.bfloat16, 74, DEV)
+    ys = []
+    for r_max in (r, 4096):
+        ffn = m.SparseFFN(D, H, torch.bfloat16, r_max=r_max, B_max=B)
+        call = ffn.sparse_ffn_forward_q8 if q8 else ffn.sparse_ffn_forward
+        ys.append(call(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu"))
+        torch.cuda.synchronize()
+        assert ffn.device_status() == 0
+    assert torch.equal(ys[0], ys[1])
