@@ -317,7 +317,8 @@ const char* sffn_status_string(int status);
  * sffn_test_fused_plan: geometry of the single-token CUDA-core kernel for a shape, as nine integers: ok, rows per
  *   gate slot, gate slot bytes, gate slots, gate warps, act slot bytes, act slots, chunks per act thread, shared
  *   memory bytes (wkind: 0 fp32, 1 bf16, 2 int8 rows).  sffn_test_umma_tiling: tiling of the batched gate GEMM over short
- *   rows; sffn_test_umma_row_tiling: over rows of K elements.
+ *   rows; sffn_test_umma_row_tiling: over rows of K elements; sffn_test_umma_pass_tiling: over rows of K elements (qbits 0:
+ *   bf16) or codes (8 / 4; 1 / 2: against limbs) in a pass of B tokens.
  * sffn_test_set_knob(knob, value):
  *   PDL                 programmatic dependent launch between calls (default 1)
  *   TENSOR_GATE         1 / 0: single-token calls take the tensor-core gate kernel wherever it applies / nowhere,
@@ -347,6 +348,7 @@ typedef enum {
 void sffn_test_fused_plan(int wkind, int D, int H, int K, int lopa, int sm_count, int* out9);
 void sffn_test_umma_tiling(int R, int sm_count, int* tile_rows, int* n_tiles, int* own_list);
 void sffn_test_umma_row_tiling(int R, int K, int sm_count, int* tile_rows, int* n_tiles, int* own_list);
+void sffn_test_umma_pass_tiling(int R, int K, int qbits, int B, int sm_count, int* tile_rows, int* n_tiles, int* own_list);
 int sffn_test_set_knob(int knob, long long value);
 
 #ifdef __cplusplus

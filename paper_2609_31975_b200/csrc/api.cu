@@ -204,8 +204,11 @@ void sffn_test_umma_tiling(int R, int sm_count, int* tile_rows, int* n_tiles, in
   sffn_test_umma_row_tiling(R, 0, sm_count, tile_rows, n_tiles, own_list);
 }
 void sffn_test_umma_row_tiling(int R, int K, int sm_count, int* tile_rows, int* n_tiles, int* own_list) {
-  sffn::umma_gate_tiling(R, K, sm_count, tile_rows, n_tiles);
-  *own_list = sffn::umma_own_list_supported(R, K, sm_count) ? 1 : 0;
+  sffn_test_umma_pass_tiling(R, K, 0, 2, sm_count, tile_rows, n_tiles, own_list);
+}
+void sffn_test_umma_pass_tiling(int R, int K, int qbits, int B, int sm_count, int* tile_rows, int* n_tiles, int* own_list) {
+  sffn::umma_gate_tiling(R, K, qbits, B, sm_count, tile_rows, n_tiles);
+  *own_list = sffn::umma_own_list_supported(R, K, qbits, B, sm_count) ? 1 : 0;
 }
 int sffn_test_set_knob(int knob, long long value) {
   sffn::FusedTestKnobs& k = sffn::fused_test_knobs();
@@ -396,10 +399,10 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
   }
   // The tcgen05 gate kernel can leave its "fired" flags as bit masks, which the up kernel compacts itself
   // (and publishes list and length): no byte flags, no compaction launch.
-  const bool own_list = umma && !dense && umma_own_list_supported(H, lopa ? g->r : D, h->sm_count);
+  const bool own_list = umma && !dense && umma_own_list_supported(H, lopa ? g->r : D, wq_rows, B, h->sm_count);
   uint32_t* words = reinterpret_cast<uint32_t*>(flag);  // the flag buffer holds either form
   int gate_tile_rows = 0, gate_tiles = 0;
-  umma_gate_tiling(H, lopa ? g->r : D, h->sm_count, &gate_tile_rows, &gate_tiles);
+  umma_gate_tiling(H, lopa ? g->r : D, wq_rows, B, h->sm_count, &gate_tile_rows, &gate_tiles);
   void* x2 = h->ws + h->L.x2;
   if (umma) {
     UmmaRowsParams p{};

@@ -332,13 +332,21 @@ __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.
 // multiple of 8, the swizzle period), so that every SM streams a share.  Two tiles of equal height, not tiles of 128 rows
 // whose second wave leaves most SMs idle: 24000 rows are 273 tiles of 88 rows, where 188 of 128 kept 40 of 148 SMs busy in the
 // second half (bf16, 5120 x 20000, 2 / 32 tokens: 80.7 / 155 -> 70.5 / 127 us; int4, 8192 x 24000, 64: 484 -> 339).  128
-// where a CTA owns more than two, and for short rows (the LoPA gate), whose tiles are gone before the imbalance shows (r =
-// 512 / 1024: 0 to 1 % faster; r = 1536: equal tiles 1 to 3 % faster).
+// where a CTA owns more than two, for short rows (the LoPA gate), whose tiles are gone before the imbalance shows (r = 512 /
+// 1024: 0 to 1 % faster; r = 1536: equal tiles 1 to 3 % faster), and for most wide passes: bf16 rows against more than 128 tokens
+// are bound by the token rows that every tile reads through L2, and tiles of 128 are fewer.  There equal tiles pay only where
+// their stages are enough smaller for more of them in the ring (tiles of 128 / equal ones: 7168 x 20000, 200 tokens, 4 / 6 slots
+// 353 / 329 us, 160 tokens, 6 / 6 slots 270 / 287; 8192 x 20000, 256, 4 / 4: 414 / 474; 6144 x 24576, 200, 4 / 4: 324 / 345).
 constexpr int kShortRow = 1024;
-__host__ __device__ inline int tile_rows_for(int n_rows, int grid, int K) {
+constexpr int kRowsSmem = 226 * 1024, kRingBytes = kRowsSmem - 1024 - kHeaderBytes;
+// token columns of a wide pass, else 0
+__host__ __device__ inline int wide_cols(int qbits, int B) { return qbits == 0 && B > 128 ? (B + 15) / 16 * 16 : 0; }
+__host__ __device__ inline int wide_slots(int tile_rows, int cols) { return kRingBytes / ((tile_rows + cols) * 128) & ~1; }
+__host__ __device__ inline int tile_rows_for(int n_rows, int grid, int K, int wide) {
   const int per_cta = n_rows > kTileRows * grid ? 2 : 1;
   if (n_rows > 2 * kTileRows * grid || (per_cta == 2 && K <= kShortRow)) return kTileRows;
   int t = ((n_rows + per_cta * grid - 1) / (per_cta * grid) + 7) & ~7;
+  if (per_cta == 2 && wide && wide_slots(t, wide) <= wide_slots(kTileRows, wide)) return kTileRows;
   return t < 8 ? 8 : t > kTileRows ? kTileRows : t;
 }
 
@@ -573,7 +581,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
   const bool walk_all = MODE == kUpMayWalk && own_list && p.walk_all &&
                         (long long)n_listed * 100 >= (long long)p.R * kWalkAllPercent;
   if (walk_all) n_rows = p.R;
-  const int tile_rows = tile_rows_for(n_rows, gridDim.x, p.K);
+  const int tile_rows = tile_rows_for(n_rows, gridDim.x, p.K, wide_cols(QB, p.B));
   const int n_tiles = (n_rows + tile_rows - 1) / tile_rows;
   if (own_list && walk_all) {
     // publish the list only: word w is written out by CTA w mod grid
@@ -1651,15 +1659,15 @@ __global__ void __launch_bounds__(kVecMaxThreads) rmsnorm_limbs_kernel(Vec vec, 
 
 
 // Tiling of the gate GEMM over R rows (the up kernel needs it to read the gate's bit masks).
-void umma_gate_tiling(int R, int K, int sm_count, int* tile_rows, int* n_tiles) {
+void umma_gate_tiling(int R, int K, int qbits, int B, int sm_count, int* tile_rows, int* n_tiles) {
   const int grid = R < 8 * sm_count ? (R + 7) / 8 : sm_count;
-  *tile_rows = tile_rows_for(R, grid, K);
+  *tile_rows = tile_rows_for(R, grid, K, wide_cols(qbits, B));
   *n_tiles = (R + *tile_rows - 1) / *tile_rows;
 }
 
-bool umma_own_list_supported(int R, int K, int sm_count) {
+bool umma_own_list_supported(int R, int K, int qbits, int B, int sm_count) {
   int tr, nt;
-  umma_gate_tiling(R, K, sm_count, &tr, &nt);
+  umma_gate_tiling(R, K, qbits, B, sm_count, &tr, &nt);
   return 4 * nt <= kScanChunks * kThreadsRows && R <= (long long)kMaxOwnTiles * kTileRows * sm_count;
 }
 
@@ -1807,15 +1815,15 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
   if (splits > 1 && (up || p.exact || p.b_g || p.g_idx || p.flag || p.words_out || p.act != kUmmaActIdentity)) return cudaErrorInvalidValue;
   const int grid = splits > 1 ? p.k_tiles : p.R < 8 * sm_count ? (p.R + 7) / 8 : sm_count;
   // all the dynamic shared memory a CTA can have; the kernel cuts its ring out of it once it knows its tiles
-  const size_t smem = 226 * 1024;
-  p.ring_bytes = (int)smem - 1024 - kHeaderBytes;
+  const size_t smem = kRowsSmem;
+  p.ring_bytes = kRingBytes;
   alignas(64) CUtensorMap map_w, map_x;
   if (p.qbits != 0 && p.qbits != 8 && p.qbits != 4 && p.qbits != 1 && p.qbits != 2) return cudaErrorInvalidValue;
   const bool i8 = p.qbits == 1 || p.qbits == 2;  // kind::i8 MMAs: X holds the tokens' int8 limbs
   if (p.npad > kUmmaMaxCols) return cudaErrorInvalidValue;
   if (i8 && (p.K % 128 || !p.tok_scale)) return cudaErrorInvalidValue;
   // weights: all R rows; boxes of one tile's rows for the gate, single-row boxes for the gather
-  if (!make_weight_map(&map_w, p.W, p.K, p.R, up ? 1 : tile_rows_for(p.R, grid, p.K), p.qbits)) return cudaErrorNotSupported;
+  if (!make_weight_map(&map_w, p.W, p.K, p.R, up ? 1 : tile_rows_for(p.R, grid, p.K, wide_cols(p.qbits, p.B)), p.qbits)) return cudaErrorNotSupported;
   // tokens: only the rows that exist; the box covers npad rows and the rest reads as zero
   if (i8 ? !make_map_i8(&map_x, p.X, p.K, p.ncols_valid, (size_t)p.x_stride, p.npad)
                    : !make_map(&map_x, p.X, p.K, p.ncols_valid, (size_t)p.x_stride, p.npad))
@@ -1825,7 +1833,7 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
     // wide batches: the union may cover most rows; the kernel then walks every row with tiled boxes of the tile
     // height of R rows (decided on the device from the union's size, so it depends on this call's inputs only)
     WalkMap<true> map_t;
-    if (!make_weight_map(&map_t.m, p.W, p.K, p.R, tile_rows_for(p.R, grid, p.K), p.qbits)) return cudaErrorNotSupported;
+    if (!make_weight_map(&map_t.m, p.W, p.K, p.R, tile_rows_for(p.R, grid, p.K, wide_cols(p.qbits, p.B)), p.qbits)) return cudaErrorNotSupported;
     return launch_rows_mode<kUpMayWalk>(p, dim3(grid), smem, s, map_w, map_x, map_t);
   }
   return launch_rows_mode<kUp>(p, dim3(grid), smem, s, map_w, map_x, WalkMap<false>{});

@@ -90,8 +90,9 @@ cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s);
 bool umma_rows_supported(int K, int cols);
 // Batches wide enough for the up kernel to consider walking every row instead of the union list.
 bool umma_may_walk(int B);
-bool umma_own_list_supported(int R, int K, int sm_count);  // R gate rows of K elements
-void umma_gate_tiling(int R, int K, int sm_count, int* tile_rows, int* n_tiles);
+// R gate rows of K elements or codes (qbits as in UmmaRowsParams) against B tokens
+bool umma_own_list_supported(int R, int K, int qbits, int B, int sm_count);
+void umma_gate_tiling(int R, int K, int qbits, int B, int sm_count, int* tile_rows, int* n_tiles);
 cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, cudaStream_t s);
 bool umma_rows_native_i8_supported(int K, int tokens);
 // Tokens [B][K] bf16 as four int8 limbs each ([4 B][K], most significant first, 7 bits apart) and one scale per token;

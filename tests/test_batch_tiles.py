@@ -35,8 +35,31 @@ def test_two_equal_tiles_for_each_cta(sms):
     assert tiling(lib, 24000, 8192) == (88, 273, 1)
 
 
+@pytest.mark.parametrize("sms", [132, 148])
+def test_wide_passes_of_bf16_rows_take_equal_tiles_only_for_a_deeper_ring(sms):
+    import paper_2609_31975_b200 as m
+
+    lib = m.load_library()
+    tr, nt, own = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
+    slots = lambda rows, B: 225280 // ((rows + -(-B // 16) * 16) * 128) // 2  # noqa: E731  (pairs of ring slots)
+    kept = 0
+    for R in (600, 14336, 128 * sms, 128 * sms + 1, 20000, 24576, 256 * sms, 60000):
+        equal = tiling(lib, R, 4096, sms)
+        for qbits in (0, 8, 4, 1, 2):
+            for B in (2, 64, 128, 129, 136, 160, 200, 256):
+                lib.sffn_test_umma_pass_tiling(R, 4096, qbits, B, sms, ctypes.byref(tr), ctypes.byref(nt), ctypes.byref(own))
+                if qbits == 0 and B > 128 and R > 128 * sms and slots(equal[0], B) <= slots(128, B):
+                    assert (tr.value, nt.value) == (128, -(-R // 128))
+                    kept += 1
+                else:
+                    assert (tr.value, nt.value, own.value) == equal
+    assert kept >= 10
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("D,H,B,s", [
+    (1280, 24001, 160, 0.9),  # a pass of more than 128 tokens: tiles of 128, a ragged second wave
+    (1280, 19001, 200, 0.9),  # and one in equal tiles
     (1280, 18945, 3, 0.9),    # one row more than one tile per CTA holds; the union is one tile per CTA
     (1280, 24001, 40, 0.5),   # a ragged last tile; the union is (nearly) every row, walked in the same tiles
     (1280, 20000, 20, 0.3),   # the union is most rows, listed: two tiles per CTA
