@@ -1439,163 +1439,19 @@ __global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarp
   }
 }
 
-// The vector of a token for the small kernels below: entry k = threadIdx.x + i * blockDim.x of a row of up to kKept *
-// blockDim.x entries stays in register i from the first look at it; the rest of a longer row is read again.
-constexpr int kVecThreads = 256, kKept = 8;
-// An entry is the sum of `runs` values, `step` apart (see umma_k_splits).
-struct KeptVec {
-  const float* v;
-  int r, runs;
+// The entries of v for the norm kernels below: the sum of `runs` fp32 values, `step` apart, or the four limbs' integer sums over
+// all runs of K (see umma_k_splits), from which v gets the bits that it has without runs.
+struct SumVec {
+  float* v;
+  int stride, runs;
   size_t step;
-  float kept[kKept];
-  __device__ __forceinline__ float at(int k) const {
+  __device__ __forceinline__ void token(int b) { v += (size_t)b * stride; }
+  __device__ __forceinline__ float entry(int k) const {
     float e = v[k];
-#pragma unroll 4
+#pragma unroll 8
     for (int i = 1; i < runs; ++i) e += v[i * step + k];
     return e;
   }
-  __device__ __forceinline__ KeptVec(const float* v_, int r_, int runs_, size_t step_) : v(v_), r(r_), runs(runs_), step(step_) {
-#pragma unroll
-    for (int i = 0; i < kKept; ++i) kept[i] = 0.f;
-    // four runs of all entries in flight, each entry added up in the order of the runs
-#pragma unroll 4
-    for (int run = 0; run < runs; ++run)
-#pragma unroll
-      for (int i = 0; i < kKept; ++i) {
-        const int k = threadIdx.x + i * kVecThreads;
-        if (k < r) kept[i] += v[run * step + k];
-      }
-  }
-  template <typename F>
-  __device__ __forceinline__ void each(F f) const {  // f(k, entry) in ascending order of k
-#pragma unroll
-    for (int i = 0; i < kKept; ++i) {
-      const int k = threadIdx.x + i * kVecThreads;
-      if (k < r) f(k, kept[i]);
-    }
-    for (int k = threadIdx.x + kKept * kVecThreads; k < r; k += kVecThreads) f(k, at(k));
-  }
-};
-// 1 / rms of the vector.
-__device__ __forceinline__ float inverse_rms(const KeptVec& vec, float eps, float* red) {
-  float ss = 0.f;
-  vec.each([&](int, float e) { ss = fmaf(e, e, ss); });
-  ss = warp_sum(ss);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-  __syncthreads();
-  float tot = 0.f;
-#pragma unroll
-  for (int w = 0; w < kVecThreads / 32; ++w) tot += red[w];
-  return rsqrtf(tot / (float)vec.r + eps);
-}
-
-// LoPA gate, batched: n = RMSNorm(v) (or v itself) as a sum of two bf16 vectors for the tensor cores: row b of
-// x2 holds the high part of token b's vector, row cols + b the low part (v - bf16(v)), so that the gate's U n keeps
-// close to fp32 accuracy.  `exact`: row 2 cols + b holds what those two leave (24 bits in all).  One CTA per token.
-__global__ void __launch_bounds__(kVecThreads) rmsnorm_split_kernel(const float* v, int r, int v_stride, int runs, size_t step, const float* gain,
-                                                                    float eps, int use_rms, int cols, int exact,
-                                                                    __nv_bfloat16* x2) {
-  __shared__ float red[kVecThreads / 32];
-  pdl_launch_dependents();
-  pdl_wait();
-  const int b = blockIdx.x;
-  const KeptVec vec(v + (size_t)b * v_stride, r, runs, step);
-  const float inv = use_rms ? inverse_rms(vec, eps, red) : 1.f;
-  vec.each([&](int k, float e) {
-    float n = use_rms ? (gain ? gain[k] : 1.f) * e * inv : e;
-    x2[(size_t)b * r + k] = take_bf16(n);
-    x2[(size_t)(cols + b) * r + k] = take_bf16(n);
-    if (exact) x2[(size_t)(2 * cols + b) * r + k] = __float2bfloat16(n);
-  });
-}
-
-// Tokens as int8 limbs for the kind::i8 MMAs: t[k] = scale * (q0 + q1 / 128 + q2 / 128^2 + q3 / 128^3) up to
-// scale * 2^-22, with scale = max |t| / 127, |q0| <= 127 and the other limbs <= 64 in magnitude.  Row 4 b + l of
-// `limbs` holds limb l of token b.  One CTA per token.
-// scale of a token whose threads have seen entries of at most m
-__device__ __forceinline__ float limb_scale(float m, float* red, int warps) {
-#pragma unroll
-  for (int d = 16; d >= 1; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
-  float mx = 0.f;
-  for (int w = 0; w < warps; ++w) mx = fmaxf(mx, red[w]);
-  return mx > 0.f ? mx / 127.f : 1.f;
-}
-// the limbs of one entry
-__device__ __forceinline__ void limbs_of(float e, float inv, int* q4) {
-  float t = fminf(fmaxf(e * inv, -127.f), 127.f);
-#pragma unroll
-  for (int l = 0; l < 4; ++l) {
-    const float q = rintf(t);
-    q4[l] = (int)q;
-    t = (t - q) * 128.f;
-  }
-}
-
-// A thread takes eight consecutive entries (16 bytes) at a time and keeps those of its first two rounds; it stores eight
-// limbs at a time.  Bound by its own latency, which stands between the predecessor and the first gate MMA: one round trip to
-// the token instead of two dozen (4096 entries by 256 threads, an entry at a time, twice: calls of
-// 4096 x 14336 with 2 to 64 tokens 8 to 9 us longer, of 8192 x 24000 20 us).
-constexpr int kLimbThreads = 512, kLimbRounds = 2;
-__global__ void __launch_bounds__(kLimbThreads) token_limbs_kernel(const __nv_bfloat16* x, int K, int x_stride, int8_t* limbs,
-                                                                   float* scale, int4* zero, int zero_n) {
-  __shared__ float red[kLimbThreads / 32];
-  pdl_launch_dependents();
-  pdl_wait();
-  const int b = blockIdx.x;
-  const uint4* xb = reinterpret_cast<const uint4*>(x + (size_t)b * x_stride);
-  const int n8 = K / 8;
-  uint4 kept[kLimbRounds];
-  float m = 0.f;
-  auto largest = [&](const uint4& w) {
-    float e[8];
-    Elem<__nv_bfloat16>::unpack(w, e);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) m = fmaxf(m, fabsf(e[q]));
-  };
-#pragma unroll
-  for (int i = 0; i < kLimbRounds; ++i) {
-    const int k = threadIdx.x + i * kLimbThreads;
-    kept[i] = k < n8 ? xb[k] : make_uint4(0, 0, 0, 0);
-  }
-  for (int k = threadIdx.x; k < zero_n; k += kLimbThreads) zero[(size_t)b * zero_n + k] = make_int4(0, 0, 0, 0);
-#pragma unroll
-  for (int i = 0; i < kLimbRounds; ++i) largest(kept[i]);
-  for (int k = threadIdx.x + kLimbRounds * kLimbThreads; k < n8; k += kLimbThreads) largest(xb[k]);
-  const float s = limb_scale(m, red, kLimbThreads / 32);
-  if (threadIdx.x == 0) scale[b] = s;
-  const float inv = 1.f / s;
-  int8_t* out = limbs + (size_t)4 * b * K;
-  auto put = [&](int k, const uint4& w) {
-    float e[8];
-    Elem<__nv_bfloat16>::unpack(w, e);
-    uint2 o[4] = {};
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      int l4[4];
-      limbs_of(e[q], inv, l4);
-#pragma unroll
-      for (int l = 0; l < 4; ++l) (q < 4 ? o[l].x : o[l].y) |= (uint32_t)(l4[l] & 0xff) << (8 * (q & 3));
-    }
-#pragma unroll
-    for (int l = 0; l < 4; ++l) *reinterpret_cast<uint2*>(out + (size_t)l * K + 8 * k) = o[l];
-  };
-#pragma unroll
-  for (int i = 0; i < kLimbRounds; ++i) {
-    const int k = threadIdx.x + i * kLimbThreads;
-    if (k < n8) put(k, kept[i]);
-  }
-  for (int k = threadIdx.x + kLimbRounds * kLimbThreads; k < n8; k += kLimbThreads) put(k, xb[k]);
-}
-
-// The entries of v for the kernel below: fp32 values, or the four limbs' integer sums over all runs of K (see umma_k_splits), from
-// which v gets the bits that it has without runs.
-struct PlainVec {
-  float* v;
-  int stride;
-  __device__ __forceinline__ void token(int b) { v += (size_t)b * stride; }
-  __device__ __forceinline__ float entry(int k) const { return v[k]; }
   __device__ __forceinline__ float& home(int k) const { return v[k]; }
 };
 struct LimbSumsVec {
@@ -1610,46 +1466,195 @@ struct LimbSumsVec {
   __device__ __forceinline__ float& home(int k) const { return *reinterpret_cast<float*>(v + k); }
 };
 
-// LoPA gate with int8 rows: n = RMSNorm(v) (or v itself) as limbs.  One CTA per token.  An entry is fetched once, by a thread
-// that keeps it in shared memory (past kVecKept entries: at its home); the squares are added by the first kVecThreads threads
-// whatever the block, which fixes the order of that sum.
-constexpr int kVecMaxThreads = 1024, kVecKept = 4096;
+// The norm kernels, one CTA per token.  An entry is fetched once, by a thread that keeps it in shared memory (past kVecKept
+// entries: at its home); the squares are added as kVecThreads threads take them whatever the block, which fixes the order of
+// that sum.  Bound by their own latency, a part of which is the fetch of their instructions: the loops are hardly unrolled.
+// (Split kernel alone, r = 64 / 896 / 1024 / 2048: 2.1 / 3.3 / 3.0 / 4.2 us, the last three from 10, 9 and 4 runs; with a thread's
+// entries in eight registers and every loop over them unrolled 2.4 / 5.4 / 4.8 / 3.6, with blocks of 256 2.1 / 5.8 / 4.4 / 9.4.)
+constexpr int kVecThreads = 256, kVecMaxThreads = 1024, kVecKept = 4096;
+inline int vec_threads(int r) { return r <= 256 ? 256 : r <= 512 ? 512 : kVecMaxThreads; }
 template <typename Vec>
-__global__ void __launch_bounds__(kVecMaxThreads) rmsnorm_limbs_kernel(Vec vec, int r, const float* gain, float eps, int use_rms,
-                                                                       int8_t* limbs, float* scale) {
-  __shared__ float kept[kVecKept], red[kVecMaxThreads / 32], red2[kVecMaxThreads / 32];
+struct Kept {
+  const Vec& vec;
+  float* sm;
+  __device__ __forceinline__ float get(int k) const { return k < kVecKept ? sm[k] : vec.home(k); }
+  __device__ __forceinline__ void put(int k, float e) const {
+    if (k < kVecKept) sm[k] = e;
+    else vec.home(k) = e;
+  }
+};
+// Fetches the entries (thread k mod blockDim.x's are there for itself) and returns 1 / rms, or 1.
+template <typename Vec>
+__device__ __forceinline__ float take_vec(const Kept<Vec>& v, int r, float eps, int use_rms, float* red) {
+  const int tid = threadIdx.x;
+  float ss = 0.f;
+#pragma unroll 2
+  for (int k = tid; k < r; k += blockDim.x) {
+    const float e = v.vec.entry(k);
+    ss = fmaf(e, e, ss);
+    v.put(k, e);
+  }
+  if (!use_rms) return 1.f;
+  if (blockDim.x != kVecThreads) {
+    __syncthreads();
+    ss = 0.f;
+    if (tid < kVecThreads)
+#pragma unroll 4
+      for (int k = tid; k < r; k += kVecThreads) ss = fmaf(v.get(k), v.get(k), ss);
+  }
+  if (tid < kVecThreads) {
+    ss = warp_sum(ss);
+    if ((tid & 31) == 0) red[tid >> 5] = ss;
+  }
+  __syncthreads();
+  float tot = 0.f;
+#pragma unroll
+  for (int w = 0; w < kVecThreads / 32; ++w) tot += red[w];
+  return rsqrtf(tot / (float)r + eps);
+}
+__device__ __forceinline__ float normed(float e, float inv, const float* gain, int use_rms, int k) {
+  return use_rms ? (gain ? gain[k] : 1.f) * e * inv : e;
+}
+
+// LoPA gate, batched: n = RMSNorm(v) (or v itself) as a sum of two bf16 vectors for the tensor cores: row b of
+// x2 holds the high part of token b's vector, row cols + b the low part (v - bf16(v)), so that the gate's U n keeps
+// close to fp32 accuracy.  `exact`: row 2 cols + b holds what those two leave (24 bits in all).
+__global__ void __launch_bounds__(kVecMaxThreads) rmsnorm_split_kernel(SumVec vec, int r, const float* gain, float eps, int use_rms,
+                                                                       int cols, int exact, __nv_bfloat16* x2) {
+  __shared__ float kept[kVecKept], red[kVecThreads / 32];
+  pdl_launch_dependents();
+  pdl_wait();
+  const int b = blockIdx.x;
+  vec.token(b);
+  const Kept<SumVec> v{vec, kept};
+  const float inv = take_vec(v, r, eps, use_rms, red);
+#pragma unroll 1
+  for (int k = threadIdx.x; k < r; k += blockDim.x) {
+    float n = normed(v.get(k), inv, gain, use_rms, k);
+    x2[(size_t)b * r + k] = take_bf16(n);
+    x2[(size_t)(cols + b) * r + k] = take_bf16(n);
+    if (exact) x2[(size_t)(2 * cols + b) * r + k] = __float2bfloat16(n);
+  }
+}
+
+// Tokens as int8 limbs for the kind::i8 MMAs: t[k] = scale * (q0 + q1 / 128 + q2 / 128^2 + q3 / 128^3) up to
+// scale * 2^-22, with scale = max |t| / 127, |q0| <= 127 and the other limbs <= 64 in magnitude.  Row 4 b + l of
+// `limbs` holds limb l of token b.  One CTA per token.
+// scale of a token whose threads have seen entries of at most m
+__device__ __forceinline__ float limb_scale(float m, float* red) {
+#pragma unroll
+  for (int d = 16; d >= 1; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  float mx = 0.f;
+  for (int w = 0; w < blockDim.x / 32; ++w) mx = fmaxf(mx, red[w]);
+  return mx > 0.f ? mx / 127.f : 1.f;
+}
+// the limbs of one entry
+__device__ __forceinline__ void limbs_of(float e, float inv, int* q4) {
+  float t = fminf(fmaxf(e * inv, -127.f), 127.f);
+#pragma unroll
+  for (int l = 0; l < 4; ++l) {
+    const float q = rintf(t);
+    q4[l] = (int)q;
+    t = (t - q) * 128.f;
+  }
+}
+
+// A thread takes N consecutive entries at a time, stores N limbs at a time and keeps its first entries, which are all there are up
+// to N * 1024 columns.  Bound by its own latency, which stands between the predecessor and the first gate MMA: one round trip to
+// the token instead of two dozen (4096 entries by 256 threads, an entry at a time, twice: calls of 4096 x 14336 with 2 to 64
+// tokens 8 to 9 us longer, of 8192 x 24000 20 us).
+constexpr int kLimbMaxThreads = 1024;
+template <int N>
+struct LimbGroup;
+template <>
+struct LimbGroup<8> {
+  using In = uint4;
+  using Out = uint2;
+};
+template <>
+struct LimbGroup<2> {
+  using In = uint32_t;
+  using Out = uint16_t;
+};
+template <int N>
+__global__ void __launch_bounds__(kLimbMaxThreads) token_limbs_kernel(const __nv_bfloat16* x, int K, int x_stride, int8_t* limbs,
+                                                                      float* scale, int4* zero, int zero_n) {
+  using In = typename LimbGroup<N>::In;
+  using Out = typename LimbGroup<N>::Out;
+  union Entries {
+    In in;
+    __nv_bfloat16 e[N];
+    __device__ Entries() : in() {}
+  };
+  union Limbs {
+    Out out;
+    int8_t q[N];
+    __device__ Limbs() : out() {}
+  };
+  __shared__ float red[kLimbMaxThreads / 32];
   pdl_launch_dependents();
   pdl_wait();
   const int b = blockIdx.x, tid = threadIdx.x;
-  vec.token(b);
-  auto at = [&](int k) -> float& { return k < kVecKept ? kept[k] : vec.home(k); };
-#pragma unroll 1
-  for (int k = tid; k < r; k += blockDim.x) at(k) = vec.entry(k);
-  if (use_rms) {
-    __syncthreads();
-    if (tid < kVecThreads) {
-      float ss = 0.f;
-      for (int k = tid; k < r; k += kVecThreads) ss = fmaf(at(k), at(k), ss);
-      ss = warp_sum(ss);
-      if ((tid & 31) == 0) red[tid >> 5] = ss;
-    }
-    __syncthreads();
-    float tot = 0.f;
-#pragma unroll
-    for (int w = 0; w < kVecThreads / 32; ++w) tot += red[w];
-    const float inv_rms = rsqrtf(tot / (float)r + eps);
-#pragma unroll 1
-    for (int k = tid; k < r; k += blockDim.x) at(k) = (gain ? gain[k] : 1.f) * at(k) * inv_rms;
-  }
+  const In* xb = reinterpret_cast<const In*>(x + (size_t)b * x_stride);
+  const int n = K / N;
+  Entries first;
+  if (tid < n) first.in = xb[tid];
+  for (int k = tid; k < zero_n; k += blockDim.x) zero[(size_t)b * zero_n + k] = make_int4(0, 0, 0, 0);
   float m = 0.f;
-  for (int k = tid; k < r; k += blockDim.x) m = fmaxf(m, fabsf(at(k)));
-  const float s = limb_scale(m, red2, blockDim.x / 32);
+  auto largest = [&](const Entries& w) {
+#pragma unroll
+    for (int q = 0; q < N; ++q) m = fmaxf(m, fabsf(__bfloat162float(w.e[q])));
+  };
+  Entries w = first;
+#pragma unroll 1
+  for (int k = tid; k < n; w.in = xb[k]) {
+    largest(w);
+    if ((k += blockDim.x) >= n) break;
+  }
+  const float s = limb_scale(m, red);
   if (tid == 0) scale[b] = s;
   const float inv = 1.f / s;
+  int8_t* out = limbs + (size_t)4 * b * K;
+  w = first;
 #pragma unroll 1
-  for (int k = tid; k < r; k += blockDim.x) {
+  for (int k = tid; k < n; w.in = xb[k]) {
+    Limbs o[4];
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      int l4[4];
+      limbs_of(__bfloat162float(w.e[q]), inv, l4);
+#pragma unroll
+      for (int l = 0; l < 4; ++l) o[l].q[q] = (int8_t)l4[l];
+    }
+#pragma unroll
+    for (int l = 0; l < 4; ++l) *reinterpret_cast<Out*>(out + (size_t)l * K + N * k) = o[l].out;
+    if ((k += blockDim.x) >= n) break;
+  }
+}
+
+// LoPA gate with rows of codes: n = RMSNorm(v) (or v itself) as limbs.
+template <typename Vec>
+__global__ void __launch_bounds__(kVecMaxThreads) rmsnorm_limbs_kernel(Vec vec, int r, const float* gain, float eps, int use_rms,
+                                                                       int8_t* limbs, float* scale) {
+  __shared__ float kept[kVecKept], red[kVecThreads / 32], red2[kVecMaxThreads / 32];
+  pdl_launch_dependents();
+  pdl_wait();
+  const int b = blockIdx.x;
+  vec.token(b);
+  const Kept<Vec> v{vec, kept};
+  const float inv_rms = take_vec(v, r, eps, use_rms, red);
+  float m = 0.f;
+#pragma unroll 1
+  for (int k = threadIdx.x; k < r; k += blockDim.x) m = fmaxf(m, fabsf(normed(v.get(k), inv_rms, gain, use_rms, k)));
+  const float s = limb_scale(m, red2);
+  if (threadIdx.x == 0) scale[b] = s;
+  const float inv = 1.f / s;
+#pragma unroll 1
+  for (int k = threadIdx.x; k < r; k += blockDim.x) {
     int q4[4];
-    limbs_of(at(k), inv, q4);
+    limbs_of(normed(v.get(k), inv_rms, gain, use_rms, k), inv, q4);
 #pragma unroll
     for (int l = 0; l < 4; ++l) limbs[((size_t)4 * b + l) * r + k] = (int8_t)q4[l];
   }
@@ -1912,24 +1917,30 @@ cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s) {
                         : launch_down_q<0>(p, g, smem, s, map_wg, map_wt, map_hm);
 }
 
+// Pairs of entries up to this many columns: groups of eight left a token of 256 columns to one warp (whole calls, 256 x 700, 4 /
+// 16 tokens, eights / pairs: int4 23.3 / 26.1 us -> 22.3 / 25.4).  Pairs up to 2048 are no faster.
+constexpr int kShortToken = 1024;
 cudaError_t launch_token_limbs(const void* x, int B, int K, int x_stride, void* limbs, float* scale, void* zero, int zero_bytes,
                                cudaStream_t s) {
-  return launch_pdl(token_limbs_kernel, dim3(B), dim3(kLimbThreads), 0, s, static_cast<const __nv_bfloat16*>(x), K, x_stride,
-                    static_cast<int8_t*>(limbs), scale, static_cast<int4*>(zero), zero_bytes / 16);
+  const bool pairs = K <= kShortToken;
+  const int groups = (K / (pairs ? 2 : 8) + 31) / 32 * 32;
+  return launch_pdl(pairs ? token_limbs_kernel<2> : token_limbs_kernel<8>, dim3(B), dim3(groups < kLimbMaxThreads ? groups : kLimbMaxThreads),
+                    0, s, static_cast<const __nv_bfloat16*>(x), K, x_stride, static_cast<int8_t*>(limbs), scale, static_cast<int4*>(zero),
+                    zero_bytes / 16);
 }
 
 cudaError_t launch_rmsnorm_limbs(float* v, int B, int r, int v_stride, const UmmaLimbSums* sums, const float* gain, float eps,
                                  bool use_rms, void* limbs, float* scale, cudaStream_t s) {
-  const dim3 block(r <= 256 ? 256 : r <= 512 ? 512 : kVecMaxThreads);
+  const dim3 block(vec_threads(r));
   int8_t* out = static_cast<int8_t*>(limbs);
-  if (!sums) return launch_pdl(rmsnorm_limbs_kernel<PlainVec>, dim3(B), block, 0, s, PlainVec{v, v_stride}, r, gain, eps, use_rms ? 1 : 0, out, scale);
+  if (!sums) return launch_pdl(rmsnorm_limbs_kernel<SumVec>, dim3(B), block, 0, s, SumVec{v, v_stride, 1, 0}, r, gain, eps, use_rms ? 1 : 0, out, scale);
   const LimbSumsVec vec{reinterpret_cast<int*>(v), v_stride, sums->row_scale, sums->tok_scale, sums->code_scale, 0.f};
   return launch_pdl(rmsnorm_limbs_kernel<LimbSumsVec>, dim3(B), block, 0, s, vec, r, gain, eps, use_rms ? 1 : 0, out, scale);
 }
 
-cudaError_t launch_rmsnorm_split(const float* v, int B, int r, int v_stride, int runs, size_t step, const float* gain, float eps,
+cudaError_t launch_rmsnorm_split(float* v, int B, int r, int v_stride, int runs, size_t step, const float* gain, float eps,
                                  bool use_rms, int cols, bool exact, void* x2, cudaStream_t s) {
-  return launch_pdl(rmsnorm_split_kernel, dim3(B), dim3(kVecThreads), 0, s, v, r, v_stride, runs, step, gain, eps, use_rms ? 1 : 0,
+  return launch_pdl(rmsnorm_split_kernel, dim3(B), dim3(vec_threads(r)), 0, s, SumVec{v, v_stride, runs, step}, r, gain, eps, use_rms ? 1 : 0,
                     cols, exact ? 1 : 0, static_cast<__nv_bfloat16*>(x2));
 }
 

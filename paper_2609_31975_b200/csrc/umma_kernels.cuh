@@ -109,7 +109,7 @@ struct UmmaLimbSums {
 cudaError_t launch_rmsnorm_limbs(float* v, int B, int r, int v_stride, const UmmaLimbSums* sums, const float* gain, float eps,
                                  bool use_rms, void* limbs, float* scale, cudaStream_t s);
 // The bf16 pairs (or triples) of n.  v is the sum of `runs` vectors, `step` floats apart.
-cudaError_t launch_rmsnorm_split(const float* v, int B, int r, int v_stride, int runs, size_t step, const float* gain, float eps,
+cudaError_t launch_rmsnorm_split(float* v, int B, int r, int v_stride, int runs, size_t step, const float* gain, float eps,
                                  bool use_rms, int cols, bool exact, void* x2, cudaStream_t s);
 
 }  // namespace sffn

@@ -205,3 +205,35 @@ def test_lopa_batches_are_the_same_bits_whatever_rank_the_handle_allows(q8):
         torch.cuda.synchronize()
         assert ffn.device_status() == 0
     assert torch.equal(ys[0], ys[1])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("qbits", [8, 4])
+@pytest.mark.parametrize("D", [256, 768, 1024, 1280, 4096, 8192, 8448, 14336])
+def test_every_limb_of_every_column_arrives(D, qbits):
+    """Columns 1 to D - 2 have a neuron each, whose pre-activation is that column's entry beside two products of 127 and the largest
+    code that cancel.  The entry lies in the token's second, third or fourth limb, and which neurons fire says whether each
+    limb of each column is where it belongs, with its sign.  Widths: pairs and groups of eight entries a thread, one group
+    a thread and more."""
+    import paper_2609_31975_b200 as m
+
+    gen = torch.Generator().manual_seed(D + qbits)
+    top, B, n = 2 ** (qbits - 1) - 1, 2, min(D - 2, 8192)
+    col = 1 + torch.randperm(D - 2, generator=gen)[:n]
+    part, positive = small_parts(D, B, gen)
+    owner = torch.randint(0, B, (D,), generator=gen)
+    x = -part.repeat(B, 1)
+    for b in range(B):
+        x[b, positive & (owner == b)] *= -1
+    x[:, 0] = x[:, D - 1] = 127.0
+    W = torch.zeros((n, D), dtype=torch.int8)
+    W[:, 0], W[:, D - 1] = top, -top
+    W[torch.arange(n), col] = 1
+    ffn = m.SparseFFN(D, n, torch.bfloat16, B_max=B)
+    gate = {"W_g": dict(q=pack(W, qbits), s=torch.ones(n, device=DEV))}
+    w = dict(q=pack(torch.ones((n, D), dtype=torch.int8), qbits), s=torch.full((n,), 0.01, device=DEV))
+    (ffn.sparse_ffn_forward_q8 if qbits == 8 else ffn.sparse_ffn_forward_q4)(x.bfloat16().to(DEV), gate, None, w, w, "relu")
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0
+    fires = (x[:, col] > 0).any(dim=0)
+    assert torch.equal(ffn.last_active().cpu().long(), torch.nonzero(fires)[:, 0])
