@@ -481,11 +481,12 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
   constexpr int kAtomElems = kNat ? 128 : kAtomK;              // elements of one 128-byte swizzle row
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // Gate mode: a second grid dimension cuts K into runs of blocks (see umma_k_splits); each writes sums of its own.
+  // Gate mode: a second grid dimension cuts K into runs of blocks (see umma_k_splits), the first `longer_runs` of them one block
+  // longer; each writes sums of its own, or adds its own to the others'.  (Not a mode of its own: the gate that follows V x finds
+  // its code in the caches, without which calls of bf16 rows take 1 us more.)
   constexpr bool kSplits = MODE == kGate && !EX;
-  const int k_run = kSplits ? (p.K / kAtomElems + (int)gridDim.y - 1) / (int)gridDim.y : p.K / kAtomElems;
-  const int kb_first = kSplits ? (int)blockIdx.y * k_run : 0;
-  const int kblocks = min(k_run, p.K / kAtomElems - kb_first);
+  const int kb_first = kSplits ? (int)blockIdx.y * p.run_blocks + min((int)blockIdx.y, p.longer_runs) : 0;
+  const int kblocks = kSplits ? p.run_blocks + ((int)blockIdx.y < p.longer_runs) : p.K / kAtomElems;
   float* const a_out = p.a_out + (kSplits ? (size_t)blockIdx.y * p.split_stride : 0);
 
   // Set-up that needs nothing from earlier kernels runs while the predecessor in the stream finishes.
@@ -745,6 +746,18 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
       __nv_bfloat16* hm = static_cast<__nv_bfloat16*>(p.hmT) + li;
       float* arow = a_out + j;
       const __nv_bfloat16* xg = static_cast<const __nv_bfloat16*>(p.xtok) + (gi >= 0 ? gi : 0);
+      if (kSplits && p.k_splits > 1) {  // a run of K: added to the integer sums of the others, in whatever order
+#pragma unroll 1
+        for (int c0 = 8 * part; c0 < npad; c0 += 8 * nparts) {
+          int iv[8];
+          tmem_ld8_int(taddr + c0, nacc, npad, iv);
+          int* sums = reinterpret_cast<int*>(a_out) + (size_t)c0 * p.a_stride + j;  // column c0 is limb c0 mod 4 of token c0 / 4
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            if (row_ok && c0 + q < 4 * B) atomicAdd(sums + (size_t)q * p.a_stride, iv[q]);
+        }
+        return true;
+      }
       for (int c0 = 8 * part; c0 < npad; c0 += 8 * nparts) {
         int iv[8];
         tmem_ld8_int(taddr + c0, nacc, npad, iv);
@@ -752,11 +765,6 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
         for (int q = 0; q < 2; ++q) {
           const int b = c0 / 4 + q;
           if (row_ok && b < B) {
-            if (kSplits && p.k_splits > 1) {  // a run of K: added to the integer sums of the others, in whatever order
-#pragma unroll
-              for (int l = 0; l < 4; ++l) atomicAdd(reinterpret_cast<int*>(a_out) + (size_t)(4 * b + l) * p.a_stride + j, iv[4 * q + l]);
-              continue;
-            }
             const float val = p.tok_scale[b] * sc * limb_sum(iv[4 * q], iv[4 * q + 1], iv[4 * q + 2], iv[4 * q + 3]);
             if (UP) {
               const float av = p.a[(size_t)b * p.a_stride + j];
@@ -1818,6 +1826,9 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
   p.drop_stage = fused_test_knobs().drop_stage;
   const int splits = p.k_splits > 1 ? p.k_splits : 1;
   if (splits > 1 && (up || p.exact || p.b_g || p.g_idx || p.flag || p.words_out || p.act != kUmmaActIdentity)) return cudaErrorInvalidValue;
+  const int kb = p.K / (p.qbits == 1 || p.qbits == 2 ? 128 : kAtomK);
+  p.run_blocks = kb / splits;
+  p.longer_runs = kb % splits;
   const int grid = splits > 1 ? p.k_tiles : p.R < 8 * sm_count ? (p.R + 7) / 8 : sm_count;
   // all the dynamic shared memory a CTA can have; the kernel cuts its ring out of it once it knows its tiles
   const size_t smem = kRowsSmem;
