@@ -1485,32 +1485,40 @@ template <typename Vec>
 struct Kept {
   const Vec& vec;
   float* sm;
-  __device__ __forceinline__ float get(int k) const { return k < kVecKept ? sm[k] : vec.home(k); }
+  int room;  // entries of sm
+  __device__ __forceinline__ float get(int k) const { return k < room ? sm[k] : vec.home(k); }
   __device__ __forceinline__ void put(int k, float e) const {
-    if (k < kVecKept) sm[k] = e;
+    if (k < room) sm[k] = e;
     else vec.home(k) = e;
   }
 };
-// Fetches the entries (thread k mod blockDim.x's are there for itself) and returns 1 / rms, or 1.
-template <typename Vec>
+// Fetches the entries (thread k mod blockDim.x's are there for itself) and returns 1 / rms, or 1.  ONE: a block of kVecThreads
+// for at most as many entries.
+template <bool ONE, typename Vec>
 __device__ __forceinline__ float take_vec(const Kept<Vec>& v, int r, float eps, int use_rms, float* red) {
   const int tid = threadIdx.x;
   float ss = 0.f;
+  if (ONE) {
+    const float e = tid < r ? v.vec.entry(tid) : 0.f;
+    ss = e * e;
+    v.put(tid, e);
+  } else {
 #pragma unroll 2
-  for (int k = tid; k < r; k += blockDim.x) {
-    const float e = v.vec.entry(k);
-    ss = fmaf(e, e, ss);
-    v.put(k, e);
+    for (int k = tid; k < r; k += blockDim.x) {
+      const float e = v.vec.entry(k);
+      ss = fmaf(e, e, ss);
+      v.put(k, e);
+    }
   }
   if (!use_rms) return 1.f;
-  if (blockDim.x != kVecThreads) {
+  if (!ONE && blockDim.x != kVecThreads) {
     __syncthreads();
     ss = 0.f;
     if (tid < kVecThreads)
 #pragma unroll 4
       for (int k = tid; k < r; k += kVecThreads) ss = fmaf(v.get(k), v.get(k), ss);
   }
-  if (tid < kVecThreads) {
+  if (ONE || tid < kVecThreads) {
     ss = warp_sum(ss);
     if ((tid & 31) == 0) red[tid >> 5] = ss;
   }
@@ -1527,17 +1535,19 @@ __device__ __forceinline__ float normed(float e, float inv, const float* gain, i
 // LoPA gate, batched: n = RMSNorm(v) (or v itself) as a sum of two bf16 vectors for the tensor cores: row b of
 // x2 holds the high part of token b's vector, row cols + b the low part (v - bf16(v)), so that the gate's U n keeps
 // close to fp32 accuracy.  `exact`: row 2 cols + b holds what those two leave (24 bits in all).
-__global__ void __launch_bounds__(kVecMaxThreads) rmsnorm_split_kernel(SumVec vec, int r, const float* gain, float eps, int use_rms,
+template <bool ONE>
+__global__ void __launch_bounds__(ONE ? kVecThreads : kVecMaxThreads) rmsnorm_split_kernel(SumVec vec, int r, const float* gain, float eps, int use_rms,
                                                                        int cols, int exact, __nv_bfloat16* x2) {
-  __shared__ float kept[kVecKept], red[kVecThreads / 32];
+  constexpr int kRoom = ONE ? kVecThreads : kVecKept;
+  __shared__ float kept[kRoom], red[kVecThreads / 32];
   pdl_launch_dependents();
   pdl_wait();
   const int b = blockIdx.x;
   vec.token(b);
-  const Kept<SumVec> v{vec, kept};
-  const float inv = take_vec(v, r, eps, use_rms, red);
+  const Kept<SumVec> v{vec, kept, kRoom};
+  const float inv = take_vec<ONE>(v, r, eps, use_rms, red);
 #pragma unroll 1
-  for (int k = threadIdx.x; k < r; k += blockDim.x) {
+  for (int k = threadIdx.x; k < r; k += ONE ? kVecThreads : blockDim.x) {
     float n = normed(v.get(k), inv, gain, use_rms, k);
     x2[(size_t)b * r + k] = take_bf16(n);
     x2[(size_t)(cols + b) * r + k] = take_bf16(n);
@@ -1643,16 +1653,17 @@ __global__ void __launch_bounds__(kLimbMaxThreads) token_limbs_kernel(const __nv
 }
 
 // LoPA gate with rows of codes: n = RMSNorm(v) (or v itself) as limbs.
-template <typename Vec>
-__global__ void __launch_bounds__(kVecMaxThreads) rmsnorm_limbs_kernel(Vec vec, int r, const float* gain, float eps, int use_rms,
+template <bool ONE, typename Vec>
+__global__ void __launch_bounds__(ONE ? kVecThreads : kVecMaxThreads) rmsnorm_limbs_kernel(Vec vec, int r, const float* gain, float eps, int use_rms,
                                                                        int8_t* limbs, float* scale) {
-  __shared__ float kept[kVecKept], red[kVecThreads / 32], red2[kVecMaxThreads / 32];
+  constexpr int kRoom = ONE ? kVecThreads : kVecKept;
+  __shared__ float kept[kRoom], red[kVecThreads / 32], red2[kVecMaxThreads / 32];
   pdl_launch_dependents();
   pdl_wait();
   const int b = blockIdx.x;
   vec.token(b);
-  const Kept<Vec> v{vec, kept};
-  const float inv_rms = take_vec(v, r, eps, use_rms, red);
+  const Kept<Vec> v{vec, kept, kRoom};
+  const float inv_rms = take_vec<ONE>(v, r, eps, use_rms, red);
   float m = 0.f;
 #pragma unroll 1
   for (int k = threadIdx.x; k < r; k += blockDim.x) m = fmaxf(m, fabsf(normed(v.get(k), inv_rms, gain, use_rms, k)));
@@ -1944,15 +1955,22 @@ cudaError_t launch_rmsnorm_limbs(float* v, int B, int r, int v_stride, const Umm
                                  bool use_rms, void* limbs, float* scale, cudaStream_t s) {
   const dim3 block(vec_threads(r));
   int8_t* out = static_cast<int8_t*>(limbs);
-  if (!sums) return launch_pdl(rmsnorm_limbs_kernel<SumVec>, dim3(B), block, 0, s, SumVec{v, v_stride, 1, 0}, r, gain, eps, use_rms ? 1 : 0, out, scale);
+  const bool one = r <= kVecThreads;
+  if (!sums) {
+    const SumVec vec{v, v_stride, 1, 0};
+    return launch_pdl(one ? rmsnorm_limbs_kernel<true, SumVec> : rmsnorm_limbs_kernel<false, SumVec>, dim3(B), block, 0, s, vec, r, gain, eps,
+                      use_rms ? 1 : 0, out, scale);
+  }
   const LimbSumsVec vec{reinterpret_cast<int*>(v), v_stride, sums->row_scale, sums->tok_scale, sums->code_scale, 0.f};
-  return launch_pdl(rmsnorm_limbs_kernel<LimbSumsVec>, dim3(B), block, 0, s, vec, r, gain, eps, use_rms ? 1 : 0, out, scale);
+  return launch_pdl(one ? rmsnorm_limbs_kernel<true, LimbSumsVec> : rmsnorm_limbs_kernel<false, LimbSumsVec>, dim3(B), block, 0, s, vec, r, gain,
+                    eps, use_rms ? 1 : 0, out, scale);
 }
 
 cudaError_t launch_rmsnorm_split(float* v, int B, int r, int v_stride, int runs, size_t step, const float* gain, float eps,
                                  bool use_rms, int cols, bool exact, void* x2, cudaStream_t s) {
-  return launch_pdl(rmsnorm_split_kernel, dim3(B), dim3(vec_threads(r)), 0, s, SumVec{v, v_stride, runs, step}, r, gain, eps, use_rms ? 1 : 0,
-                    cols, exact ? 1 : 0, static_cast<__nv_bfloat16*>(x2));
+  const SumVec vec{v, v_stride, runs, step};
+  return launch_pdl(r <= kVecThreads ? rmsnorm_split_kernel<true> : rmsnorm_split_kernel<false>, dim3(B), dim3(vec_threads(r)), 0, s, vec, r,
+                    gain, eps, use_rms ? 1 : 0, cols, exact ? 1 : 0, static_cast<__nv_bfloat16*>(x2));
 }
 
 }  // namespace sffn
