@@ -318,7 +318,8 @@ const char* sffn_status_string(int status);
  *   gate slot, gate slot bytes, gate slots, gate warps, act slot bytes, act slots, chunks per act thread, shared
  *   memory bytes (wkind: 0 fp32, 1 bf16, 2 int8 rows).  sffn_test_umma_tiling: tiling of the batched gate GEMM over short
  *   rows; sffn_test_umma_row_tiling: over rows of K elements; sffn_test_umma_pass_tiling: over rows of K elements (qbits 0:
- *   bf16) or codes (8 / 4; 1 / 2: against limbs) in a pass of B tokens.
+ *   bf16) or codes (8 / 4; 1 / 2: against limbs) in a pass of B tokens.  sffn_test_umma_k_splits: runs of K and tiles of
+ *   rows of V x, R rows of K elements (limbs: codes) against B tokens, at most max_splits runs.
  * sffn_test_set_knob(knob, value):
  *   PDL                 programmatic dependent launch between calls (default 1)
  *   TENSOR_GATE         1 / 0: single-token calls take the tensor-core gate kernel wherever it applies / nowhere,
@@ -349,6 +350,7 @@ void sffn_test_fused_plan(int wkind, int D, int H, int K, int lopa, int sm_count
 void sffn_test_umma_tiling(int R, int sm_count, int* tile_rows, int* n_tiles, int* own_list);
 void sffn_test_umma_row_tiling(int R, int K, int sm_count, int* tile_rows, int* n_tiles, int* own_list);
 void sffn_test_umma_pass_tiling(int R, int K, int qbits, int B, int sm_count, int* tile_rows, int* n_tiles, int* own_list);
+void sffn_test_umma_k_splits(int R, int K, int limbs, int B, int sm_count, int max_splits, int* tiles, int* splits);
 int sffn_test_set_knob(int knob, long long value);
 
 #ifdef __cplusplus

@@ -210,6 +210,9 @@ void sffn_test_umma_pass_tiling(int R, int K, int qbits, int B, int sm_count, in
   sffn::umma_gate_tiling(R, K, qbits, B, sm_count, tile_rows, n_tiles);
   *own_list = sffn::umma_own_list_supported(R, K, qbits, B, sm_count) ? 1 : 0;
 }
+void sffn_test_umma_k_splits(int R, int K, int limbs, int B, int sm_count, int max_splits, int* tiles, int* splits) {
+  sffn::umma_k_splits(R, K, limbs != 0, B, sm_count, max_splits, tiles, splits);
+}
 int sffn_test_set_knob(int knob, long long value) {
   sffn::FusedTestKnobs& k = sffn::fused_test_knobs();
   switch (knob) {
@@ -359,7 +362,7 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
   int v_tiles = 1, v_runs = 1, vs = rs;
   if (lopa && umma && !exact) {
     const long long room = (long long)kMaxUpDownGrid * kMaxChunk * D / ((long long)B * g->r);
-    umma_k_splits(g->r, D, native, h->sm_count, !native ? (int)room : room >= 4 ? 16 : 1, &v_tiles, &v_runs);
+    umma_k_splits(g->r, D, native, B, h->sm_count, !native ? (int)room : room >= 4 ? 16 : 1, &v_tiles, &v_runs);
     if (v_runs > 1) {
       v = h->at<float>(h->L.partial);
       vs = g->r;

@@ -1816,16 +1816,19 @@ cudaError_t launch_rows_mode(const UmmaRowsParams& p, dim3 grid, size_t smem, cu
 // calls of r >= 1280 were 2 us longer: one SM read 130 KB).  Whole calls, 4096 x 14336, r = 512, 5 / 64 tokens, not cut / cut:
 // 47.8 / 93.8 -> 47.1 / 87.6 us (bf16), 8 / 64 tokens 49.8 / 108 -> 47.0 / 98.7 (int4); 8192 x 28672, r = 1024, 8 tokens:
 // 101 -> 96.5 (int8).
-void umma_k_splits(int R, int K, bool codes, int sm_count, int max_splits, int* tiles, int* splits) {
+// Rows of up to kShortRow columns are cut from 16 tokens on: fewer hand little over, and the cut costs the norm more round trips
+// (1024 x 3000, r = 128, 2 / 8 / 16 / 64 tokens, not cut / cut: bf16 25.5 / 28.4 / 29.9 / 42.8 us against 26.4 / 28.5 / 30.0 / 41.3;
+// int4 29.6 / 32.9 / 36.4 / 56.6 against 29.8 / 32.6 / 35.4 / 55.5).  The runs differ by at most one block of K.
+void umma_k_splits(int R, int K, bool codes, int B, int sm_count, int max_splits, int* tiles, int* splits) {
   const int kb = K / (codes ? 128 : kAtomK);
   auto least = [](int a, int b) { return a < b ? a : b; };
   int t = (R + 63) / 64, n = least(least(max_splits, 16), least(sm_count / t, kb / 4));
   *tiles = *splits = 1;
-  if (n < 2) return;
+  if (n < 2 || (K <= kShortRow && B < 16)) return;
   if (4 * t * n < 3 * sm_count) t = least((R + 7) / 8, sm_count / n);
-  const int rows = ((R + t - 1) / t + 7) & ~7, run = (kb + n - 1) / n;
+  const int rows = ((R + t - 1) / t + 7) & ~7;
   *tiles = (R + rows - 1) / rows;
-  *splits = (kb + run - 1) / run;
+  *splits = n;
 }
 
 cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, cudaStream_t s) {

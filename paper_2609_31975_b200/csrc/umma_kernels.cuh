@@ -100,8 +100,9 @@ bool umma_rows_native_i8_supported(int K, int tokens);
 // zeroes B * zero_bytes (a multiple of 16) beside it.
 cudaError_t launch_token_limbs(const void* x, int B, int K, int x_stride, void* limbs, float* scale, void* zero, int zero_bytes,
                                cudaStream_t s);
-// How v = V x (R rows of K elements or codes) is cut: `splits` runs of K (1: not), each over `tiles` tiles of rows.
-void umma_k_splits(int R, int K, bool codes, int sm_count, int max_splits, int* tiles, int* splits);
+// How v = V x (R rows of K elements, or codes against limbs; B tokens) is cut: `splits` runs of K (1: not), each over `tiles` tiles
+// of rows.
+void umma_k_splits(int R, int K, bool codes, int B, int sm_count, int max_splits, int* tiles, int* splits);
 // The same for the LoPA vector n = RMSNorm(v) (or v): from fp32 (`sums` null), or from integer sums, four rows of v_stride a token.
 struct UmmaLimbSums {
   const float *row_scale, *tok_scale;  // of V's rows and of the tokens' limbs

@@ -97,14 +97,44 @@ def test_token_limbs_of_every_width(D):
     assert ((y - one).norm() / one.norm()).item() < 1e-2
 
 
+def runs_of(lib, R, K, limbs, B, sms=148, most=16):
+    tiles, runs = ctypes.c_int(), ctypes.c_int()
+    lib.sffn_test_umma_k_splits(R, K, limbs, B, sms, most, ctypes.byref(tiles), ctypes.byref(runs))
+    return tiles.value, runs.value
+
+
+@pytest.mark.parametrize("limbs", [0, 1])
+@pytest.mark.parametrize("sms", [132, 148])
+def test_runs_of_columns_are_whole_and_fit_the_grid(sms, limbs):
+    import paper_2609_31975_b200 as m
+
+    lib = m.load_library()
+    block, cut = 128 if limbs else 64, 0
+    for K in (256, 512, 768, 1024, 1280, 3840, 4096, 4352, 8192, 14336):
+        for R in (8, 64, 72, 128, 448, 512, 896, 1024, 1088, 2048, 4224, 20000):
+            for B in (2, 15, 16, 64):
+                for most in (0, 1, 2, 5, 16):
+                    tiles, runs = runs_of(lib, R, K, limbs, B, sms, most)
+                    if runs == 1:
+                        continue
+                    cut += 1
+                    assert runs <= most and tiles * runs <= sms                  # a CTA for each
+                    assert K // block // runs >= 4                               # the shorter runs have four blocks
+                    rows = (-(-R // tiles) + 7) // 8 * 8                         # as the kernel takes them
+                    assert rows <= 128 and (tiles - 1) * rows < R <= tiles * rows
+                    assert K > 1024 or B >= 16
+    assert cut > 500
+    assert runs_of(lib, 896, 4096, 0, 2) == (14, 10) and runs_of(lib, 512, 4096, 1, 64) == (16, 8)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("D,r,B", [
     (256, 64, 2),       # too few columns to cut
-    (512, 128, 3),      # two runs
-    (4096, 64, 5),      # sixteen runs of one tile's rows
+    (512, 128, 3),      # too few tokens
+    (4096, 64, 5),      # sixteen runs of one tile's rows (int8: eight)
     (3840, 448, 16),    # runs of unequal length
     (4352, 1088, 70),   # unequal runs, a ragged last tile of rows
-    (2304, 2112, 4),    # a vector longer than what the norm kernel's threads keep
+    (2304, 2112, 4),    # several entries for each thread of the norm kernel
 ])
 @pytest.mark.parametrize("q8", [False, True])
 def test_lopa_batches_with_v_from_several_runs_of_columns(D, r, B, q8):
@@ -148,19 +178,20 @@ def small_parts(n, B, gen):
 @pytest.mark.gpu
 @pytest.mark.parametrize("qbits", [8, 4])
 @pytest.mark.parametrize("rms", [False, True])
-@pytest.mark.parametrize("D,r,B", [
-    (512, 128, 3),      # not cut
-    (1024, 256, 5),     # two runs
-    (4096, 128, 64),    # eight
-    (3840, 896, 16),    # runs of unequal length
-    (8192, 512, 2),     # sixteen
-    (1024, 4224, 3),    # a vector longer than what the norm kernel keeps in shared memory
+@pytest.mark.parametrize("D,r,B,runs", [
+    (512, 128, 3, 1),       # not cut
+    (1024, 256, 16, 2),
+    (4096, 128, 64, 8),     # one entry a thread of the norm kernel
+    (3840, 896, 16, 7),     # runs of four and five blocks
+    (8192, 512, 2, 16),
+    (1280, 4224, 3, 2),     # a vector longer than what the norm kernel keeps in shared memory
 ])
-def test_quantised_lopa_vectors_cut_into_runs_keep_integer_sums(D, r, B, rms, qbits):
+def test_quantised_lopa_vectors_cut_into_runs_keep_integer_sums(D, r, B, runs, rms, qbits):
     """Every entry of v is a small part beside two products of 127 and the largest code that cancel, one in the first and one in
     the last run of columns: integer sums keep the part and its sign, fp32 sums of runs lose all below 2^-24 of the products."""
     import paper_2609_31975_b200 as m
 
+    assert runs_of(m.load_library(), r, D, 1, B)[1] == runs
     gen = torch.Generator().manual_seed(D + r)
     top, H = 2 ** (qbits - 1) - 1, r
     col = torch.randint(1, D - 1, (r,), generator=gen)
@@ -185,6 +216,30 @@ def test_quantised_lopa_vectors_cut_into_runs_keep_integer_sums(D, r, B, rms, qb
     # V's products are exact; the limbs of n reach 2^-22 of its largest entry, far below 2^-18 / 2^-4
     fires = (x[:, col] > 0).any(dim=0)
     assert torch.equal(ffn.last_active().cpu().long(), torch.nonzero(fires)[:, 0])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("D,r,B", [
+    (512, 64, 16),      # two runs, one entry a thread of the norm kernel
+    (1024, 256, 128),   # four runs
+    (2304, 4160, 4),    # two runs, a vector longer than what the norm kernel keeps in shared memory
+])
+def test_bf16_lopa_batches_with_sums_of_runs(D, r, B):
+    """Against the oracle, the fired set included."""
+    import paper_2609_31975_b200 as m
+
+    assert runs_of(m.load_library(), r, D, 0, B)[1] > 1
+    H = 600
+    w = syn.lopa_ffn(D, H, r, torch.bfloat16, 75, DEV, sparsity=0.7)
+    gate = {"V": w["V"], "U": w["U"], "g_idx": m.g_diagonal(H, D, DEV)}
+    ffn = m.SparseFFN(D, H, torch.bfloat16, r_max=r, B_max=B)
+    x = syn.tokens(B, D, torch.bfloat16, 75, DEV)
+    y = ffn.sparse_ffn_forward(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0
+    ref = run_oracle(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+    assert_y_close(y, ref["y"], what=f"{D} r={r} B={B}")
+    assert_active_set(ffn.last_active(), ref, what=f"{D} r={r} B={B}")
 
 
 @pytest.mark.gpu
