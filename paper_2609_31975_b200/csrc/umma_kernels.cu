@@ -20,18 +20,19 @@
 //              lets the copies run at memory speed; warp 8 allocates and frees the TMEM columns
 //   warps 4-7  epilogue: tcgen05.ld the accumulator row of "their" neuron (all accumulators added), apply the
 //              gate / scale epilogue; for wide batches all twelve warps share the epilogue of the CTA's last tile
-// A problem of up to 256 rows per SM is cut into one or two tiles per SM, all of one height (see tile_rows_for).  The ring of
+// A problem of up to 256 rows per SM is cut into one or two tiles per SM, all of one height, but short rows and most wide
+// batches over more than 128 into tiles of 128 (see tile_rows_for).  The ring of
 // stages (up to 12) is cut out of the dynamic shared memory on the device, once the tile height is known.
 // Every kernel here is launched with programmatic dependent launch: set-up first, griddepcontrol.wait before the
 // first dependent read or global write.
 // Weight-only int8 / int4 rows (QB = 8 / 4): the copies bring the codes (and the token rows) into the ring slots;
 // four more warps (the last four of the CTA, two pairs that alternate over the stages) expand the codes to bf16 --
 // every code is an integer bf16 holds exactly -- in the swizzled layout, into a short ring of expanded blocks of
-// its own (rows kernels) or the slot's block area (down kernel), and arrive on a "ready" barrier that the MMA
-// issuers wait for instead of "full"; the row scales are applied to the accumulator rows in the epilogue (the
-// down projection's are folded into Hm).  With the weights as the A operand the tensor core takes 32 bytes of
-// bf16 per cycle and SM whatever the token count, i.e. 16 codes per cycle: quantised batches are bound by that
-// rate, not by their bytes.
+// its own (rows kernels; down kernel, where that leaves more slots for the copies) or the slot's block area, and
+// arrive on a "ready" barrier that the MMA issuers wait for instead of "full"; the row scales are applied to the
+// accumulator rows in the epilogue (the down projection's are folded into Hm).  With the weights as the A operand
+// the tensor core takes 32 bytes of bf16 per cycle and SM whatever the token count, i.e. 16 codes per cycle:
+// quantised batches are bound by that rate, not by their bytes.
 // Up to 256 token columns go through in one pass.  Wide batches (npad > 128) leave room for two accumulators and a ring
 // of four stages of ~40 KB (two with expanded codes and 241 columns or more); they are bound by the token rows every CTA reads again (200 tokens x 4096: 1.6 MB a CTA
 // through L2 beside 0.8 MB of weights), still far cheaper than further passes over the weights (200 tokens, 4096 x
@@ -61,7 +62,7 @@ constexpr int kProducerWarps = 4;
 constexpr int kMaxStages = 16;                       // barrier slots; bf16 rows use up to 12
 constexpr int kMaxStagesBf16 = 12;
 constexpr int kExpandSlots = 4;                      // quantised rows: ring of expanded bf16 blocks
-constexpr int kDownExpand = 4;                       // the same in the down kernel, at most (2 or 4, see launch_umma_down)
+constexpr int kDownExpand = 4;                       // the same in the down kernel's, where it has two rings (2 or 4)
 constexpr int kWalkMinTokens = 32;                   // batches from which the up kernel may walk every row
 constexpr int kWalkAllPercent = 70;                  // union share of the rows from which "every row" is walked
 constexpr int kMaxIssuers = 4;
@@ -1180,7 +1181,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
 // gathered row delivers 64 contiguous d per swizzle row) and HmT[b][u] is the K-major B operand.
 // Same pipeline as above: 4 producer warps (gather4 per lane: 2 column halves x 16 row quads = one 64-row
 // stage), 2 MMA issuers with their own accumulators, 4 epilogue warps; two CTAs share an SM.
-template <int QB, bool EX = false>
+template <int QB, bool EX = false, bool TWO = false>
 __global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarps : 0), EX ? 1 : 2) umma_down_kernel(const UmmaDownParams p,
                                                                   const __grid_constant__ CUtensorMap map_wg,
                                                                   const __grid_constant__ CUtensorMap map_wt,
@@ -1188,11 +1189,12 @@ __global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarp
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const int npad = p.npad;
   constexpr int kRawBytes = QB * kTileRows * kAtomK / 8;  // quantised rows: the codes of a stage's 64 rows x 128 columns
-  // Quantised rows: a ring slot holds what the copies bring (h, then the codes); the expanded blocks have a short ring of
-  // their own in front of it (stage kb uses block kb mod E), as in the rows kernels.  One ring of slots with room for both was
-  // two slots deep from 24 tokens of int8 rows on (whole calls, 4096 x 14336, 24 / 64 tokens: 70.6 / 96.8 -> 62.5 / 88.6 us;
-  // 8192 x 24000, 24 tokens: 178 -> 145).  Exact sums keep the one ring.
-  constexpr bool kTwo = QB != 0 && !EX;
+  // Quantised rows.  One ring: a slot holds the expanded block, h, then the codes.  TWO: it holds what the copies bring (h, then
+  // the codes); the expanded blocks have a short ring of their own in front of it (stage kb uses block kb mod E), as in the rows
+  // kernels.  That is for the slots that with room for both are two or four (see launch_umma_down; whole calls, int8, 4096 x
+  // 14336, 24 / 64 tokens, one ring / two: 70.6 / 97.5 -> 62.4 / 88.7 us; 8192 x 18000, 24 tokens: 142 -> 116).
+  constexpr bool kTwo = TWO;
+  static_assert(!TWO || (QB != 0 && !EX), "two rings: codes, plain sums");
   const int E = p.expand, expand_bytes = kTwo ? E * kAAtomBytes : 0;
   const int b_off = kTwo ? 0 : kAAtomBytes;               // h within a slot
   const int raw_off = b_off + npad * 128;
@@ -1366,7 +1368,7 @@ __global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarp
         if (nacc == 2 && (s & 1) != m) continue;
         const int e = kb & (E - 1);
         if (!(kTwo ? mbar_wait(ready + 8 * e, (kb & E) ? 1u : 0u, abort_flag, p.status, p.wait_cycles)
-                   : mbar_wait(full + 8 * s, ph, abort_flag, p.status, p.wait_cycles))) { ok = false; break; }
+                   : mbar_wait((QB ? ready : full) + 8 * s, ph, abort_flag, p.status, p.wait_cycles))) { ok = false; break; }
         tc_fence_after();
         const uint32_t sbase = stage0 + s * stage_bytes;
         const uint32_t abase = kTwo ? expand0 + e * kAAtomBytes : sbase;
@@ -1892,13 +1894,13 @@ int umma_down_splits(int D, int cols, bool exact, int sm_count, int max_splits) 
 bool umma_down_supported(int D, int cols) { return D % kTileRows == 0 && cols >= 1 && cols <= kUmmaMaxCols; }
 
 namespace {
-template <int QB, bool EX = false>
+template <int QB, bool EX = false, bool TWO = false>
 cudaError_t launch_down_q(const UmmaDownParams& p, int grid, size_t smem, cudaStream_t s, const CUtensorMap& map_wg,
                           const CUtensorMap& map_wt, const CUtensorMap& map_hm) {
   static unsigned long long configured = 0;
-  const cudaError_t e = allow_dynamic_smem(umma_down_kernel<QB, EX>, 227 * 1024, configured);
+  const cudaError_t e = allow_dynamic_smem(umma_down_kernel<QB, EX, TWO>, 227 * 1024, configured);
   if (e != cudaSuccess) return e;
-  return launch_pdl(umma_down_kernel<QB, EX>, dim3(grid), dim3((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarps : 0)), smem, s, p, map_wg,
+  return launch_pdl(umma_down_kernel<QB, EX, TWO>, dim3(grid), dim3((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarps : 0)), smem, s, p, map_wg,
                     map_wt, map_hm);
 }
 }  // namespace
@@ -1911,17 +1913,25 @@ cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s) {
   p.npad = (own + 15) / 16 * 16;
   if (p.cols % 8 || p.cols < p.B || p.npad > kUmmaMaxCols) return cudaErrorInvalidValue;
   p.wait_cycles = fused_test_knobs().wait_cycles;
-  const bool two = p.qbits && !p.exact;  // rings of copies and of expanded blocks
-  const int stage_bytes = (two ? 0 : kAAtomBytes) + p.npad * 128 + p.qbits * kTileRows * kAtomK / 8;
-  // Expanded blocks: two leave more slots for the copies, which is worth more (int8, 4096 x 14336, 16 tokens, 2 / 4: 56.9 /
-  // 58.1 us; int4, 8192 x 24000, 24: 155 / 165), but four where a CTA has the SM to itself (int4, 2688 x 8000, 64: 67.2 /
-  // 65.7) and for 4-bit codes from 32 columns on, while four slots remain (8192 x 24000, 32: 255 / 252).
   const int room = (down_pairs(own, p.exact) ? 111 : 225) * 1024 - 1024 - 1024;
-  p.expand = !down_pairs(own, p.exact) || (p.qbits == 4 && own >= 32 && room - 4 * kAAtomBytes >= 4 * stage_bytes) ? kDownExpand : 2;
+  const int copies = p.npad * 128 + p.qbits * kTileRows * kAtomK / 8;  // of a stage: h, and the codes of quantised rows
+  auto slots = [&](int expand) {  // ring slots beside `expand` expanded blocks, or with a block each (0)
+    const int n = (room - expand * kAAtomBytes) / (copies + (expand ? 0 : kAAtomBytes));
+    return (n > 12 ? 12 : n) & (p.exact ? ~3 : ~1);
+  };
+  // Expanded blocks: two leave more slots for the copies, which is worth more (int8, 4096 x 14336, 16 tokens, 2 / 4: 56.9 / 58.1
+  // us), but four where a CTA has the SM to itself and four slots are left (int8, 4480 x 13000, 64 tokens, 6 slots: 114 / 110;
+  // 128 tokens, where they leave two slots: 147 / 167).
+  p.expand = !down_pairs(own, p.exact) && slots(kDownExpand) >= 4 ? kDownExpand : 2;
+  // One ring where it has six slots or no fewer than two rings would, and for 4-bit codes that are walked rather than gathered
+  // (from 32 tokens on) where it has four: nothing is left to gain, and a block for each slot keeps the expansion further ahead
+  // (one ring / two: int8, 4480 x 13000, 48 and 96 tokens 105.5 / 107.0 and 121.1 / 121.9 us; int4, 40 and 128 tokens 109.0 /
+  // 110.0 and 130.9 / 131.8; int4, 8192 x 18000, 32 tokens 152.7 / 156.4, but 24 tokens 131.6 / 124.7).
+  const bool two = p.qbits && !p.exact && slots(0) < 6 && slots(p.expand) > slots(0) &&
+                   !(p.qbits == 4 && p.B >= kWalkMinTokens && slots(0) >= 4);
   const int expanded = two ? p.expand * kAAtomBytes : 0;
-  int stages = (room - expanded) / stage_bytes;
-  if (stages > 12) stages = 12;
-  stages &= p.exact ? ~3 : ~1;
+  const int stage_bytes = copies + (two ? 0 : kAAtomBytes);
+  const int stages = slots(two ? p.expand : 0);
   if (stages < 2) return cudaErrorInvalidValue;
   p.stages = stages;
   const size_t smem = 1024 + expanded + (size_t)stages * stage_bytes + (3 * stages + 4 + 2 * kMaxIssuers + 2 * kDownExpand) * 8 + 64;
@@ -1937,6 +1947,9 @@ cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s) {
     return p.qbits == 8   ? launch_down_q<8, true>(p, g, smem, s, map_wg, map_wt, map_hm)
            : p.qbits == 4 ? launch_down_q<4, true>(p, g, smem, s, map_wg, map_wt, map_hm)
                           : launch_down_q<0, true>(p, g, smem, s, map_wg, map_wt, map_hm);
+  if (two)
+    return p.qbits == 8 ? launch_down_q<8, false, true>(p, g, smem, s, map_wg, map_wt, map_hm)
+                        : launch_down_q<4, false, true>(p, g, smem, s, map_wg, map_wt, map_hm);
   return p.qbits == 8   ? launch_down_q<8>(p, g, smem, s, map_wg, map_wt, map_hm)
          : p.qbits == 4 ? launch_down_q<4>(p, g, smem, s, map_wg, map_wt, map_hm)
                         : launch_down_q<0>(p, g, smem, s, map_wg, map_wt, map_hm);

@@ -292,3 +292,31 @@ def test_every_limb_of_every_column_arrives(D, qbits):
     assert ffn.device_status() == 0
     fires = (x[:, col] > 0).any(dim=0)
     assert torch.equal(ffn.last_active().cpu().long(), torch.nonzero(fires)[:, 0])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("qbits,D,H,B", [
+    (8, 4096, 9000, 16),    # two rings, two CTAs per SM
+    (8, 4096, 9000, 64),    # the same, four slots of copies
+    (8, 4224, 3000, 40),    # one ring: a CTA alone, six slots
+    (8, 4224, 3000, 64),    # two rings, four expanded blocks
+    (8, 4224, 3000, 96),    # one ring of four slots
+    (8, 4224, 3000, 128),   # two rings, two expanded blocks
+    (4, 4096, 9000, 24),    # two rings: gathered rows
+    (4, 4096, 9000, 40),    # one ring: every row
+    (4, 4224, 3000, 128),
+])
+def test_down_projection_of_codes_in_one_ring_and_two(qbits, D, H, B):
+    """Rings that wrap several times, against the single-token calls (a bf16 h in the batch where the width is even: 1e-2)."""
+    import paper_2609_31975_b200 as m
+
+    w = (syn.standard_ffn_q8 if qbits == 8 else syn.standard_ffn_q4)(D, H, 76, DEV, sparsity=0.4)
+    ffn = m.SparseFFN(D, H, torch.bfloat16, B_max=B)
+    x = syn.tokens(B, D, torch.bfloat16, 76, DEV)
+    call = ffn.sparse_ffn_forward_q8 if qbits == 8 else ffn.sparse_ffn_forward_q4
+    args = ({"W_g": w["W_g"]}, w["b_g"], w["W_up"], w["W_down"], "relu")
+    y = call(x, *args)
+    one = torch.stack([call(x[b], *args) for b in range(B)])
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0
+    assert ((y - one).norm(dim=1) / one.norm(dim=1)).max().item() < 1e-2
