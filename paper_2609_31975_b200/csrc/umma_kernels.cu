@@ -1955,9 +1955,12 @@ cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s) {
                         : launch_down_q<0>(p, g, smem, s, map_wg, map_wt, map_hm);
 }
 
-// Pairs of entries up to this many columns: groups of eight left a token of 256 columns to one warp (whole calls, 256 x 700, 4 /
-// 16 tokens, eights / pairs: int4 23.3 / 26.1 us -> 22.3 / 25.4).  Pairs up to 2048 are no faster.
-constexpr int kShortToken = 1024;
+// Pairs of entries up to this many columns: groups of eight leave a token of 256 columns to one warp (whole calls, 256 x 700, 4 /
+// 16 tokens, eights / pairs: int4 23.3 / 26.1 us -> 22.3 / 25.4; int8, 768 x 2300, 24 tokens 30.1 -> 29.6).  At 1024 columns pairs
+// are 512 threads, beside which an SM has no registers left for a CTA of the 4-bit gate (512 threads of 106), so that it starts
+// late where the grid needs that SM (int4, 1024 x 3000, 32 / 40 tokens, pairs / eights: 35.5 / 38.1 -> 34.4 / 37.1).  Longer tokens
+// want their threads nevertheless (256 at most instead of 512 at 4096 columns, 1024 at 8192: 1 to 2 % slower).
+constexpr int kShortToken = 768;
 cudaError_t launch_token_limbs(const void* x, int B, int K, int x_stride, void* limbs, float* scale, void* zero, int zero_bytes,
                                cudaStream_t s) {
   const bool pairs = K <= kShortToken;
