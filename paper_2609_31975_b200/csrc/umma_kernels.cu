@@ -334,7 +334,8 @@ __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.
 // whose second wave leaves most SMs idle: 24000 rows are 273 tiles of 88 rows, where 188 of 128 kept 40 of 148 SMs busy in the
 // second half (bf16, 5120 x 20000, 2 / 32 tokens: 80.7 / 155 -> 70.5 / 127 us; int4, 8192 x 24000, 64: 484 -> 339).  128
 // where a CTA owns more than two, for short rows (the LoPA gate), whose tiles are gone before the imbalance shows (r = 512 /
-// 1024: 0 to 1 % faster; r = 1536: equal tiles 1 to 3 % faster), and for most wide passes: bf16 rows against more than 128 tokens
+// 1024: 0 to 1 % faster; r = 1536, and int4 rows of 2048 codes, which are as many bytes as 512 bf16 elements: equal tiles 0 to 3 %
+// faster), and for most wide passes: bf16 rows against more than 128 tokens
 // are bound by the token rows that every tile reads through L2, and tiles of 128 are fewer.  There equal tiles pay only where
 // their stages are enough smaller for more of them in the ring (tiles of 128 / equal ones: 7168 x 20000, 200 tokens, 4 / 6 slots
 // 353 / 329 us, 160 tokens, 6 / 6 slots 270 / 287; 8192 x 20000, 256, 4 / 4: 414 / 474; 6144 x 24576, 200, 4 / 4: 324 / 345).
@@ -1815,9 +1816,9 @@ cudaError_t launch_rows_mode(const UmmaRowsParams& p, dim3 grid, size_t smem, cu
 // them: with tiles of up to 64 rows and K cut into runs all CTAs together read an eighth of that, and ranks below 8 rows per SM
 // fill the SMs too.  The next kernel adds the fp32 sums of the runs in their order; integer sums (limbs) are added in memory, so
 // that what cancels across runs leaves nothing behind and v has the bits of one run (as int4 of every run, added by the norm,
-// calls of r >= 1280 were 2 us longer: one SM read 130 KB).  Whole calls, 4096 x 14336, r = 512, 5 / 64 tokens, not cut / cut:
-// 47.8 / 93.8 -> 47.1 / 87.6 us (bf16), 8 / 64 tokens 49.8 / 108 -> 47.0 / 98.7 (int4); 8192 x 28672, r = 1024, 8 tokens:
-// 101 -> 96.5 (int8).
+// calls of r >= 1280 were 2 us longer: one SM read 130 KB).  Whole calls, power-law firing, not cut / cut: 4096 x 14336, r = 512,
+// 4 / 64 tokens, bf16 46.2 / 94.3 -> 44.5 / 86.8 us, int4 44.2 / 108 -> 42.1 / 97.7; 8192 x 28672, r = 1024, 8 tokens, int8
+// 101 -> 95.7.
 // Rows of up to kShortRow columns are cut from 16 tokens on: fewer hand little over, and the cut costs the norm more round trips
 // (1024 x 3000, r = 128, 2 / 8 / 16 / 64 tokens, not cut / cut: bf16 25.5 / 28.4 / 29.9 / 42.8 us against 26.4 / 28.5 / 30.0 / 41.3;
 // int4 29.6 / 32.9 / 36.4 / 56.6 against 29.8 / 32.6 / 35.4 / 55.5).  The runs differ by at most one block of K.

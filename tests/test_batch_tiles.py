@@ -82,8 +82,9 @@ def test_batches_over_two_equal_tiles(D, H, B, s):
 @pytest.mark.gpu
 @pytest.mark.parametrize("D", [256, 1280, 4096, 8192, 8448])
 def test_token_limbs_of_every_width(D):
-    """Widths below, at and above what the limb kernel's threads keep in registers: the batch against the single-token calls,
-    whose tokens go through other code (their error is 3e-5 of a group's largest entry, the batch's a bf16 h: 1e-2)."""
+    """Whole calls of several widths: the batch against the single-token calls, whose tokens go through other code (their error is
+    3e-5 of a group's largest entry, the batch's a bf16 h: 1e-2, which the third and fourth limb are far below; see
+    test_every_limb_of_every_column_arrives for these)."""
     import paper_2609_31975_b200 as m
 
     w = syn.standard_ffn_q8(D, 300, 72, DEV, sparsity=0.5)
@@ -138,8 +139,8 @@ def test_runs_of_columns_are_whole_and_fit_the_grid(sms, limbs):
 ])
 @pytest.mark.parametrize("q8", [False, True])
 def test_lopa_batches_with_v_from_several_runs_of_columns(D, r, B, q8):
-    """bf16: against the oracle.  int8: against the single-token calls, whose gate vector is summed elsewhere (fp32 sums on both
-    sides, a bf16 h in the batch: 1e-2)."""
+    """bf16: against the oracle.  int8: against the single-token calls, whose gate vector is summed elsewhere (a bf16 h in the batch:
+    1e-2; that the sums are exact is test_quantised_lopa_vectors_cut_into_runs_keep_integer_sums)."""
     import paper_2609_31975_b200 as m
 
     H = 600
