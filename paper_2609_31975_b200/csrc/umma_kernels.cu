@@ -341,14 +341,19 @@ __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.
 // 353 / 329 us, 160 tokens, 6 / 6 slots 270 / 287; 8192 x 20000, 256, 4 / 4: 414 / 474; 6144 x 24576, 200, 4 / 4: 324 / 345).
 constexpr int kShortRow = 1024;
 constexpr int kRowsSmem = 226 * 1024, kRingBytes = kRowsSmem - 1024 - kHeaderBytes;
-// token columns of a wide pass, else 0
-__host__ __device__ inline int wide_cols(int qbits, int B) { return qbits == 0 && B > 128 ? (B + 15) / 16 * 16 : 0; }
-__host__ __device__ inline int wide_slots(int tile_rows, int cols) { return kRingBytes / ((tile_rows + cols) * 128) & ~1; }
-__host__ __device__ inline int tile_rows_for(int n_rows, int grid, int K, int wide) {
+// The tallest tiles that two equal ones may be, else 128 (over rows of K elements, qbits as in UmmaRowsParams, B tokens).
+inline int equal_tiles_max(int K, int qbits, int B) {
+  if (K <= kShortRow) return 0;
+  if (qbits != 0 || B <= 128) return kTileRows;
+  const int cols = (B + 15) / 16 * 16;
+  auto slots = [&](int rows) { return kRingBytes / ((rows + cols) * 128) & ~1; };
+  return kRingBytes / (128 * (slots(kTileRows) + 2)) - cols;
+}
+__host__ __device__ inline int tile_rows_for(int n_rows, int grid, int equal_max) {
   const int per_cta = n_rows > kTileRows * grid ? 2 : 1;
-  if (n_rows > 2 * kTileRows * grid || (per_cta == 2 && K <= kShortRow)) return kTileRows;
-  int t = ((n_rows + per_cta * grid - 1) / (per_cta * grid) + 7) & ~7;
-  if (per_cta == 2 && wide && wide_slots(t, wide) <= wide_slots(kTileRows, wide)) return kTileRows;
+  if (n_rows > 2 * kTileRows * grid) return kTileRows;
+  const int t = ((n_rows + per_cta * grid - 1) / (per_cta * grid) + 7) & ~7;
+  if (per_cta == 2 && t > equal_max) return kTileRows;
   return t < 8 ? 8 : t > kTileRows ? kTileRows : t;
 }
 
@@ -584,7 +589,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
   const bool walk_all = MODE == kUpMayWalk && own_list && p.walk_all &&
                         (long long)n_listed * 100 >= (long long)p.R * kWalkAllPercent;
   if (walk_all) n_rows = p.R;
-  const int tile_rows = tile_rows_for(n_rows, gridDim.x, p.K, wide_cols(QB, p.B));
+  const int tile_rows = tile_rows_for(n_rows, gridDim.x, p.equal_max);
   const int n_tiles = (n_rows + tile_rows - 1) / tile_rows;
   if (own_list && walk_all) {
     // publish the list only: word w is written out by CTA w mod grid
@@ -1688,7 +1693,7 @@ __global__ void __launch_bounds__(ONE ? kVecThreads : kVecMaxThreads) rmsnorm_li
 // Tiling of the gate GEMM over R rows (the up kernel needs it to read the gate's bit masks).
 void umma_gate_tiling(int R, int K, int qbits, int B, int sm_count, int* tile_rows, int* n_tiles) {
   const int grid = R < 8 * sm_count ? (R + 7) / 8 : sm_count;
-  *tile_rows = tile_rows_for(R, grid, K, wide_cols(qbits, B));
+  *tile_rows = tile_rows_for(R, grid, equal_tiles_max(K, qbits, B));
   *n_tiles = (R + *tile_rows - 1) / *tile_rows;
 }
 
@@ -1844,6 +1849,7 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
   const int splits = p.k_splits > 1 ? p.k_splits : 1;
   if (splits > 1 && (up || p.exact || p.b_g || p.g_idx || p.flag || p.words_out || p.act != kUmmaActIdentity)) return cudaErrorInvalidValue;
   const int kb = p.K / (p.qbits == 1 || p.qbits == 2 ? 128 : kAtomK);
+  p.equal_max = equal_tiles_max(p.K, p.qbits, p.B);
   p.run_blocks = kb / splits;
   p.longer_runs = kb % splits;
   const int grid = splits > 1 ? p.k_tiles : p.R < 8 * sm_count ? (p.R + 7) / 8 : sm_count;
@@ -1856,7 +1862,7 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
   if (p.npad > kUmmaMaxCols) return cudaErrorInvalidValue;
   if (i8 && (p.K % 128 || !p.tok_scale)) return cudaErrorInvalidValue;
   // weights: all R rows; boxes of one tile's rows for the gate, single-row boxes for the gather
-  if (!make_weight_map(&map_w, p.W, p.K, p.R, up ? 1 : tile_rows_for(p.R, grid, p.K, wide_cols(p.qbits, p.B)), p.qbits)) return cudaErrorNotSupported;
+  if (!make_weight_map(&map_w, p.W, p.K, p.R, up ? 1 : tile_rows_for(p.R, grid, p.equal_max), p.qbits)) return cudaErrorNotSupported;
   // tokens: only the rows that exist; the box covers npad rows and the rest reads as zero
   if (i8 ? !make_map_i8(&map_x, p.X, p.K, p.ncols_valid, (size_t)p.x_stride, p.npad)
                    : !make_map(&map_x, p.X, p.K, p.ncols_valid, (size_t)p.x_stride, p.npad))
@@ -1866,7 +1872,7 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
     // wide batches: the union may cover most rows; the kernel then walks every row with tiled boxes of the tile
     // height of R rows (decided on the device from the union's size, so it depends on this call's inputs only)
     WalkMap<true> map_t;
-    if (!make_weight_map(&map_t.m, p.W, p.K, p.R, tile_rows_for(p.R, grid, p.K, wide_cols(p.qbits, p.B)), p.qbits)) return cudaErrorNotSupported;
+    if (!make_weight_map(&map_t.m, p.W, p.K, p.R, tile_rows_for(p.R, grid, p.equal_max), p.qbits)) return cudaErrorNotSupported;
     return launch_rows_mode<kUpMayWalk>(p, dim3(grid), smem, s, map_w, map_x, map_t);
   }
   return launch_rows_mode<kUp>(p, dim3(grid), smem, s, map_w, map_x, WalkMap<false>{});
@@ -1916,9 +1922,13 @@ cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s) {
   p.wait_cycles = fused_test_knobs().wait_cycles;
   const int room = (down_pairs(own, p.exact) ? 111 : 225) * 1024 - 1024 - 1024;
   const int copies = p.npad * 128 + p.qbits * kTileRows * kAtomK / 8;  // of a stage: h, and the codes of quantised rows
+  // Codes: no more slots than a CTA has blocks of 64 rows, so that narrow models, whose many splits get a block or two, keep
+  // one ring (the second one's barriers and hand-overs: 0.3 us of 6.3 at 256 columns).
+  const int blocks = ((p.R + kAtomK - 1) / kAtomK + p.splits - 1) / p.splits;
+  const int most = !p.qbits || p.exact || blocks > 12 ? 12 : (blocks + 1) & ~1;
   auto slots = [&](int expand) {  // ring slots beside `expand` expanded blocks, or with a block each (0)
     const int n = (room - expand * kAAtomBytes) / (copies + (expand ? 0 : kAAtomBytes));
-    return (n > 12 ? 12 : n) & (p.exact ? ~3 : ~1);
+    return (n > most ? most : n) & (p.exact ? ~3 : ~1);
   };
   // Expanded blocks: two leave more slots for the copies, which is worth more (int8, 4096 x 14336, 16 tokens, 2 / 4: 56.9 / 58.1
   // us), but four where a CTA has the SM to itself and four slots are left (int8, 4480 x 13000, 64 tokens, 6 slots: 114 / 110;
@@ -1935,7 +1945,11 @@ cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s) {
   const int stages = slots(two ? p.expand : 0);
   if (stages < 2) return cudaErrorInvalidValue;
   p.stages = stages;
-  const size_t smem = 1024 + expanded + (size_t)stages * stage_bytes + (3 * stages + 4 + 2 * kMaxIssuers + 2 * kDownExpand) * 8 + 64;
+  size_t smem = 1024 + expanded + (size_t)stages * stage_bytes + (3 * stages + 4 + 2 * kMaxIssuers + 2 * kDownExpand) * 8 + 64;
+  // Never so little that an SM takes more CTAs than its TMEM has room for: they would wait for it (int8, 640 x 1408, 87 tokens:
+  // 36.5 -> 39.8 us).
+  const size_t least = (down_pairs(own, p.exact) ? 80 : 120) * 1024;
+  if (smem < least) smem = least;
   const int grid = (p.D / kTileRows) * p.splits;
   alignas(64) CUtensorMap map_wg, map_wt, map_hm;
   // W_down [H, D]: inner dimension d; single-row boxes for the gather, 64-row boxes for the dense walk

@@ -49,7 +49,7 @@ struct UmmaRowsParams {
   float* a_out;          // GATE: gate values a_out[b * a_stride + j]
   int k_splits, k_tiles; // GATE, raw products only (0: not cut): runs of K and tiles of rows (umma_k_splits); run i writes
   size_t split_stride;   //   at a_out + i * split_stride; limbs (qbits = 1 / 2): all add their integers to rows 4 b + l of a_out
-  int run_blocks, longer_runs;  // filled by the launcher
+  int run_blocks, longer_runs, equal_max;  // filled by the launcher
   uint8_t* flag;         // GATE: [R] any token fires, or null
   uint32_t* words_out;   // GATE: the same as bit masks, word 4 * tile + epilogue warp, or null
   const float* a;        // UP: gate values
