@@ -36,6 +36,11 @@ constexpr int kActSilu = 4;  // z * sigmoid(z) on both sides: only ever A_3 on t
 // compare and a max per element instead of a speculated exponential and division.
 static __device__ __noinline__ float rsplus_of_nonnegative(float p) { return p / (1.f + __expf(-p)); }
 
+// Four at once, so that their exponentials and divisions overlap.
+static __device__ __noinline__ float4 rsplus4_of_nonnegative(float4 p) {
+  return make_float4(p.x / (1.f + __expf(-p.x)), p.y / (1.f + __expf(-p.y)), p.z / (1.f + __expf(-p.z)), p.w / (1.f + __expf(-p.w)));
+}
+
 __device__ __forceinline__ float activation(int act, float z) {
   if (act == kActNone) return z;
   if (act == kActSilu) return rsplus_of_nonnegative(z);  // the same expression on the whole axis (-0 for z -> -inf)
@@ -43,6 +48,29 @@ __device__ __forceinline__ float activation(int act, float z) {
   if (act == kActRelu) return p;
   if (act == kActSqRelu) return p * p;
   return rsplus_of_nonnegative(p);               // R-S+: z * sigmoid(z) on the non-negative side, 0 at 0
+}
+
+// The same for the first n of N values (and what shares a group of four with them), the choice made once.
+template <int N>
+__device__ __forceinline__ void activate(int act, float* z, int n) {
+  static_assert(N % 4 == 0, "fours");
+  if (act == kActNone) return;
+  if (act != kActSilu) {
+#pragma unroll
+    for (int q = 0; q < N; ++q) z[q] = fmaxf(z[q], 0.f);
+  }
+  if (act == kActRelu) return;
+  if (act == kActSqRelu) {
+#pragma unroll
+    for (int q = 0; q < N; ++q) z[q] = z[q] * z[q];
+  } else {
+#pragma unroll
+    for (int q = 0; q < N; q += 4) {
+      if (q >= n) break;
+      const float4 r = rsplus4_of_nonnegative(make_float4(z[q], z[q + 1], z[q + 2], z[q + 3]));
+      z[q] = r.x; z[q + 1] = r.y; z[q + 2] = r.z; z[q + 3] = r.w;
+    }
+  }
 }
 
 // Element traits: 16-byte vectors of the storage type, unpacked to fp32.

@@ -207,6 +207,46 @@ __device__ __forceinline__ void tmem_ld8_int(uint32_t taddr, int nacc, int strid
   }
 }
 
+// 16 int32 columns of this thread's lane, summed over the accumulators.
+__device__ __forceinline__ void tmem_ld16_int(uint32_t taddr, int nacc, int stride, int* v) {
+  uint32_t r[16];
+  tmem_ld8_raw(taddr, r);
+  tmem_ld8_raw(taddr + 8, r + 8);
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = (int)r[i];
+#pragma unroll 1
+  for (int a = 1; a < nacc; ++a) {
+    tmem_ld8_raw(taddr + a * stride, r);
+    tmem_ld8_raw(taddr + a * stride + 8, r + 8);
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] += (int)r[i];
+  }
+}
+
+// Loads (0 where `on` is false) and stores that a predicate turns off: the epilogues' straight-line code has a dozen of them, and
+// a branch around each costs more than the access.
+__device__ __forceinline__ float ld_f32_if(const float* p, bool on) {
+  float v;
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\tmov.f32 %0, 0f00000000;\n\t@p ld.global.f32 %0, [%1];\n\t}"
+               : "=f"(v) : "l"(p), "r"((uint32_t)on) : "memory");
+  return v;
+}
+__device__ __forceinline__ float ld_bf16_if(const __nv_bfloat16* p, bool on) {
+  uint16_t v;
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\tmov.b16 %0, 0;\n\t@p ld.global.u16 %0, [%1];\n\t}"
+               : "=h"(v) : "l"(p), "r"((uint32_t)on) : "memory");
+  return __uint_as_float((uint32_t)v << 16);
+}
+__device__ __forceinline__ void st_f32_if(float* p, float v, bool on) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.global.f32 [%0], %1;\n\t}" ::"l"(p), "f"(v), "r"((uint32_t)on) : "memory");
+}
+__device__ __forceinline__ void st_bf16_if(__nv_bfloat16* p, __nv_bfloat16 v, bool on) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.global.b16 [%0], %1;\n\t}" ::"l"(p), "h"(__bfloat16_as_ushort(v)), "r"((uint32_t)on)
+               : "memory");
+}
+
 // What the products with a token's four limbs (most significant first, 7 bits apart) amount to: i0 + i1 / 128 + i2 / 128^2 +
 // i3 / 128^3.
 __device__ __forceinline__ float limb_sum(int i0, int i1, int i2, int i3) {
@@ -713,20 +753,30 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
     const float sc = ((kQ && row_ok && p.w_scale) ? p.w_scale[j] : 1.f) * (QB == 2 ? 0.0625f : 1.f);  // scale of the weight row
     const float osc = (kQ && UP && row_ok && p.out_scale) ? p.out_scale[j] : 1.f;  // scale of the down row, folded into Hm
     int gi = -1;
-    float pre[16];  // union rows: the gate values of this thread's first two column groups
-    if (UP) {
-#pragma unroll
-      for (int g = 0; g < 2; ++g)
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int b = 8 * (part + g * nparts) + q;
-          pre[8 * g + q] = (row_ok && b < B) ? p.a[(size_t)b * p.a_stride + j] : 0.f;
-        }
-    } else {
+    if (!UP) {
       bias = (row_ok && p.b_g) ? p.b_g[j] : 0.f;
       gi = (row_ok && p.g_idx) ? p.g_idx[j] : -1;
       sg = (row_ok && p.g_sign && p.g_sign[j] < 0) ? -1.f : 1.f;
     }
+    // What a step of the loops below (kStep tokens) needs of each token beside its sums: gate value (union rows) or fixed-matrix
+    // entry (gate), and the scale of its limbs.  Two steps are always under way: with the loads where they are used a step waited
+    // for each of them in turn.
+    constexpr int kStep = kNat ? 4 : 8;
+    const __nv_bfloat16* xg = static_cast<const __nv_bfloat16*>(p.xtok) + (gi >= 0 ? gi : 0);
+    struct Pre { float e[kStep], ts[kNat ? kStep : 1]; };
+    auto fetch = [&](int b0) -> Pre {
+      Pre w;
+#pragma unroll
+      for (int q = 0; q < kStep; ++q) {
+        const int b = b0 + q;
+        if (UP) w.e[q] = ld_f32_if(p.a + (size_t)b * p.a_stride + j, row_ok && b < B);
+        else w.e[q] = ld_bf16_if(xg + (size_t)b * p.xtok_stride, gi >= 0 && b < B);
+        if (kNat) w.ts[q] = ld_f32_if(p.tok_scale + b, b < B);
+      }
+      return w;
+    };
+    const int b_first = kStep * part, b_step = kStep * nparts;
+    Pre now = fetch(b_first), next = fetch(b_first + b_step);
     int okw = 1;
     if (!shared || (warp >= 4 && warp < 8)) {
       if (lane == 0) okw = mbar_wait(acc_full, tcount & 1, abort_flag, p.status, p.wait_cycles) ? 1 : 0;
@@ -739,20 +789,8 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
     }
     if (!okw) return false;
     tc_fence_after();
-    // h of one (neuron, token): one bf16 value, or (quantised rows of some widths) two that add up to 16 bits of it
-    auto store_h = [&](__nv_bfloat16* dst, float h) {
-      if (kQ && p.h_terms == 2) {
-        *dst = take_bf16(h);
-        dst[(size_t)p.h_cols * p.hm_stride] = __float2bfloat16(h);
-      } else {
-        *dst = __float2bfloat16(h);
-      }
-    };
     if constexpr (kNat) {
       // int32 accumulators, four columns per token (its limbs): value = token scale * row scale * their sum
-      __nv_bfloat16* hm = static_cast<__nv_bfloat16*>(p.hmT) + li;
-      float* arow = a_out + j;
-      const __nv_bfloat16* xg = static_cast<const __nv_bfloat16*>(p.xtok) + (gi >= 0 ? gi : 0);
       if (kSplits && p.k_splits > 1) {  // a run of K: added to the integer sums of the others, in whatever order
 #pragma unroll 1
         for (int c0 = 8 * part; c0 < npad; c0 += 8 * nparts) {
@@ -765,71 +803,63 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
         }
         return true;
       }
-      for (int c0 = 8 * part; c0 < npad; c0 += 8 * nparts) {
-        int iv[8];
-        tmem_ld8_int(taddr + c0, nacc, npad, iv);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int b = c0 / 4 + q;
-          if (row_ok && b < B) {
-            const float val = p.tok_scale[b] * sc * limb_sum(iv[4 * q], iv[4 * q + 1], iv[4 * q + 2], iv[4 * q + 3]);
-            if (UP) {
-              const float av = p.a[(size_t)b * p.a_stride + j];
-              hm[(size_t)b * p.hm_stride] = __float2bfloat16(av * activation(p.act_up, val) * osc);
-            } else {
-              float z = val + bias;
-              if (gi >= 0) z += sg * __bfloat162float(xg[(size_t)b * p.xtok_stride]);
-              fired |= z > 0.f;
-              arow[(size_t)b * p.a_stride] = activation(p.act, z);
-            }
-          }
-        }
-      }
-      return true;
     }
-    if (UP) {
-      __nv_bfloat16* hm = static_cast<__nv_bfloat16*>(p.hmT) + li;
-      const float* arow = p.a + j;
-      const int act_up = p.act_up;
-      int g = 0;
-      for (int c0 = 8 * part; c0 < npad; c0 += 8 * nparts, ++g) {
-        float av[8];
+    // Bound by instruction issue: three warps a scheduler, and code that is fetched anew by every launch.  A step's tokens go
+    // through straight-line code, accesses predicated and the activation chosen once for all of them: with a branch around each
+    // token a step of eight took 1640 cycles (4096 x 14336, 200 tokens, bf16, after the last MMA of the gate / up kernel: 8.6 / 8.0
+    // us, now 5.6 / 5.2; int8, 64 tokens: 4.9 / 7.0 -> 2.9 / 2.6; whole calls 129 -> 123, 88.5 -> 80.7).  Steps of 16 and of 4
+    // bf16 tokens are slower (whole calls of 4096 x 14336, 24 / 200 tokens, 16 / 8 / 4: 70.1 / 68.0 / 68.7, 134 / 127 / 129).
+#pragma unroll 1
+    for (int b0 = b_first; b0 < B; b0 += b_step) {
+      float v[kStep];
+      if constexpr (kNat) {
+        int iv[16];
+        tmem_ld16_int(taddr + 4 * b0, nacc, npad, iv);
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          av[q] = g == 0 ? pre[q] : g == 1 ? pre[8 + q] : (row_ok && c0 + q < B) ? arow[(size_t)(c0 + q) * p.a_stride] : 0.f;
-        float v[8];
-        tmem_ld8(taddr + c0, nacc, npad, v);
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (row_ok && c0 + q < B)
-            store_h(hm + (size_t)(c0 + q) * p.hm_stride,
-                    fired_part(av[q], kQ ? av[q] * activation(act_up, v[q] * sc) * osc : av[q] * activation(act_up, v[q])));
-      }
-    } else {
-      const int act = p.act;
-      float* arow = a_out + j;
-      const __nv_bfloat16* xg = static_cast<const __nv_bfloat16*>(p.xtok) + (gi >= 0 ? gi : 0);
-      // LoPA: a token's vector is the sum of two bf16 vectors (columns b and x_cols + b), whose products are added here
-      const int cols = p.x_cols ? p.x_cols : npad;
-      for (int c0 = 8 * part; c0 < cols; c0 += 8 * nparts) {
-        float v[8];
-        tmem_ld8(taddr + c0, nacc, npad, v);
-        if (p.x_cols) {
+        for (int q = 0; q < kStep; ++q) v[q] = now.ts[q] * sc * limb_sum(iv[4 * q], iv[4 * q + 1], iv[4 * q + 2], iv[4 * q + 3]);
+      } else {
+        tmem_ld8(taddr + b0, nacc, npad, v);
+        if (!UP && p.x_cols) {  // LoPA: a token's vector is the sum of two bf16 vectors (columns b and x_cols + b)
           float w[8];
-          tmem_ld8(taddr + p.x_cols + c0, nacc, npad, w);
+          tmem_ld8(taddr + p.x_cols + b0, nacc, npad, w);
 #pragma unroll
           for (int q = 0; q < 8; ++q) v[q] += w[q];
         }
+      }
+      const Pre w = now;
+      now = next;
+      next = fetch(b0 + 2 * b_step);
+      if (UP) {
+        if (kQ && !kNat) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int b = c0 + q;
-          if (row_ok && b < B) {
-            float z = kQ ? v[q] * sc + bias : v[q] + bias;
-            if (gi >= 0) z += sg * __bfloat162float(xg[(size_t)b * p.xtok_stride]);
-            fired |= z > 0.f;
-            arow[(size_t)b * p.a_stride] = activation(act, z);
+          for (int q = 0; q < kStep; ++q) v[q] *= sc;
+        }
+        activate<kStep>(p.act_up, v, B - b0);
+        __nv_bfloat16* hm = static_cast<__nv_bfloat16*>(p.hmT) + (size_t)b0 * p.hm_stride + li;
+#pragma unroll
+        for (int q = 0; q < kStep; ++q) {
+          float h = kQ ? w.e[q] * v[q] * osc : w.e[q] * v[q];
+          if (!kNat) h = fired_part(w.e[q], h);
+          const bool on = row_ok && b0 + q < B;
+          // one bf16 value, or (quantised rows of some widths) two that add up to 16 bits of h
+          if (kQ && !kNat && p.h_terms == 2) {
+            st_bf16_if(hm + (size_t)q * p.hm_stride, take_bf16(h), on);
+            st_bf16_if(hm + (size_t)(p.h_cols + q) * p.hm_stride, __float2bfloat16(h), on);
+          } else {
+            st_bf16_if(hm + (size_t)q * p.hm_stride, __float2bfloat16(h), on);
           }
         }
+      } else {
+#pragma unroll
+        for (int q = 0; q < kStep; ++q) {
+          v[q] = kQ && !kNat ? v[q] * sc + bias : v[q] + bias;
+          v[q] = gi >= 0 ? v[q] + sg * w.e[q] : v[q];
+          fired |= (b0 + q < B) & (v[q] > 0.f);
+        }
+        activate<kStep>(p.act, v, B - b0);
+        float* arow = a_out + (size_t)b0 * p.a_stride + j;
+#pragma unroll
+        for (int q = 0; q < kStep; ++q) st_f32_if(arow + (size_t)q * p.a_stride, v[q], row_ok && b0 + q < B);
       }
     }
     return true;
