@@ -404,7 +404,7 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
   // (and publishes list and length): no byte flags, no compaction launch.
   const bool own_list = umma && !dense && umma_own_list_supported(H, lopa ? g->r : D, wq_rows, B, h->sm_count);
   uint32_t* words = reinterpret_cast<uint32_t*>(flag);  // the flag buffer holds either form
-  int gate_tile_rows = 0, gate_tiles = 0;
+  int gate_tile_rows = 0, gate_tiles = 0, gate_rows_per_word = 32;
   umma_gate_tiling(H, lopa ? g->r : D, wq_rows, B, h->sm_count, &gate_tile_rows, &gate_tiles);
   void* x2 = h->ws + h->L.x2;
   if (umma) {
@@ -440,6 +440,7 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
       p.W = g->W_g; p.K = D; p.X = x; p.x_stride = D;
     }
     p.ncols_valid = cols;
+    gate_rows_per_word = umma_gate_rows_per_word(p.R, p.K, p.qbits, B, cols, exact, h->sm_count);
     SFFN_CUDA(launch_umma_rows(false, p, cols, h->sm_count, s));
   } else {
     RowsMmaParams p{};
@@ -481,7 +482,7 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
     p.qbits = wq_rows; p.w_scale = q8 ? q8->s_up : nullptr; p.out_scale = q8 ? q8->s_down : nullptr;
     if (own_list) {
       p.words_in = words; p.n_words = 4 * gate_tiles; p.gate_tile_rows = gate_tile_rows;
-      p.gate_rows_per_word = gate_tile_rows <= 64 ? 16 : 32;
+      p.gate_rows_per_word = gate_rows_per_word;
       p.idx_out = idx; p.count_out = count; p.walk_all = may_walk ? count + 1 : nullptr;
     } else {
       p.idx = lidx; p.count = lcount;

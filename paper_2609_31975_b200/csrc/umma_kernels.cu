@@ -34,9 +34,9 @@
 // the tensor core takes 32 bytes of bf16 per cycle and SM whatever the token count, i.e. 16 codes per cycle:
 // quantised batches are bound by that rate, not by their bytes.
 // Up to 256 token columns go through in one pass.  Wide batches (npad > 128) leave room for two accumulators and a ring
-// of four stages of ~40 KB (two with expanded codes and 241 columns or more); they are bound by the token rows every CTA reads again (200 tokens x 4096: 1.6 MB a CTA
-// through L2 beside 0.8 MB of weights), still far cheaper than further passes over the weights (200 tokens, 4096 x
-// 14336, bf16: 137 us in one pass against 333 us in four of at most 64).
+// of four stages of ~40 KB (two with expanded codes and 241 columns or more), too few for the token rows that every CTA reads again
+// (200 tokens x 4096: 1.6 MB a CTA through L2 beside 0.8 MB of weights).  There the rows kernels run in pairs of CTAs that hold half
+// of the token rows each (PAIR, see rows_pairs): 200 tokens, 4096 x 14336, bf16: 112 us in one pass, 130 without pairs.
 // Every wait is bounded by a cycle budget; on expiry the status word is set, all roles wind down and the TMEM
 // columns are released before the CTA exits.
 #include "umma_kernels.cuh"
@@ -160,6 +160,49 @@ __device__ __forceinline__ void umma_i8(uint32_t tmem_d, uint64_t adesc, uint64_
       ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// The same three for a pair of CTAs (cta_group::2): one thread of the even CTA issues for both.  A's rows m and m + 128 and B's
+// columns n and n + N / 2 are in the two CTAs' shared memory at the same offsets, accumulator rows m and m + 128 in their TMEM;
+// the commit arrives at the barrier of that offset in both.
+__device__ __forceinline__ void umma_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+__device__ __forceinline__ void umma_pair_i8(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::i8 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+               "h"((uint16_t)3)
+               : "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The address, in the cluster's window, of this CTA's shared-memory address in the CTA of rank `rank`.
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
@@ -261,6 +304,21 @@ __device__ __forceinline__ void tma_tile_2d(uint32_t dst, const CUtensorMap* map
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
       "l"(map), "r"(c0), "r"(c1), "r"(bar)
+      : "memory");
+}
+// The same, and the gather below, for a CTA of a pair: `bar` may be the other CTA's.
+__device__ __forceinline__ void tma_tile_2d_pair(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+      "l"(map), "r"(c0), "r"(c1), "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void tma_gather4_pair(uint32_t dst, const CUtensorMap* map, int c0, int r0, int r1, int r2,
+                                                 int r3, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
+      "%3, %4, %5, %6}], [%7];" ::"r"(dst),
+      "l"(map), "r"(c0), "r"(r0), "r"(r1), "r"(r2), "r"(r3), "r"(bar)
       : "memory");
 }
 // Gather copy: four rows r0..r3 (any order) x 64 elements starting at element c0 land as four
@@ -497,12 +555,13 @@ __device__ __forceinline__ bool named_bar_any(int id, int threads, bool v) {
 
 enum RowsMode { kGate = 0, kUp = 1, kUpMayWalk = 2 };  // kUpMayWalk: wide batches, see walk_all below
 
-template <int MODE, int QB, bool EX = false>
+template <int MODE, int QB, bool EX = false, bool PAIR = false>
 __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || QB == 4 || QB == 2) ? 32 * kExpandWarps : 0), 1) umma_rows_kernel(const UmmaRowsParams p,
                                                                   const __grid_constant__ CUtensorMap map_w,
                                                                   const __grid_constant__ CUtensorMap map_x,
                                                                   const __grid_constant__ WalkMap<MODE == kUpMayWalk> map_t) {
   constexpr bool UP = MODE != kGate;
+  static_assert(!(EX && PAIR) && (!PAIR || QB <= 1), "pairs: bf16 rows, or int8 rows against limbs");
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   // carve: stages first (1024-byte aligned), then barriers and control words
   const int npad = p.npad;
@@ -528,10 +587,12 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
   constexpr int kAtomElems = kNat ? 128 : kAtomK;              // elements of one 128-byte swizzle row
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // PAIR: the pair's CTAs go through their tiles together (the second one's last tile may not exist); `first` is the even CTA
+  const int rank = PAIR ? (int)cluster_rank() : 0, first = (int)blockIdx.x - rank;
   // Gate mode: a second grid dimension cuts K into runs of blocks (see umma_k_splits), the first `longer_runs` of them one block
   // longer; each writes sums of its own, or adds its own to the others'.  (Not a mode of its own: the gate that follows V x finds
   // its code in the caches, without which calls of bf16 rows take 1 us more.)
-  constexpr bool kSplits = MODE == kGate && !EX;
+  constexpr bool kSplits = MODE == kGate && !EX && !PAIR;
   const int kb_first = kSplits ? (int)blockIdx.y * p.run_blocks + min((int)blockIdx.y, p.longer_runs) : 0;
   const int kblocks = kSplits ? p.run_blocks + ((int)blockIdx.y < p.longer_runs) : p.K / kAtomElems;
   float* const a_out = p.a_out + (kSplits ? (size_t)blockIdx.y * p.split_stride : 0);
@@ -559,16 +620,21 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
         mbar_init(place_full + 8 * q, 1);
         mbar_init(place_empty + 8 * q, 8);  // one arrival per epilogue warp
       }
-    mbar_init(acc_empty, 128);
+    mbar_init(acc_empty, PAIR ? 256 : 128);
     *abort_flag = 0;
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_w) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
   }
   if (warp == 8) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(tmem_cols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (PAIR) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(tmem_cols)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(tmem_cols)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   // The up kernel needs the gate's results from here on.  The gate kernel's tiles depend on nothing but its
   // own arguments, and its weights are parameters: its producers fill the ring before they wait (see below),
@@ -577,7 +643,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
 
   // Union rows: either the list is given (idx, count), or every CTA compacts the gate's "fired" bit masks
   // itself.  The gate kernel leaves one 32-bit word per epilogue warp and tile (word 4 * tile + warp, bit =
-  // lane = row rows_per_word * warp + lane of the tile, 32 rows per word for M = 128 tiles, 16 for M = 64); thread t takes word t of each chunk of `threads` words, a
+  // lane = row rows_per_word * warp + lane of the tile, 32 rows per word for M = 128 tiles and pairs, 16 for M = 64); thread t takes word t of each chunk of `threads` words, a
   // warp scan plus the warp totals of all chunks give the list position of its first set bit.
   const bool own_list = UP && p.words_in != nullptr;
   uint32_t bits[kScanChunks];
@@ -687,12 +753,12 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
   // not shrink with the tile -- followed by the token rows of the same K blocks.  Block a sits tile_rows * 128
   // bytes after block a - 1; its MMA reads M rows from its start, i.e. on into the following blocks and the
   // token rows of the same stage (rows that are ignored); the stage is sized so that it never reads past it.
-  const bool m64 = tile_rows <= 64;
+  const bool m64 = !PAIR && tile_rows <= 64;
   const int mrows = m64 ? 64 : kTileRows;
   int atoms = kTileRows / tile_rows;
   const int atoms_cap = npad <= 16 ? 4 : npad <= 32 ? 2 : 1;  // at most 8 KB of token rows per stage
   atoms = atoms > atoms_cap ? atoms_cap : atoms;
-  const int a_block_bytes = tile_rows * 128, b_block_bytes = npad * 128;
+  const int a_block_bytes = tile_rows * 128, b_cols = PAIR ? npad / 2 : npad, b_block_bytes = b_cols * 128;
   // bytes of the bf16 weight blocks of a stage, including what the last block's MMA reads past its rows
   const int a_bytes = (max(atoms * a_block_bytes, (atoms - 1) * a_block_bytes + mrows * 128) + 1023) & ~1023;
   const int raw_block_bytes = tile_rows * kRawRow;
@@ -727,7 +793,8 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   tc_fence_before();
-  __syncthreads();
+  if constexpr (PAIR) cluster_sync();  // the other CTA's barriers are initialised too
+  else __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
@@ -946,8 +1013,16 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
     // which a parity wait could not tell from "ready".  Lane 0 waits for the slot and announces the byte
     // count, then the copies go out: one tiled copy for the tile's consecutive rows (gate), or one
     // gather4 per lane for four listed rows each (union rows); the token block is one more tiled copy.
-    const int my_tiles = (int)blockIdx.x < n_tiles ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    const int my_tiles = first < n_tiles ? (n_tiles - 1 - first) / (int)gridDim.x + 1 : 0;
     const int total = my_tiles * kstages;
+    auto copy_tile = [&](uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
+      if constexpr (PAIR) tma_tile_2d_pair(dst, map, c0, c1, bar);
+      else tma_tile_2d(dst, map, c0, c1, bar);
+    };
+    auto copy_gather = [&](uint32_t dst, int c0, const int* r, uint32_t bar) {
+      if constexpr (PAIR) tma_gather4_pair(dst, &map_w, c0, r[0], r[1], r[2], r[3], bar);
+      else tma_gather4(dst, &map_w, c0, r[0], r[1], r[2], r[3], bar);
+    };
     // Stages [it0, it1) of this CTA's sequence; with_w / with_x say which of the two operands are copied.  A
     // stage is armed (slot waited for, byte count announced) together with its weight copy.
     auto produce = [&](int it0, int it1, bool with_w, bool with_x) -> bool {
@@ -960,7 +1035,9 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
         if ((s & (kProducerWarps - 1)) != warp) continue;
         const int tile = blockIdx.x + tl * gridDim.x;
         const int na = min(atoms, kblocks - kb * atoms);
-        const uint32_t tx_bytes = kExp ? (uint32_t)(na * (tile_rows * kRawRow + npad * 128)) : (uint32_t)(na * (tile_rows + npad)) * 128;
+        // PAIR: the bytes of both CTAs, whose copies complete on the even one's barrier
+        const uint32_t tx_bytes = (PAIR ? 2 : 1) * (kExp ? (uint32_t)(na * (tile_rows * kRawRow + b_cols * 128)) : (uint32_t)(na * (tile_rows + b_cols)) * 128);
+        const uint32_t bar = PAIR ? map_rank(full + 8 * s, 0) : full + 8 * s;
         if (UP && !walk_all && tl != rows_of) {
           rows_of = tl;
 #pragma unroll
@@ -976,7 +1053,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
           int ok = 1;
           if (lane == 0) {
             ok = mbar_wait(empty + 8 * s, ph ^ 1, abort_flag, p.status, p.wait_cycles) ? 1 : 0;
-            if (ok) mbar_expect_tx(full + 8 * s, tx_bytes);
+            if (ok && rank == 0) mbar_expect_tx(full + 8 * s, tx_bytes);
           }
           ok = __shfl_sync(0xffffffffu, ok, 0);
           if (!ok) return false;
@@ -991,14 +1068,14 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
           if (with_w && !(MODE == kGate && blockIdx.x == 0 && it == p.drop_stage)) {  // test hook: a copy that never comes
             if (UP && !walk_all) {
               if (lane * 4 < tile_rows)
-                tma_gather4(wdst + lane * 4 * wrow, &map_w, wc0, r[0], r[1], r[2], r[3], full + 8 * s);
+                copy_gather(wdst + lane * 4 * wrow, wc0, r, bar);
             } else if (UP) {
-              if (lane == 0) tma_tile_2d(wdst, map_t.get(), wc0, tile * tile_rows, full + 8 * s);
+              if (lane == 0) copy_tile(wdst, map_t.get(), wc0, tile * tile_rows, bar);
             } else if (lane == 0) {
-              tma_tile_2d(wdst, &map_w, wc0, tile * tile_rows, full + 8 * s);
+              copy_tile(wdst, &map_w, wc0, tile * tile_rows, bar);
             }
           }
-          if (with_x && lane == 0) tma_tile_2d(abase + b_off + a * b_block_bytes, &map_x, k0, 0, full + 8 * s);
+          if (with_x && lane == 0) copy_tile(abase + b_off + a * b_block_bytes, &map_x, k0, rank * b_cols, bar);
         }
       }
       return true;
@@ -1017,7 +1094,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
     // ======================= expanders (quantised rows): codes -> bf16 block of the slot ==========
     // Two pairs of warps; a pair takes the slots of its parity (S is even), in the producers' order, so it meets
     // every phase of its slots and cannot fall two phases behind; while one pair waits the other one converts.
-    const int my_tiles = (int)blockIdx.x < n_tiles ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    const int my_tiles = first < n_tiles ? (n_tiles - 1 - first) / (int)gridDim.x + 1 : 0;
     const int total = my_tiles * kstages;
     const int pair = (tid - kExpand0) / (16 * kExpandWarps);
     const int et = (tid - kExpand0) % (16 * kExpandWarps);
@@ -1047,7 +1124,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
       if (lane == 0 && m < issuers) {
         const uint32_t idesc = make_idesc(npad, mrows);
         const uint32_t place = tmem_base + m * place_cols;
-        const int my_tiles = (int)blockIdx.x < n_tiles ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+        const int my_tiles = first < n_tiles ? (n_tiles - 1 - first) / (int)gridDim.x + 1 : 0;
         int s = 0, ph = 0, kb = 0;
         for (int it = 0; it < my_tiles * kstages; ++it, ++s, ++kb) {
           if (s == S) { s = 0; ph ^= 1; }
@@ -1071,12 +1148,22 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
           umma_commit(place_full + 8 * m);
         }
       }
-    } else if (lane == 0 && m < nacc) {
-      const uint32_t idesc = kNat ? make_idesc_i8(npad, mrows) : make_idesc(npad, mrows);
+    } else if (lane == 0 && m < nacc && rank == 0) {
+      const uint32_t idesc = kNat ? make_idesc_i8(npad, PAIR ? 2 * mrows : mrows) : make_idesc(npad, PAIR ? 2 * mrows : mrows);
+      auto mma = [&](uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
+        if constexpr (PAIR && kNat) umma_pair_i8(d, adesc, bdesc, idesc, accumulate);
+        else if constexpr (PAIR) umma_pair(d, adesc, bdesc, idesc, accumulate);
+        else if constexpr (kNat) umma_i8(d, adesc, bdesc, idesc, accumulate);
+        else umma(d, adesc, bdesc, idesc, accumulate);
+      };
+      auto commit = [&](uint32_t bar) {
+        if constexpr (PAIR) umma_commit_pair(bar);
+        else umma_commit(bar);
+      };
       const uint32_t acc = tmem_base + m * npad;
       int tcount = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; ok && tile < n_tiles; tile += gridDim.x, ++tcount) {
+      for (int tile = first; ok && tile < n_tiles; tile += gridDim.x, ++tcount) {
         if (!mbar_wait(acc_empty, (tcount & 1) ^ 1, abort_flag, p.status, p.wait_cycles)) break;
         tc_fence_after();
         const int it0 = tcount * kstages;
@@ -1094,20 +1181,14 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
           for (int a = 0; a < na; ++a) {
             const uint64_t adesc = make_desc(wbase + a * a_block_bytes);
             const uint64_t bdesc = make_desc(sbase + b_off + a * b_block_bytes);
-            if (kNat) {
-              umma_i8(acc, adesc, bdesc, idesc, (kb >= nacc || a > 0) ? 1u : 0u);
+            mma(acc, adesc, bdesc, (kb >= nacc || a > 0) ? 1u : 0u);
 #pragma unroll
-              for (int k = 1; k < 4; ++k) umma_i8(acc, adesc + 2 * k, bdesc + 2 * k, idesc, 1u);
-            } else {
-              umma(acc, adesc, bdesc, idesc, (kb >= nacc || a > 0) ? 1u : 0u);
-#pragma unroll
-              for (int k = 1; k < kAtomK / 16; ++k) umma(acc, adesc + 2 * k, bdesc + 2 * k, idesc, 1u);
-            }
+            for (int k = 1; k < 4; ++k) mma(acc, adesc + 2 * k, bdesc + 2 * k, 1u);
           }
-          umma_commit(empty + 8 * s);   // slot free once these MMAs have read it
-          if (kExp) umma_commit(afree + 8 * t);
+          commit(empty + 8 * s);   // slot free once these MMAs have read it
+          if (kExp) commit(afree + 8 * t);
         }
-        if (ok) umma_commit(acc_full);  // this issuer's accumulator is complete
+        if (ok) commit(acc_full);  // this issuer's accumulator is complete
       }
     }
     __syncwarp();
@@ -1126,7 +1207,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
         }
     }
     int tcount = 0, it = 0, s = 0;
-    int tile = blockIdx.x;
+    int tile = blockIdx.x;  // PAIR: all of the pair's tiles but its last one here, whose shared epilogue both CTAs go through
     // which rows of the tile fired, as the up kernel or the compaction reads it
     auto publish = [&](bool fired) {
       const int li = tile * tile_rows + row_thr;
@@ -1134,10 +1215,10 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
       if (p.flag && valid) p.flag[li] = fired ? 1 : 0;
       if (p.words_out) {
         const unsigned m = __ballot_sync(0xffffffffu, fired && valid);
-        if (lane == 0) p.words_out[4 * tile + (warp & 3)] = m;
+        if (lane == 0 && tile < n_tiles) p.words_out[4 * tile + (warp & 3)] = m;
       }
     };
-    for (; tile + (share_last ? (int)gridDim.x : 0) < n_tiles; tile += gridDim.x, ++tcount) {
+    for (; tile - rank + (share_last ? (int)gridDim.x : 0) < n_tiles; tile += gridDim.x, ++tcount) {
       bool fired = false;
       if constexpr (EX) {
         const bool done = exact_epilogue(tile, tcount, set, it, s, fired);
@@ -1158,12 +1239,13 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
       if (!UP) publish(fired);
       if (EX) continue;
       tc_fence_before();
-      mbar_arrive(acc_empty);
+      if constexpr (PAIR) mbar_arrive_cluster(map_rank(acc_empty, 0));
+      else mbar_arrive(acc_empty);
     }
     // after a wait that ran out: nothing fired in the tiles that are left (the masks there are an earlier call's, or
     // the bytes of another route, whose bits need not stand for rows at all)
     if (!UP && set == 0)
-      for (; tile + (share_last ? (int)gridDim.x : 0) < n_tiles; tile += gridDim.x) {
+      for (; tile - rank + (share_last ? (int)gridDim.x : 0) < n_tiles; tile += gridDim.x) {
         pdl_wait();
         publish(false);
       }
@@ -1172,8 +1254,8 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
   // ---- the CTA's last tile (wide batches): by now the producer and issuer warps have nothing left to do, so
   // all twelve warps share its epilogue.  A warp reads the TMEM lanes of its quarter (warp mod 4); the three warps of
   // a quarter take every third group of eight token columns.
-  if (share_last && (int)blockIdx.x < n_tiles && warp < kThreadsRows / 32) {
-    const int my_tiles = (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
+  if (share_last && first < n_tiles && warp < kThreadsRows / 32) {
+    const int my_tiles = (n_tiles - 1 - first) / (int)gridDim.x + 1;
     const int last_tile = blockIdx.x + (my_tiles - 1) * gridDim.x;
     const int part = warp >= 8 ? 2 : warp >= 4 ? 0 : 1;
     bool fired = false;
@@ -1191,7 +1273,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
         if (p.flag && valid) p.flag[li] = any ? 1 : 0;
         if (p.words_out) {
           const unsigned m = __ballot_sync(0xffffffffu, any && valid);
-          if (lane == 0) p.words_out[4 * last_tile + (warp & 3)] = m;
+          if (lane == 0 && last_tile < n_tiles) p.words_out[4 * last_tile + (warp & 3)] = m;
         }
       }
     }
@@ -1203,8 +1285,13 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
   if (*abort_flag)
     for (int i = 0; i < 50; ++i) __nanosleep(1000);
   tc_fence_before();
-  __syncthreads();
-  if (warp == 8) {
+  // (PAIR: nor is there shared memory left behind that the even CTA's MMAs, or its commits, reach for)
+  if constexpr (PAIR) cluster_sync();
+  else __syncthreads();
+  if (PAIR && warp == 8) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
+  } else if (warp == 8) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
   }
@@ -1819,6 +1906,14 @@ cudaError_t launch_rows_mode(const UmmaRowsParams& p, dim3 grid, size_t smem, cu
       return launch_pdl(k, grid, dim3(kThreadsRows + 128 + (p.qbits ? 32 * kExpandWarps : 0)), smem, s, p, map_w, map_x, map_t);
     }
   }
+  if constexpr (MODE != kUp) {
+    if (p.pair) {
+      static unsigned long long configured_pair[2] = {0, 0};
+      auto k = p.qbits ? umma_rows_kernel<MODE, 1, false, true> : umma_rows_kernel<MODE, 0, false, true>;
+      if ((e = allow_dynamic_smem(k, 227 * 1024, configured_pair[p.qbits])) != cudaSuccess) return e;
+      return launch_clusters(2, k, grid, dim3(kThreadsRows), smem, s, p, map_w, map_x, map_t);
+    }
+  }
   if (p.qbits == 1) {
     auto k = umma_rows_kernel<MODE, 1>;
     if ((e = allow_dynamic_smem(k, 227 * 1024, configured[3])) != cudaSuccess) return e;
@@ -1869,6 +1964,25 @@ void umma_k_splits(int R, int K, bool codes, int B, int sm_count, int max_splits
   *splits = n;
 }
 
+// Pairs of CTAs (cta_group::2) where a CTA by itself has fewer than six ring slots: each holds half of the token rows, which every
+// CTA reads through L2 otherwise, and the ring gets eight slots instead of four.  4096 x 14336, alone / in pairs: bf16, 200 and
+// 256 tokens 130 / 112 and 137 / 122 us; int8, 48 and 64 tokens 75.3 / 69.3 and 80.5 / 75.9; 8192 x 24000: 394 / 348, 235 / 210.
+// With six slots nothing is gained (4096 x 14336, 160 tokens 99.9 / 100.7; 2048 x 6000, 200 tokens 59.7 / 61.6), and the clusters
+// cost a kernel 0.5 to 1 us (1024 x 3000, 72 tokens 29.7 / 33.3).  Codes that are expanded stay alone (int4, 4096 x 14336, 64
+// tokens 97.5 / 112: two CTAs' expansions to wait for).
+static bool rows_pairs(int R, int K, int qbits, int B, int cols, bool exact, int sm_count) {
+  if (exact || qbits > 1 || sm_count % 2) return false;
+  int tile_rows, n_tiles;
+  umma_gate_tiling(R, K, qbits, B, sm_count, &tile_rows, &n_tiles);
+  return kRingBytes / ((tile_rows + (cols + 15) / 16 * 16) * 128) < 6;
+}
+
+int umma_gate_rows_per_word(int R, int K, int qbits, int B, int cols, bool exact, int sm_count) {
+  int tile_rows, n_tiles;
+  umma_gate_tiling(R, K, qbits, B, sm_count, &tile_rows, &n_tiles);
+  return tile_rows <= 64 && !rows_pairs(R, K, qbits, B, cols, exact, sm_count) ? 16 : 32;
+}
+
 cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, cudaStream_t s) {
   p.npad = (cols + 15) / 16 * 16;
   if (p.exact ? (p.B > (p.qbits ? kExactHalfTerms + 16 : kExactTokens) || p.npad > kUmmaExactCols || p.qbits == 1 || p.qbits == 2 || (up && p.h_terms != 3))
@@ -1882,7 +1996,11 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
   p.equal_max = equal_tiles_max(p.K, p.qbits, p.B);
   p.run_blocks = kb / splits;
   p.longer_runs = kb % splits;
-  const int grid = splits > 1 ? p.k_tiles : p.R < 8 * sm_count ? (p.R + 7) / 8 : sm_count;
+  const bool may_walk = up && p.walk_all && umma_may_walk(p.B) && !p.exact;
+  int grid = splits > 1 ? p.k_tiles : p.R < 8 * sm_count ? (p.R + 7) / 8 : sm_count;
+  p.pair = splits == 1 && (!up || may_walk) && rows_pairs(p.R, p.K, p.qbits, p.B, cols, p.exact, sm_count);
+  grid += p.pair ? grid % 2 : 0;  // (one CTA more of eight rows each: the same tiles)
+  if (p.pair && p.qbits) p.npad = (p.npad + 31) / 32 * 32;  // what the pairs' int8 MMAs take
   // all the dynamic shared memory a CTA can have; the kernel cuts its ring out of it once it knows its tiles
   const size_t smem = kRowsSmem;
   p.ring_bytes = kRingBytes;
@@ -1893,12 +2011,13 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
   if (i8 && (p.K % 128 || !p.tok_scale)) return cudaErrorInvalidValue;
   // weights: all R rows; boxes of one tile's rows for the gate, single-row boxes for the gather
   if (!make_weight_map(&map_w, p.W, p.K, p.R, up ? 1 : tile_rows_for(p.R, grid, p.equal_max), p.qbits)) return cudaErrorNotSupported;
-  // tokens: only the rows that exist; the box covers npad rows and the rest reads as zero
-  if (i8 ? !make_map_i8(&map_x, p.X, p.K, p.ncols_valid, (size_t)p.x_stride, p.npad)
-                   : !make_map(&map_x, p.X, p.K, p.ncols_valid, (size_t)p.x_stride, p.npad))
+  // tokens: only the rows that exist; the box covers npad rows (half of them in each CTA of a pair) and the rest reads as zero
+  const int x_box = p.pair ? p.npad / 2 : p.npad;
+  if (i8 ? !make_map_i8(&map_x, p.X, p.K, p.ncols_valid, (size_t)p.x_stride, x_box)
+                   : !make_map(&map_x, p.X, p.K, p.ncols_valid, (size_t)p.x_stride, x_box))
     return cudaErrorNotSupported;
   if (!up) return launch_rows_mode<kGate>(p, dim3(grid, splits), smem, s, map_w, map_x, WalkMap<false>{});
-  if (p.walk_all && umma_may_walk(p.B) && !p.exact) {
+  if (may_walk) {
     // wide batches: the union may cover most rows; the kernel then walks every row with tiled boxes of the tile
     // height of R rows (decided on the device from the union's size, so it depends on this call's inputs only)
     WalkMap<true> map_t;

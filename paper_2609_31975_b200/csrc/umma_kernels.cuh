@@ -29,7 +29,7 @@ struct UmmaRowsParams {
   const uint32_t* words_in;  // UP, instead of idx / count: the gate kernel's "fired" bit masks (n_words of
   int n_words;               //   them, 4 per gate tile of gate_tile_rows rows); the kernel compacts them itself
   int gate_tile_rows;
-  int gate_rows_per_word;    //   rows covered by one mask word: 32 for gate tiles of more than 64 rows, else 16
+  int gate_rows_per_word;    //   rows covered by one mask word (umma_gate_rows_per_word)
   int32_t* idx_out;          //   ... and writes the ascending list
   int32_t* count_out;        //   ... and its length
   int32_t* walk_all;         //   ... and 1 here when it walked every row instead of the list (the down kernel must too), else 0
@@ -59,7 +59,7 @@ struct UmmaRowsParams {
   int h_terms, h_cols;   //   2 terms: quantised rows only (0: 1); exact: 3
   int act_up;            // UP: activation on the up projection (double activation), kUmmaActIdentity = none
   int32_t* status;       // device status word
-  int npad, ring_bytes;  // filled by the launcher
+  int npad, ring_bytes, pair;  // filled by the launcher
   long long wait_cycles; // budget of every device-side wait (filled by the launcher)
   int drop_stage;        // test hook: CTA 0 of the gate kernel never copies the weights of this stage (-1: none)
 };
@@ -94,6 +94,8 @@ bool umma_may_walk(int B);
 // R gate rows of K elements or codes (qbits as in UmmaRowsParams) against B tokens
 bool umma_own_list_supported(int R, int K, int qbits, int B, int sm_count);
 void umma_gate_tiling(int R, int K, int qbits, int B, int sm_count, int* tile_rows, int* n_tiles);
+// Rows that a word of that gate's "fired" masks covers (`cols`: its token columns, limbs or terms included).
+int umma_gate_rows_per_word(int R, int K, int qbits, int B, int cols, bool exact, int sm_count);
 cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, cudaStream_t s);
 bool umma_rows_native_i8_supported(int K, int tokens);
 // Tokens [B][K] bf16 as four int8 limbs each ([4 B][K], most significant first, 7 bits apart) and one scale per token;

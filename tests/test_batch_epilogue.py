@@ -51,3 +51,68 @@ def test_tokens_of_short_and_full_steps_of_codes(B, D, qbits):
     torch.cuda.synchronize()
     assert ffn.device_status() == 0
     assert ((y - one).norm(dim=1) / one.norm(dim=1)).max().item() < 1e-2
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("qbits,D,H,B,s", [
+    (0, 256, 6001, 250, 0.5),    # pairs of CTAs; every row walked, a ragged last tile
+    (0, 256, 6001, 250, 0.999),  # the union listed, in tiles of eight rows or so
+    (0, 256, 28003, 200, 0.9),   # 219 tiles: the last pair has one
+    (0, 256, 28003, 180, 0.999),
+    (0, 1280, 24001, 256, 0.9),  # two tiles for each CTA of a pair
+    (8, 256, 6001, 64, 0.5),
+    (8, 256, 6001, 61, 0.97),    # 244 limbs in 256 columns
+    (8, 256, 28003, 45, 0.9),    # 180 limbs in 192
+    (8, 1280, 24001, 57, 0.97),
+])
+def test_pairs_of_ctas_share_the_token_rows(qbits, D, H, B, s):
+    """Two calls of one handle, the second on other tokens.  bf16 rows against the oracle, codes against the single-token calls (a
+    bf16 h in the batch: 1e-2)."""
+    import paper_2609_31975_b200 as m
+
+    w = syn.standard_ffn_q8(D, H, 83, DEV, sparsity=s) if qbits else syn.standard_ffn(D, H, torch.bfloat16, 83, DEV, sparsity=s)
+    ffn = m.SparseFFN(D, H, torch.bfloat16, B_max=B)
+    call = ffn.sparse_ffn_forward_q8 if qbits else ffn.sparse_ffn_forward
+    args = ({"W_g": w["W_g"]}, w["b_g"], w["W_up"], w["W_down"], "relu")
+    xs = syn.tokens(2 * B, D, torch.bfloat16, 83, DEV)
+    for x in (xs[:B], xs[B:]):
+        y = call(x, *args)
+        torch.cuda.synchronize()
+        assert ffn.device_status() == 0
+        if qbits:
+            one = torch.stack([call(x[b], *args) for b in range(B)])
+            torch.cuda.synchronize()
+            assert ((y - one).norm(dim=1) / one.norm(dim=1).clamp(min=1e-3)).max().item() < 1e-2
+        else:
+            ref = run_oracle(x, args[0], w["b_g"], w["W_up"], w["W_down"], "relu", threads=16)
+            active = ffn.last_active()
+            assert_y_close(y, ref["y"], what=f"{D}x{H} B={B}")
+            assert_active_set(active, ref, what=f"{D}x{H} B={B}")
+
+
+@pytest.mark.gpu
+def test_a_copy_that_never_comes_ends_both_ctas_of_a_pair():
+    """A wait that runs out in the even CTA, whose barrier the copies of both complete on: a status, and the next call is right."""
+    import paper_2609_31975_b200 as m
+    from paper_2609_31975_b200 import binding
+
+    D, H, B = 256, 6001, 250
+    w = syn.standard_ffn(D, H, torch.bfloat16, 84, DEV, sparsity=0.9)
+    ffn = m.SparseFFN(D, H, torch.bfloat16, B_max=B)
+    args = (syn.tokens(B, D, torch.bfloat16, 84, DEV), {"W_g": w["W_g"]}, w["b_g"], w["W_up"], w["W_down"], "relu")
+    want = ffn.sparse_ffn_forward(*args).clone()
+    torch.cuda.synchronize()
+    try:
+        binding.test_set_knob("wait_cycles", 20_000_000)
+        binding.test_set_knob("drop_stage", 1)
+        ffn.sparse_ffn_forward(*args)
+        torch.cuda.synchronize()
+        assert ffn.device_status() == 5
+    finally:
+        binding.test_set_knob("drop_stage", -1)
+        binding.test_set_knob("wait_cycles", 0)
+    ffn.reset()
+    got = ffn.sparse_ffn_forward(*args)
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0
+    assert torch.equal(got, want)
