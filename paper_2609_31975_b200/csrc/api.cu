@@ -510,21 +510,27 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
   const int down_max = umma ? (exact ? kUmmaExactCols : kUmmaMaxCols) / h_terms / 8 * 8 : B;
   for (int b0 = 0; b0 < B; b0 += down_max) {
     const int nb = B - b0 < down_max ? B - b0 : down_max;
-    int splits;
     if (umma) {
       UmmaDownParams d{};
       d.W_down = W_down; d.R = H; d.D = D; d.qbits = wq;
       d.idx = lidx; d.count = lcount;
       d.hmT = hmT; d.hm_stride = h->L.hm_stride; d.terms = h_terms; d.h_cols = h_cols; d.exact = exact;
       d.tok0 = b0; d.B = nb; d.cols = round8(nb);
-      // (the workspace holds most_splits() partials of nb tokens; the first argument bounds what the SMs can use)
+      // (the workspace holds most_splits() partials of nb tokens)
       const int cap = nb <= kMaxMmaTokens ? kMaxSplits : most_splits(D, nb);
-      d.splits = splits = umma_down_splits(D, h_terms * d.cols, exact, h->sm_count, cap);
+      const bool clustered = umma_down_splits(D, H, wq, h_terms * d.cols, exact, h->sm_count, cap, &d.splits);
       d.walk_all = (own_list && may_walk) ? count + 1 : nullptr;
-      d.partial = partial; d.status = h->at<int32_t>(h->L.status);
+      if (clustered) d.y = y + (size_t)b0 * D;
+      else d.partial = partial;
+      d.status = h->at<int32_t>(h->L.status);
       SFFN_CUDA(launch_umma_down(d, s));
+      ++h->launches;
+      if (!clustered) {
+        SFFN_CUDA(launch_reduce(partial, d.splits, nb, D, y + (size_t)b0 * D, D, s));
+        ++h->launches;
+      }
     } else {
-      splits = h->sm_count / (D / 256);
+      int splits = h->sm_count / (D / 256);
       splits = splits < 1 ? 1 : splits > kMaxSplits ? kMaxSplits : splits;
       DownMmaParams d{};
       d.status = h->at<int32_t>(h->L.status);
@@ -533,9 +539,9 @@ int run_batched(sffn_handle* h, const void* x, int B, const sffn_gate* g, const 
       d.hmT = hmT; d.hm_stride = h->L.hm_stride; d.B = nb;
       d.partial = partial;
       SFFN_CUDA(launch_down_mma(d, splits, s));
+      SFFN_CUDA(launch_reduce(partial, splits, nb, D, y + (size_t)b0 * D, D, s));
+      h->launches += 2;
     }
-    SFFN_CUDA(launch_reduce(partial, splits, nb, D, y + (size_t)b0 * D, D, s));
-    h->launches += 2;
   }
   return SFFN_OK;
 }

@@ -4,7 +4,7 @@
 //                           "any token fires" bit per neuron             (Eq. 1 gate / LoPA U and V stages, batched)
 //   umma_rows_kernel<UP>    compacts those bits into the union list of fired neurons (Sec. 5.4), then over that
 //                           list: Up = W_up[idx] X^T, Hm = a . A_3(Up), stored as bf16 HmT[b][u]
-//   umma_down_kernel        partial[split][b][d] = sum over the split's list rows u of HmT[b][u] W_down[idx[u]][d]
+//   umma_down_kernel        y[b][d] = sum over the list rows u of HmT[b][u] W_down[idx[u]][d]
 //   rmsnorm_split_kernel    LoPA: n = RMSNorm(v) as bf16 high / low pairs (the B operand of the U stage)
 //
 // Rows kernels: one CTA owns a tile of up to 128 weight rows (TMEM lanes) x Npad token columns (Npad = columns
@@ -42,6 +42,8 @@
 #include "umma_kernels.cuh"
 
 #include <cuda.h>
+
+#include <atomic>
 
 #include "common.cuh"
 #include "fused_kernel.cuh"
@@ -1298,14 +1300,17 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
 }
 
 // ------------------------------------------------------------------------------------------------
-// Down projection over the union list (Sec. 5.4): partial[sp][b][d] = sum over the split's listed rows u of
-// Hm[b][u] * W_down[idx[u]][d].  One CTA owns 128 output columns d (TMEM lanes) and one split of the list;
+// Down projection over the union list (Sec. 5.4): y[b][d] = sum over the listed rows u of Hm[b][u] * W_down[idx[u]][d].
+// One CTA owns 128 output columns d (TMEM lanes) and one split of the list, a cluster (if any) all splits of those columns;
 // the contraction runs over list rows, so the gathered W_down rows are the MN-major A operand (each
 // gathered row delivers 64 contiguous d per swizzle row) and HmT[b][u] is the K-major B operand.
 // Same pipeline as above: 4 producer warps (gather4 per lane: 2 column halves x 16 row quads = one 64-row
 // stage), 2 MMA issuers with their own accumulators, 4 epilogue warps; two CTAs share an SM.
+// Threads, rounded up to whole warps for each scheduler: registers are handed out by scheduler, and two CTAs of 14 warps with 72
+// registers a thread, which fit an SM's file, do not fit those of the first two (int4 rows ran in two waves of CTAs).
+constexpr int down_bound(int qb, bool exact) { return ((exact ? 512 : kThreads) + (qb ? 32 * kExpandWarps : 0) + 127) / 128 * 128; }
 template <int QB, bool EX = false, bool TWO = false>
-__global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarps : 0), EX ? 1 : 2) umma_down_kernel(const UmmaDownParams p,
+__global__ void __launch_bounds__(down_bound(QB, EX), EX ? 1 : 2) umma_down_kernel(const UmmaDownParams p,
                                                                   const __grid_constant__ CUtensorMap map_wg,
                                                                   const __grid_constant__ CUtensorMap map_wt,
                                                                   const __grid_constant__ CUtensorMap map_hm) {
@@ -1324,7 +1329,7 @@ __global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarp
   const int stage_bytes = raw_off + kRawBytes;
   const int S = p.stages;
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + expand_bytes + (size_t)S * stage_bytes);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.ring_bytes);  // (the rings, or as much as the sums of the tokens take)
   const uint32_t expand0 = smem_u32(smem), stage0 = expand0 + expand_bytes;
   const uint32_t full = smem_u32(bars), empty = smem_u32(bars + S);
   const uint32_t acc_full = smem_u32(bars + 2 * S);
@@ -1335,7 +1340,8 @@ __global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarp
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int d_tiles = p.D / kTileRows;
-  const int dt = blockIdx.x % d_tiles, sp = blockIdx.x / d_tiles;
+  const bool clustered = p.y != nullptr;  // the splits of a tile are one cluster
+  const int dt = clustered ? blockIdx.x / p.splits : blockIdx.x % d_tiles, sp = clustered ? blockIdx.x % p.splits : blockIdx.x / d_tiles;
   const int d0 = dt * kTileRows;
 
   pdl_launch_dependents();
@@ -1506,47 +1512,63 @@ __global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarp
     }
     __syncwarp();
   } else {
-    // ======================= epilogue: lane = output column d, TMEM columns = tokens ============
+    // (below: every warp that has nothing left to do takes part in the epilogue)
+  }
+
+  // ======================= epilogue: lane = output column d, TMEM columns = tokens ================
+  // Clustered: the split's sums go to shared memory, [token][128 columns] over the ring, which nothing is copied into or multiplied
+  // from any more; then each CTA of the cluster adds a share of the tokens up over all splits, in their order.  Else they go to the
+  // partials, which a kernel adds up in the same order.
+  float* sums = reinterpret_cast<float*>(smem);
+  const int B = p.B;
+  {
     const int ew = warp & 3;
-    const int d = d0 + ew * 32 + lane;
-    const int B = p.B;
-    float* out = p.partial + (size_t)sp * B * p.D + d;
+    float* mine = clustered ? sums + ew * 32 + lane : p.partial + (size_t)sp * B * p.D + d0 + ew * 32 + lane;
+    const size_t pitch = clustered ? kTileRows : p.D;
     const uint32_t taddr = tmem_base + ((uint32_t)(ew * 32) << 16);
-    const int set = EX && warp >= 12 ? 1 : 0;
-    if (kblocks <= 0) {
-      for (int b = 0; set == 0 && b < B; ++b) out[(size_t)b * p.D] = 0.f;
-    } else if constexpr (EX) {
-      constexpr int kHalf = QB ? kExactHalfTerms : kExactHalf;
-      float sum[kHalf], low[kHalf];
+    if constexpr (EX) {
+      if ((warp >= 4 && warp < 8) || (warp >= 12 && warp < 16)) {
+        constexpr int kHalf = QB ? kExactHalfTerms : kExactHalf;
+        const int set = warp >= 12 ? 1 : 0;
+        float sum[kHalf], low[kHalf];
 #pragma unroll
-      for (int c = 0; c < kHalf; ++c) sum[c] = low[c] = 0.f;
-      const int half = ((p.cols + 1) / 2 + 7) & ~7, c0 = set * half, c1 = set ? p.cols : half;
-      int ok = 1, s = 0;
-      for (int kb = 0; kb < kblocks; ++kb, ++s) {
-        if (s == S) s = 0;
-        const int m = kb & (issuers - 1);
-        if (lane == 0) ok = mbar_wait(place_full + 8 * m, (kb / issuers) & 1, abort_flag, p.status, p.wait_cycles) ? 1 : 0;
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        if (!ok) break;
-        if (warp == 4 && lane == 0) mbar_arrive(empty + 8 * s);  // the stage's MMAs are done with their operands
-        tc_fence_after();
-        add_stage<kHalf>(taddr + m * place_cols, kExactPer, npad, c0, c1, p.terms, p.cols, sum, low);
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(place_empty + 8 * m);
+        for (int c = 0; c < kHalf; ++c) sum[c] = low[c] = 0.f;
+        const int half = ((p.cols + 1) / 2 + 7) & ~7, c0 = set * half, c1 = set ? p.cols : half;
+        int ok = 1, s = 0;
+        for (int kb = 0; kb < kblocks; ++kb, ++s) {
+          if (s == S) s = 0;
+          const int m = kb & (issuers - 1);
+          if (lane == 0) ok = mbar_wait(place_full + 8 * m, (kb / issuers) & 1, abort_flag, p.status, p.wait_cycles) ? 1 : 0;
+          ok = __shfl_sync(0xffffffffu, ok, 0);
+          if (!ok) break;
+          if (warp == 4 && lane == 0) mbar_arrive(empty + 8 * s);  // the stage's MMAs are done with their operands
+          tc_fence_after();
+          add_stage<kHalf>(taddr + m * place_cols, kExactPer, npad, c0, c1, p.terms, p.cols, sum, low);
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(place_empty + 8 * m);
+        }
+        finish_sums<kHalf>(sum, low);
+#pragma unroll
+        for (int i = 0; i < kHalf; ++i)
+          if (c0 + i < c1 && c0 + i < B) mine[(c0 + i) * pitch] = sum[i];
       }
-      finish_sums<kHalf>(sum, low);
-#pragma unroll
-      for (int i = 0; i < kHalf; ++i)
-        if (ok && c0 + i < c1 && c0 + i < B) out[(size_t)(c0 + i) * p.D] = sum[i];
-    } else {
+    } else if (warp < 8) {
+      // two warps for each quarter of the lanes, on alternate groups of eight tokens (there is one phase of this barrier, so any
+      // warp may wait for it)
       int okw = 1;
-      if (lane == 0) okw = mbar_wait(acc_full, 0, abort_flag, p.status, p.wait_cycles) ? 1 : 0;
-      okw = __shfl_sync(0xffffffffu, okw, 0);
-      if (okw) {
-        tc_fence_after();
-        for (int c0 = 0; c0 < p.cols; c0 += 8) {
-          float v[8];
+      if (kblocks > 0) {
+        if (lane == 0) okw = mbar_wait(acc_full, 0, abort_flag, p.status, p.wait_cycles) ? 1 : 0;
+        okw = __shfl_sync(0xffffffffu, okw, 0);
+      }
+      tc_fence_after();
+      const bool some = okw && kblocks > 0;
+#pragma unroll 1
+      for (int c0 = warp < 4 ? 8 : 0; c0 < B; c0 += 16) {
+        float v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = 0.f;
+        if (some) {
           tmem_ld8(taddr + c0, nacc, npad, v);
           if (QB && p.terms == 2) {
             float w[8];
@@ -1554,10 +1576,10 @@ __global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarp
 #pragma unroll
             for (int q = 0; q < 8; ++q) v[q] += w[q];
           }
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            if (c0 + q < B) out[(size_t)(c0 + q) * p.D] = v[q];
         }
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (c0 + q < B) mine[(c0 + q) * pitch] = v[q];
       }
     }
   }
@@ -1565,11 +1587,38 @@ __global__ void __launch_bounds__((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarp
   if (*abort_flag)
     for (int i = 0; i < 50; ++i) __nanosleep(1000);
   tc_fence_before();
-  __syncthreads();
+  if (clustered) cluster_sync();
+  else __syncthreads();
   if (warp == 8) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
   }
+  if (!clustered) return;
+  // a warp takes a token at a time, a lane four columns of it
+  const int n_warps = blockDim.x >> 5;
+  const uint32_t at = smem_u32(sums) + lane * 16;
+  for (int b = sp * n_warps + warp; b < B; b += p.splits * n_warps) {
+    float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int r0 = 0; r0 < p.splits; r0 += 4) {
+      float4 v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r0 + i < p.splits)
+          asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v[i].x), "=f"(v[i].y), "=f"(v[i].z), "=f"(v[i].w)
+                       : "r"(map_rank(at + b * (kTileRows * 4), r0 + i)) : "memory");
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        t.x += v[i].x;
+        t.y += v[i].y;
+        t.z += v[i].z;
+        t.w += v[i].w;
+      }
+    }
+    *reinterpret_cast<float4*>(p.y + (size_t)b * p.D + d0 + 4 * lane) = t;
+  }
+  cluster_sync();  // no CTA leaves while another reads its sums
 }
 
 // The entries of v for the norm kernels below: the sum of `runs` fp32 values, `step` apart, or the four limbs' integer sums over
@@ -2031,20 +2080,72 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
 // at least four ring stages); wider batches give one CTA the whole SM, and so do exact sums, whose accumulators fill
 // the TMEM.
 constexpr int kDownPairCols = 64;
+constexpr int kMaxDownCluster = 8;  // CTAs of a cluster
 static bool down_pairs(int cols, bool exact) { return cols <= kDownPairCols && !exact; }
 
-int umma_down_splits(int D, int cols, bool exact, int sm_count, int max_splits) {
+// Clusters of `size` CTAs of the down kernel that the device runs at once, two CTAs per SM or one.  (It depends on how many SMs
+// each of its GPCs has.)  Asked for a kernel that does nothing in as many threads and as much shared memory: for one that
+// allocates TMEM the runtime answers as if an SM took a single CTA.
+static __global__ void __launch_bounds__(down_bound(8, false), 2) down_place_kernel() {}
+static int down_clusters(int size, bool pairs) {
+  static std::atomic<int> known[16][2][kMaxDownCluster + 1];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= 16) return 0;
+  std::atomic<int>& k = known[dev][pairs ? 1 : 0][size];
+  if (k.load(std::memory_order_relaxed) == 0) {
+    static unsigned long long configured = 0;
+    auto kernel = down_place_kernel;
+    int n = 0;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(size);
+    cfg.blockDim = dim3(down_bound(8, false));
+    cfg.dynamicSmemBytes = (pairs ? 111 : 225) * 1024;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = size;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (allow_dynamic_smem(kernel, 227 * 1024, configured) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    k.store(n + 1, std::memory_order_relaxed);
+  }
+  return k.load(std::memory_order_relaxed) - 1;
+}
+
+// Splits of the list, and whether they are a cluster that adds its sums up itself.  That saves the partials' way through memory and
+// a kernel (4096 x 14336, bf16, partials / clusters: 200 tokens 108.3 / 101.2 us, 72 tokens 83.3 / 79.4, 16 tokens 62.9 / 61.6; 512 x
+// 1500, int8, 2 tokens 21.5 / 18.9), and costs splits where more CTAs would run than clusters fit the GPCs: up to a ninth of them
+// (codes, whose blocks take longer: none) is worth it (int8, 4096 x 14336, 8 tokens, nine splits / clusters of eight 44.6 / 45.1;
+// bf16, 6144 x 20000, 160 tokens, three / two 229 / 242; exact sums, 2688 x 8000, 24 tokens, seven / six 78.5 / 80.2), or any number
+// where a CTA has a dozen blocks at most (2048 x 6000, 16 / 8: bf16, 64 tokens 40.0 / 39.1, int4, 2 / 24 / 64 tokens 27.3 / 38.5 /
+// 53.6 against 25.5 / 39.1 / 49.9).  Clusters of up to 16 where they fit are slower (512 x 1500, bf16, 24 tokens, 8 / 16: 19.4 / 20.4).
+bool umma_down_splits(int D, int R, int qbits, int cols, bool exact, int sm_count, int max_splits, int* splits) {
   const int tiles = D >= kTileRows ? D / kTileRows : 1;
+  const bool pairs = down_pairs(cols, exact);
+  int cluster = kMaxDownCluster;
+  while (cluster > 1 && down_clusters(cluster, pairs) < tiles) --cluster;
   auto splits_of = [&](int ctas) {
     const int n = ctas / tiles;
     return n < 1 ? 1 : n > max_splits ? max_splits : n;
   };
-  if (down_pairs(cols, exact)) return splits_of(2 * sm_count);
   const int one = splits_of(sm_count), two = splits_of(2 * sm_count);
+  int n = pairs ? two : one;
   // Exact sums: two waves of CTAs, each with a set-up of its own (about 6 us), only where they shorten the contraction by a
   // tenth: wide rows, whose tiles leave SMs idle in one wave.  16 tokens, one wave / two: 2688 x 8000 67 / 74 us, 6528 x
   // 20000 (102 and 255 CTAs) 312 / 301.
-  return exact && 10 * (two - 2 * one) >= one * two ? two : one;
+  if (exact && 10 * (two - 2 * one) >= one * two) n = two;
+  const int blocks = (R + kAtomK - 1) / kAtomK;
+  const bool clustered = qbits ? cluster >= n : 9 * cluster >= 8 * n;
+  if (clustered || blocks <= 12 * cluster) {
+    *splits = cluster;
+    return true;
+  }
+  *splits = n;
+  return false;
 }
 
 bool umma_down_supported(int D, int cols) { return D % kTileRows == 0 && cols >= 1 && cols <= kUmmaMaxCols; }
@@ -2056,7 +2157,7 @@ cudaError_t launch_down_q(const UmmaDownParams& p, int grid, size_t smem, cudaSt
   static unsigned long long configured = 0;
   const cudaError_t e = allow_dynamic_smem(umma_down_kernel<QB, EX, TWO>, 227 * 1024, configured);
   if (e != cudaSuccess) return e;
-  return launch_pdl(umma_down_kernel<QB, EX, TWO>, dim3(grid), dim3((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarps : 0)), smem, s, p, map_wg,
+  return launch_clusters(p.y ? p.splits : 1, umma_down_kernel<QB, EX, TWO>, dim3(grid), dim3((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarps : 0)), smem, s, p, map_wg,
                     map_wt, map_hm);
 }
 }  // namespace
@@ -2094,7 +2195,9 @@ cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s) {
   const int stages = slots(two ? p.expand : 0);
   if (stages < 2) return cudaErrorInvalidValue;
   p.stages = stages;
-  size_t smem = 1024 + expanded + (size_t)stages * stage_bytes + (3 * stages + 4 + 2 * kMaxIssuers + 2 * kDownExpand) * 8 + 64;
+  p.ring_bytes = expanded + stages * stage_bytes;
+  if (p.ring_bytes < p.cols * kTileRows * 4) p.ring_bytes = p.cols * kTileRows * 4;
+  size_t smem = 1024 + p.ring_bytes + (3 * stages + 4 + 2 * kMaxIssuers + 2 * kDownExpand) * 8 + 64;
   // Never so little that an SM takes more CTAs than its TMEM has room for: they would wait for it (int8, 640 x 1408, 87 tokens:
   // 36.5 -> 39.8 us).
   const size_t least = (down_pairs(own, p.exact) ? 80 : 120) * 1024;

@@ -77,15 +77,17 @@ struct UmmaDownParams {
   int exact;             // see UmmaRowsParams
   int tok0, B;           // tokens [tok0, tok0 + B) of those rows
   int cols;              // B rounded up to a multiple of 8 (token columns of one term)
-  int splits;            // the list is cut into this many runs of 64-row blocks
+  int splits;            // the list is cut into this many runs of 64-row blocks (umma_down_splits)
   const int32_t* walk_all;  // device word: nonzero = walk every row of W_down instead of the list (set by the up kernel), or null
-  float* partial;        // [splits][B][D]
+  float* y;              // [B][D]: the splits are clusters (umma_down_splits), or null:
+  float* partial;        //   [splits][B][D]
   int32_t* status;
-  int npad, stages, expand;  // filled by the launcher
+  int npad, stages, expand, ring_bytes;  // filled by the launcher
   long long wait_cycles; // budget of every device-side wait (filled by the launcher)
 };
 
-int umma_down_splits(int D, int cols, bool exact, int sm_count, int max_splits);  // cols: token columns of all terms
+// How the list (of up to R rows) is split; true: `y`, in clusters, false: `partial` (at most max_splits).  cols: token columns of all terms.
+bool umma_down_splits(int D, int R, int qbits, int cols, bool exact, int sm_count, int max_splits, int* splits);
 bool umma_down_supported(int D, int cols);
 cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s);
 bool umma_rows_supported(int K, int cols);
