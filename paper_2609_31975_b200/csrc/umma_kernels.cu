@@ -69,7 +69,6 @@ constexpr int kWalkMinTokens = 32;                   // batches from which the u
 constexpr int kWalkAllPercent = 70;                  // union share of the rows from which "every row" is walked
 constexpr int kMaxIssuers = 4;
 constexpr int kExpandWarps = 4;                      // quantised rows: warps that expand the codes to bf16
-constexpr int kScanChunks = 4;                       // in-kernel compaction: up to 4 * 384 mask words = 384 gate tiles
 constexpr int kMaxOwnTiles = 8;                      // tiles of one CTA whose rows are kept in shared memory
 constexpr int kHeaderBytes = 1024 + kMaxOwnTiles * kTileRows * 4;  // barriers + scratch, then the row lists
 
@@ -571,7 +570,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
   // header: barriers (for the largest ring) and control words, scan scratch, this CTA's rows of the union
   // list; then the ring of stages, whose geometry is decided below once the tile height is known
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem);
-  int* scan_wt = reinterpret_cast<int*>(smem + 512);   // [kScanChunks][warps]
+  int* scan_wt = reinterpret_cast<int*>(smem + 512);   // [warps]
   int* rows_sm = reinterpret_cast<int*>(smem + 1024);  // [kMaxOwnTiles][128]
   const uint32_t stage0 = smem_u32(smem) + kHeaderBytes;
   const uint32_t full = smem_u32(bars), empty = smem_u32(bars + kMaxStages);
@@ -645,48 +644,35 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
 
   // Union rows: either the list is given (idx, count), or every CTA compacts the gate's "fired" bit masks
   // itself.  The gate kernel leaves one 32-bit word per epilogue warp and tile (word 4 * tile + warp, bit =
-  // lane = row rows_per_word * warp + lane of the tile, 32 rows per word for M = 128 tiles and pairs, 16 for M = 64); thread t takes word t of each chunk of `threads` words, a
-  // warp scan plus the warp totals of all chunks give the list position of its first set bit.
+  // lane = row rows_per_word * warp + lane of the tile, 32 rows per word for M = 128 tiles and pairs, 16 for M = 64); thread t takes
+  // the four words of tile t, and a warp scan plus the warps' totals give the list position of their first set bit.
   const bool own_list = UP && p.words_in != nullptr;
-  uint32_t bits[kScanChunks];
-  int first_pos[kScanChunks];
+  uint32_t bits[4] = {0, 0, 0, 0};
+  int fired_here = 0, first_pos = 0;
   int n_rows;
-  const int nch = own_list ? (p.n_words + kThreadsRows - 1) / kThreadsRows : 0;
   if (own_list) {
-#pragma unroll
-    for (int k = 0; k < kScanChunks; ++k) {
-      const int w = k * kThreadsRows + tid;
-      bits[k] = (k < nch && tid < kThreadsRows && w < p.n_words) ? __ldcg(p.words_in + w) : 0u;
+    if (tid < kThreadsRows && 4 * tid < p.n_words) {
+      const uint4 w = __ldcg(reinterpret_cast<const uint4*>(p.words_in) + tid);
+      bits[0] = w.x; bits[1] = w.y; bits[2] = w.z; bits[3] = w.w;
     }
+    fired_here = __popc(bits[0]) + __popc(bits[1]) + __popc(bits[2]) + __popc(bits[3]);
+    int incl = fired_here;
 #pragma unroll
-    for (int k = 0; k < kScanChunks; ++k) {
-      if (k < nch) {
-        int incl = __popc(bits[k]);
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-          const int t = __shfl_up_sync(0xffffffffu, incl, d);
-          if (lane >= d) incl += t;
-        }
-        first_pos[k] = incl - __popc(bits[k]);
-        if (lane == 31 && warp < kThreadsRows / 32) scan_wt[k * (kThreadsRows / 32) + warp] = incl;
-      }
+    for (int d = 1; d < 32; d <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += t;
     }
+    if (lane == 31 && warp < kThreadsRows / 32) scan_wt[warp] = incl;
     __syncthreads();
-    int run = 0;
+    int before = 0, total = 0;
 #pragma unroll
-    for (int k = 0; k < kScanChunks; ++k) {
-      if (k < nch) {
-        int before = 0, total = 0;
-        for (int w = 0; w < kThreadsRows / 32; ++w) {
-          const int t = scan_wt[k * (kThreadsRows / 32) + w];
-          before += w < warp ? t : 0;
-          total += t;
-        }
-        first_pos[k] += run + before;
-        run += total;
-      }
+    for (int w = 0; w < kThreadsRows / 32; ++w) {
+      const int t = scan_wt[w];
+      before += w < warp ? t : 0;
+      total += t;
     }
-    n_rows = run;
+    first_pos = incl - fired_here + before;
+    n_rows = total;
   } else {
     n_rows = p.count ? *p.count : p.R;
   }
@@ -699,22 +685,25 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
   if (walk_all) n_rows = p.R;
   const int tile_rows = tile_rows_for(n_rows, gridDim.x, p.equal_max);
   const int n_tiles = (n_rows + tile_rows - 1) / tile_rows;
-  if (own_list && walk_all) {
-    // publish the list only: word w is written out by CTA w mod grid
+  // Calls put(list position, row) for the rows of the gate tiles of this warp's lanes with `mine`: a lane a row, 32 at a time.  (A
+  // thread that went through the set bits of its own word took a microsecond for them.)
+  auto each_row = [&](bool mine, auto&& put) {
+    unsigned todo = __ballot_sync(0xffffffffu, mine);
+    while (todo) {
+      const int src = __ffs(todo) - 1;
+      todo &= todo - 1;
+      int pos = __shfl_sync(0xffffffffu, first_pos, src), j = (tid - lane + src) * p.gate_tile_rows + lane;
 #pragma unroll
-    for (int k = 0; k < kScanChunks; ++k) {
-      const int w = k * kThreadsRows + tid;
-      if (k < nch && bits[k] && w % (int)gridDim.x == (int)blockIdx.x) {
-        const int j0 = (w >> 2) * p.gate_tile_rows + (w & 3) * p.gate_rows_per_word;
-        uint32_t rest = bits[k];
-        int li = first_pos[k];
-        while (rest) {
-          const int q = __ffs(rest) - 1;
-          rest &= rest - 1;
-          p.idx_out[li++] = j0 + q;
-        }
+      for (int i = 0; i < 4; ++i, j += p.gate_rows_per_word) {
+        const uint32_t b = __shfl_sync(0xffffffffu, bits[i], src);
+        if (b >> lane & 1) put(pos + __popc(b & ((1u << lane) - 1u)), j);
+        pos += __popc(b);
       }
     }
+  };
+  if (own_list && walk_all) {
+    // publish the list only: a tile's part is written out by CTA tile mod grid
+    each_row(fired_here && tid % (int)gridDim.x == (int)blockIdx.x, [&](int li, int j) { p.idx_out[li] = j; });
     if (blockIdx.x == 0 && tid == 0) {
       *p.count_out = n_listed;
       *p.walk_all = 1;
@@ -723,29 +712,15 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
     if (blockIdx.x == 0 && tid == 0 && p.walk_all) *p.walk_all = 0;
     // keep the rows of this CTA's tiles in shared memory and publish them (and the length) for the
     // down projection and the caller: every list position belongs to exactly one CTA's tile
-#pragma unroll
-    for (int k = 0; k < kScanChunks; ++k) {
-      if (k < nch && bits[k]) {
-        const int cnt = __popc(bits[k]);
-        const int w = k * kThreadsRows + tid;
-        const int j0 = (w >> 2) * p.gate_tile_rows + (w & 3) * p.gate_rows_per_word;  // row of bit 0
-        int m = 0;
-        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++m) {
-          const int lo = tile * tile_rows, hi = lo + tile_rows;
-          if (first_pos[k] + cnt <= lo || first_pos[k] >= hi) continue;
-          uint32_t rest = bits[k];
-          int li = first_pos[k];
-          while (rest) {
-            const int q = __ffs(rest) - 1;
-            rest &= rest - 1;
-            if (li >= lo && li < hi) {
-              rows_sm[m * kTileRows + li - lo] = j0 + q;
-              p.idx_out[li] = j0 + q;
-            }
-            ++li;
-          }
+    int m = 0;
+    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++m) {
+      const int lo = tile * tile_rows, hi = lo + tile_rows;
+      each_row(fired_here && first_pos < hi && first_pos + fired_here > lo, [&](int li, int j) {
+        if (li >= lo && li < hi) {
+          rows_sm[m * kTileRows + li - lo] = j;
+          p.idx_out[li] = j;
         }
-      }
+      });
     }
     if (blockIdx.x == 0 && tid == 0) *p.count_out = n_rows;
   }
@@ -1866,7 +1841,7 @@ void umma_gate_tiling(int R, int K, int qbits, int B, int sm_count, int* tile_ro
 bool umma_own_list_supported(int R, int K, int qbits, int B, int sm_count) {
   int tr, nt;
   umma_gate_tiling(R, K, qbits, B, sm_count, &tr, &nt);
-  return 4 * nt <= kScanChunks * kThreadsRows && R <= (long long)kMaxOwnTiles * kTileRows * sm_count;
+  return nt <= kThreadsRows && R <= (long long)kMaxOwnTiles * kTileRows * sm_count;
 }
 
 bool umma_may_walk(int B) { return B >= kWalkMinTokens; }
