@@ -106,7 +106,7 @@ struct SmemLayout {
   int gate_ring, act_ring, sx, sn, aval, slot_a, red, ctl, bars, row_params, row_scales, slot_scales, gated_bars, gated_vals, xlimb, total;
   __host__ __device__ SmemLayout(int D, int K, bool lopa, int n_gate_slots, int gate_slot_bytes,
                                  int n_act_slots, int act_slot_bytes, int slab_max, bool scaled, int act_extra = 0,
-                                 bool gated = false, bool limbs = false) {
+                                 bool gated = false, bool limbs = false, bool pair = false) {
     int off = 0;
     auto take = [&](int bytes) {
       int o = off;
@@ -117,7 +117,7 @@ struct SmemLayout {
     act_ring = take(n_act_slots * act_slot_bytes);
     sx = take(D * 4);
     sn = take(lopa ? K * 4 : 0);
-    aval = take(slab_max * 4);
+    aval = take((pair ? 2 : 1) * slab_max * 4);  // this CTA's rows, and the other's of a pair
     slot_a = take((n_act_slots + act_extra) * 4);
     red = take(6 * kRedStride * 4);  // two buffers per act group (four warps each), up to three groups
     ctl = take((8 + 16) * 4);  // control words, then one sum of squares per staging warp (LoPA)
@@ -162,6 +162,9 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// The barrier of a pair of CTAs: thread by thread, first all arrive, then all wait.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 // Whether a phase has completed, without waiting for it.
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
   uint32_t ok;
@@ -355,9 +358,15 @@ __device__ __forceinline__ long long global_ns() {
 // the published h in order and copies the W_down rows that are needed into the "down" ring, which the act warps
 // consume one round behind (whatever is left after the stop marker).  Rows are added in the same order as in the
 // other variant and a skipped row would have added zeros, so y is bitwise the same.
-template <typename T, int CPT, bool LOPA, bool GATED = false>
+// PAIR (LoPA, wide rows; see launch_fused): CTAs 2 i and 2 i + 1 are a cluster and share out the rows of their fired neurons.  Gate
+// results go to both, and of the fired rows of both, in an order of their own (sixteen of the even CTA, sixteen of the odd one ...),
+// the even CTA does every other one, beginning with the first.  How many rows a CTA is left with varies twofold (97 neurons that
+// fire one time in ten: 10 +- 3, at most 20 in 148 CTAs, 15 in 74 pairs), and a call with a short gate waits for the CTA with most.
+// Who does a row depends on what fired alone: y is bitwise the same on every run.
+template <typename T, int CPT, bool LOPA, bool GATED = false, bool PAIR = false>
 __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParams p) {
   static_assert(!(GATED && LOPA), "the gated variant is built for the standard gate");
+  static_assert(!PAIR || (LOPA && !TokenOf<T>::kScaled), "pairs: LoPA gate, rows without scales");
   // Warp roles: 2 gate producers, 2 act producers, then gate warps and act warps.  The standard gate needs its
   // eight gate warps to keep up with the stream; the LoPA gate is short (r elements per row), the call's time
   // is then set by the up/down rows, so eight of the twelve workers are act warps there.
@@ -400,7 +409,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
   // an error of 3e-5 of the chunk's largest |x| per entry, about 1e-4 of a typical |z| or |u|.
   constexpr int kGateLimbs = kTokenLimbs;
   constexpr int kUpLimbs = kTokenLimbs;
-  const SmemLayout L(D, K, LOPA, NG, p.gate_slot_bytes, NAown, p.act_slot_bytes, p.slab_max, kScaled, p.act_extra, GATED, kLimbs || kLimbs4);
+  const SmemLayout L(D, K, LOPA, NG, p.gate_slot_bytes, NAown, p.act_slot_bytes, p.slab_max, kScaled, p.act_extra, GATED, kLimbs || kLimbs4, PAIR);
 
   unsigned char* gate_ring = smem + L.gate_ring;
   unsigned char* act_ring = smem + L.act_ring;
@@ -414,6 +423,10 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
   // A single 32-bit store publishes value and state together, so no fence is needed on either side
   // (a fence in the producers would also wait for their bulk copies in flight).
   volatile uint32_t* row_state = reinterpret_cast<volatile uint32_t*>(smem + L.aval);
+  const int side = cta & 1;
+  volatile uint32_t* peer_state = row_state + p.slab_max;
+  uint32_t peer_dst = 0;  // where the other CTA keeps this one's
+  if (PAIR) asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer_dst) : "r"(smem_u32(smem + L.aval) + 4 * p.slab_max), "r"(side ^ 1));
   float* slot_a = reinterpret_cast<float*>(smem + L.slot_a);  // per act slot: gate value, < 0 = stop
   // Per-neuron gate parameters of the slab, fetched before the dependency wait (parameters, like the weights), where
   // a neuron has several of them (LoPA: bias, fixed-matrix column and sign; int8 rows: bias and scale): the gate warps
@@ -462,9 +475,13 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
   const int n_gslots = cta < n_blocks ? (n_blocks - cta + G - 1) / G : 0;
   const int slab_rows =
       n_gslots == 0 ? 0 : (n_gslots - 1) * nr + min(nr, p.H - (cta + (n_gslots - 1) * G) * nr);
+  const int other = cta ^ 1, other_gslots = other < n_blocks ? (n_blocks - other + G - 1) / G : 0;  // the same of the pair's other CTA
+  const int other_rows =
+      !PAIR || other_gslots == 0 ? 0 : (other_gslots - 1) * nr + min(nr, p.H - (other + (other_gslots - 1) * G) * nr);
   auto slot_first_neuron = [&](int s) { return (cta + s * G) * nr; };
 
   if (warp < kGateProducers) {
+    if (PAIR) cluster_arrive();
     // ======================= gate producers ===================================================
     // Warp 0 sets up the barriers; both producer warps then start streaming at once (alternate
     // ring slots): the weights do not depend on anything earlier in the stream.
@@ -526,8 +543,16 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
     }
     __syncwarp();
     abort_grace(ctl);
+    if (PAIR) {
+      cluster_wait();
+      cluster_arrive();
+      cluster_wait();
+    }
     return;
   }
+  // Nothing is computed yet, in this CTA or the other of a pair, which may write here once both have arrived.
+  for (int i = tid - kStageBase; i < (PAIR ? 2 : 1) * p.slab_max; i += kStageThreads) row_state[i] = 0xffffffffu;
+  if (PAIR) cluster_arrive();
 
   // The token itself may still be written by the predecessor, so it is not read before the wait -- but its lines can
   // be asked into L2 (a hint: whatever is written later lands in the same L2), which turns the staging loads right
@@ -570,7 +595,6 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
   if (tid == kStageBase) SFFN_GSTAMP(11);
   // this call's number: the tag of the partials and of the LoPA exchange values
   const uint32_t ep = (LOPA || warp >= kFirstGateWarp) ? __ldcg(p.epoch_word) + 1u : 0u;
-  for (int i = tid - kStageBase; i < slab_rows; i += kStageThreads) row_state[i] = 0xffffffffu;
   constexpr int XEPV = Elem<X>::kPerVec;  // token elements per 16 bytes (the weights' EPV unless those are int8)
   // Quantised rows under a standard gate: the token is also split, 16 (int8) or 32 (int4) entries at a time -- the
   // entries one 16-byte chunk of a row meets -- into two int8 limbs and one scale per chunk:
@@ -718,6 +742,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
     if (lane == 0) wss[sw] = ss;
   }
   named_bar_sync(3, kThreads);
+  if (PAIR) cluster_wait();  // gate results may go to the other CTA from here on
   if (LOPA && use_rms) {
     // the warps' sums of squares, added in a fixed order by everyone
     float tot = 0.f;
@@ -960,7 +985,9 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
       const bool fired = z > 0.f;
       if (!p.dense && (fired || !p.flag_or) && SFFN_IN_BOUNDS(j0 + lane < p.H && r0 + lane < p.slab_max, p.status, 3))
         p.flag[j0 + lane] = fired ? 1 : 0;
-      row_state[r0 + lane] = fired ? __float_as_uint(fmaxf(activation(p.act, z), 0.f)) : 0x80000000u;
+      const uint32_t st = fired ? __float_as_uint(fmaxf(activation(p.act, z), 0.f)) : 0x80000000u;
+      row_state[r0 + lane] = st;
+      if (PAIR) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_dst + 4 * (r0 + lane)), "r"(st) : "memory");
     }
     __syncwarp();
     if (lane == 0 && (kLimbs || kLimbs4 || !ctl[kAbort])) {
@@ -971,6 +998,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
   };
 
   if (warp < kFirstGateWarp) {
+    if (PAIR) cluster_arrive();  // (no gate results from this warp)
     // ======================= act producers: rows of fired neurons, ascending ===================
     // Both walk the published gate results in the same order; producer 0 copies the W_up row of a
     // fired neuron, producer 1 its W_down row, into the same ring slot.
@@ -1035,9 +1063,13 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
     // the copies of the fired ones in ascending order.  Only the leading run of finished rows is
     // consumed, so the order never depends on which gate warp was faster.
     long long t_idle = 0;
-    for (int base = 0; ok && base < slab_rows;) {
-      const int row = base + lane;
-      const uint32_t st = row < slab_rows ? row_state[row] : 0x80000000u;
+    int n_fired = 0;  // of the pair's rows so far
+    const int n_scan = PAIR ? 2 * ((max(slab_rows, other_rows) + 15) & ~15) : slab_rows;
+    for (int base = 0; ok && base < n_scan;) {
+      // place base + lane of the scan: row `row` of this CTA, or of the pair's other one
+      const int at = base + lane, row = PAIR ? (at >> 5 << 4) + (at & 15) : at;
+      const bool own = !PAIR || ((at >> 4) & 1) == side, there = row < (own ? slab_rows : other_rows);
+      const uint32_t st = there ? (own ? row_state : peer_state)[row] : 0x80000000u;
       const unsigned done = __ballot_sync(0xffffffffu, st != 0xffffffffu);
       const int prefix = done == 0xffffffffu ? 32 : __ffs(~done) - 1;
       if (prefix == 0) {  // the next row's gate is not computed yet
@@ -1049,8 +1081,13 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
         continue;
       }
       t_idle = 0;
-      const bool take = row < slab_rows && lane < prefix && (p.dense || st != 0x80000000u);
+      bool take = there && lane < prefix && (p.dense || st != 0x80000000u);
       unsigned fired = __ballot_sync(0xffffffffu, take);
+      if (PAIR) {
+        take = take && ((n_fired + __popc(fired & ((1u << lane) - 1u))) & 1) == side;
+        n_fired += __popc(fired);
+        fired = __ballot_sync(0xffffffffu, take);
+      }
       // Every lane issues the copy of its own row into the ring slot of its place among the fired rows (one lane issuing
       // them one after the other manages a row every ~500 cycles, which is what bounds a call with a short gate).  Where
       // the ring is short (wide rows) a step takes the leading rows whose slots are free right now, and waits only when
@@ -1090,7 +1127,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
               slot_su[ms] = row_su[row];
               slot_sd[ms] = row_sd[row];
             }
-            size_t j = (size_t)(slot_first_neuron(row / nr) + row % nr);
+            size_t j = (size_t)(((own ? cta : other) + row / nr * G) * nr + row % nr);
             if (!SFFN_IN_BOUNDS(j < (size_t)p.H && ms >= 0 && ms < NR, p.status, 2)) j = 0;
             mbar_expect_tx(pfull + 8 * ms, (uint32_t)row_bytes);
             const uint32_t dst = GATED ? smem_u32(act_ring) + (uint32_t)(ms * row_bytes)
@@ -1155,6 +1192,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
       for (int s = gw; gw < p.gate_warps && s < n_gslots; s += p.gate_workers)
         if (!gate_slot(s)) break;
       if (lane == 0 && gw == (n_gslots - 1) % p.gate_workers) SFFN_STAMP(3);
+      if (PAIR) cluster_arrive();  // every gate result of this warp has gone out
     }
     // ======================= act warps =========================================================
     // (LoPA with three act groups: the four gate warps, done with the short gate, are the third group)
@@ -1170,6 +1208,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
         if (p.gate_warps + aw >= p.gate_workers || !gate_slot(s)) break;
       if (lane == 0 && p.gate_warps + aw == (n_gslots - 1) % p.gate_workers) SFFN_STAMP(3);
     }
+    if (PAIR && !gate_warp) cluster_arrive();
     float acc[CPT][EPV];
 #pragma unroll
     for (int i = 0; i < CPT; ++i)
@@ -1567,8 +1606,10 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
   // still carry an older call's number (bounded).  Thread (u, rg) takes two columns (one 16-byte unit) in the rows
   // rg, rg + RG, ...; the RG row groups are then added in order through shared memory.  The other CTAs leave at once
   // and their SMs take the next kernel of the stream.
+  // (pairs: nobody leaves before the other CTA's gate results have all arrived)
   if (warp < kFirstGateWarp) {  // act producers (the gate producers left long ago)
     abort_grace(ctl);
+    if (PAIR) cluster_wait();
     return;
   }
   constexpr int kTail = 32 * (kGW + kAW);
@@ -1586,6 +1627,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
   // between two threads' looks at it)
   if (slice < 0) {
     abort_grace(ctl);
+    if (PAIR) cluster_wait();
     return;
   }
   if (tt == 0) SFFN_GSTAMP(8);
@@ -1654,6 +1696,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
   }
   if (tt == 0) SFFN_GSTAMP(13);
   abort_grace(ctl);
+  if (PAIR) cluster_wait();
 }
 
 // ---- host side --------------------------------------------------------------------------------
@@ -1822,6 +1865,15 @@ int fused_grid(int sm_count, int H) {
   return grid > H ? H : grid;
 }
 
+// (PAIR: in the width that plan() gives the rows it is for)
+template <typename T>
+cudaError_t launch_pairs(const FusedParams& p, const Geometry& g, int grid, cudaStream_t s) {
+  auto k = fused_ffn_kernel<T, 8, true, false, true>;
+  static unsigned long long configured = 0;
+  const cudaError_t e = allow_dynamic_smem(k, kSmemBudget, configured);
+  return e != cudaSuccess ? e : launch_clusters(2, k, dim3(grid), dim3(kThreads), (size_t)g.smem, s, p);
+}
+
 template <typename T, bool LOPA, bool GATED = false>
 cudaError_t launch_main(const FusedParams& p, const Geometry& g, int grid, cudaStream_t s) {
   void (*k)(const FusedParams) = nullptr;
@@ -1904,6 +1956,20 @@ cudaError_t launch_fused(const FusedCall& c, cudaStream_t s, int* launched) {
     if (with.total <= kSmemBudget) g.smem = with.total;
     else gated = false;
   }
+  // Pairs of CTAs where a row of a fired neuron is long, so that the CTA with most of them is what a call waits for, and eight gate
+  // rows or more, so that it is not the gate: the two SMs of a pair start a call together, 1 us later than alone.  Alone / in pairs,
+  // firing 30 / 10 / 4 %: fp32, 4096 x 14336, r = 512 45.2 / 27.6 / 21.6 -> 42.1 / 26.3 / 21.5 us, r = 1024 47.7 / 31.4 / 30.0 -> 46.8 /
+  // 32.4 / 31.4; bf16, 8192 x 24000, r = 1024 67.9 / 40.7 / 36.4 -> 66.3 / 39.4 / 36.8, but 4096 x 14336, r = 512 26.7 / 18.6 / 15.5 ->
+  // 26.2 / 18.5 / 16.9; eight layers of fp32, 3840 x 14230, r = 480, 229 -> 215.
+  constexpr int kLongRow = 15 * 1024;
+  bool pairs = false;
+  if (lopa && (c.wkind == kWBF16 || c.wkind == kWF32) && grid % 2 == 0 && g.cpt == 8) {
+    const int row_bytes = c.D * 16 / weight_epv(c.wkind), gate_row_bytes = K * 16 / weight_epv(c.wkind);
+    const SmemLayout with(c.D, K, true, g.n_gate_slots, g.gate_slot_bytes, g.n_act_slots, g.act_slot_bytes, g.slab_max, false, g.act_extra,
+                          false, false, true);
+    pairs = row_bytes >= kLongRow && row_bytes >= 8 * gate_row_bytes && with.total <= kSmemBudget;
+    if (pairs) g.smem = with.total;
+  }
   char* ws = static_cast<char*>(c.workspace);
   int n = 0;
   cudaError_t e;
@@ -1935,10 +2001,12 @@ cudaError_t launch_fused(const FusedCall& c, cudaStream_t s, int* launched) {
   else if (c.wkind == kWQ4)
     e = lopa ? launch_main<q4_t, true>(p, g, grid, s) : launch_main<q4_t, false>(p, g, grid, s);
   else if (c.wkind == kWBF16)
-    e = lopa ? launch_main<__nv_bfloat16, true>(p, g, grid, s)
+    e = pairs ? launch_pairs<__nv_bfloat16>(p, g, grid, s)
+        : lopa ? launch_main<__nv_bfloat16, true>(p, g, grid, s)
              : gated ? launch_main<__nv_bfloat16, false, true>(p, g, grid, s) : launch_main<__nv_bfloat16, false>(p, g, grid, s);
   else
-    e = lopa ? launch_main<float, true>(p, g, grid, s)
+    e = pairs ? launch_pairs<float>(p, g, grid, s)
+        : lopa ? launch_main<float, true>(p, g, grid, s)
              : gated ? launch_main<float, false, true>(p, g, grid, s) : launch_main<float, false>(p, g, grid, s);
   if (e != cudaSuccess) return e;
   ++n;

@@ -1,0 +1,82 @@
+"""Single-token LoPA calls whose CTAs share out the rows of fired neurons in pairs (rows of 15 KB and more, a gate of short rows)."""
+import pytest
+import torch
+
+import synthetic_inputs as syn
+from parity import assert_active_set, assert_y_close, run_oracle
+
+DEV = "cuda:0"
+pytestmark = pytest.mark.gpu
+
+
+def make(m, D, H, r, dtype, s):
+    w = syn.lopa_ffn(D, H, r, dtype, 88, DEV, sparsity=s)
+    return {"V": w["V"], "U": w["U"], "g_idx": m.g_diagonal(H, D, DEV)}, w
+
+
+@pytest.mark.parametrize("D,H,r,dtype,s", [
+    (3840, 1531, 480, torch.float32, 0.9),    # slabs of unequal length
+    (3840, 300, 480, torch.float32, 0.5),     # two rows a CTA, CTAs without rows
+    (3840, 149, 64, torch.float32, 0.05),
+    (4096, 5003, 512, torch.float32, 0.97),
+    (4096, 5003, 512, torch.float32, 0.2),    # many rows a CTA: the rings wrap
+    (8192, 3001, 1024, torch.bfloat16, 0.8),
+])
+def test_pairs_share_the_fired_rows(D, H, r, dtype, s):
+    import paper_2609_31975_b200 as m
+
+    gate, w = make(m, D, H, r, dtype, s)
+    ffn = m.SparseFFN(D, H, dtype, r_max=r, B_max=1)
+    x = syn.tokens(3, D, dtype, 88, DEV)
+    ys = []
+    for t in (0, 1, 2, 0):
+        ys.append(ffn.sparse_ffn_forward(x[t], gate, w["b_g"], w["W_up"], w["W_down"], "relu").clone())
+        active = ffn.last_active()
+        torch.cuda.synchronize()
+        assert ffn.device_status() == 0, ffn.status_words()
+        ref = run_oracle(x[t:t + 1], gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+        tol = 1e-5 if dtype == torch.float32 else 1e-2  # fp32: sums of up to 5000 terms, in another order
+        assert_y_close(ys[-1], ref["y"][0], rel_l2=tol, max_abs=2 * tol, what=f"{D}x{H} r={r} token {t}")
+        assert_active_set(active, ref, what=f"{D}x{H} r={r} token {t}")
+    assert torch.equal(ys[0], ys[3])
+
+
+def test_pairs_do_every_row_of_a_dense_call_once():
+    import paper_2609_31975_b200 as m
+
+    gate, w = make(m, 3840, 700, 480, torch.float32, None)
+    ffn = m.SparseFFN(3840, 700, torch.float32, r_max=480, B_max=1)
+    x = syn.tokens(1, 3840, torch.float32, 88, DEV)[0]
+    hi = torch.full((700,), 1e3, device=DEV)
+    y = ffn.sparse_ffn_forward(x, gate, hi, w["W_up"], w["W_down"], "relu").clone()
+    assert torch.equal(y, ffn.dense_ffn_forward(x, gate, hi, w["W_up"], w["W_down"], "relu"))  # same rows, same order
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0
+
+
+@pytest.mark.parametrize("knob,value", [("skip_arrival_cta", 3), ("wait_cycles", 2000), ("wait_cycles", 20000)])
+def test_pairs_end_together_when_a_wait_runs_out(knob, value):
+    """A CTA that never hands in its sums, and budgets that run out in the middle of the call: a status, and a good call after a
+    reset."""
+    import paper_2609_31975_b200 as m
+
+    gate, w = make(m, 3840, 1531, 480, torch.float32, 0.9)
+    ffn = m.SparseFFN(3840, 1531, torch.float32, r_max=480, B_max=1)
+    x = syn.tokens(1, 3840, torch.float32, 88, DEV)[0]
+    args = (x, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+    want = ffn.sparse_ffn_forward(*args).clone()
+    torch.cuda.synchronize()
+    try:
+        m.test_set_knob("wait_cycles", 20_000_000)
+        m.test_set_knob(knob, value)
+        ffn.sparse_ffn_forward(*args)
+        torch.cuda.synchronize()
+        assert ffn.device_status() in ((5,) if knob == "skip_arrival_cta" else (0, 5))
+    finally:
+        m.test_set_knob("skip_arrival_cta", -1)
+        m.test_set_knob("wait_cycles", 0)
+    ffn.reset()
+    got = ffn.sparse_ffn_forward(*args)
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0
+    assert torch.equal(got, want)
