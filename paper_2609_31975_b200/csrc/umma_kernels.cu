@@ -404,25 +404,45 @@ __device__ __forceinline__ void expand_block(uint32_t raw, uint32_t dst, int row
 // receives [rows][128] bytes, each 16 x its code (the nibble moved to the upper half of the byte: exact, and the factor
 // goes into the row scale), in the same swizzled layout.  Thread t takes the 32 codes of quarter t % 4 of its rows: one
 // 16-byte load, two 16-byte stores; per word of eight nibbles two masks and two byte permutes.
+// kUnroll rows of a thread are in flight.  Tiles of more than 64 rows: eight, which is all that a thread has, one latency for a stage
+// instead of one a row (4096 x 14336, 5 / 24 tokens 47.0 / 62.6 -> 45.8 / 61.2 us, 8192 x 24000 102.6 / 149 -> 98.2 / 146; four in
+// flight gain a third of that).  Others, a kernel of their own: one, as more code to fetch costs them more (1024 x 3000, tiles of 24
+// rows, 5 tokens 23.2 / 23.6), and the LoPA gate, whose few stages come with the code of V x in the caches (4096 x 14336, r = 512, 2
+// tokens 36.0 / 37.8).
+constexpr int kTallTile = 64;
+template <int kUnroll>
 __device__ __forceinline__ void expand_block_q4_i8(uint32_t raw, uint32_t dst, int rows, int t, int nthr) {
   const int c = t & 3, step = nthr >> 2;
-  for (int row = t >> 2; row < rows; row += step) {
-    uint32_t w[4], o[8];
-    asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(raw + row * 64 + c * 16));
+#pragma unroll 1
+  for (int row0 = t >> 2; row0 < rows; row0 += kUnroll * step) {
+    uint32_t w[kUnroll][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const uint32_t ev = (w[i] << 4) & 0xf0f0f0f0u, od = w[i] & 0xf0f0f0f0u;  // even / odd columns, times 16
-      o[2 * i] = __byte_perm(ev, od, 0x5140);
-      o[2 * i + 1] = __byte_perm(ev, od, 0x7362);
+    for (int u = 0; u < kUnroll; ++u) {
+      const int row = row0 + u * step;
+      w[u][0] = w[u][1] = w[u][2] = w[u][3] = 0;
+      if (kUnroll == 1 || row < rows)
+        asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(w[u][0]), "=r"(w[u][1]), "=r"(w[u][2]), "=r"(w[u][3]) : "r"(raw + row * 64 + c * 16));
     }
-    const uint32_t drow = dst + row * 128;
-    const int sw = row & 7;
-    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(drow + (((2 * c) ^ sw) << 4)), "r"(o[0]), "r"(o[1]),
-                 "r"(o[2]), "r"(o[3])
-                 : "memory");
-    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(drow + (((2 * c + 1) ^ sw) << 4)), "r"(o[4]), "r"(o[5]),
-                 "r"(o[6]), "r"(o[7])
-                 : "memory");
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) {
+      const int row = row0 + u * step;
+      if (row >= rows) break;
+      uint32_t o[8];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t ev = (w[u][i] << 4) & 0xf0f0f0f0u, od = w[u][i] & 0xf0f0f0f0u;  // even / odd columns, times 16
+        o[2 * i] = __byte_perm(ev, od, 0x5140);
+        o[2 * i + 1] = __byte_perm(ev, od, 0x7362);
+      }
+      const uint32_t drow = dst + row * 128;
+      const int sw = row & 7;
+      asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(drow + (((2 * c) ^ sw) << 4)), "r"(o[0]), "r"(o[1]),
+                   "r"(o[2]), "r"(o[3])
+                   : "memory");
+      asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(drow + (((2 * c + 1) ^ sw) << 4)), "r"(o[4]), "r"(o[5]),
+                   "r"(o[6]), "r"(o[7])
+                   : "memory");
+    }
   }
 }
 // Makes this thread's shared-memory stores visible to the tensor core's reads.
@@ -557,7 +577,7 @@ __device__ __forceinline__ bool named_bar_any(int id, int threads, bool v) {
 enum RowsMode { kGate = 0, kUp = 1, kUpMayWalk = 2 };  // kUpMayWalk: wide batches, see walk_all below
 
 template <int MODE, int QB, bool EX = false, bool PAIR = false>
-__global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || QB == 4 || QB == 2) ? 32 * kExpandWarps : 0), 1) umma_rows_kernel(const UmmaRowsParams p,
+__global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || QB == 4 || QB == 2 || QB == 3) ? 32 * kExpandWarps : 0), 1) umma_rows_kernel(const UmmaRowsParams p,
                                                                   const __grid_constant__ CUtensorMap map_w,
                                                                   const __grid_constant__ CUtensorMap map_x,
                                                                   const __grid_constant__ WalkMap<MODE == kUpMayWalk> map_t) {
@@ -579,12 +599,14 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const uint32_t ready = smem_u32(bars + 2 * kMaxStages + 4);  // quantised rows: slot t of the bf16 ring is written ...
   const uint32_t afree = ready + 8 * kExpandSlots;             // ... and has been read by its MMAs
-  constexpr int kRawRow = QB == 2 ? 64 : 8 * QB;               // bytes of the codes of one K block (as copied)
+  // QB = 3: the same for tall tiles (see expand_block_q4_i8).
+  constexpr bool kI4 = QB == 2 || QB == 3;
+  constexpr int kRawRow = kI4 ? 64 : 8 * QB;                   // bytes of the codes of one K block (as copied)
   // QB = 1: int8 rows and the tokens as int8 limbs (four per token, see token_limbs_kernel) go straight into
   // kind::i8 MMAs with int32 accumulators: nothing to expand, a K block is 128 codes.  QB = 8 / 4: codes expanded
   // to bf16 by four more warps.
   // QB = 2: int4 rows expanded to int8 (16 x the code, a byte each) for the same kind::i8 MMAs.
-  constexpr bool kNat = QB == 1 || QB == 2, kExp = QB == 8 || QB == 4 || QB == 2, kQ = QB != 0;
+  constexpr bool kNat = QB == 1 || kI4, kExp = QB == 8 || QB == 4 || kI4, kQ = QB != 0;
   constexpr int kAtomElems = kNat ? 128 : kAtomK;              // elements of one 128-byte swizzle row
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -794,7 +816,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
     // everything that does not depend on the accumulator is fetched before the wait
     if (MODE == kGate) pdl_wait();  // before the first read of a buffer an earlier kernel may write, and the first store
     float bias = 0.f, sg = 1.f;
-    const float sc = ((kQ && row_ok && p.w_scale) ? p.w_scale[j] : 1.f) * (QB == 2 ? 0.0625f : 1.f);  // scale of the weight row
+    const float sc = ((kQ && row_ok && p.w_scale) ? p.w_scale[j] : 1.f) * (kI4 ? 0.0625f : 1.f);  // scale of the weight row
     const float osc = (kQ && UP && row_ok && p.out_scale) ? p.out_scale[j] : 1.f;  // scale of the down row, folded into Hm
     int gi = -1;
     if (!UP) {
@@ -1040,7 +1062,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
           const int k0 = (kb_first + kb * atoms + a) * kAtomElems;
           // where the weight block lands, the byte column it starts at, and the bytes of one landed row
           const uint32_t wdst = abase + w_off + a * (kExp ? raw_block_bytes : a_block_bytes);
-          const int wc0 = QB == 2 ? k0 / 2 : kExp ? k0 * QB / 8 : k0;
+          const int wc0 = kI4 ? k0 / 2 : kExp ? k0 * QB / 8 : k0;
           const int wrow = kExp ? kRawRow : 128;
           if (with_w && !(MODE == kGate && blockIdx.x == 0 && it == p.drop_stage)) {  // test hook: a copy that never comes
             if (UP && !walk_all) {
@@ -1088,7 +1110,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
       const uint32_t src = ring0 + s * stage_bytes + w_off, dst = stage0 + t * a_bytes;
       const int na = min(atoms, kblocks - kb * atoms);
       for (int a = 0; a < na; ++a)
-        if (QB == 2) expand_block_q4_i8(src + a * raw_block_bytes, dst + a * a_block_bytes, tile_rows, et, 16 * kExpandWarps);
+        if (kI4) expand_block_q4_i8<QB == 3 ? 8 : 1>(src + a * raw_block_bytes, dst + a * a_block_bytes, tile_rows, et, 16 * kExpandWarps);
         else expand_block<(QB == 8 || QB == 4) ? QB : 8>(src + a * raw_block_bytes, dst + a * a_block_bytes, tile_rows, et, 16 * kExpandWarps);
       fence_proxy_async();
       __syncwarp();
@@ -1944,9 +1966,10 @@ cudaError_t launch_rows_mode(const UmmaRowsParams& p, dim3 grid, size_t smem, cu
     return launch_pdl(k, grid, dim3(kThreadsRows), smem, s, p, map_w, map_x, map_t);
   }
   if (p.qbits == 2) {
-    static unsigned long long configured2 = 0;
-    auto k = umma_rows_kernel<MODE, 2>;
-    if ((e = allow_dynamic_smem(k, 227 * 1024, configured2)) != cudaSuccess) return e;
+    static unsigned long long configured2[2] = {0, 0};
+    const bool tall = p.K > kShortRow && tile_rows_for(p.R, grid.x, p.equal_max) > kTallTile;
+    auto k = tall ? umma_rows_kernel<MODE, 3> : umma_rows_kernel<MODE, 2>;
+    if ((e = allow_dynamic_smem(k, 227 * 1024, configured2[tall])) != cudaSuccess) return e;
     return launch_pdl(k, grid, dim3(kThreadsRows + 32 * kExpandWarps), smem, s, p, map_w, map_x, map_t);
   }
   if (p.qbits == 8) {
