@@ -333,13 +333,25 @@ __device__ __forceinline__ void tma_gather4(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
+// Eight 4-bit codes of a word as bf16: o[i] holds codes i and i + 4, which are the halves of one shift and mask.  Under the exponent
+// of 128 the nibble ^ 8 reads 136 + code, and 136 is subtracted from both at once.
+__device__ __forceinline__ void q4_halves(uint32_t w, uint32_t* o) {
+  const __nv_bfloat162 bias = __halves2bfloat162(__ushort_as_bfloat16(0x4308), __ushort_as_bfloat16(0x4308));
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t both = ((w >> (4 * i)) & 0x000f000fu) ^ 0x43084308u;
+    const __nv_bfloat162 v = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&both), bias);
+    o[i] = *reinterpret_cast<const uint32_t*>(&v);
+  }
+}
+
 // Expands a block of weight codes to bf16: `raw` holds [rows][64] codes (QB = 8: a byte each, +-127; QB = 4: two's-
 // complement nibbles, even column in the low nibble), `dst` (1024-byte aligned) receives [rows][64] bf16 in the
 // 128-byte-swizzled K-major layout (16-byte chunk c of row i at i * 128 + ((c ^ (i & 7)) * 16)).  Thread t of nthr
 // takes the 16-code quarter t % 4 of rows t / 4, t / 4 + nthr / 4, ... (four of them in flight): a quarter warp reads two whole raw rows
-// and writes chunks of two rows that share no bank.  A code c becomes the fp32 2^23 + (c + bias) by a byte
-// permute, the bias and 2^23 are subtracted exactly, and the upper half of that fp32 is the bf16.
-template <int QB>
+// and writes chunks of two rows that share no bank.  An int8 code c becomes the fp32 2^23 + (c + bias) by a byte
+// permute, the bias and 2^23 are subtracted exactly, and the upper half of that fp32 is the bf16.  ALL: rows = nthr, four a thread.
+template <int QB, bool ALL = false>
 __device__ __forceinline__ void expand_block(uint32_t raw, uint32_t dst, int rows, int t, int nthr) {
   constexpr int kRawRow = 8 * QB;  // bytes of 64 codes
   constexpr int kUnroll = 4;       // rows of one thread in flight
@@ -351,7 +363,7 @@ __device__ __forceinline__ void expand_block(uint32_t raw, uint32_t dst, int row
       const int row = row0 + u * step;
       const uint32_t src = raw + row * kRawRow + c * (kRawRow / 4);
       w[u][0] = w[u][1] = w[u][2] = w[u][3] = 0;
-      if (row < rows) {
+      if (ALL || row < rows) {
         if (QB == 8) {
           asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];"
                        : "=r"(w[u][0]), "=r"(w[u][1]), "=r"(w[u][2]), "=r"(w[u][3])
@@ -364,30 +376,26 @@ __device__ __forceinline__ void expand_block(uint32_t raw, uint32_t dst, int row
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
       const int row = row0 + u * step;
-      if (row >= rows) break;
+      if (!ALL && row >= rows) break;
+      uint32_t o[8];  // o[i] = codes 2i, 2i+1 of the quarter
       if (QB == 4) {
-        const uint32_t a = w[u][0] ^ 0x88888888u, b = w[u][1] ^ 0x88888888u;
-        // bytes of w[2i]: even columns of word i, of w[2i+1]: odd columns
-        w[u][0] = a & 0x0f0f0f0fu; w[u][1] = (a >> 4) & 0x0f0f0f0fu;
-        w[u][2] = b & 0x0f0f0f0fu; w[u][3] = (b >> 4) & 0x0f0f0f0fu;
-      }
-      uint32_t o[8];
-      const float off = QB == 8 ? 8388736.f : 8388616.f;  // 2^23 + 128, 2^23 + 8
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        // o[i] = codes 2i, 2i+1 of the quarter
-        uint32_t lo, hi;
-        if (QB == 8) {
-          const uint32_t v = w[u][i >> 1] ^ 0x80808080u;
-          lo = __byte_perm(v, 0x4b000000u, (i & 1) ? 0x7442 : 0x7440);
-          hi = __byte_perm(v, 0x4b000000u, (i & 1) ? 0x7443 : 0x7441);
-        } else {
-          const uint32_t sel = 0x7440 + (i & 3);
-          lo = __byte_perm(w[u][(i >> 2) * 2], 0x4b000000u, sel);
-          hi = __byte_perm(w[u][(i >> 2) * 2 + 1], 0x4b000000u, sel);
+        for (int q = 0; q < 2; ++q) {
+          uint32_t h[4];
+          q4_halves(w[u][q], h);
+          o[4 * q] = __byte_perm(h[0], h[1], 0x5410);
+          o[4 * q + 1] = __byte_perm(h[2], h[3], 0x5410);
+          o[4 * q + 2] = __byte_perm(h[0], h[1], 0x7632);
+          o[4 * q + 3] = __byte_perm(h[2], h[3], 0x7632);
         }
-        const float fl = __uint_as_float(lo) - off, fh = __uint_as_float(hi) - off;
-        o[i] = __byte_perm(__float_as_uint(fl), __float_as_uint(fh), 0x7632);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const uint32_t v = w[u][i >> 1] ^ 0x80808080u;
+          const uint32_t lo = __byte_perm(v, 0x4b000000u, (i & 1) ? 0x7442 : 0x7440), hi = __byte_perm(v, 0x4b000000u, (i & 1) ? 0x7443 : 0x7441);
+          const float2 f = add2(make_float2(__uint_as_float(lo), __uint_as_float(hi)), make_float2(-8388736.f, -8388736.f));  // 2^23 + 128
+          o[i] = __byte_perm(__float_as_uint(f.x), __float_as_uint(f.y), 0x7632);
+        }
       }
       const uint32_t drow = dst + row * 128;
       const int sw = row & 7;
@@ -396,6 +404,31 @@ __device__ __forceinline__ void expand_block(uint32_t raw, uint32_t dst, int row
                    : "memory");
       asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(drow + (((2 * c + 1) ^ sw) << 4)), "r"(o[4]), "r"(o[5]),
                    "r"(o[6]), "r"(o[7])
+                   : "memory");
+    }
+    if (ALL) break;
+  }
+}
+// int4 codes for the down projection, whose columns are the rows m of the MMA and may come in the order of q4_halves, which its
+// epilogue undoes: m = 8 k + 2 i + h holds column 8 k + i + 4 h.  64 rows of 64 codes.  (1.4 instructions a code, where fp32 and
+// columns in order took 3: 4096 x 14336, 5 / 64 tokens 45.8 / 87.5 -> 45.0 / 83.9 us, 8192 x 24000, 24 tokens 146 -> 139.)
+__device__ __forceinline__ int column_of_row(int m) { return (m & ~7) + ((m & 7) >> 1) + ((m & 1) << 2); }
+__device__ __forceinline__ void expand_block_q4_mn(uint32_t raw, uint32_t dst, int t) {
+  constexpr int kRows = kAtomK, kStep = 32 * kExpandWarps / 2 / 4, kUnroll = kRows / kStep;  // by a pair of warps, all rows in flight
+  const int c = t & 3;
+  uint32_t w[kUnroll][2];
+#pragma unroll
+  for (int u = 0; u < kUnroll; ++u)
+    asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(w[u][0]), "=r"(w[u][1]) : "r"(raw + ((t >> 2) + u * kStep) * 32 + c * 8));
+#pragma unroll
+  for (int u = 0; u < kUnroll; ++u) {
+    const int row = (t >> 2) + u * kStep, sw = row & 7;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      uint32_t o[4];
+      q4_halves(w[u][q], o);
+      asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst + row * 128 + (((2 * c + q) ^ sw) << 4)), "r"(o[0]), "r"(o[1]),
+                   "r"(o[2]), "r"(o[3])
                    : "memory");
     }
   }
@@ -1456,8 +1489,14 @@ __global__ void __launch_bounds__(down_bound(QB, EX), EX ? 1 : 2) umma_down_kern
       if (!__all_sync(0xffffffffu, ok)) break;
       const uint32_t raw = stage0 + s * stage_bytes + raw_off;
       const uint32_t dst = kTwo ? expand0 + e * kAAtomBytes : stage0 + s * stage_bytes;
-      expand_block<QB ? QB : 8>(raw, dst, kAtomK, et, 16 * kExpandWarps);
-      expand_block<QB ? QB : 8>(raw + kRawBytes / 2, dst + kAAtomBytes / 2, kAtomK, et, 16 * kExpandWarps);
+      if constexpr (QB == 4) {
+        expand_block_q4_mn(raw, dst, et);
+        expand_block_q4_mn(raw + kRawBytes / 2, dst + kAAtomBytes / 2, et);
+      } else {
+        static_assert(kAtomK == 16 * kExpandWarps, "four rows a thread");
+        expand_block<8, true>(raw, dst, kAtomK, et, 16 * kExpandWarps);
+        expand_block<8, true>(raw + kRawBytes / 2, dst + kAAtomBytes / 2, kAtomK, et, 16 * kExpandWarps);
+      }
       fence_proxy_async();
       __syncwarp();
       if (lane == 0) mbar_arrive(ready + 8 * (kTwo ? e : s));
@@ -1520,7 +1559,8 @@ __global__ void __launch_bounds__(down_bound(QB, EX), EX ? 1 : 2) umma_down_kern
   const int B = p.B;
   {
     const int ew = warp & 3;
-    float* mine = clustered ? sums + ew * 32 + lane : p.partial + (size_t)sp * B * p.D + d0 + ew * 32 + lane;
+    const int col = QB == 4 ? column_of_row(ew * 32 + lane) : ew * 32 + lane;
+    float* mine = clustered ? sums + col : p.partial + (size_t)sp * B * p.D + d0 + col;
     const size_t pitch = clustered ? kTileRows : p.D;
     const uint32_t taddr = tmem_base + ((uint32_t)(ew * 32) << 16);
     if constexpr (EX) {
