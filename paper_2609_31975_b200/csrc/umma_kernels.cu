@@ -36,7 +36,7 @@
 // Up to 256 token columns go through in one pass.  Wide batches (npad > 128) leave room for two accumulators and a ring
 // of four stages of ~40 KB (two with expanded codes and 241 columns or more), too few for the token rows that every CTA reads again
 // (200 tokens x 4096: 1.6 MB a CTA through L2 beside 0.8 MB of weights).  There the rows kernels run in pairs of CTAs that hold half
-// of the token rows each (PAIR, see rows_pairs): 200 tokens, 4096 x 14336, bf16: 112 us in one pass, 130 without pairs.
+// of the token rows each (PAIR, see rows_pairs): 200 tokens, 4096 x 14336, bf16: 130 us without pairs, 112 with them.
 // Every wait is bounded by a cycle budget; on expiry the status word is set, all roles wind down and the TMEM
 // columns are released before the CTA exits.
 #include "umma_kernels.cuh"
@@ -1335,7 +1335,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
 // the contraction runs over list rows, so the gathered W_down rows are the MN-major A operand (each
 // gathered row delivers 64 contiguous d per swizzle row) and HmT[b][u] is the K-major B operand.
 // Same pipeline as above: 4 producer warps (gather4 per lane: 2 column halves x 16 row quads = one 64-row
-// stage), 2 MMA issuers with their own accumulators, 4 epilogue warps; two CTAs share an SM.
+// stage), 2 MMA issuers with their own accumulators, 4 epilogue warps, which the producers join; two CTAs share an SM.
 // Threads, rounded up to whole warps for each scheduler: registers are handed out by scheduler, and two CTAs of 14 warps with 72
 // registers a thread, which fit an SM's file, do not fit those of the first two (int4 rows ran in two waves of CTAs).
 constexpr int down_bound(int qb, bool exact) { return ((exact ? 512 : kThreads) + (qb ? 32 * kExpandWarps : 0) + 127) / 128 * 128; }
