@@ -657,7 +657,7 @@ int run(sffn_handle* h, const void* x, int B, const sffn_gate* g, const float* b
   // 128 from a few tokens on (see h_terms_for and odd_width_tokens); a LoPA rank of a multiple of 64.
   // Larger batches are cut into passes of as many tokens as one launch chain holds: a pass reads every gate row and the
   // rows of its own union, so fewer passes read fewer bytes (bf16, 4096 x 14336, 200 tokens: 4 passes of 64 took 333 us, one
-  // takes 137).  The mma.sync kernels (selected, or a bf16 LoPA rank that is no multiple of 64) take passes of 64 and rows
+  // takes 100).  The mma.sync kernels (selected, or a bf16 LoPA rank that is no multiple of 64) take passes of 64 and rows
   // of a multiple of 256 elements.
   const bool umma_ok = h->path != SFFN_PATH_MMA_SYNC && sffn::umma_rows_supported(gate_k, 1) &&
                        sffn::umma_rows_supported(h->D, 1) && sffn::umma_down_supported(h->D, 1) &&
@@ -665,6 +665,8 @@ int run(sffn_handle* h, const void* x, int B, const sffn_gate* g, const float* b
   const int pass_max = umma_ok ? umma_pass_tokens(h->D, gate_k, q8 != nullptr, lopa_gate) : kMaxMmaTokens;
   const bool tensor_batch = h->dtype == SFFN_BF16 && B >= 2 && h->path != SFFN_PATH_GENERAL && h->path != SFFN_PATH_FUSED &&
                             (umma_ok || (!q8 && sffn::batched_mma_supported(h->D, gate_k, 1)));
+  // Asked for by name, the fused path takes the 4-bit LoPA rows that it always took; narrower ones are for the automatic choice.
+  if (h->path == SFFN_PATH_FUSED && wkind == sffn::kWQ4 && g->kind == SFFN_GATE_LOPA && h->D <= 896) return SFFN_ERR_UNSUPPORTED;
   // Any other batch (fp32 operands, a row width the tensor-core kernels do not tile, SFFN_PATH_FUSED): the single-token
   // kernel once per token, where it serves the shape.  The CUDA-core batch kernels are slower than B single-token calls
   // (int8, 4096 x 14336, B = 16: 1.66 ms against 0.33 ms; bf16 rows of 4000 elements: 1.03 ms against 0.46 ms; fp32:

@@ -1759,6 +1759,9 @@ Geometry plan(int wkind, int D, int H, int K, bool lopa, int grid) {
   g.rows_per_gate_slot = nr;
   g.gate_slot_bytes = (nr * gate_row_bytes + 127) / 128 * 128;
   g.act_slot_bytes = (2 * row_bytes + 127) / 128 * 128;
+  // LoPA: the act groups' sums, which meet in the act ring, must fit sixteen slots of it (4-bit rows of less than 1024 codes: 512 x
+  // 1500, r = 64 took the CUDA-core path's 44.6 us, 12.5 here)
+  if (lopa && wkind == kWQ4 && D >= 256 && 16 * g.act_slot_bytes < g.cpt * epv * act_threads * 4) g.act_slot_bytes = g.cpt * epv * act_threads * 4 / 16;
   g.slab_max = (((H + nr - 1) / nr + grid - 1) / grid) * nr;  // most rows one CTA can own
   const bool limbs = (wkind == kWQ8 || wkind == kWQ4) && !lopa;
   const SmemLayout fixed(D, K, lopa, 0, 0, 0, 0, g.slab_max, scaled, 0, false, limbs);
