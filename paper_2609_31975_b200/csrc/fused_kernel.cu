@@ -165,6 +165,16 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
 // The barrier of a pair of CTAs: thread by thread, first all arrive, then all wait.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// A word of the other CTA's shared memory (`addr` from mapa), and a look at one that it may be writing.  Both name the cluster: between
+// CTAs a plain store that a load runs into is a data race, whatever its size.  Nothing else is published by the word.
+__device__ __forceinline__ void st_peer(uint32_t addr, uint32_t v) {
+  asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t ld_pair(uint32_t words, int i) {
+  uint32_t v;
+  asm volatile("ld.relaxed.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(words + 4 * i) : "memory");
+  return v;
+}
 // Whether a phase has completed, without waiting for it.
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
   uint32_t ok;
@@ -424,9 +434,9 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
   // (a fence in the producers would also wait for their bulk copies in flight).
   volatile uint32_t* row_state = reinterpret_cast<volatile uint32_t*>(smem + L.aval);
   const int side = cta & 1;
-  volatile uint32_t* peer_state = row_state + p.slab_max;
+  const uint32_t states = smem_u32(smem + L.aval);  // the same words; PAIR: the other CTA's follow
   uint32_t peer_dst = 0;  // where the other CTA keeps this one's
-  if (PAIR) asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer_dst) : "r"(smem_u32(smem + L.aval) + 4 * p.slab_max), "r"(side ^ 1));
+  if (PAIR) asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer_dst) : "r"(states + 4 * p.slab_max), "r"(side ^ 1));
   float* slot_a = reinterpret_cast<float*>(smem + L.slot_a);  // per act slot: gate value, < 0 = stop
   // Per-neuron gate parameters of the slab, fetched before the dependency wait (parameters, like the weights), where
   // a neuron has several of them (LoPA: bias, fixed-matrix column and sign; int8 rows: bias and scale): the gate warps
@@ -987,7 +997,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
         p.flag[j0 + lane] = fired ? 1 : 0;
       const uint32_t st = fired ? __float_as_uint(fmaxf(activation(p.act, z), 0.f)) : 0x80000000u;
       row_state[r0 + lane] = st;
-      if (PAIR) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_dst + 4 * (r0 + lane)), "r"(st) : "memory");
+      if (PAIR) st_peer(peer_dst + 4 * (r0 + lane), st);
     }
     __syncwarp();
     if (lane == 0 && (kLimbs || kLimbs4 || !ctl[kAbort])) {
@@ -1069,7 +1079,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
       // place base + lane of the scan: row `row` of this CTA, or of the pair's other one
       const int at = base + lane, row = PAIR ? (at >> 5 << 4) + (at & 15) : at;
       const bool own = !PAIR || ((at >> 4) & 1) == side, there = row < (own ? slab_rows : other_rows);
-      const uint32_t st = there ? (own ? row_state : peer_state)[row] : 0x80000000u;
+      const uint32_t st = !there ? 0x80000000u : PAIR ? ld_pair(own ? states : states + 4 * p.slab_max, row) : row_state[row];
       const unsigned done = __ballot_sync(0xffffffffu, st != 0xffffffffu);
       const int prefix = done == 0xffffffffu ? 32 : __ffs(~done) - 1;
       if (prefix == 0) {  // the next row's gate is not computed yet
