@@ -316,7 +316,9 @@ const char* sffn_status_string(int status);
  *
  * sffn_test_fused_plan: geometry of the single-token CUDA-core kernel for a shape, as nine integers: ok, rows per
  *   gate slot, gate slot bytes, gate slots, gate warps, act slot bytes, act slots, chunks per act thread, shared
- *   memory bytes (wkind: 0 fp32, 1 bf16, 2 int8 rows).  sffn_test_umma_tiling: tiling of the batched gate GEMM over short
+ *   memory bytes (wkind: 0 fp32, 1 bf16, 2 int8 rows).  sffn_test_fused_pairs: 1 = a single-token LoPA call of rank r goes
+ *   to the kernel of pairs of CTAs on a device that runs at_once pairs at once (-1: the current device, as a call does).
+ *   sffn_test_umma_tiling: tiling of the batched gate GEMM over short
  *   rows; sffn_test_umma_row_tiling: over rows of K elements; sffn_test_umma_pass_tiling: over rows of K elements (qbits 0:
  *   bf16) or codes (8 / 4; 1 / 2: against limbs) in a pass of B tokens.  sffn_test_umma_k_splits: runs of K and tiles of
  *   rows of V x, R rows of K elements (limbs: codes) against B tokens, at most max_splits runs.
@@ -339,14 +341,18 @@ const char* sffn_status_string(int status);
  *                       overwrites the first entry of its list of fired neurons with a number far beyond H before
  *                       the up / down kernel reads it, so that the kernel's index check has something to find (it
  *                       records SFFN_ERR_BOUNDS and takes row 0 instead; the bad index is never used as an address)
+ *   CLUSTER_QUERY_FAILS 1 = the runtime has no answer to how many clusters of CTAs the device runs at once: the kernels that
+ *                       have to know take the form without them (default 0)
  *   TRACE_BUFFER        device address of [grid][16] int64 time stamps, written only by libraries built with
  *                       -DSFFN_TRACE (0 = none) */
 typedef enum {
   SFFN_KNOB_PDL = 0, SFFN_KNOB_TENSOR_GATE = 1, SFFN_KNOB_WAIT_CYCLES = 2, SFFN_KNOB_SKIP_ARRIVAL_CTA = 3,
   SFFN_KNOB_RING_GATE_SLOTS = 4, SFFN_KNOB_RING_ACT_SLOTS = 5, SFFN_KNOB_TRACE_BUFFER = 6,
-  SFFN_KNOB_RING_PARKED_STAGES = 7, SFFN_KNOB_L2_HINTS = 8, SFFN_KNOB_DROP_STAGE = 9, SFFN_KNOB_POISON_LIST = 10
+  SFFN_KNOB_RING_PARKED_STAGES = 7, SFFN_KNOB_L2_HINTS = 8, SFFN_KNOB_DROP_STAGE = 9, SFFN_KNOB_POISON_LIST = 10,
+  SFFN_KNOB_CLUSTER_QUERY_FAILS = 11
 } sffn_test_knob;
 void sffn_test_fused_plan(int wkind, int D, int H, int K, int lopa, int sm_count, int* out9);
+int sffn_test_fused_pairs(int wkind, int D, int H, int r, int sm_count, int at_once);
 void sffn_test_umma_tiling(int R, int sm_count, int* tile_rows, int* n_tiles, int* own_list);
 void sffn_test_umma_row_tiling(int R, int K, int sm_count, int* tile_rows, int* n_tiles, int* own_list);
 void sffn_test_umma_pass_tiling(int R, int K, int qbits, int B, int sm_count, int* tile_rows, int* n_tiles, int* own_list);

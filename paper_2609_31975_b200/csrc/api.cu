@@ -200,6 +200,9 @@ int sffn_set_path(sffn_handle* h, int path) {
 void sffn_test_fused_plan(int wkind, int D, int H, int K, int lopa, int sm_count, int* out9) {
   sffn::debug_fused_plan(wkind, D, H, K, lopa != 0, sm_count, out9);  // wkind: 0 fp32, 1 bf16, 2 int8 rows
 }
+int sffn_test_fused_pairs(int wkind, int D, int H, int r, int sm_count, int at_once) {
+  return sffn::debug_fused_pairs(wkind, D, H, r, sm_count, at_once) ? 1 : 0;
+}
 void sffn_test_umma_tiling(int R, int sm_count, int* tile_rows, int* n_tiles, int* own_list) {
   sffn_test_umma_row_tiling(R, 0, sm_count, tile_rows, n_tiles, own_list);
 }
@@ -232,6 +235,7 @@ int sffn_test_set_knob(int knob, long long value) {
 #else
       return value ? SFFN_ERR_UNSUPPORTED : SFFN_OK;
 #endif
+    case SFFN_KNOB_CLUSTER_QUERY_FAILS: sffn::cluster_query_fails() = value != 0; return SFFN_OK;
     case SFFN_KNOB_TRACE_BUFFER: k.trace = reinterpret_cast<long long*>(static_cast<uintptr_t>(value)); return SFFN_OK;
     default: return SFFN_ERR_INVALID_ARG;
   }

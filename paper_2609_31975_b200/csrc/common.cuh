@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace sffn {
 
 // Debug builds (-DSFFN_DEBUG, `python -m paper_2609_31975_b200.build --debug`): an index that is about to address
@@ -268,6 +270,12 @@ inline bool& pdl_enabled() {
   return on;
 }
 
+// Test hook: true = the question how many clusters fit the device finds no answer.
+inline bool& cluster_query_fails() {
+  static bool fails = false;
+  return fails;
+}
+
 // Raises a kernel's dynamic shared-memory limit once per device (the attribute belongs to the device's copy of
 // the kernel); `done` holds one bit per device ordinal.
 template <typename K>
@@ -307,6 +315,32 @@ cudaError_t launch_clusters(int cluster, void (*k)(KArgs...), dim3 grid, dim3 bl
   cfg.attrs = attr;
   cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, k, args...);
+}
+// How many clusters of `size` blocks (this many threads, this much dynamic shared memory) of a kernel the current device runs at
+// once: it depends on how many SMs each of its GPCs has.  0 where it cannot be told, and then asked again by the next call.  An
+// answer is kept for each device (`known`: 0 = none yet, else the answer + 1).
+constexpr int kKnownDevices = 64;
+template <typename K>
+int clusters_at_once(K kernel, int size, int threads, int smem, unsigned long long& configured, std::atomic<int>* known) {
+  int dev = 0, n = 0;
+  if (cluster_query_fails() || cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if (dev < kKnownDevices && (n = known[dev].load(std::memory_order_relaxed)) != 0) return n - 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(size);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = size;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (allow_dynamic_smem(kernel, smem, configured) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  if (dev < kKnownDevices) known[dev].store(n + 1, std::memory_order_relaxed);
+  return n;
 }
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {

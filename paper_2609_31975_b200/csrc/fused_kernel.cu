@@ -1886,6 +1886,33 @@ cudaError_t launch_pairs(const FusedParams& p, const Geometry& g, int grid, cuda
   const cudaError_t e = allow_dynamic_smem(k, kSmemBudget, configured);
   return e != cudaSuccess ? e : launch_clusters(2, k, dim3(grid), dim3(kThreads), (size_t)g.smem, s, p);
 }
+template <typename T>
+int pairs_at_once() {
+  static unsigned long long configured = 0;
+  static std::atomic<int> known[kKnownDevices];
+  return clusters_at_once(fused_ffn_kernel<T, 8, true, false, true>, 2, kThreads, kSmemBudget, configured, known);
+}
+
+// Whether a LoPA call goes to the kernel of pairs, and the shared memory that takes.  `at_once`: pairs that the device runs at once,
+// -1 = it is asked.  They have to be all of the call's: its CTAs wait for one another (the exchange of V x), so a device whose GPCs
+// leave some of them no second SM takes the kernel without pairs.
+// Pairs of CTAs where a row of a fired neuron is long, so that the CTA with most of them is what a call waits for, and eight gate
+// rows or more, so that it is not the gate: the two SMs of a pair start a call together, 1 us later than alone.  Alone / in pairs,
+// firing 30 / 10 / 4 %: fp32, 4096 x 14336, r = 512 45.2 / 27.6 / 21.6 -> 42.1 / 26.3 / 21.5 us, r = 1024 47.7 / 31.4 / 30.0 -> 46.8 /
+// 32.4 / 31.4; bf16, 8192 x 24000, r = 1024 67.9 / 40.7 / 36.4 -> 66.3 / 39.4 / 36.8, but 4096 x 14336, r = 512 26.7 / 18.6 / 15.5 ->
+// 26.2 / 18.5 / 16.9; eight layers of fp32, 3840 x 14230, r = 480, 229 -> 215.
+bool in_pairs(const Geometry& g, int wkind, int D, int K, int grid, int at_once, int* smem) {
+  constexpr int kLongRow = 15 * 1024;
+  if ((wkind != kWBF16 && wkind != kWF32) || grid % 2 || g.cpt != 8) return false;
+  const int row_bytes = D * 16 / weight_epv(wkind), gate_row_bytes = K * 16 / weight_epv(wkind);
+  const SmemLayout with(D, K, true, g.n_gate_slots, g.gate_slot_bytes, g.n_act_slots, g.act_slot_bytes, g.slab_max, false, g.act_extra,
+                        false, false, true);
+  if (row_bytes < kLongRow || row_bytes < 8 * gate_row_bytes || with.total > kSmemBudget) return false;
+  if (at_once < 0) at_once = wkind == kWBF16 ? pairs_at_once<__nv_bfloat16>() : pairs_at_once<float>();
+  if (2 * at_once < grid) return false;
+  *smem = with.total;
+  return true;
+}
 
 template <typename T, bool LOPA, bool GATED = false>
 cudaError_t launch_main(const FusedParams& p, const Geometry& g, int grid, cudaStream_t s) {
@@ -1935,6 +1962,12 @@ void debug_fused_plan(int wkind, int D, int H, int K, bool lopa, int sm_count, i
   for (int i = 0; i < 9; ++i) out[i] = v[i];
 }
 
+bool debug_fused_pairs(int wkind, int D, int H, int r, int sm_count, int at_once) {
+  const int grid = fused_grid(sm_count, H);
+  Geometry g = plan(wkind, D, H, r, true, grid);
+  return g.ok && in_pairs(g, wkind, D, r, grid, at_once, &g.smem);
+}
+
 // Whether this call's gate goes to the tensor cores (see sffn_set_gate_engine).
 static bool wants_tensor_gate(const FusedCall& c) {
   const int knob = fused_test_knobs().tensor_gate;
@@ -1969,20 +2002,7 @@ cudaError_t launch_fused(const FusedCall& c, cudaStream_t s, int* launched) {
     if (with.total <= kSmemBudget) g.smem = with.total;
     else gated = false;
   }
-  // Pairs of CTAs where a row of a fired neuron is long, so that the CTA with most of them is what a call waits for, and eight gate
-  // rows or more, so that it is not the gate: the two SMs of a pair start a call together, 1 us later than alone.  Alone / in pairs,
-  // firing 30 / 10 / 4 %: fp32, 4096 x 14336, r = 512 45.2 / 27.6 / 21.6 -> 42.1 / 26.3 / 21.5 us, r = 1024 47.7 / 31.4 / 30.0 -> 46.8 /
-  // 32.4 / 31.4; bf16, 8192 x 24000, r = 1024 67.9 / 40.7 / 36.4 -> 66.3 / 39.4 / 36.8, but 4096 x 14336, r = 512 26.7 / 18.6 / 15.5 ->
-  // 26.2 / 18.5 / 16.9; eight layers of fp32, 3840 x 14230, r = 480, 229 -> 215.
-  constexpr int kLongRow = 15 * 1024;
-  bool pairs = false;
-  if (lopa && (c.wkind == kWBF16 || c.wkind == kWF32) && grid % 2 == 0 && g.cpt == 8) {
-    const int row_bytes = c.D * 16 / weight_epv(c.wkind), gate_row_bytes = K * 16 / weight_epv(c.wkind);
-    const SmemLayout with(c.D, K, true, g.n_gate_slots, g.gate_slot_bytes, g.n_act_slots, g.act_slot_bytes, g.slab_max, false, g.act_extra,
-                          false, false, true);
-    pairs = row_bytes >= kLongRow && row_bytes >= 8 * gate_row_bytes && with.total <= kSmemBudget;
-    if (pairs) g.smem = with.total;
-  }
+  const bool pairs = lopa && in_pairs(g, c.wkind, c.D, K, grid, -1, &g.smem);
   char* ws = static_cast<char*>(c.workspace);
   int n = 0;
   cudaError_t e;
