@@ -343,13 +343,15 @@ const char* sffn_status_string(int status);
  *                       records SFFN_ERR_BOUNDS and takes row 0 instead; the bad index is never used as an address)
  *   CLUSTER_QUERY_FAILS 1 = the runtime has no answer to how many clusters of CTAs the device runs at once: the kernels that
  *                       have to know take the form without them (default 0)
+ *   PAIRS               1 / 0: single-token LoPA calls go to the kernel of pairs of CTAs wherever it can run them / nowhere;
+ *                       -1 (the default): by their sizes
  *   TRACE_BUFFER        device address of [grid][16] int64 time stamps, written only by libraries built with
  *                       -DSFFN_TRACE (0 = none) */
 typedef enum {
   SFFN_KNOB_PDL = 0, SFFN_KNOB_TENSOR_GATE = 1, SFFN_KNOB_WAIT_CYCLES = 2, SFFN_KNOB_SKIP_ARRIVAL_CTA = 3,
   SFFN_KNOB_RING_GATE_SLOTS = 4, SFFN_KNOB_RING_ACT_SLOTS = 5, SFFN_KNOB_TRACE_BUFFER = 6,
   SFFN_KNOB_RING_PARKED_STAGES = 7, SFFN_KNOB_L2_HINTS = 8, SFFN_KNOB_DROP_STAGE = 9, SFFN_KNOB_POISON_LIST = 10,
-  SFFN_KNOB_CLUSTER_QUERY_FAILS = 11
+  SFFN_KNOB_CLUSTER_QUERY_FAILS = 11, SFFN_KNOB_PAIRS = 12
 } sffn_test_knob;
 void sffn_test_fused_plan(int wkind, int D, int H, int K, int lopa, int sm_count, int* out9);
 int sffn_test_fused_pairs(int wkind, int D, int H, int r, int sm_count, int at_once);

@@ -99,7 +99,7 @@ def load_library() -> ctypes.CDLL:
 GATE_ENGINE = {"auto": 0, "cuda_core": 1, "tensor_core": 2}
 KNOB = {"pdl": 0, "tensor_gate": 1, "wait_cycles": 2, "skip_arrival_cta": 3, "ring_gate_slots": 4,
         "ring_act_slots": 5, "trace_buffer": 6, "ring_parked_stages": 7, "l2_hints": 8, "drop_stage": 9,
-        "poison_list": 10, "cluster_query_fails": 11}
+        "poison_list": 10, "cluster_query_fails": 11, "pairs": 12}
 
 
 def test_set_knob(name: str, value: int):

@@ -236,6 +236,7 @@ int sffn_test_set_knob(int knob, long long value) {
       return value ? SFFN_ERR_UNSUPPORTED : SFFN_OK;
 #endif
     case SFFN_KNOB_CLUSTER_QUERY_FAILS: sffn::cluster_query_fails() = value != 0; return SFFN_OK;
+    case SFFN_KNOB_PAIRS: k.pairs = value < 0 ? -1 : (value != 0); return SFFN_OK;
     case SFFN_KNOB_TRACE_BUFFER: k.trace = reinterpret_cast<long long*>(static_cast<uintptr_t>(value)); return SFFN_OK;
     default: return SFFN_ERR_INVALID_ARG;
   }

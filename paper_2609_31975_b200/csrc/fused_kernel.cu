@@ -1896,18 +1896,27 @@ int pairs_at_once() {
 // Whether a LoPA call goes to the kernel of pairs, and the shared memory that takes.  `at_once`: pairs that the device runs at once,
 // -1 = it is asked.  They have to be all of the call's: its CTAs wait for one another (the exchange of V x), so a device whose GPCs
 // leave some of them no second SM takes the kernel without pairs.
-// Pairs of CTAs where a row of a fired neuron is long, so that the CTA with most of them is what a call waits for, and eight gate
-// rows or more, so that it is not the gate: the two SMs of a pair start a call together, 1 us later than alone.  Alone / in pairs,
-// firing 30 / 10 / 4 %: fp32, 4096 x 14336, r = 512 45.2 / 27.6 / 21.6 -> 42.1 / 26.3 / 21.5 us, r = 1024 47.7 / 31.4 / 30.0 -> 46.8 /
-// 32.4 / 31.4; bf16, 8192 x 24000, r = 1024 67.9 / 40.7 / 36.4 -> 66.3 / 39.4 / 36.8, but 4096 x 14336, r = 512 26.7 / 18.6 / 15.5 ->
-// 26.2 / 18.5 / 16.9; eight layers of fp32, 3840 x 14230, r = 480, 229 -> 215.
-bool in_pairs(const Geometry& g, int wkind, int D, int K, int grid, int at_once, int* smem) {
-  constexpr int kLongRow = 15 * 1024;
-  if ((wkind != kWBF16 && wkind != kWF32) || grid % 2 || g.cpt != 8) return false;
+// Where: a call waits for the CTA with most fired neurons, and what a pair evens out is worth more than the 1 us that two SMs that
+// start a call together take longer, at the firing rates from 3 to 30 % that the calls are made for.
+// - Rows of 15 KB and more (kLongRow).  At 3 % firing and 80 to 130 neurons a CTA, time alone over time in pairs: fp32, 3072 columns 0.93
+//   to 1.0, 3328 0.98, 3584 and 3712 0.97 to 1.025, 3840 and 4096 0.99 to 1.03; bf16, 5632 0.96 to 1.02, 6656 0.99 to 1.05, 7680 0.99 to
+//   1.05, 8192 0.985 to 1.02.  (bf16 of 7168 would gain as well.)
+// - 80 neurons a CTA and more (kLongShare): at 3 % firing, rows of 3840 and 4096 fp32, 50 / 65 / 80 / 100 neurons: 0.98 to 1.01 / 0.98
+//   to 1.0 / 1.0 to 1.03 / 0.99 to 1.015; 55 of 4096, r = 256: 0.95.
+// - Eight gate rows or more to a row (kGateRows): above that the gate is what a call waits for.  At 10 % firing, r = D / 8 / D / 7.5 /
+//   D / 7: fp32, 3840 x 14230 1.026 / 1.030 / 0.984, 3456 x 13000 1.049 / 1.035 / 1.018; bf16, 8192 x 28000 1.022 / 0.991 / 1.006.
+// Times alone / in pairs at 30 / 10 / 3 % firing: fp32, 4096 x 13926, r = 512 44.4 / 27.9 / 20.6 -> 42.5 / 26.8 / 21.3 us, r = 256 44.2 /
+// 27.8 / 18.6 -> 42.9 / 26.3 / 19.0; bf16, 8192 x 27852, r = 1024 78.2 / 44.5 / 38.9 -> 72.2 / 43.7 / 39.4; eight layers of fp32, 3840 x
+// 14230, r = 480, at 10 %: 229 -> 216.
+constexpr int kLongRow = 15 * 1024, kLongShare = 80, kGateRows = 8;
+bool in_pairs(const Geometry& g, int wkind, int D, int H, int K, int grid, int at_once, int* smem) {
+  const int knob = fused_test_knobs().pairs;
+  if (knob == 0 || (wkind != kWBF16 && wkind != kWF32) || grid % 2 || g.cpt != 8) return false;
   const int row_bytes = D * 16 / weight_epv(wkind), gate_row_bytes = K * 16 / weight_epv(wkind);
   const SmemLayout with(D, K, true, g.n_gate_slots, g.gate_slot_bytes, g.n_act_slots, g.act_slot_bytes, g.slab_max, false, g.act_extra,
                         false, false, true);
-  if (row_bytes < kLongRow || row_bytes < 8 * gate_row_bytes || with.total > kSmemBudget) return false;
+  if (with.total > kSmemBudget) return false;
+  if (knob < 0 && (row_bytes < kLongRow || H < kLongShare * grid || row_bytes < kGateRows * gate_row_bytes)) return false;
   if (at_once < 0) at_once = wkind == kWBF16 ? pairs_at_once<__nv_bfloat16>() : pairs_at_once<float>();
   if (2 * at_once < grid) return false;
   *smem = with.total;
@@ -1965,7 +1974,7 @@ void debug_fused_plan(int wkind, int D, int H, int K, bool lopa, int sm_count, i
 bool debug_fused_pairs(int wkind, int D, int H, int r, int sm_count, int at_once) {
   const int grid = fused_grid(sm_count, H);
   Geometry g = plan(wkind, D, H, r, true, grid);
-  return g.ok && in_pairs(g, wkind, D, r, grid, at_once, &g.smem);
+  return g.ok && in_pairs(g, wkind, D, H, r, grid, at_once, &g.smem);
 }
 
 // Whether this call's gate goes to the tensor cores (see sffn_set_gate_engine).
@@ -2002,7 +2011,7 @@ cudaError_t launch_fused(const FusedCall& c, cudaStream_t s, int* launched) {
     if (with.total <= kSmemBudget) g.smem = with.total;
     else gated = false;
   }
-  const bool pairs = lopa && in_pairs(g, c.wkind, c.D, K, grid, -1, &g.smem);
+  const bool pairs = lopa && in_pairs(g, c.wkind, c.D, c.H, K, grid, -1, &g.smem);
   char* ws = static_cast<char*>(c.workspace);
   int n = 0;
   cudaError_t e;

@@ -58,6 +58,7 @@ struct FusedTestKnobs {
   int ring_S = 0, ring_NA = 0;   // tensor-core gate: ring split override (0 = planned)
   int l2_hints = 2;              // tensor-core gate: bit 0 weights evict-first, bit 1 partials evict-last
   int ring_E = -1;               // tensor-core gate: gate stages parked in the act ring at the start (-1 = planned)
+  int pairs = -1;                // single-token LoPA calls in pairs of CTAs: 1 / 0 wherever they fit / nowhere; -1: by their sizes
   long long* trace = nullptr;    // SFFN_TRACE builds: [grid][16] time stamps
 };
 FusedTestKnobs& fused_test_knobs();

@@ -1,4 +1,4 @@
-"""Single-token LoPA calls whose CTAs share out the rows of fired neurons in pairs (rows of 15 KB and more, a gate of short rows)."""
+"""Single-token LoPA calls whose CTAs share out the rows of fired neurons in pairs, at sizes that are quick to check."""
 import pytest
 import torch
 
@@ -7,6 +7,16 @@ from parity import assert_active_set, assert_y_close, run_oracle
 
 DEV = "cuda:0"
 pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def in_pairs():
+    import paper_2609_31975_b200 as m
+
+    m.test_set_knob("pairs", 1)  # (by their sizes these calls would go alone: too few neurons a CTA)
+    yield lambda D, H, r, dtype: m.load_library().sffn_test_fused_pairs(
+        0 if dtype == torch.float32 else 1, D, H, r, torch.cuda.get_device_properties(0).multi_processor_count, -1)
+    m.test_set_knob("pairs", -1)
 
 
 def make(m, D, H, r, dtype, s):
@@ -22,8 +32,10 @@ def make(m, D, H, r, dtype, s):
     (4096, 5003, 512, torch.float32, 0.2),    # many rows a CTA: the rings wrap
     (8192, 3001, 1024, torch.bfloat16, 0.8),
 ])
-def test_pairs_share_the_fired_rows(D, H, r, dtype, s):
+def test_pairs_share_the_fired_rows(D, H, r, dtype, s, in_pairs):
     import paper_2609_31975_b200 as m
+
+    assert in_pairs(D, H, r, dtype)
 
     gate, w = make(m, D, H, r, dtype, s)
     ffn = m.SparseFFN(D, H, dtype, r_max=r, B_max=1)
@@ -41,8 +53,10 @@ def test_pairs_share_the_fired_rows(D, H, r, dtype, s):
     assert torch.equal(ys[0], ys[3])
 
 
-def test_pairs_do_every_row_of_a_dense_call_once():
+def test_pairs_do_every_row_of_a_dense_call_once(in_pairs):
     import paper_2609_31975_b200 as m
+
+    assert in_pairs(3840, 700, 480, torch.float32)
 
     gate, w = make(m, 3840, 700, 480, torch.float32, None)
     ffn = m.SparseFFN(3840, 700, torch.float32, r_max=480, B_max=1)
@@ -55,10 +69,12 @@ def test_pairs_do_every_row_of_a_dense_call_once():
 
 
 @pytest.mark.parametrize("knob,value", [("skip_arrival_cta", 3), ("wait_cycles", 2000), ("wait_cycles", 20000)])
-def test_pairs_end_together_when_a_wait_runs_out(knob, value):
+def test_pairs_end_together_when_a_wait_runs_out(knob, value, in_pairs):
     """A CTA that never hands in its sums, and budgets that run out in the middle of the call: a status, and a good call after a
     reset."""
     import paper_2609_31975_b200 as m
+
+    assert in_pairs(3840, 1531, 480, torch.float32)
 
     gate, w = make(m, 3840, 1531, 480, torch.float32, 0.9)
     ffn = m.SparseFFN(3840, 1531, torch.float32, r_max=480, B_max=1)

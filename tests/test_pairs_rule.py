@@ -19,6 +19,18 @@ def test_all_pairs_of_a_call_have_to_fit_at_once(wkind, D, H, r):
     assert in_pairs(wkind, D, H, r, sms=147, at_once=100) == 0  # an odd one out
 
 
+@pytest.mark.parametrize("wkind,D,H,r,want", [
+    (0, 4096, 14336, 512, 1), (0, 3840, 12000, 224, 1), (1, 8192, 28672, 1024, 1), (1, 7680, 15769, 448, 1),
+    (0, 3836, 14336, 256, 0), (1, 7672, 24000, 448, 0),       # rows below 15 KB
+    (0, 4096, 80 * 148, 512, 1), (0, 4096, 80 * 148 - 1, 512, 0), (1, 8192, 9000, 512, 0),  # CTAs of few neurons
+    (0, 4096, 14336, 516, 0), (1, 8192, 28672, 1032, 0),      # a gate row longer than an eighth of a row
+    (2, 8192, 28672, 512, 0), (3, 8192, 28672, 512, 0),       # codes
+])
+def test_calls_that_gain(wkind, D, H, r, want):
+    """Calls whose CTAs have few fired neurons lose the microsecond that two SMs take longer to start together."""
+    assert in_pairs(wkind, D, H, r, at_once=74) == want
+
+
 @pytest.mark.gpu
 def test_without_an_answer_a_call_goes_alone():
     import paper_2609_31975_b200 as m
