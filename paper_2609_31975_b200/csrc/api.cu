@@ -670,15 +670,13 @@ int run(sffn_handle* h, const void* x, int B, const sffn_gate* g, const float* b
   const int pass_max = umma_ok ? umma_pass_tokens(h->D, gate_k, q8 != nullptr, lopa_gate) : kMaxMmaTokens;
   const bool tensor_batch = h->dtype == SFFN_BF16 && B >= 2 && h->path != SFFN_PATH_GENERAL && h->path != SFFN_PATH_FUSED &&
                             (umma_ok || (!q8 && sffn::batched_mma_supported(h->D, gate_k, 1)));
-  // Asked for by name, the fused path takes the 4-bit LoPA rows that it always took; narrower ones are for the automatic choice.
-  if (h->path == SFFN_PATH_FUSED && wkind == sffn::kWQ4 && g->kind == SFFN_GATE_LOPA && h->D <= 896) return SFFN_ERR_UNSUPPORTED;
   // Any other batch (fp32 operands, a row width the tensor-core kernels do not tile, SFFN_PATH_FUSED): the single-token
   // kernel once per token, where it serves the shape.  The CUDA-core batch kernels are slower than B single-token calls
   // (int8, 4096 x 14336, B = 16: 1.66 ms against 0.33 ms; bf16 rows of 4000 elements: 1.03 ms against 0.46 ms; fp32:
   // 0.86 against 0.77 ms).
   // The fired flags of the tokens are OR-ed: the list is the batch's union.
   if (B > 1 && !tensor_batch && h->path != SFFN_PATH_GENERAL && h->path != SFFN_PATH_MMA_SYNC &&
-      sffn::fused_supported(wkind, h->D, h->H, 1, g, h->sm_count)) {
+      sffn::fused_supported(wkind, h->D, h->H, 1, g, h->sm_count, h->path == SFFN_PATH_AUTO)) {
     const size_t tok_bytes = (size_t)h->D * ((q8 || h->dtype == SFFN_BF16) ? 2 : 4);
     for (int b = 0; b < B; ++b) {
       sffn::FusedCall c{};
@@ -702,7 +700,7 @@ int run(sffn_handle* h, const void* x, int B, const sffn_gate* g, const float* b
     if (!dense) h->list_state = 2;
     return SFFN_OK;
   }
-  const bool fused_ok = sffn::fused_supported(wkind, h->D, h->H, B, g, h->sm_count);
+  const bool fused_ok = sffn::fused_supported(wkind, h->D, h->H, B, g, h->sm_count, h->path == SFFN_PATH_AUTO);
   if (h->path == SFFN_PATH_FUSED && !fused_ok) return SFFN_ERR_UNSUPPORTED;
   if (fused_ok && h->path != SFFN_PATH_GENERAL) {
     sffn::FusedCall c{};

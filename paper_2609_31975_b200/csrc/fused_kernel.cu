@@ -1717,6 +1717,7 @@ struct Geometry {
   int act_used;    // act slots the ring cycles through (<= n_act_slots + act_extra)
   int act_groups;  // groups of four warps that take alternate rounds of the act ring (LoPA: 2 or 3)
   bool v_in_smem;  // LoPA: the CTA's rows of V are copied into the idle act ring ahead of the rank-r stage
+  bool auto_only;  // the automatic choice takes the shape, a path asked for by name does not
   bool ok;
 };
 
@@ -1770,8 +1771,10 @@ Geometry plan(int wkind, int D, int H, int K, bool lopa, int grid) {
   g.gate_slot_bytes = (nr * gate_row_bytes + 127) / 128 * 128;
   g.act_slot_bytes = (2 * row_bytes + 127) / 128 * 128;
   // LoPA: the act groups' sums, which meet in the act ring, must fit sixteen slots of it (4-bit rows of less than 1024 codes: 512 x
-  // 1500, r = 64 took the CUDA-core path's 44.6 us, 12.5 here)
-  if (lopa && wkind == kWQ4 && D >= 256 && 16 * g.act_slot_bytes < g.cpt * epv * act_threads * 4) g.act_slot_bytes = g.cpt * epv * act_threads * 4 / 16;
+  // 1500, r = 64 took the CUDA-core path's 44.6 us, 12.5 here).  Asked for by name, the single-token paths refuse such rows, as they
+  // always did.
+  g.auto_only = lopa && wkind == kWQ4 && D >= 256 && 16 * g.act_slot_bytes < g.cpt * epv * act_threads * 4;
+  if (g.auto_only) g.act_slot_bytes = g.cpt * epv * act_threads * 4 / 16;
   g.slab_max = (((H + nr - 1) / nr + grid - 1) / grid) * nr;  // most rows one CTA can own
   const bool limbs = (wkind == kWQ8 || wkind == kWQ4) && !lopa;
   const SmemLayout fixed(D, K, lopa, 0, 0, 0, 0, g.slab_max, scaled, 0, false, limbs);
@@ -1985,12 +1988,13 @@ static bool wants_tensor_gate(const FusedCall& c) {
   return c.engine == SFFN_GATE_ENGINE_TENSOR_CORE;
 }
 
-bool fused_supported(int wkind, int D, int H, int B, const sffn_gate* gate, int sm_count) {
+bool fused_supported(int wkind, int D, int H, int B, const sffn_gate* gate, int sm_count, bool automatic) {
   if (B != 1) return false;
   if (fused_test_knobs().tensor_gate != 0 && fused_tc_supported(wkind, D, H, B, gate, sm_count)) return true;
   const bool lopa = gate->kind == SFFN_GATE_LOPA;
   const int K = lopa ? gate->r : D;
-  return plan(wkind, D, H, K, lopa, fused_grid(sm_count, H)).ok;
+  const Geometry g = plan(wkind, D, H, K, lopa, fused_grid(sm_count, H));
+  return g.ok && (automatic || !g.auto_only);
 }
 
 cudaError_t launch_fused(const FusedCall& c, cudaStream_t s, int* launched) {

@@ -37,7 +37,8 @@ struct FusedCall {
 
 size_t fused_workspace_bytes(int D, int H, int r_max);
 size_t fused_tagged_partials_offset(int D, int r_max);  // where the tensor-core kernel's tagged partials start
-bool fused_supported(int wkind, int D, int H, int B, const sffn_gate* gate, int sm_count);
+// automatic: the path was not asked for by name
+bool fused_supported(int wkind, int D, int H, int B, const sffn_gate* gate, int sm_count, bool automatic);
 void debug_fused_plan(int wkind, int D, int H, int K, bool lopa, int sm_count, int* out);
 bool debug_fused_pairs(int wkind, int D, int H, int r, int sm_count, int at_once);
 cudaError_t launch_fused(const FusedCall& c, cudaStream_t s, int* launched);

@@ -45,3 +45,26 @@ def test_the_fused_path_by_name_keeps_its_widths():
     ffn.set_path("fused")
     with pytest.raises(m.SFFNError):
         ffn.sparse_ffn_forward_q4(syn.tokens(1, 512, torch.bfloat16, 91, DEV)[0], gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+
+
+@pytest.mark.parametrize("D,refused", [(256, True), (896, True), (928, False), (1024, False)])
+def test_the_fused_path_by_name_ends_where_slots_are_longer_than_rows(D, refused):
+    """One token and three, sparse and dense: the automatic choice takes all of them."""
+    import paper_2609_31975_b200 as m
+
+    w = syn.lopa_ffn_q4(D, 300, 64, 91, DEV, sparsity=0.9)
+    gate = {"V": w["V"], "U": w["U"], "g_idx": m.g_diagonal(300, D, DEV)}
+    ffn = m.SparseFFN(D, 300, torch.bfloat16, r_max=64, B_max=3)
+    x = syn.tokens(3, D, torch.bfloat16, 91, DEV)
+    for path in ("fused", "auto"):
+        ffn.set_path(path)
+        for call in (ffn.sparse_ffn_forward_q4, ffn.dense_ffn_forward_q4):
+            for tokens in (x[0], x):
+                args = (tokens, gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+                if refused and path == "fused":
+                    with pytest.raises(m.SFFNError):
+                        call(*args)
+                else:
+                    call(*args)
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0
