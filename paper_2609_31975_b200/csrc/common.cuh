@@ -316,14 +316,22 @@ cudaError_t launch_clusters(int cluster, void (*k)(KArgs...), dim3 grid, dim3 bl
   cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, k, args...);
 }
-// How many clusters of `size` blocks (this many threads, this much dynamic shared memory) of a kernel the current device runs at
-// once: it depends on how many SMs each of its GPCs has.  0 where it cannot be told, and then asked again by the next call.  An
-// answer is kept for each device (`known`: 0 = none yet, else the answer + 1).
+// The current device, -1 where there is none.
+inline int current_device() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess) return dev;
+  cudaGetLastError();
+  return -1;
+}
+
+// How many clusters of `size` blocks (this many threads, this much dynamic shared memory) of a kernel the current device, `dev`,
+// runs at once: it depends on how many SMs each of its GPCs has.  0 where it cannot be told, and then asked again by the next call.
+// An answer is kept for each device (`known`: 0 = none yet, else the answer + 1).
 constexpr int kKnownDevices = 64;
 template <typename K>
-int clusters_at_once(K kernel, int size, int threads, int smem, unsigned long long& configured, std::atomic<int>* known) {
-  int dev = 0, n = 0;
-  if (cluster_query_fails() || cudaGetDevice(&dev) != cudaSuccess) return 0;
+int clusters_at_once(int dev, K kernel, int size, int threads, int smem, unsigned long long& configured, std::atomic<int>* known) {
+  int n = 0;
+  if (cluster_query_fails() || dev < 0) return 0;
   if (dev < kKnownDevices && (n = known[dev].load(std::memory_order_relaxed)) != 0) return n - 1;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(size);
@@ -335,7 +343,7 @@ int clusters_at_once(K kernel, int size, int threads, int smem, unsigned long lo
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (allow_dynamic_smem(kernel, smem, configured) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+  if (allow_dynamic_smem(kernel, 227 * 1024, configured) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }

@@ -1893,7 +1893,7 @@ template <typename T>
 int pairs_at_once() {
   static unsigned long long configured = 0;
   static std::atomic<int> known[kKnownDevices];
-  return clusters_at_once(fused_ffn_kernel<T, 8, true, false, true>, 2, kThreads, kSmemBudget, configured, known);
+  return clusters_at_once(current_device(), fused_ffn_kernel<T, 8, true, false, true>, 2, kThreads, kSmemBudget, configured, known);
 }
 
 // Whether a LoPA call goes to the kernel of pairs, and the shared memory that takes.  `at_once`: pairs that the device runs at once,

@@ -43,8 +43,6 @@
 
 #include <cuda.h>
 
-#include <atomic>
-
 #include "common.cuh"
 #include "fused_kernel.cuh"
 #include "sparse_ffn.h"
@@ -2121,37 +2119,13 @@ constexpr int kDownPairCols = 64;
 constexpr int kMaxDownCluster = 8;  // CTAs of a cluster
 static bool down_pairs(int cols, bool exact) { return cols <= kDownPairCols && !exact; }
 
-// Clusters of `size` CTAs of the down kernel that the device runs at once, two CTAs per SM or one.  (It depends on how many SMs
-// each of its GPCs has.)  Asked for a kernel that does nothing in as many threads and as much shared memory: for one that
-// allocates TMEM the runtime answers as if an SM took a single CTA.
+// Clusters of `size` CTAs of the down kernel that the device runs at once, two CTAs per SM or one.  Asked for a kernel that does
+// nothing in as many threads and as much shared memory: for one that allocates TMEM the runtime answers as if an SM took a single CTA.
 static __global__ void __launch_bounds__(down_bound(8, false), 2) down_place_kernel() {}
-static int down_clusters(int size, bool pairs) {
-  static std::atomic<int> known[16][2][kMaxDownCluster + 1];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev >= 16) return 0;
-  std::atomic<int>& k = known[dev][pairs ? 1 : 0][size];
-  if (k.load(std::memory_order_relaxed) == 0) {
-    static unsigned long long configured = 0;
-    auto kernel = down_place_kernel;
-    int n = 0;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(size);
-    cfg.blockDim = dim3(down_bound(8, false));
-    cfg.dynamicSmemBytes = (pairs ? 111 : 225) * 1024;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = size;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (allow_dynamic_smem(kernel, 227 * 1024, configured) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
-      cudaGetLastError();
-      n = 0;
-    }
-    k.store(n + 1, std::memory_order_relaxed);
-  }
-  return k.load(std::memory_order_relaxed) - 1;
+static int down_clusters(int dev, int size, bool pairs) {
+  static unsigned long long configured = 0;
+  static std::atomic<int> known[2][kMaxDownCluster + 1][kKnownDevices];
+  return clusters_at_once(dev, down_place_kernel, size, down_bound(8, false), (pairs ? 111 : 225) * 1024, configured, known[pairs][size]);
 }
 
 // Splits of the list, and whether they are a cluster that adds its sums up itself.  That saves the partials' way through memory and
@@ -2161,11 +2135,12 @@ static int down_clusters(int size, bool pairs) {
 // bf16, 6144 x 20000, 160 tokens, three / two 229 / 242; exact sums, 2688 x 8000, 24 tokens, seven / six 78.5 / 80.2), or any number
 // where a CTA has a dozen blocks at most (2048 x 6000, 16 / 8: bf16, 64 tokens 40.0 / 39.1, int4, 2 / 24 / 64 tokens 27.3 / 38.5 /
 // 53.6 against 25.5 / 39.1 / 49.9).  Clusters of up to 16 where they fit are slower (512 x 1500, bf16, 24 tokens, 8 / 16: 19.4 / 20.4).
-bool umma_down_splits(int D, int R, int qbits, int cols, bool exact, int sm_count, int max_splits, int* splits) {
+bool umma_down_splits(int D, int R, int qbits, int cols, bool exact, int sm_count, int max_splits, int* splits, const int* at_once) {
   const int tiles = D >= kTileRows ? D / kTileRows : 1;
   const bool pairs = down_pairs(cols, exact);
+  const int dev = at_once ? -1 : current_device();
   int cluster = kMaxDownCluster;
-  while (cluster > 1 && down_clusters(cluster, pairs) < tiles) --cluster;
+  while (cluster > 1 && (at_once ? at_once[cluster] : down_clusters(dev, cluster, pairs)) < tiles) --cluster;
   auto splits_of = [&](int ctas) {
     const int n = ctas / tiles;
     return n < 1 ? 1 : n > max_splits ? max_splits : n;
@@ -2178,7 +2153,7 @@ bool umma_down_splits(int D, int R, int qbits, int cols, bool exact, int sm_coun
   if (exact && 10 * (two - 2 * one) >= one * two) n = two;
   const int blocks = (R + kAtomK - 1) / kAtomK;
   const bool clustered = qbits ? cluster >= n : 9 * cluster >= 8 * n;
-  if (clustered || blocks <= 12 * cluster) {
+  if (clustered || (cluster > 1 && blocks <= 12 * cluster)) {
     *splits = cluster;
     return true;
   }

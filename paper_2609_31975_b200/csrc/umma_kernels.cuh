@@ -86,8 +86,9 @@ struct UmmaDownParams {
   long long wait_cycles; // budget of every device-side wait (filled by the launcher)
 };
 
-// How the list (of up to R rows) is split; true: `y`, in clusters, false: `partial` (at most max_splits).  cols: token columns of all terms.
-bool umma_down_splits(int D, int R, int qbits, int cols, bool exact, int sm_count, int max_splits, int* splits);
+// How the list (of up to R rows) is split; true: `y`, in clusters, false: `partial` (at most max_splits).  cols: token columns of all
+// terms.  at_once[n]: clusters of n CTAs that the device runs at once (null: it is asked).
+bool umma_down_splits(int D, int R, int qbits, int cols, bool exact, int sm_count, int max_splits, int* splits, const int* at_once = nullptr);
 bool umma_down_supported(int D, int cols);
 cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s);
 bool umma_rows_supported(int K, int cols);

@@ -1,0 +1,66 @@
+"""How the batched down projection splits the list of fired neurons: the rule is host code."""
+import ctypes
+
+import pytest
+
+
+def splits(D, R, qbits, cols, at_once, exact=0, sms=148, most=16):
+    """(clustered, splits) on a device that runs at_once(n) clusters of n CTAs at once (None: the current one)."""
+    import paper_2609_31975_b200 as m
+
+    fit = (ctypes.c_int * 9)(*([0] + [at_once(n) for n in range(1, 9)])) if at_once else None
+    n = ctypes.c_int()
+    return m.load_library().sffn_test_umma_down_splits(D, R, qbits, cols, exact, sms, most, fit, ctypes.byref(n)), n.value
+
+
+def plenty(n):
+    return 296 // n
+
+
+@pytest.mark.parametrize("qbits", [0, 8, 4])
+def test_a_cluster_for_every_tile_or_partials(qbits):
+    for D, R in ((512, 1500), (4096, 14336), (8192, 24000), (640, 600)):
+        for cols in (8, 64, 72, 200):
+            clustered, n = splits(D, R, qbits, cols, plenty)
+            assert 1 <= n <= (8 if clustered else 16)
+            if clustered:
+                assert n == 1 or plenty(n) >= D // 128
+            else:
+                assert n * (D // 128) <= (296 if cols <= 64 else 148) or n == 1
+
+
+def test_without_an_answer_the_list_is_cut_into_partials():
+    """No cluster fits, or the runtime could not tell: as many splits as without clusters, short lists too."""
+    for D, R in ((512, 700), (1024, 3000), (4096, 14336), (8192, 24000)):
+        for cols in (8, 64, 200):
+            clustered, n = splits(D, R, 0, cols, lambda size: 0)
+            want = min(16, (2 if cols <= 64 else 1) * 148 // (D // 128))
+            assert n == want and clustered == (want == 1)
+
+
+@pytest.mark.gpu
+def test_a_question_that_failed_is_asked_again():
+    """Partials and the kernel that adds them up while the runtime has no answer, one launch less once it has."""
+    import paper_2609_31975_b200 as m
+    import synthetic_inputs as syn
+    import torch
+
+    D, H, B = 512, 1500, 16
+    w = syn.standard_ffn(D, H, torch.bfloat16, 92, "cuda:0", sparsity=0.8)
+    ffn = m.SparseFFN(D, H, torch.bfloat16, B_max=B)
+    x = syn.tokens(B, D, torch.bfloat16, 92, "cuda:0")
+    launches, y = [], []
+    try:
+        for fails in (1, 0, 1, 0):
+            m.test_set_knob("cluster_query_fails", fails)
+            assert splits(D, H, 0, B, None) == ((0, 16) if fails else (1, 8))
+            n = ffn.launch_count()
+            y.append(ffn.sparse_ffn_forward(x, {"W_g": w["W_g"]}, w["b_g"], w["W_up"], w["W_down"], "relu").clone())
+            launches.append(ffn.launch_count() - n)
+    finally:
+        m.test_set_knob("cluster_query_fails", 0)
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0
+    assert launches[0] == launches[2] == launches[1] + 1 == launches[3] + 1
+    assert torch.equal(y[0], y[2]) and torch.equal(y[1], y[3])
+    assert (y[0] - y[1]).norm() <= 1e-5 * y[0].norm()  # fp32 sums of the same products in another order
