@@ -2133,8 +2133,10 @@ static int down_clusters(int dev, int size, bool pairs) {
 // 1500, int8, 2 tokens 21.5 / 18.9), and costs splits where more CTAs would run than clusters fit the GPCs: up to a ninth of them
 // (codes, whose blocks take longer: none) is worth it (int8, 4096 x 14336, 8 tokens, nine splits / clusters of eight 44.6 / 45.1;
 // bf16, 6144 x 20000, 160 tokens, three / two 229 / 242; exact sums, 2688 x 8000, 24 tokens, seven / six 78.5 / 80.2), or any number
-// where a CTA has a dozen blocks at most (2048 x 6000, 16 / 8: bf16, 64 tokens 40.0 / 39.1, int4, 2 / 24 / 64 tokens 27.3 / 38.5 /
-// 53.6 against 25.5 / 39.1 / 49.9).  Clusters of up to 16 where they fit are slower (512 x 1500, bf16, 24 tokens, 8 / 16: 19.4 / 20.4).
+// where a CTA has a few blocks: a dozen where the list has codes, or the fired rows of up to eight tokens (2048 x 6144, 16 / 8: int4, 2 /
+// 24 / 64 tokens 26.7 / 36.9 / 50.7 against 24.4 / 37.6 / 49.0; bf16, 2 tokens 25.7 / 25.2), else eight (bf16, 16 / 8, 63 blocks: 1024 x
+// 3993, 16 / 32 / 64 tokens 22.5 / 24.8 / 29.9 against 23.2 / 23.8 / 28.7; 72 blocks: 1536 x 4608, 16 / 24 / 64 tokens 26.9 / 26.8 / 33.3
+// against 28.4 / 28.7 / 33.9; codes of 16 to 32 tokens between 65 and 96 blocks: clusters from 6 % slower to 4 % faster).  Clusters of up to 16 where they fit are slower (512 x 1500, bf16, 24 tokens, 8 / 16: 19.4 / 20.4).
 bool umma_down_splits(int D, int R, int qbits, int cols, bool exact, int sm_count, int max_splits, int* splits, const int* at_once) {
   const int tiles = D >= kTileRows ? D / kTileRows : 1;
   const bool pairs = down_pairs(cols, exact);
@@ -2153,7 +2155,8 @@ bool umma_down_splits(int D, int R, int qbits, int cols, bool exact, int sm_coun
   if (exact && 10 * (two - 2 * one) >= one * two) n = two;
   const int blocks = (R + kAtomK - 1) / kAtomK;
   const bool clustered = qbits ? cluster >= n : 9 * cluster >= 8 * n;
-  if (clustered || (cluster > 1 && blocks <= 12 * cluster)) {
+  const int few = (qbits || exact || cols <= 8 ? 12 : 8) * cluster;
+  if (clustered || (cluster > 1 && blocks <= few)) {
     *splits = cluster;
     return true;
   }

@@ -38,6 +38,17 @@ def test_without_an_answer_the_list_is_cut_into_partials():
             assert n == want and clustered == (want == 1)
 
 
+@pytest.mark.parametrize("D,R,qbits,cols,exact,clustered", [
+    (1024, 64 * 64, 0, 24, 0, 1), (1024, 64 * 64 + 1, 0, 24, 0, 0),   # eight blocks a CTA
+    (1024, 64 * 64 + 1, 0, 8, 0, 1), (1024, 96 * 64, 0, 8, 0, 1), (1024, 96 * 64 + 1, 0, 8, 0, 0),
+    (1024, 96 * 64, 8, 64, 0, 1), (1024, 96 * 64, 4, 64, 0, 1), (1024, 96 * 64 + 1, 4, 64, 0, 0),
+    (640, 96 * 64, 0, 24, 1, 1),                                      # exact sums
+])
+def test_clusters_for_lists_of_few_blocks(D, R, qbits, cols, exact, clustered):
+    """Narrow rows, whose tiles leave room for more splits than a cluster has."""
+    assert splits(D, R, qbits, cols, plenty, exact)[0] == clustered
+
+
 @pytest.mark.gpu
 def test_a_question_that_failed_is_asked_again():
     """Partials and the kernel that adds them up while the runtime has no answer, one launch less once it has."""
