@@ -47,10 +47,12 @@ def lib_path() -> Path:
 
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda i: torch.cuda.current_stream(i).cuda_stream)
 _lib = None
-# Where os.environ keeps the variables, and its key of one that every call looks at: os.environ.get encodes the name and raises and
-# catches an exception for a variable that is not set, 0.55 us of the 8 that a call on a small model takes.
-_environ = getattr(os.environ, "_data", os.environ)
-_SYNC_CHECK = "SFFN_SYNC_CHECK" if _environ is os.environ else os.environ.encodekey("SFFN_SYNC_CHECK")
+# The environment as this process began with it, where it keeps its variables, and how it writes the one that every call looks at:
+# os.environ.get encodes the name, and raises and catches an exception for a variable that is not set, 0.55 us of the 8 that a call
+# on a small model takes.  A program that puts another mapping in os.environ's place is asked the usual way.
+_environ = os.environ if isinstance(getattr(os.environ, "_data", None), dict) else None
+_variables = _environ._data if _environ is not None else {}
+_SYNC_CHECK, _ON = (_environ.encodekey("SFFN_SYNC_CHECK"), _environ.encodevalue("1")) if _environ is not None else ("", "1")
 
 
 def load_library() -> ctypes.CDLL:
@@ -279,7 +281,7 @@ class SparseFFN:
                 ACT[act] if isinstance(act, str) else int(act), _addr(y), self._stream(stream))
         if rc:
             raise SFFNError(name, rc)
-        if _SYNC_CHECK in _environ and os.environ["SFFN_SYNC_CHECK"] == "1":
+        if _variables.get(_SYNC_CHECK) == _ON if os.environ is _environ else os.environ.get("SFFN_SYNC_CHECK") == "1":
             self._sync_check(name, B, gate)
         return y
 
