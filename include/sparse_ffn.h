@@ -322,6 +322,8 @@ const char* sffn_status_string(int status);
  *   rows; sffn_test_umma_row_tiling: over rows of K elements; sffn_test_umma_pass_tiling: over rows of K elements (qbits 0:
  *   bf16) or codes (8 / 4; 1 / 2: against limbs) in a pass of B tokens.  sffn_test_umma_k_splits: runs of K and tiles of
  *   rows of V x, R rows of K elements (limbs: codes) against B tokens, at most max_splits runs.
+ *   sffn_test_umma_pairs: 1 = the batched gate over R rows of K elements or codes (qbits as above), cols token columns in all,
+ *   runs in pairs of CTAs; the up projection too, from 32 tokens on (cols then: of its own).
  *   sffn_test_umma_down_splits: splits of the list of up to R rows in the batched down projection (qbits 0 / 8 / 4, cols token
  *   columns of all terms, at most max_splits partials); 1 = they are clusters.  at_once[n], n up to 8: clusters of n CTAs that
  *   the device runs at once (NULL: the current device, as a call does).
@@ -362,6 +364,7 @@ void sffn_test_umma_tiling(int R, int sm_count, int* tile_rows, int* n_tiles, in
 void sffn_test_umma_row_tiling(int R, int K, int sm_count, int* tile_rows, int* n_tiles, int* own_list);
 void sffn_test_umma_pass_tiling(int R, int K, int qbits, int B, int sm_count, int* tile_rows, int* n_tiles, int* own_list);
 void sffn_test_umma_k_splits(int R, int K, int limbs, int B, int sm_count, int max_splits, int* tiles, int* splits);
+int sffn_test_umma_pairs(int R, int K, int qbits, int B, int cols, int sm_count);
 int sffn_test_umma_down_splits(int D, int R, int qbits, int cols, int exact, int sm_count, int max_splits, const int* at_once,
                                int* splits);
 int sffn_test_set_knob(int knob, long long value);

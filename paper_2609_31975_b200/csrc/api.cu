@@ -216,6 +216,9 @@ void sffn_test_umma_pass_tiling(int R, int K, int qbits, int B, int sm_count, in
 void sffn_test_umma_k_splits(int R, int K, int limbs, int B, int sm_count, int max_splits, int* tiles, int* splits) {
   sffn::umma_k_splits(R, K, limbs != 0, B, sm_count, max_splits, tiles, splits);
 }
+int sffn_test_umma_pairs(int R, int K, int qbits, int B, int cols, int sm_count) {
+  return sffn::umma_rows_pairs(R, K, qbits, B, cols, false, sm_count) ? 1 : 0;
+}
 int sffn_test_umma_down_splits(int D, int R, int qbits, int cols, int exact, int sm_count, int max_splits, const int* at_once, int* splits) {
   return sffn::umma_down_splits(D, R, qbits, cols, exact != 0, sm_count, max_splits, splits, at_once) ? 1 : 0;
 }

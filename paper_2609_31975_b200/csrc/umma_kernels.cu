@@ -36,7 +36,7 @@
 // Up to 256 token columns go through in one pass.  Wide batches (npad > 128) leave room for two accumulators and a ring
 // of four stages of ~40 KB (two with expanded codes and 241 columns or more), too few for the token rows that every CTA reads again
 // (200 tokens x 4096: 1.6 MB a CTA through L2 beside 0.8 MB of weights).  There the rows kernels run in pairs of CTAs that hold half
-// of the token rows each (PAIR, see rows_pairs): 200 tokens, 4096 x 14336, bf16: 130 us without pairs, 112 with them.
+// of the token rows each (PAIR, see umma_rows_pairs): 200 tokens, 4096 x 14336, bf16: 130 us without pairs, 112 with them.
 // Every wait is bounded by a cycle budget; on expiry the status word is set, all roles wind down and the TMEM
 // columns are released before the CTA exits.
 #include "umma_kernels.cuh"
@@ -2055,7 +2055,7 @@ void umma_k_splits(int R, int K, bool codes, int B, int sm_count, int max_splits
 // With six slots nothing is gained (4096 x 14336, 160 tokens 99.9 / 100.7; 2048 x 6000, 200 tokens 59.7 / 61.6), and the clusters
 // cost a kernel 0.5 to 1 us (1024 x 3000, 72 tokens 29.7 / 33.3).  Codes that are expanded stay alone (int4, 4096 x 14336, 64
 // tokens 97.5 / 112: two CTAs' expansions to wait for).
-static bool rows_pairs(int R, int K, int qbits, int B, int cols, bool exact, int sm_count) {
+bool umma_rows_pairs(int R, int K, int qbits, int B, int cols, bool exact, int sm_count) {
   if (exact || qbits > 1 || sm_count % 2) return false;
   int tile_rows, n_tiles;
   umma_gate_tiling(R, K, qbits, B, sm_count, &tile_rows, &n_tiles);
@@ -2065,7 +2065,7 @@ static bool rows_pairs(int R, int K, int qbits, int B, int cols, bool exact, int
 int umma_gate_rows_per_word(int R, int K, int qbits, int B, int cols, bool exact, int sm_count) {
   int tile_rows, n_tiles;
   umma_gate_tiling(R, K, qbits, B, sm_count, &tile_rows, &n_tiles);
-  return tile_rows <= 64 && !rows_pairs(R, K, qbits, B, cols, exact, sm_count) ? 16 : 32;
+  return tile_rows <= 64 && !umma_rows_pairs(R, K, qbits, B, cols, exact, sm_count) ? 16 : 32;
 }
 
 cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, cudaStream_t s) {
@@ -2083,7 +2083,7 @@ cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, 
   p.longer_runs = kb % splits;
   const bool may_walk = up && p.walk_all && umma_may_walk(p.B) && !p.exact;
   int grid = splits > 1 ? p.k_tiles : p.R < 8 * sm_count ? (p.R + 7) / 8 : sm_count;
-  p.pair = splits == 1 && (!up || may_walk) && rows_pairs(p.R, p.K, p.qbits, p.B, cols, p.exact, sm_count);
+  p.pair = splits == 1 && (!up || may_walk) && umma_rows_pairs(p.R, p.K, p.qbits, p.B, cols, p.exact, sm_count);
   grid += p.pair ? grid % 2 : 0;  // (one CTA more of eight rows each: the same tiles)
   if (p.pair && p.qbits) p.npad = (p.npad + 31) / 32 * 32;  // what the pairs' int8 MMAs take
   // all the dynamic shared memory a CTA can have; the kernel cuts its ring out of it once it knows its tiles

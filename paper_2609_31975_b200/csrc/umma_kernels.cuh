@@ -99,6 +99,8 @@ bool umma_own_list_supported(int R, int K, int qbits, int B, int sm_count);
 void umma_gate_tiling(int R, int K, int qbits, int B, int sm_count, int* tile_rows, int* n_tiles);
 // Rows that a word of that gate's "fired" masks covers (`cols`: its token columns, limbs or terms included).
 int umma_gate_rows_per_word(int R, int K, int qbits, int B, int cols, bool exact, int sm_count);
+// Whether that gate, or an up projection that may walk every row, runs in pairs of CTAs.
+bool umma_rows_pairs(int R, int K, int qbits, int B, int cols, bool exact, int sm_count);
 cudaError_t launch_umma_rows(bool up, UmmaRowsParams p, int cols, int sm_count, cudaStream_t s);
 bool umma_rows_native_i8_supported(int K, int tokens);
 // Tokens [B][K] bf16 as four int8 limbs each ([4 B][K], most significant first, 7 bits apart) and one scale per token;

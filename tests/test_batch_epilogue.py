@@ -8,6 +8,14 @@ from parity import assert_active_set, assert_y_close, run_oracle
 DEV = "cuda:0"
 
 
+def in_pairs(R, K, qbits, B, cols):
+    """Whether a gate over R rows of K columns, or an up projection of 32 tokens and more, runs in pairs of CTAs (qbits 1: int8 codes
+    against limbs)."""
+    import paper_2609_31975_b200 as m
+
+    return m.load_library().sffn_test_umma_pairs(R, K, qbits, B, cols, torch.cuda.get_device_properties(0).multi_processor_count)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("lopa", [False, True])
 @pytest.mark.parametrize("act,act_up", [("relu", None), ("sqrelu", "relu"), ("rsplus", "silu")])
@@ -36,7 +44,8 @@ def test_tokens_of_short_and_full_steps(B, act, act_up, lopa):
 @pytest.mark.parametrize("D", [512, 640])  # against limbs; codes expanded to bf16, h in two terms
 @pytest.mark.parametrize("B", [5, 13, 23, 37, 64])
 def test_tokens_of_short_and_full_steps_of_codes(B, D, qbits):
-    """Against the single-token calls (a bf16 h in the batch where D is a multiple of 256: 1e-2)."""
+    """Against the single-token calls: a bf16 h in the batch where D is a multiple of 256, 1e-2; else h has 16 bits, and the single
+    tokens' two limbs are what is left, some 1e-4 (the second term of h lost: 1.1e-3)."""
     import paper_2609_31975_b200 as m
 
     H = 603
@@ -50,7 +59,7 @@ def test_tokens_of_short_and_full_steps_of_codes(B, D, qbits):
     one = torch.stack([call(x[b], *args) for b in range(B)])
     torch.cuda.synchronize()
     assert ffn.device_status() == 0
-    assert ((y - one).norm(dim=1) / one.norm(dim=1)).max().item() < 1e-2
+    assert ((y - one).norm(dim=1) / one.norm(dim=1)).max().item() < (1e-2 if D % 256 == 0 else 4e-4)
 
 
 @pytest.mark.gpu
@@ -70,6 +79,7 @@ def test_pairs_of_ctas_share_the_token_rows(qbits, D, H, B, s):
     bf16 h in the batch: 1e-2)."""
     import paper_2609_31975_b200 as m
 
+    assert in_pairs(H, D, 1 if qbits else 0, B, 4 * B if qbits else B)
     w = syn.standard_ffn_q8(D, H, 83, DEV, sparsity=s) if qbits else syn.standard_ffn(D, H, torch.bfloat16, 83, DEV, sparsity=s)
     ffn = m.SparseFFN(D, H, torch.bfloat16, B_max=B)
     call = ffn.sparse_ffn_forward_q8 if qbits else ffn.sparse_ffn_forward
@@ -97,6 +107,7 @@ def test_a_copy_that_never_comes_ends_both_ctas_of_a_pair():
     from paper_2609_31975_b200 import binding
 
     D, H, B = 256, 6001, 250
+    assert in_pairs(H, D, 0, B, B)
     w = syn.standard_ffn(D, H, torch.bfloat16, 84, DEV, sparsity=0.9)
     ffn = m.SparseFFN(D, H, torch.bfloat16, B_max=B)
     args = (syn.tokens(B, D, torch.bfloat16, 84, DEV), {"W_g": w["W_g"]}, w["b_g"], w["W_up"], w["W_down"], "relu")

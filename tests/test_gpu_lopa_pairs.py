@@ -96,3 +96,50 @@ def test_pairs_end_together_when_a_wait_runs_out(knob, value, in_pairs):
     torch.cuda.synchronize()
     assert ffn.device_status() == 0
     assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("dtype,D,H,r", [(torch.float32, 3840, 1531, 480), (torch.bfloat16, 8192, 1001, 512)])
+@pytest.mark.parametrize("options", ["sign", "gain", "no norm", "no fixed matrix"])
+def test_pairs_take_every_option_of_the_gate(dtype, D, H, r, options, in_pairs):
+    import paper_2609_31975_b200 as m
+
+    assert in_pairs(D, H, r, dtype)
+    gate, w = make(m, D, H, r, dtype, 0.8)
+    if options == "sign":
+        gate["g_sign"] = torch.where(torch.arange(H, device=DEV) % 3 == 0, -1, 1).to(torch.int8)
+    elif options == "gain":
+        gate["rms_gain"] = 0.5 + torch.rand(r, generator=torch.Generator(device=DEV).manual_seed(5), device=DEV)
+    elif options == "no norm":
+        gate["use_rmsnorm"] = False
+    else:
+        del gate["g_idx"]
+    x = syn.tokens(1, D, dtype, 97, DEV)
+    ffn = m.SparseFFN(D, H, dtype, r_max=r, B_max=1)
+    y = ffn.sparse_ffn_forward(x[0], gate, w["b_g"], w["W_up"], w["W_down"], "sqrelu")
+    active = ffn.last_active()
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0, ffn.status_words()
+    ref = run_oracle(x, gate, w["b_g"], w["W_up"], w["W_down"], "sqrelu")
+    assert_y_close(y, ref["y"][0], rel_l2=1e-5, max_abs=2e-5, what=f"{D}x{H} {options}")  # fp32 sums of up to 1500 terms
+    assert_active_set(active, ref, what=f"{D}x{H} {options}")
+
+
+def test_pairs_token_by_token_leave_the_union_of_the_batch(in_pairs):
+    """A batch of fp32 tokens is as many calls: each the bits of a call of its own, the flags those of any."""
+    import paper_2609_31975_b200 as m
+
+    D, H, r, B = 3840, 1531, 480, 3
+    assert in_pairs(D, H, r, torch.float32)
+    gate, w = make(m, D, H, r, torch.float32, 0.9)
+    x = syn.tokens(B, D, torch.float32, 98, DEV)
+    ffn = m.SparseFFN(D, H, torch.float32, r_max=r, B_max=B)
+    args = (gate, w["b_g"], w["W_up"], w["W_down"], "relu")
+    y = ffn.sparse_ffn_forward(x, *args).clone()
+    union = set(ffn.last_active().tolist())
+    fired = set()
+    for b in range(B):
+        assert torch.equal(ffn.sparse_ffn_forward(x[b], *args), y[b])
+        fired |= set(ffn.last_active().tolist())
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0
+    assert union == fired
