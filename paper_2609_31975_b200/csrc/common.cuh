@@ -52,9 +52,12 @@ __device__ __forceinline__ float activation(int act, float z) {
   return rsplus_of_nonnegative(p);               // R-S+: z * sigmoid(z) on the non-negative side, 0 at 0
 }
 
-// The same for the first n of N values (and what shares a group of four with them), the choice made once.
+// The same for the first n of N values (and what shares a group of four with them), the choice made once.  Where `on` is false nothing
+// reads the results, and the values may be anything: R-S+ and SiLU get a one instead, as a division takes several times as long for
+// the whole warp where one of its lanes has an operand out of the ordinary (batches over rows of codes, whose tiles leave lanes without a row:
+// 640 x 2198, int4, SiLU, 64 / 203 tokens 39.9 / 81.8 -> 32.6 / 61.1 us; R-S+ and SiLU 47.5 / 104.5 -> 37.8 / 76.3).
 template <int N>
-__device__ __forceinline__ void activate(int act, float* z, int n) {
+__device__ __forceinline__ void activate(int act, float* z, int n, bool on) {
   static_assert(N % 4 == 0, "fours");
   if (act == kActNone) return;
   if (act != kActSilu) {
@@ -69,7 +72,7 @@ __device__ __forceinline__ void activate(int act, float* z, int n) {
 #pragma unroll
     for (int q = 0; q < N; q += 4) {
       if (q >= n) break;
-      const float4 r = rsplus4_of_nonnegative(make_float4(z[q], z[q + 1], z[q + 2], z[q + 3]));
+      const float4 r = rsplus4_of_nonnegative(make_float4(on ? z[q] : 1.f, on ? z[q + 1] : 1.f, on ? z[q + 2] : 1.f, on ? z[q + 3] : 1.f));
       z[q] = r.x; z[q + 1] = r.y; z[q + 2] = r.z; z[q + 3] = r.w;
     }
   }

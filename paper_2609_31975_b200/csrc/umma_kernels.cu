@@ -931,7 +931,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
 #pragma unroll
           for (int q = 0; q < kStep; ++q) v[q] *= sc;
         }
-        activate<kStep>(p.act_up, v, B - b0);
+        activate<kStep>(p.act_up, v, B - b0, row_ok);
         __nv_bfloat16* hm = static_cast<__nv_bfloat16*>(p.hmT) + (size_t)b0 * p.hm_stride + li;
 #pragma unroll
         for (int q = 0; q < kStep; ++q) {
@@ -953,7 +953,7 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
           v[q] = gi >= 0 ? v[q] + sg * w.e[q] : v[q];
           fired |= (b0 + q < B) & (v[q] > 0.f);
         }
-        activate<kStep>(p.act, v, B - b0);
+        activate<kStep>(p.act, v, B - b0, row_ok);
         float* arow = a_out + (size_t)b0 * p.a_stride + j;
 #pragma unroll
         for (int q = 0; q < kStep; ++q) st_f32_if(arow + (size_t)q * p.a_stride, v[q], row_ok && b0 + q < B);
