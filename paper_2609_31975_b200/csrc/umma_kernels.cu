@@ -2130,19 +2130,29 @@ static int down_clusters(int dev, int size, bool pairs) {
 
 // Splits of the list, and whether they are a cluster that adds its sums up itself.  That saves the partials' way through memory and
 // a kernel (4096 x 14336, bf16, partials / clusters: 200 tokens 108.3 / 101.2 us, 72 tokens 83.3 / 79.4, 16 tokens 62.9 / 61.6; 512 x
-// 1500, int8, 2 tokens 21.5 / 18.9), and costs splits where more CTAs would run than clusters fit the GPCs: up to a ninth of them
-// (codes, whose blocks take longer: none) is worth it (int8, 4096 x 14336, 8 tokens, nine splits / clusters of eight 44.6 / 45.1;
-// bf16, 6144 x 20000, 160 tokens, three / two 229 / 242; exact sums, 2688 x 8000, 24 tokens, seven / six 78.5 / 80.2), or any number
-// where a CTA has a few blocks: a dozen where the list has codes, or the fired rows of up to eight tokens (2048 x 6144, 16 / 8: int4, 2 /
-// 24 / 64 tokens 26.7 / 36.9 / 50.7 against 24.4 / 37.6 / 49.0; bf16, 2 tokens 25.7 / 25.2), else eight (bf16, 16 / 8, 63 blocks: 1024 x
-// 3993, 16 / 32 / 64 tokens 22.5 / 24.8 / 29.9 against 23.2 / 23.8 / 28.7; 72 blocks: 1536 x 4608, 16 / 24 / 64 tokens 26.9 / 26.8 / 33.3
-// against 28.4 / 28.7 / 33.9; codes of 16 to 32 tokens between 65 and 96 blocks: clusters from 6 % slower to 4 % faster).  Clusters of up to 16 where they fit are slower (512 x 1500, bf16, 24 tokens, 8 / 16: 19.4 / 20.4).
+// 1500, int8, 2 tokens 21.5 / 18.9), and costs splits where more CTAs would run than clusters fit the GPCs.  Clusters:
+// - where they cost up to a ninth of the splits (codes, whose blocks take longer: none): int8, 4096 x 14336, 8 tokens, nine splits /
+//   clusters of eight 44.6 / 45.1; bf16, 6144 x 20000, 160 tokens, three / two 229 / 242; exact sums, 2688 x 8000, 24 tokens, seven / six 78.5 / 80.2;
+// - or any number of them where a CTA has few blocks.  A dozen where the list has codes, or the fired rows of up to eight tokens (2048 x
+//   6144, 16 / 8: int4, 2 / 24 / 64 tokens 26.7 / 36.9 / 50.7 against 24.4 / 37.6 / 49.0; bf16, 2 tokens 25.7 / 25.2; codes of 16 to 32
+//   tokens between 65 and 96 blocks: from 6 % slower to 4 % faster), else eight (bf16, 16 / 8, 63 blocks: 1024 x 3993, 16 / 32 / 64
+//   tokens 22.5 / 24.8 / 29.9 against 23.2 / 23.8 / 28.7; 72 blocks: 1536 x 4608, 16 / 24 / 64 tokens 26.9 / 26.8 / 33.3 against 28.4 /
+//   28.7 / 33.9).
+// Clusters of an odd size need a sixteenth of room to spare: they split the two SMs of a TPC, and the SMs that the kernel before leaves
+// one after the other do not always come to as many clusters as an empty device takes (tiles / most that fit at once, partials /
+// clusters: 42 / 45 of three, 5376 x 16128, bf16, 100 tokens 115 / 111 us, but 45 / 45, 5760 x 17280, int8, 100 tokens 179 / 227; 52 /
+// 56 of five, 6656 x 19968, bf16, 24 tokens 139 / 137, but 56 / 56, 7168 x 21504, int8 122 / 145).  Clusters of up to 16 where they fit
+// are slower (512 x 1500, bf16, 24 tokens, 8 / 16: 19.4 / 20.4).
 bool umma_down_splits(int D, int R, int qbits, int cols, bool exact, int sm_count, int max_splits, int* splits, const int* at_once) {
   const int tiles = D >= kTileRows ? D / kTileRows : 1;
   const bool pairs = down_pairs(cols, exact);
   const int dev = at_once ? -1 : current_device();
   int cluster = kMaxDownCluster;
-  while (cluster > 1 && (at_once ? at_once[cluster] : down_clusters(dev, cluster, pairs)) < tiles) --cluster;
+  auto fits = [&](int size) {
+    const int most = at_once ? at_once[size] : down_clusters(dev, size, pairs);
+    return most >= tiles && (size % 2 == 0 || 15 * most >= 16 * tiles);
+  };
+  while (cluster > 1 && !fits(cluster)) --cluster;
   auto splits_of = [&](int ctas) {
     const int n = ctas / tiles;
     return n < 1 ? 1 : n > max_splits ? max_splits : n;

@@ -49,6 +49,19 @@ def test_clusters_for_lists_of_few_blocks(D, R, qbits, cols, exact, clustered):
     assert splits(D, R, qbits, cols, plenty, exact)[0] == clustered
 
 
+@pytest.mark.parametrize("tiles,cols,size,most,clustered", [
+    (42, 100, 3, 45, 1), (43, 100, 3, 45, 0), (45, 100, 3, 45, 0), (45, 100, 3, 48, 1),
+    (52, 24, 5, 56, 1), (54, 24, 5, 56, 0), (56, 24, 5, 56, 0),
+    (32, 100, 4, 33, 1), (32, 24, 8, 33, 1), (33, 100, 4, 33, 1),
+])
+def test_odd_clusters_need_room_to_spare(tiles, cols, size, most, clustered):
+    """As many clusters of an even size as the device takes, of an odd one 15 for every 16."""
+    got = splits(128 * tiles, 30000, 0, cols, lambda n: most if n == size else 0 if n > size else 296 // n)
+    assert got[0] == clustered
+    if clustered:
+        assert got[1] == size
+
+
 @pytest.mark.gpu
 def test_a_question_that_failed_is_asked_again():
     """Partials and the kernel that adds them up while the runtime has no answer, one launch less once it has."""
