@@ -2132,7 +2132,7 @@ static int down_clusters(int dev, int size, bool pairs) {
 // a kernel (4096 x 14336, bf16, partials / clusters: 200 tokens 108.3 / 101.2 us, 72 tokens 83.3 / 79.4, 16 tokens 62.9 / 61.6; 512 x
 // 1500, int8, 2 tokens 21.5 / 18.9), and costs splits where more CTAs would run than clusters fit the GPCs.  Clusters:
 // - where they cost up to a ninth of the splits (codes, whose blocks take longer: none): int8, 4096 x 14336, 8 tokens, nine splits /
-//   clusters of eight 44.6 / 45.1; bf16, 6144 x 20000, 160 tokens, three / two 229 / 242; exact sums, 2688 x 8000, 24 tokens, seven / six 78.5 / 80.2;
+//   clusters of eight 44.6 / 45.1; bf16, 6144 x 20000, 160 tokens, three / two 229 / 242;
 // - or any number of them where a CTA has few blocks.  A dozen where the list has codes, or the fired rows of up to eight tokens (2048 x
 //   6144, 16 / 8: int4, 2 / 24 / 64 tokens 26.7 / 36.9 / 50.7 against 24.4 / 37.6 / 49.0; bf16, 2 tokens 25.7 / 25.2; codes of 16 to 32
 //   tokens between 65 and 96 blocks: from 6 % slower to 4 % faster), else eight (bf16, 16 / 8, 63 blocks: 1024 x 3993, 16 / 32 / 64
@@ -2143,6 +2143,11 @@ static int down_clusters(int dev, int size, bool pairs) {
 // clusters: 42 / 45 of three, 5376 x 16128, bf16, 100 tokens 115 / 111 us, but 45 / 45, 5760 x 17280, int8, 100 tokens 179 / 227; 52 /
 // 56 of five, 6656 x 19968, bf16, 24 tokens 139 / 137, but 56 / 56, 7168 x 21504, int8 122 / 145).  Clusters of up to 16 where they fit
 // are slower (512 x 1500, bf16, 24 tokens, 8 / 16: 19.4 / 20.4).
+// Exact sums: three blocks a CTA, or six for up to 24 tokens (three columns each); their CTAs work longer on each block, and the sum has
+// less to hide (partials / clusters of eight: 384 x 1152, bf16, 6 / 64 tokens 34.4 / 59.2 against 31.7 / 59.1; 640 x 1920, 6 / 24 / 64
+// tokens 35.1 / 40.3 / 67.3 against 33.9 / 39.9 / 69.0; 896 x 2688, 64 / 256 tokens 77.6 / 320 against 81.3 / 336; 1152 x 3287, 13 tokens
+// 43.4 / 44.4; of three, 43 tiles: 5504 x 16512, 6 / 15 tokens 163 / 206 against 170 / 233).
+constexpr int kExactClusterCols = 72;
 bool umma_down_splits(int D, int R, int qbits, int cols, bool exact, int sm_count, int max_splits, int* splits, const int* at_once) {
   const int tiles = D >= kTileRows ? D / kTileRows : 1;
   const bool pairs = down_pairs(cols, exact);
@@ -2164,8 +2169,9 @@ bool umma_down_splits(int D, int R, int qbits, int cols, bool exact, int sm_coun
   // 20000 (102 and 255 CTAs) 312 / 301.
   if (exact && 10 * (two - 2 * one) >= one * two) n = two;
   const int blocks = (R + kAtomK - 1) / kAtomK;
-  const bool clustered = qbits ? cluster >= n : 9 * cluster >= 8 * n;
-  const int few = (qbits || exact || cols <= 8 ? 12 : 8) * cluster;
+  if (exact && n == 1) cluster = 1;
+  const bool clustered = exact ? n == 1 : qbits ? cluster >= n : 9 * cluster >= 8 * n;
+  const int few = (exact ? (cols <= kExactClusterCols ? 6 : 3) : qbits || cols <= 8 ? 12 : 8) * cluster;
   if (clustered || (cluster > 1 && blocks <= few)) {
     *splits = cluster;
     return true;

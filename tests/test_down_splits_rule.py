@@ -42,7 +42,9 @@ def test_without_an_answer_the_list_is_cut_into_partials():
     (1024, 64 * 64, 0, 24, 0, 1), (1024, 64 * 64 + 1, 0, 24, 0, 0),   # eight blocks a CTA
     (1024, 64 * 64 + 1, 0, 8, 0, 1), (1024, 96 * 64, 0, 8, 0, 1), (1024, 96 * 64 + 1, 0, 8, 0, 0),
     (1024, 96 * 64, 8, 64, 0, 1), (1024, 96 * 64, 4, 64, 0, 1), (1024, 96 * 64 + 1, 4, 64, 0, 0),
-    (640, 96 * 64, 0, 24, 1, 1),                                      # exact sums
+    (640, 48 * 64, 0, 72, 1, 1), (640, 48 * 64 + 1, 0, 72, 1, 0),     # exact sums
+    (640, 24 * 64, 0, 96, 1, 1), (640, 24 * 64 + 1, 0, 96, 1, 0),
+    (5504, 16512, 0, 24, 1, 0), (5504, 16512, 8, 120, 1, 0), (16512, 200, 0, 120, 1, 1),
 ])
 def test_clusters_for_lists_of_few_blocks(D, R, qbits, cols, exact, clustered):
     """Narrow rows, whose tiles leave room for more splits than a cluster has."""
