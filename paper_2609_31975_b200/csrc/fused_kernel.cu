@@ -560,11 +560,12 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
     }
     return;
   }
-  if (PAIR) {
-    // Nothing is computed yet, in this CTA or the other, which may write here once both have arrived.
-    for (int i = tid - kStageBase; i < 2 * p.slab_max; i += kStageThreads) row_state[i] = 0xffffffffu;
-    cluster_arrive();
-  }
+  // Nothing is computed yet, in this CTA or the other of a pair, which may write here once both have arrived.  (LoPA, alone: after the
+  // wait, beside the epoch's load.  Here it holds up what the vector's exchange waits for: six dependent layers of 512 x 1500, r = 64, fp32
+  // 69 -> 73.5 us, of 384 x 886, bf16 69 -> 72.5; the standard gate is faster so, one token, fp32, 2176 x 5182 16.0 -> 15.8.)
+  constexpr bool kLateStates = LOPA && !PAIR;
+  for (int i = tid - kStageBase; !kLateStates && i < (PAIR ? 2 : 1) * p.slab_max; i += kStageThreads) row_state[i] = 0xffffffffu;
+  if (PAIR) cluster_arrive();
 
   // The token itself may still be written by the predecessor, so it is not read before the wait -- but its lines can
   // be asked into L2 (a hint: whatever is written later lands in the same L2), which turns the staging loads right
@@ -607,10 +608,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_ffn_kernel(const FusedParam
   if (tid == kStageBase) SFFN_GSTAMP(11);
   // this call's number: the tag of the partials and of the LoPA exchange values
   const uint32_t ep = (LOPA || warp >= kFirstGateWarp) ? __ldcg(p.epoch_word) + 1u : 0u;
-  // (alone: here, beside the epoch's load; ahead of the wait, as pairs have to, it holds up what is asked for there: six dependent LoPA
-  // layers of 512 x 1500, fp32 69 -> 73.5 us, of 384 x 886, bf16 69 -> 72.5)
-  if (!PAIR)
-    for (int i = tid - kStageBase; i < slab_rows; i += kStageThreads) row_state[i] = 0xffffffffu;
+  for (int i = tid - kStageBase; kLateStates && i < slab_rows; i += kStageThreads) row_state[i] = 0xffffffffu;
   constexpr int XEPV = Elem<X>::kPerVec;  // token elements per 16 bytes (the weights' EPV unless those are int8)
   // Quantised rows under a standard gate: the token is also split, 16 (int8) or 32 (int4) entries at a time -- the
   // entries one 16-byte chunk of a row meets -- into two int8 limbs and one scale per chunk:
