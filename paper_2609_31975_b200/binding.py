@@ -49,10 +49,10 @@ _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda i:
 _lib = None
 # The environment as this process began with it, where it keeps its variables, and how it writes the one that every call looks at:
 # os.environ.get encodes the name, and raises and catches an exception for a variable that is not set, 0.55 us of the 8 that a call
-# on a small model takes.  A program that puts another mapping in os.environ's place is asked the usual way.
+# on a small model takes, so it is asked only where the variable is there or a program has put another mapping in os.environ's place.
 _environ = os.environ if isinstance(getattr(os.environ, "_data", None), dict) else None
 _variables = _environ._data if _environ is not None else {}
-_SYNC_CHECK, _ON = (_environ.encodekey("SFFN_SYNC_CHECK"), _environ.encodevalue("1")) if _environ is not None else ("", "1")
+_SYNC_CHECK = _environ.encodekey("SFFN_SYNC_CHECK") if _environ is not None else ""
 
 
 def load_library() -> ctypes.CDLL:
@@ -281,7 +281,7 @@ class SparseFFN:
                 ACT[act] if isinstance(act, str) else int(act), _addr(y), self._stream(stream))
         if rc:
             raise SFFNError(name, rc)
-        if _variables.get(_SYNC_CHECK) == _ON if os.environ is _environ else os.environ.get("SFFN_SYNC_CHECK") == "1":
+        if (_SYNC_CHECK in _variables or os.environ is not _environ) and os.environ.get("SFFN_SYNC_CHECK") == "1":
             self._sync_check(name, B, gate)
         return y
 
