@@ -667,8 +667,8 @@ int run(sffn_handle* h, const void* x, int B, const sffn_gate* g, const float* b
   // A batch the tensor-core kernels can take: bf16 tokens; bf16, int8 or int4 rows of a multiple of 256 elements, or of
   // 128 from a few tokens on (see h_terms_for and odd_width_tokens); a LoPA rank of a multiple of 64.
   // Larger batches are cut into passes of as many tokens as one launch chain holds: a pass reads every gate row and the
-  // rows of its own union, so fewer passes read fewer bytes (bf16, 4096 x 14336, 200 tokens: 4 passes of 64 took 333 us, one
-  // takes 100).  The mma.sync kernels (selected, or a bf16 LoPA rank that is no multiple of 64) take passes of 64 and rows
+  // rows of its own union, so fewer passes read fewer bytes (bf16, 4096 x 14336, 200 tokens, short runs: 4 passes of 64 took 333 us,
+  // one takes 100).  The mma.sync kernels (selected, or a bf16 LoPA rank that is no multiple of 64) take passes of 64 and rows
   // of a multiple of 256 elements.
   const bool umma_ok = h->path != SFFN_PATH_MMA_SYNC && sffn::umma_rows_supported(gate_k, 1) &&
                        sffn::umma_rows_supported(h->D, 1) && sffn::umma_down_supported(h->D, 1) &&

@@ -36,7 +36,7 @@
 // Up to 256 token columns go through in one pass.  Wide batches (npad > 128) leave room for two accumulators and a ring
 // of four stages of ~40 KB (two with expanded codes and 241 columns or more), too few for the token rows that every CTA reads again
 // (200 tokens x 4096: 1.6 MB a CTA through L2 beside 0.8 MB of weights).  There the rows kernels run in pairs of CTAs that hold half
-// of the token rows each (PAIR, see umma_rows_pairs): 200 tokens, 4096 x 14336, bf16: 130 us without pairs, 112 with them.
+// of the token rows each (PAIR, see umma_rows_pairs).  200 tokens, 4096 x 14336, bf16: 100 us in one pass (short runs), 333 in four.
 // Every wait is bounded by a cycle budget; on expiry the status word is set, all roles wind down and the TMEM
 // columns are released before the CTA exits.
 #include "umma_kernels.cuh"
@@ -2055,6 +2055,9 @@ void umma_k_splits(int R, int K, bool codes, int B, int sm_count, int max_splits
 // With six slots nothing is gained (4096 x 14336, 160 tokens 99.9 / 100.7; 2048 x 6000, 200 tokens 59.7 / 61.6), and the clusters
 // cost a kernel 0.5 to 1 us (1024 x 3000, 72 tokens 29.7 / 33.3).  Codes that are expanded stay alone (int4, 4096 x 14336, 64
 // tokens 97.5 / 112: two CTAs' expansions to wait for).
+// The up projection goes by R, as the list's length is known on the device alone: time alone over time in pairs, Zipf firing, bf16 176 to
+// 256 and int8 40 to 64 tokens, 1024 to 8192 columns, at 10 / 3 / 1.5 / 0.5 / 0.1 % firing 0.98-1.09 / 0.98-1.09 / 0.96-1.13 /
+// 0.96-1.10 / 0.92-1.01.
 bool umma_rows_pairs(int R, int K, int qbits, int B, int cols, bool exact, int sm_count) {
   if (exact || qbits > 1 || sm_count % 2) return false;
   int tile_rows, n_tiles;
@@ -2129,7 +2132,7 @@ static int down_clusters(int dev, int size, bool pairs) {
 }
 
 // Splits of the list, and whether they are a cluster that adds its sums up itself.  That saves the partials' way through memory and
-// a kernel (4096 x 14336, bf16, partials / clusters: 200 tokens 108.3 / 101.2 us, 72 tokens 83.3 / 79.4, 16 tokens 62.9 / 61.6; 512 x
+// a kernel (4096 x 14336, bf16, short runs, partials / clusters: 200 tokens 108.3 / 101.2 us, 72 tokens 83.3 / 79.4, 16 tokens 62.9 / 61.6; 512 x
 // 1500, int8, 2 tokens 21.5 / 18.9), and costs splits where more CTAs would run than clusters fit the GPCs.  Clusters:
 // - where they cost up to a ninth of the splits (codes, whose blocks take longer: none): int8, 4096 x 14336, 8 tokens, nine splits /
 //   clusters of eight 44.6 / 45.1; bf16, 6144 x 20000, 160 tokens, three / two 229 / 242;
