@@ -349,7 +349,7 @@ const char* sffn_status_string(int status);
  *   CLUSTER_QUERY_FAILS 1 = the runtime has no answer to how many clusters of CTAs the device runs at once: the kernels that
  *                       have to know take the form without them (default 0)
  *   PAIRS               1 / 0: single-token LoPA calls go to the kernel of pairs of CTAs wherever it can run them / nowhere;
- *                       -1 (the default): by their sizes
+ *                       -1 (the default): sparse calls by their sizes, dense ones nowhere
  *   TRACE_BUFFER        device address of [grid][16] int64 time stamps, written only by libraries built with
  *                       -DSFFN_TRACE (0 = none) */
 typedef enum {

@@ -1912,18 +1912,19 @@ int pairs_at_once() {
 //   to 1.0 / 1.0 to 1.03 / 0.99 to 1.015; 55 of 4096, r = 256: 0.95.
 // - Eight gate rows or more to a row (kGateRows): above that the gate is what a call waits for.  At 10 % firing, r = D / 8 / D / 7.5 /
 //   D / 7: fp32, 3840 x 14230 1.026 / 1.030 / 0.984, 3456 x 13000 1.049 / 1.035 / 1.018; bf16, 8192 x 28000 1.022 / 0.991 / 1.006.
+// Dense calls, which do every row, have nothing to even out (4096 x 14336, fp32, r = 512 87.8 alone, 90.2 in pairs).
 // Times alone / in pairs at 30 / 10 / 3 % firing: fp32, 4096 x 13926, r = 512 44.4 / 27.9 / 20.6 -> 42.5 / 26.8 / 21.3 us, r = 256 44.2 /
 // 27.8 / 18.6 -> 42.9 / 26.3 / 19.0; bf16, 8192 x 27852, r = 1024 78.2 / 44.5 / 38.9 -> 72.2 / 43.7 / 39.4; eight layers of fp32, 3840 x
 // 14230, r = 480, at 10 %: 229 -> 216.
 constexpr int kLongRow = 15 * 1024, kLongShare = 80, kGateRows = 8;
-bool in_pairs(const Geometry& g, int wkind, int D, int H, int K, int grid, int at_once, int* smem) {
+bool in_pairs(const Geometry& g, int wkind, int D, int H, int K, bool dense, int grid, int at_once, int* smem) {
   const int knob = fused_test_knobs().pairs;
   if (knob == 0 || (wkind != kWBF16 && wkind != kWF32) || grid % 2 || g.cpt != 8) return false;
   const int row_bytes = D * 16 / weight_epv(wkind), gate_row_bytes = K * 16 / weight_epv(wkind);
   const SmemLayout with(D, K, true, g.n_gate_slots, g.gate_slot_bytes, g.n_act_slots, g.act_slot_bytes, g.slab_max, false, g.act_extra,
                         false, false, true);
   if (with.total > kSmemBudget) return false;
-  if (knob < 0 && (row_bytes < kLongRow || H < kLongShare * grid || row_bytes < kGateRows * gate_row_bytes)) return false;
+  if (knob < 0 && (dense || row_bytes < kLongRow || H < kLongShare * grid || row_bytes < kGateRows * gate_row_bytes)) return false;
   if (at_once < 0) at_once = wkind == kWBF16 ? pairs_at_once<__nv_bfloat16>() : pairs_at_once<float>();
   if (2 * at_once < grid) return false;
   *smem = with.total;
@@ -1981,7 +1982,7 @@ void debug_fused_plan(int wkind, int D, int H, int K, bool lopa, int sm_count, i
 bool debug_fused_pairs(int wkind, int D, int H, int r, int sm_count, int at_once) {
   const int grid = fused_grid(sm_count, H);
   Geometry g = plan(wkind, D, H, r, true, grid);
-  return g.ok && in_pairs(g, wkind, D, H, r, grid, at_once, &g.smem);
+  return g.ok && in_pairs(g, wkind, D, H, r, false, grid, at_once, &g.smem);
 }
 
 // Whether this call's gate goes to the tensor cores (see sffn_set_gate_engine).
@@ -2019,7 +2020,7 @@ cudaError_t launch_fused(const FusedCall& c, cudaStream_t s, int* launched) {
     if (with.total <= kSmemBudget) g.smem = with.total;
     else gated = false;
   }
-  const bool pairs = lopa && in_pairs(g, c.wkind, c.D, c.H, K, grid, -1, &g.smem);
+  const bool pairs = lopa && in_pairs(g, c.wkind, c.D, c.H, K, c.dense, grid, -1, &g.smem);
   char* ws = static_cast<char*>(c.workspace);
   int n = 0;
   cudaError_t e;

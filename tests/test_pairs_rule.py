@@ -55,3 +55,29 @@ def test_without_an_answer_a_call_goes_alone():
         m.test_set_knob("cluster_query_fails", 0)
     assert torch.equal(y[0], y[2])
     assert (y[0] - y[1]).norm() <= 1e-5 * y[0].norm()  # sums of some 700 terms in another order
+
+
+@pytest.mark.gpu
+def test_dense_calls_go_alone():
+    """Every row is done: nothing to even out between two CTAs."""
+    import paper_2609_31975_b200 as m
+    import synthetic_inputs as syn
+    import torch
+
+    D, H, r = 3840, 12000, 256
+    w = syn.lopa_ffn(D, H, r, torch.float32, 99, "cuda:0")
+    gate = {"V": w["V"], "U": w["U"], "g_idx": m.g_diagonal(H, D, "cuda:0")}
+    x = syn.tokens(1, D, torch.float32, 99, "cuda:0")[0]
+    ffn = m.SparseFFN(D, H, torch.float32, r_max=r, B_max=1)
+    assert in_pairs(0, D, H, r, torch.cuda.get_device_properties(0).multi_processor_count)
+    y = {}
+    try:
+        for knob in (-1, 0, 1):
+            m.test_set_knob("pairs", knob)
+            y[knob] = ffn.dense_ffn_forward(x, gate, w["b_g"], w["W_up"], w["W_down"], "relu").clone()
+    finally:
+        m.test_set_knob("pairs", -1)
+    torch.cuda.synchronize()
+    assert ffn.device_status() == 0
+    assert torch.equal(y[-1], y[0]) and not torch.equal(y[1], y[0])  # sums of 12000 rows in another order
+    assert (y[1] - y[0]).norm() <= 1e-5 * y[0].norm()
