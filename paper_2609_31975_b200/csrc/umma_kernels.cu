@@ -188,10 +188,17 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-__device__ __forceinline__ void cluster_sync() {
+__device__ __forceinline__ void cluster_arrive() {
   __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+  cluster_arrive();
+  cluster_wait();
 }
 // The address, in the cluster's window, of this CTA's shared-memory address in the CTA of rank `rank`.
 __device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
@@ -1622,13 +1629,17 @@ __global__ void __launch_bounds__(down_bound(QB, EX), EX ? 1 : 2) umma_down_kern
   if (*abort_flag)
     for (int i = 0; i < 50; ++i) __nanosleep(1000);
   tc_fence_before();
-  if (clustered) cluster_sync();
-  else __syncthreads();
+  // The TMEM goes back before this CTA waits for the others of its cluster.  A CTA whose allocation waits for columns waits without a
+  // limit, for a CTA of another stream's call that holds them on its SM; were that one waiting for its own cluster meanwhile, whose
+  // other CTA may be the one that cannot allocate on the next SM, neither would ever go on.
+  if (clustered) cluster_arrive();
+  __syncthreads();
   if (warp == 8) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
   }
   if (!clustered) return;
+  cluster_wait();
   // a warp takes a token at a time, a lane four columns of it
   const int n_warps = blockDim.x >> 5;
   const uint32_t at = smem_u32(sums) + lane * 16;

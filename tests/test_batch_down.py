@@ -84,3 +84,27 @@ def test_nothing_fires(D, B):
     y = ffn.sparse_ffn_forward(syn.tokens(B, D, torch.bfloat16, 87, DEV), {"W_g": w["W_g"]}, w["b_g"] - 100.0, w["W_up"], w["W_down"], "relu")
     torch.cuda.synchronize()
     assert ffn.device_status() == 0 and not y.any() and len(ffn.last_active()) == 0
+
+
+@pytest.mark.gpu
+def test_batches_of_two_streams_share_sms():
+    """Clusters of two calls whose CTAs fit an SM together but for the tensor memory of one that has it all: each as if alone."""
+    import paper_2609_31975_b200 as m
+
+    calls, want = [], []
+    for D, H, B in ((256, 300, 200), (512, 700, 33), (256, 500, 256), (512, 300, 16)):
+        w = syn.standard_ffn(D, H, torch.bfloat16, 88, DEV, sparsity=0.8)
+        ffn = m.SparseFFN(D, H, torch.bfloat16, B_max=B)
+        x = syn.tokens(B, D, torch.bfloat16, 88, DEV)
+        y = torch.empty(B, D, dtype=torch.float32, device=DEV)
+        calls.append((ffn, (x, {"W_g": w["W_g"]}, w["b_g"], w["W_up"], w["W_down"], "relu", y)))
+        want.append(ffn.sparse_ffn_forward(*calls[-1][1]).clone())
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in calls]
+    for _ in range(200):
+        for (ffn, args), stream in zip(calls, streams):
+            ffn.sparse_ffn_forward(*args, stream=stream)
+    torch.cuda.synchronize()
+    for (ffn, args), y in zip(calls, want):
+        assert ffn.device_status() == 0
+        assert torch.equal(args[-1], y)
