@@ -1344,7 +1344,10 @@ __global__ void __launch_bounds__(kThreadsRows + (EX ? 128 : 0) + ((QB == 8 || Q
 // Threads, rounded up to whole warps for each scheduler: registers are handed out by scheduler, and two CTAs of 14 warps with 72
 // registers a thread, which fit an SM's file, do not fit those of the first two (int4 rows ran in two waves of CTAs).
 constexpr int down_bound(int qb, bool exact) { return ((exact ? 512 : kThreads) + (qb ? 32 * kExpandWarps : 0) + 127) / 128 * 128; }
-template <int QB, bool EX = false, bool TWO = false>
+// CL: calls whose splits may be clusters.  Exact sums of codes, whose kernel fills its registers and spills a few, have another one without
+// that code for the calls that have none (LoPA gate, 7296 x 21888, 39 / 64 tokens, with / without: int8 495 / 864 -> 487 / 851 us, int4 488 /
+// 851 -> 480 / 837; bf16 rows, which spill nothing, are 2 % slower so: 746 -> 756).
+template <int QB, bool EX = false, bool TWO = false, bool CL = true>
 __global__ void __launch_bounds__(down_bound(QB, EX), EX ? 1 : 2) umma_down_kernel(const UmmaDownParams p,
                                                                   const __grid_constant__ CUtensorMap map_wg,
                                                                   const __grid_constant__ CUtensorMap map_wt,
@@ -1375,7 +1378,7 @@ __global__ void __launch_bounds__(down_bound(QB, EX), EX ? 1 : 2) umma_down_kern
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int d_tiles = p.D / kTileRows;
-  const bool clustered = p.y != nullptr;  // the splits of a tile are one cluster
+  const bool clustered = CL && p.y != nullptr;  // the splits of a tile are one cluster
   const int dt = clustered ? blockIdx.x / p.splits : blockIdx.x % d_tiles, sp = clustered ? blockIdx.x % p.splits : blockIdx.x / d_tiles;
   const int d0 = dt * kTileRows;
 
@@ -2197,13 +2200,13 @@ bool umma_down_splits(int D, int R, int qbits, int cols, bool exact, int sm_coun
 bool umma_down_supported(int D, int cols) { return D % kTileRows == 0 && cols >= 1 && cols <= kUmmaMaxCols; }
 
 namespace {
-template <int QB, bool EX = false, bool TWO = false>
+template <int QB, bool EX = false, bool TWO = false, bool CL = true>
 cudaError_t launch_down_q(const UmmaDownParams& p, int grid, size_t smem, cudaStream_t s, const CUtensorMap& map_wg,
                           const CUtensorMap& map_wt, const CUtensorMap& map_hm) {
   static unsigned long long configured = 0;
-  const cudaError_t e = allow_dynamic_smem(umma_down_kernel<QB, EX, TWO>, 227 * 1024, configured);
+  const cudaError_t e = allow_dynamic_smem(umma_down_kernel<QB, EX, TWO, CL>, 227 * 1024, configured);
   if (e != cudaSuccess) return e;
-  return launch_clusters(p.y ? p.splits : 1, umma_down_kernel<QB, EX, TWO>, dim3(grid), dim3((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarps : 0)), smem, s, p, map_wg,
+  return launch_clusters(p.y ? p.splits : 1, umma_down_kernel<QB, EX, TWO, CL>, dim3(grid), dim3((EX ? 512 : kThreads) + (QB ? 32 * kExpandWarps : 0)), smem, s, p, map_wg,
                     map_wt, map_hm);
 }
 }  // namespace
@@ -2257,9 +2260,11 @@ cudaError_t launch_umma_down(UmmaDownParams p, cudaStream_t s) {
   if (!make_map(&map_hm, p.hmT, p.hm_stride, p.terms * p.h_cols, (size_t)p.hm_stride, p.cols)) return cudaErrorNotSupported;
   const int g = grid;
   if (p.exact)
-    return p.qbits == 8   ? launch_down_q<8, true>(p, g, smem, s, map_wg, map_wt, map_hm)
-           : p.qbits == 4 ? launch_down_q<4, true>(p, g, smem, s, map_wg, map_wt, map_hm)
-                          : launch_down_q<0, true>(p, g, smem, s, map_wg, map_wt, map_hm);
+    return p.qbits == 0 ? launch_down_q<0, true>(p, g, smem, s, map_wg, map_wt, map_hm)
+           : p.qbits == 8
+               ? p.y ? launch_down_q<8, true>(p, g, smem, s, map_wg, map_wt, map_hm) : launch_down_q<8, true, false, false>(p, g, smem, s, map_wg, map_wt, map_hm)
+           : p.y ? launch_down_q<4, true>(p, g, smem, s, map_wg, map_wt, map_hm)
+                 : launch_down_q<4, true, false, false>(p, g, smem, s, map_wg, map_wt, map_hm);
   if (two)
     return p.qbits == 8 ? launch_down_q<8, false, true>(p, g, smem, s, map_wg, map_wt, map_hm)
                         : launch_down_q<4, false, true>(p, g, smem, s, map_wg, map_wt, map_hm);
